@@ -1,4 +1,6 @@
-// FP64 GEMM for the plain double-precision form of the OMM CG step.
+// FP64 GEMM on the CUDA cores: omm_op_dgemm (which has no workspace), the FP64
+// refinement of the mixed form, and dense FP64 handles too large for residue planes
+// (crt.cu, 4 to 33 times faster from m = 144 to 1996 and no slower at m = 8).
 //
 // GB300 executes FP64 on its CUDA cores only (no FP64 tensor-core kind in
 // tcgen05), at a small fraction of the BF16 tensor rate, so this kernel is

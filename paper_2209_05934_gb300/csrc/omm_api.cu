@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "chol.cuh"
+#include "crt.cuh"
 #include "omm_internal.cuh"
 #include "sparse.cuh"
 #include "tc_exact.cuh"
@@ -67,6 +68,25 @@ struct ExactBufs {
     CUtensorMap mapHS_A, mapW, mapHWSW_B, mapSWHW_A, mapHSW_B;
 };
 
+// Residue planes of the FP64 form's products (crt.cu; 16 planes, row-scaled), each
+// with its per-row exponents:
+//   HSr   [16][2m][ldm]  rows of [H' ; S]         A of H'D, SD (and H'W, SW)
+//   WDr   [16][2n][ldm]  columns of [W | D]       B of those; A of Z
+//   HDSDr [16][2n][ldm]  columns of [H'D | SD]    B of Z (start: [SW | H'W])
+//   SWHWr [16][m][ld2n]  rows of [SW | H'W]       A of the gradient
+//   HSWr  [16][n][ld2n]  columns of [H_W ; S_W]   B of the gradient
+// words: the residue planes of a product; part: partial row norms.
+struct CrtBufs {
+    int64_t ldm = 0, ld2n = 0;
+    __nv_bfloat16 *HSr = nullptr, *WDr = nullptr, *HDSDr = nullptr, *SWHWr = nullptr, *HSWr = nullptr;
+    __nv_bfloat16 *Pr = nullptr, *Gr = nullptr;   // preconditioner: rows of P, columns of G
+    int *e = nullptr;
+    int *eHS = nullptr, *eWD = nullptr, *eHDSD = nullptr, *eSWHW = nullptr, *eHSW = nullptr, *eP = nullptr, *eG = nullptr;
+    float2 *part = nullptr;
+    uint32_t *words = nullptr;
+    CUtensorMap mapHS, mapWD, mapHDSD, mapSWHW, mapHSW, mapP, mapG;
+};
+
 // Device copy of a persistent tile list (one problem) of a handle's split product.
 struct HandleList {
     omm::tc::TileProblem *probs = nullptr;
@@ -108,6 +128,7 @@ struct omm_handle {
     int graph_eager[kPhases] = {};
     MixedBufs mx;
     ExactBufs ex;
+    CrtBufs cr;               // FP64 form on the tensor cores (cr.words == nullptr: CUDA-core products)
     HandleList lists[3];      // persistent tile lists of the step's split products (gemm_persistent)
     double *L = nullptr;      // Cholesky variant: factor of S (m x m)
     double *Wsave = nullptr;  // Cholesky variant: W in the original basis (m x n)
@@ -154,6 +175,13 @@ int dalloc(T **p, size_t count) {
     return OMM_OK;
 }
 
+void crt_free(CrtBufs &c) {
+    for (void *p : {(void *)c.HSr, (void *)c.WDr, (void *)c.HDSDr, (void *)c.SWHWr, (void *)c.HSWr, (void *)c.Pr,
+                    (void *)c.Gr, (void *)c.e, (void *)c.part, (void *)c.words})
+        cudaFree(p);
+    c = CrtBufs{};
+}
+
 void free_handle(omm_handle *h) {
     if (h == nullptr) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
@@ -189,6 +217,7 @@ void free_handle(omm_handle *h) {
     cudaFree(h->ex.SWHWx);
     cudaFree(h->ex.HSWx);
     cudaFree(h->ex.e);
+    crt_free(h->cr);
     cudaFree(h->L);
     cudaFree(h->Wsave);
     cudaFree(h->S0);
@@ -275,8 +304,6 @@ double *scr(omm_handle *h, int i) {
     return h->scratch + (int64_t)i * omm::kRedBlocksMax * omm::kRedSlots;
 }
 
-// One CG step of the dense FP64 form (products, contractions, line search,
-// update, energy + convergence, gradient, direction).
 // Cholesky variant: the overlap of the reduced problem is I, so S D = D and
 // S W = W are copies, not products.
 bool s_identity(const omm_handle *h) { return h->opt.cholesky != 0 && !h->sparse; }
@@ -284,6 +311,64 @@ bool s_identity(const omm_handle *h) { return h->opt.cholesky != 0 && !h->sparse
 // electron pairs counted in the energy's 2 eta n_occ term: n, or fewer with the
 // Kim functional's extra columns
 int64_t n_occ(const omm_handle *h) { return h->opt.n_occupied > 0 ? h->opt.n_occupied : h->n; }
+
+// ---------------------------------------------------------------- FP64 form
+// The products run on the tensor cores through residue planes (crt.cu) where the
+// handle holds them, else on the CUDA cores (dense_fp64.cu).
+bool crt_on(const omm_handle *h) { return h->cr.words != nullptr; }
+
+omm::crt::Args crt_args(omm_handle *h, int64_t M, int64_t N, int64_t K) {
+    omm::crt::Args a{};
+    a.M = (int)M;
+    a.N = (int)N;
+    a.K = (int)K;
+    a.alpha = 1.0;
+    a.words = h->cr.words;
+    a.state = h->dstate;
+    a.err = &h->dstate->wait_timeout;
+    return a;
+}
+
+// C, C + c_step <- [H' ; S] B (S: omitted for the Cholesky variant) for the n packed
+// columns b_row0.. of [W | D]
+int crt_products(omm_handle *h, int b_row0, double *C, int64_t c_step) {
+    const int64_t m = h->m, n = h->n;
+    CrtBufs &c = h->cr;
+    omm::crt::Args a = crt_args(h, m, n, m);
+    a.a_row_step = (int)m;
+    a.b_row0 = b_row0;
+    a.C = C;
+    a.ldc = m;
+    a.c_step = c_step;
+    a.eA = c.eHS;
+    a.eA_step = m;
+    a.eB = c.eWD + b_row0;
+    return omm::crt::gemm(c.mapHS, c.mapWD, a, s_identity(h) ? 1 : 2, h->stream);
+}
+
+// G = 4 H'W - 2 [SW H'W][H_W ; S_W]
+int dense_gradient(omm_handle *h) {
+    const int64_t m = h->m, n = h->n, mn = m * n;
+    cudaStream_t st = h->stream;
+    if (crt_on(h)) {
+        CrtBufs &c = h->cr;
+        TRY(omm::crt::pack_rows(m, 2 * n, h->SWHW, m, c.eSWHW, c.part, c.SWHWr, c.ld2n, m * c.ld2n, false, h->dstate, st));
+        TRY(omm::crt::pack_cols(2 * n, n, h->h0s0, 2 * n, c.eHSW, c.HSWr, c.ld2n, n * c.ld2n, true, h->dstate, st));
+        omm::crt::Args a = crt_args(h, m, n, 2 * n);
+        a.alpha = -2.0;
+        a.beta = 4.0;
+        a.Cin = h->SWHW + mn;
+        a.ldcin = m;
+        a.C = h->G;
+        a.ldc = m;
+        a.eA = c.eSWHW;
+        a.eB = c.eHSW;
+        return omm::crt::gemm(c.mapSWHW, c.mapHSW, a, 1, st);
+    }
+    omm::GemmBatch g{};
+    g.A[0] = h->SWHW; g.B[0] = h->h0s0; g.Cin[0] = h->SWHW + mn; g.C[0] = h->G;
+    return omm::dgemm_batched(false, false, m, n, 2 * n, -2.0, g, 1, m, 2 * n, 4.0, m, m, h->dstate, st);
+}
 
 // CG dots, beta and direction of the dense FP64 form; with the kinetic-energy
 // preconditioner the gradient is first multiplied by P (Eq. 6): Z = P G.
@@ -293,9 +378,20 @@ int dense_direction(omm_handle *h, int first) {
     const double *Zg = h->G;
     if (h->precon_on) {
         StageTimer t(h, OMM_STAGE_PRECON);
-        omm::GemmBatch p{};
-        p.A[0] = h->P; p.B[0] = h->G; p.C[0] = h->PG; p.Cin[0] = nullptr;
-        TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, p, 1, m, m, 0.0, m, m, h->dstate, st));
+        if (crt_on(h)) {
+            CrtBufs &c = h->cr;
+            TRY(omm::crt::pack_cols(m, n, h->G, m, c.eG, c.Gr, c.ldm, n * c.ldm, false, h->dstate, st));
+            omm::crt::Args a = crt_args(h, m, n, m);
+            a.C = h->PG;
+            a.ldc = m;
+            a.eA = c.eP;
+            a.eB = c.eG;
+            TRY(omm::crt::gemm(c.mapP, c.mapG, a, 1, st));
+        } else {
+            omm::GemmBatch p{};
+            p.A[0] = h->P; p.B[0] = h->G; p.C[0] = h->PG; p.Cin[0] = nullptr;
+            TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, p, 1, m, m, 0.0, m, m, h->dstate, st));
+        }
         Zg = h->PG;
     }
     StageTimer t(h, OMM_STAGE_DIRECTION);
@@ -307,20 +403,41 @@ int dense_iteration(omm_handle *h) {
     const int64_t m = h->m, n = h->n, mn = m * n;
     cudaStream_t st = h->stream;
     omm::DevState *s = h->dstate;
-    omm::GemmBatch b{};
     // H'D and S D
-    b.A[0] = h->HS;          b.B[0] = h->WD + mn; b.C[0] = h->HDSD;      b.Cin[0] = nullptr;
-    b.A[1] = h->HS + m * m;  b.B[1] = h->WD + mn; b.C[1] = h->HDSD + mn; b.Cin[1] = nullptr;
     {
         StageTimer t(h, OMM_STAGE_PRODUCTS);
-        TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, b, s_identity(h) ? 1 : 2, m, m, 0.0, m, m, s, st));
+        if (crt_on(h)) {
+            // residues of W and D: D is the products' operand, both are the contraction's
+            CrtBufs &c = h->cr;
+            TRY(omm::crt::pack_cols(m, 2 * n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, s, st));
+            TRY(crt_products(h, (int)n, h->HDSD, mn));
+        } else {
+            omm::GemmBatch b{};
+            b.A[0] = h->HS;          b.B[0] = h->WD + mn; b.C[0] = h->HDSD;      b.Cin[0] = nullptr;
+            b.A[1] = h->HS + m * m;  b.B[1] = h->WD + mn; b.C[1] = h->HDSD + mn; b.Cin[1] = nullptr;
+            TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, b, s_identity(h) ? 1 : 2, m, m, 0.0, m, m, s, st));
+        }
         if (s_identity(h))
             OMM_CUDA_TRY(cudaMemcpyAsync(h->HDSD + mn, h->WD + mn, mn * sizeof(double), cudaMemcpyDeviceToDevice, st));
     }
     // Z = [W D]^T [H'D SD]
-    omm::GemmBatch z{};
-    z.A[0] = h->WD; z.B[0] = h->HDSD; z.C[0] = h->Z;
-    { StageTimer t(h, OMM_STAGE_CONTRACT); TRY(omm::dgemm_batched(true, false, 2 * n, 2 * n, m, 1.0, z, 1, m, m, 0.0, 2 * n, 2 * n, s, st)); }
+    {
+        StageTimer t(h, OMM_STAGE_CONTRACT);
+        if (crt_on(h)) {
+            CrtBufs &c = h->cr;
+            TRY(omm::crt::pack_cols(m, 2 * n, h->HDSD, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, s, st));
+            omm::crt::Args a = crt_args(h, 2 * n, 2 * n, m);
+            a.C = h->Z;
+            a.ldc = 2 * n;
+            a.eA = c.eWD;
+            a.eB = c.eHDSD;
+            TRY(omm::crt::gemm(c.mapWD, c.mapHDSD, a, 1, st));
+        } else {
+            omm::GemmBatch z{};
+            z.A[0] = h->WD; z.B[0] = h->HDSD; z.C[0] = h->Z;
+            TRY(omm::dgemm_batched(true, false, 2 * n, 2 * n, m, 1.0, z, 1, m, m, 0.0, 2 * n, 2 * n, s, st));
+        }
+    }
     // quartic coefficients and its minimum
     { StageTimer t(h, OMM_STAGE_LINESEARCH);
       TRY(omm::launch_coeffs_linemin((int)n, h->h0s0, h->h0s0 + n, 2 * n, h->Z, 2 * n, scr(h, 0),
@@ -332,9 +449,7 @@ int dense_iteration(omm_handle *h) {
       TRY(omm::launch_nn_update_energy((int)n, h->h0s0, h->h0s0 + n, 2 * n, h->Z, 2 * n, scr(h, 1),
                                        ctr(h, 1), s, 0, st)); }
     // G = 4 H'W - 2 [SW H'W][H_W ; S_W]
-    omm::GemmBatch g{};
-    g.A[0] = h->SWHW; g.B[0] = h->h0s0; g.Cin[0] = h->SWHW + mn; g.C[0] = h->G;
-    { StageTimer t(h, OMM_STAGE_GRADIENT); TRY(omm::dgemm_batched(false, false, m, n, 2 * n, -2.0, g, 1, m, 2 * n, 4.0, m, m, s, st)); }
+    { StageTimer t(h, OMM_STAGE_GRADIENT); TRY(dense_gradient(h)); }
     return dense_direction(h, 0);
 }
 
@@ -342,24 +457,92 @@ int dense_start(omm_handle *h) {
     const int64_t m = h->m, n = h->n, mn = m * n;
     cudaStream_t st = h->stream;
     omm::DevState *s = h->dstate;
-    omm::GemmBatch b{};
     // SW = S W, H'W = H' W
-    b.A[0] = h->HS;         b.B[0] = h->WD; b.C[0] = h->SWHW + mn;
-    b.A[1] = h->HS + m * m; b.B[1] = h->WD; b.C[1] = h->SWHW;
-    TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, b, s_identity(h) ? 1 : 2, m, m, 0.0, m, m, s, st));
+    if (crt_on(h)) {
+        CrtBufs &c = h->cr;
+        TRY(omm::crt::pack_cols(m, n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, s, st));
+        TRY(crt_products(h, 0, h->SWHW + mn, -mn));
+    } else {
+        omm::GemmBatch b{};
+        b.A[0] = h->HS;         b.B[0] = h->WD; b.C[0] = h->SWHW + mn;
+        b.A[1] = h->HS + m * m; b.B[1] = h->WD; b.C[1] = h->SWHW;
+        TRY(omm::dgemm_batched(false, false, m, n, m, 1.0, b, s_identity(h) ? 1 : 2, m, m, 0.0, m, m, s, st));
+    }
     if (s_identity(h))
         OMM_CUDA_TRY(cudaMemcpyAsync(h->SWHW, h->WD, mn * sizeof(double), cudaMemcpyDeviceToDevice, st));
     // H_W = W^T H'W, S_W = W^T S W
-    omm::GemmBatch c{};
-    c.A[0] = h->WD; c.B[0] = h->SWHW + mn; c.C[0] = h->h0s0;
-    c.A[1] = h->WD; c.B[1] = h->SWHW;      c.C[1] = h->h0s0 + n;
-    TRY(omm::dgemm_batched(true, false, n, n, m, 1.0, c, 2, m, m, 0.0, 2 * n, 2 * n, s, st));
+    if (crt_on(h)) {
+        CrtBufs &c = h->cr;
+        TRY(omm::crt::pack_cols(m, 2 * n, h->SWHW, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, s, st));
+        omm::crt::Args a = crt_args(h, n, n, m);
+        a.b_row0 = (int)n;          // z = 0: H'W -> rows [0, n) of h0s0;  z = 1: SW -> rows [n, 2n)
+        a.b_row_step = -(int)n;
+        a.C = h->h0s0;
+        a.ldc = 2 * n;
+        a.c_step = n;
+        a.eA = c.eWD;
+        a.eB = c.eHDSD + n;
+        a.eB_step = -n;
+        TRY(omm::crt::gemm(c.mapWD, c.mapHDSD, a, 2, st));
+    } else {
+        omm::GemmBatch c{};
+        c.A[0] = h->WD; c.B[0] = h->SWHW + mn; c.C[0] = h->h0s0;
+        c.A[1] = h->WD; c.B[1] = h->SWHW;      c.C[1] = h->h0s0 + n;
+        TRY(omm::dgemm_batched(true, false, n, n, m, 1.0, c, 2, m, m, 0.0, 2 * n, 2 * n, s, st));
+    }
     TRY(omm::launch_nn_update_energy((int)n, h->h0s0, h->h0s0 + n, 2 * n, h->Z, 2 * n, scr(h, 1),
                                      ctr(h, 1), s, 1, st));
-    omm::GemmBatch g{};
-    g.A[0] = h->SWHW; g.B[0] = h->h0s0; g.Cin[0] = h->SWHW + mn; g.C[0] = h->G;
-    TRY(omm::dgemm_batched(false, false, m, n, 2 * n, -2.0, g, 1, m, 2 * n, 4.0, m, m, s, st));
+    TRY(dense_gradient(h));
     return dense_direction(h, 1);
+}
+
+// Residue planes of an FP64 dense handle.  They take about 60 bytes per element of
+// [H' ; S] against 8 for the matrices themselves, so a handle whose planes would
+// exceed an eighth of the device's memory (m ~ 17000 at n = m / 4), or for which
+// the allocation fails, keeps the CUDA-core products.  There is no lower size limit:
+// a step takes 100 us against 104 at m = 8, 104 against 224 at m = 64.
+int crt_alloc(omm_handle *h) {
+    const int64_t m = h->m, n = h->n;
+    CrtBufs &c = h->cr;
+    constexpr int64_t L = omm::crt::kModuli;
+    c.ldm = (m + 7) / 8 * 8;
+    c.ld2n = (2 * n + 7) / 8 * 8;
+    const bool pre = h->opt.precon != 0;
+    const int64_t nHS = L * 2 * m * c.ldm, nWD = L * 2 * n * c.ldm, nSWHW = L * m * c.ld2n, nHSW = L * n * c.ld2n;
+    const int64_t w1 = 2 * omm::crt::words_of(m, n), w2 = omm::crt::words_of(2 * n, 2 * n);
+    const int64_t words = w1 > w2 ? w1 : w2;
+    const int64_t nP = pre ? L * m * c.ldm : 0, nG = pre ? L * n * c.ldm : 0;
+    const int64_t bytes = 2 * (nHS + 2 * nWD + nSWHW + nHSW + nP + nG) + 4 * words;
+    size_t free_b = 0, total_b = 0;
+    OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+    if (bytes > (int64_t)(total_b / 8)) return OMM_OK;
+    int rc;
+    if ((rc = dalloc(&c.HSr, (size_t)nHS)) || (rc = dalloc(&c.WDr, (size_t)nWD)) ||
+        (rc = dalloc(&c.HDSDr, (size_t)nWD)) || (rc = dalloc(&c.SWHWr, (size_t)nSWHW)) ||
+        (rc = dalloc(&c.HSWr, (size_t)nHSW)) || (pre && (rc = dalloc(&c.Pr, (size_t)nP))) ||
+        (pre && (rc = dalloc(&c.Gr, (size_t)nG))) || (rc = dalloc(&c.e, (size_t)(2 * m + 4 * n + m + n + m + n))) ||
+        (rc = dalloc(&c.part, (size_t)(omm::crt::kRowSlices * m))) || (rc = dalloc(&c.words, (size_t)words))) {
+        cudaGetLastError();   // the handle works without them
+        crt_free(c);
+        return OMM_OK;
+    }
+    c.eHS = c.e;
+    c.eWD = c.eHS + 2 * m;
+    c.eHDSD = c.eWD + 2 * n;
+    c.eSWHW = c.eHDSD + 2 * n;
+    c.eHSW = c.eSWHW + m;
+    c.eP = c.eHSW + n;
+    c.eG = c.eP + m;
+    const int l = (int)L;
+    if ((rc = omm::tc::make_digit_map(&c.mapHS, c.HSr, m, 2 * m, c.ldm, 2 * m * c.ldm, l, 128)) ||
+        (rc = omm::tc::make_digit_map(&c.mapWD, c.WDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128)) ||
+        (rc = omm::tc::make_digit_map(&c.mapHDSD, c.HDSDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128)) ||
+        (rc = omm::tc::make_digit_map(&c.mapSWHW, c.SWHWr, 2 * n, m, c.ld2n, m * c.ld2n, l, 128)) ||
+        (rc = omm::tc::make_digit_map(&c.mapHSW, c.HSWr, 2 * n, n, c.ld2n, n * c.ld2n, l, 128)) ||
+        (pre && (rc = omm::tc::make_digit_map(&c.mapP, c.Pr, m, m, c.ldm, m * c.ldm, l, 128))) ||
+        (pre && (rc = omm::tc::make_digit_map(&c.mapG, c.Gr, m, n, c.ldm, n * c.ldm, l, 128))))
+        return rc;
+    return OMM_OK;
 }
 
 // ---------------------------------------------------------------- mixed precision
@@ -1041,6 +1224,9 @@ int precon_build(omm_handle *h) {
         if (h->opt.precision == OMM_PREC_MIXED)
             TRY(omm::tc::pack_cm(m, m, h->P, m, h->mx.Pd, h->mx.ldm, m * h->mx.ldm, kDig, nullptr, st));
     }
+    if (crt_on(h))
+        TRY(omm::crt::pack_rows(m, m, h->P, m, h->cr.eP, h->cr.part, h->cr.Pr, h->cr.ldm, m * h->cr.ldm, true, nullptr,
+                                st));
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
     if (h->hstate->status != OMM_OK) return h->hstate->status;
@@ -1104,6 +1290,15 @@ int dense_set(omm_handle *h, const double *H, const double *S, bool on_device) {
         if (h->opt.refine == OMM_REFINE_EXACT)
             TRY(omm::tc::exact_pack(true, m, cols, h->HS, m, h->ex.eHS, h->ex.HSx, h->mx.ldm, 2 * m * h->mx.ldm,
                                     h->ex.s < 6 ? h->ex.s : 6, nullptr, st));
+    }
+    if (crt_on(h)) {
+        // rows of H' and S; omm_set_H and the Cholesky variant's S = I repack H' only
+        StageTimer t(h, OMM_STAGE_PACK);
+        CrtBufs &c = h->cr;
+        TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, nullptr, st));
+        if (S != nullptr && !s_identity(h))
+            TRY(omm::crt::pack_rows(m, m, h->HS + mm, m, c.eHS + m, c.part, c.HSr + m * c.ldm, c.ldm, 2 * m * c.ldm, true,
+                                    nullptr, st));
     }
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaEventRecord(h->ev1, st));
@@ -1298,6 +1493,11 @@ int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *patt
         return rc;
     }
     if (!h->sparse && h->opt.precon != 0 && (rc = precon_alloc(h))) {
+        free_handle(h);
+        return rc;
+    }
+    // last: what the handle cannot do without is allocated by now
+    if (!h->sparse && h->opt.precision == OMM_PREC_FP64 && (rc = crt_alloc(h))) {
         free_handle(h);
         return rc;
     }

@@ -67,6 +67,9 @@ class SolveRecord:
         return self.finish - self.submit
 
 
+DEVICE_BYTES = 284208 << 20   # HBM of one GB300
+
+
 def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7) -> int:
     """Device memory of one dense handle (what omm_create allocates)."""
     f64 = 8 * (2 * m * m + 6 * m * n + 2 * n * n + 4 * n * n + 2 * m * n)
@@ -76,6 +79,11 @@ def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7) -> in
         f64 += 2 * 3 * (2 * m * ldm + 4 * n * ldm + m * ld2n + n * ld2n)          # split digits
         f64 += 4 * (2 * m * n + 4 * n * n + 4 * m * n)                             # FP32 increments
         f64 += 2 * exact_digits * (2 * m * ldm + 3 * n * ldm + m * ld2n + n * ld2n)  # exact digits
+    else:
+        ldm, ld2n = (m + 7) // 8 * 8, (2 * n + 7) // 8 * 8
+        planes = 32 * (2 * m * ldm + 4 * n * ldm + m * ld2n + n * ld2n) + 16 * max(2 * m * n, 4 * n * n)
+        if planes <= DEVICE_BYTES // 8:                                             # residue planes
+            f64 += planes
     return int(f64)
 
 
