@@ -63,6 +63,7 @@ struct MixedBufs {
 struct ExactBufs {
     int s = 0;
     __nv_bfloat16 *HSx = nullptr, *Wx = nullptr, *HWSWx = nullptr, *SWHWx = nullptr, *HSWx = nullptr;
+    uint32_t *planes = nullptr;   // level planes of a product
     int *e = nullptr;   // exponents: [2m HS | n W | 2n HWSW | m SWHW | n HSW]
     int *eHS = nullptr, *eW = nullptr, *eHWSW = nullptr, *eSWHW = nullptr, *eHSW = nullptr;
     CUtensorMap mapHS_A, mapW, mapHWSW_B, mapSWHW_A, mapHSW_B;
@@ -216,6 +217,7 @@ void free_handle(omm_handle *h) {
     cudaFree(h->ex.HWSWx);
     cudaFree(h->ex.SWHWx);
     cudaFree(h->ex.HSWx);
+    cudaFree(h->ex.planes);
     cudaFree(h->ex.e);
     crt_free(h->cr);
     cudaFree(h->L);
@@ -819,6 +821,8 @@ int exact_alloc(omm_handle *h) {
     TRY(dalloc(&e.SWHWx, (size_t)(s * m * x.ld2n)));
     TRY(dalloc(&e.HSWx, (size_t)(s * n * x.ld2n)));
     TRY(dalloc(&e.e, (size_t)(2 * m + n + 2 * n + m + n)));
+    // the anchor's [H';S] W is the largest product; both it and the gradient take six digits
+    TRY(dalloc(&e.planes, (size_t)omm::tc::exact_plane_words(m, n, 2, s < 6 ? s : 6)));
     e.eHS = e.e;
     e.eW = e.eHS + 2 * m;
     e.eHWSW = e.eW + n;
@@ -834,7 +838,8 @@ int exact_alloc(omm_handle *h) {
 
 omm::tc::ExactArgs exact_args(omm_handle *h, int M, int N, int K) {
     omm::tc::ExactArgs a{};
-    omm::tc::exact_pairs(h->ex.s, a);
+    a.s = h->ex.s;
+    a.planes = h->ex.planes;
     a.M = M;
     a.N = N;
     a.K = K;
@@ -864,7 +869,7 @@ int exact_gradient(omm_handle *h) {
     }
     StageTimer t(h, OMM_STAGE_GRADIENT);
     omm::tc::ExactArgs a = exact_args(h, (int)m, (int)n, (int)(2 * n));
-    omm::tc::exact_pairs(sg, a);
+    a.s = sg;
     a.alpha = -2.0;
     a.beta = 4.0;
     a.Cin = h->SWHW + m * n;
@@ -892,7 +897,7 @@ int exact_anchor(omm_handle *h) {
         TRY(omm::tc::exact_pack(true, m, n, h->WD, m, e.eW, e.Wx, x.ldm, n * x.ldm, sa, s, st));
         // z = 0: H'W -> SWHW + mn;  z = 1: SW -> SWHW
         omm::tc::ExactArgs a = exact_args(h, (int)m, (int)n, (int)m);
-        omm::tc::exact_pairs(sa, a);
+        a.s = sa;
         a.a_row_step = (int)m;
         a.C = h->SWHW + mn;
         a.ldc = m;
@@ -908,7 +913,7 @@ int exact_anchor(omm_handle *h) {
                                 s, st));
         // z = 0: H_W = W^T H'W -> rows [0, n) of h0s0;  z = 1: S_W -> rows [n, 2n)
         omm::tc::ExactArgs b = exact_args(h, (int)n, (int)n, (int)m);
-        omm::tc::exact_pairs(sa, b);
+        b.s = sa;
         b.b_row_step = (int)n;
         b.C = h->h0s0;
         b.ldc = 2 * n;

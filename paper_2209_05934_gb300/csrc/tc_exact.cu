@@ -12,13 +12,9 @@
 // t + u <= s + 1 are kept; pairs of one level L = t + u share the weight
 // 2^-(7L-2).
 //
-// One CTA computes a 128 x 128 tile.  Warp 0 streams (A_t, B_u) digit tiles of
-// each pair through a 6-stage TMA ring; warp 1 accumulates each (pair, chunk)
-// unit in one of two tensor-memory buffers; warps 2..5 read a finished unit,
-// convert its exact integers to int32 and add them to the level's integer
-// sum (registers), and at the end of each level fold that sum into an FP64
-// running sum kept in tensor memory.  The final epilogue scales by
-// 2^(e_i + f_j) and writes C = alpha * A B + beta * Cin in FP64.
+// The GEMM (tc_units.cu) leaves one int32 plane per level; the fold below combines
+// the levels of an element as an integer, converts it once and writes
+// C = alpha * A B + beta * Cin.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -27,269 +23,80 @@
 #include "omm_internal.cuh"
 #include "tc_exact.cuh"
 #include "tc_gemm.cuh"
-#include "tc_ptx.cuh"
+#include "tc_units.cuh"
 
 namespace omm {
 namespace tc {
 namespace {
 
-using namespace ptx;
+constexpr int kChunkMax = 4096;             // 4096 * 64 * 64 = 2^24: exact FP32 integer sums
+constexpr int64_t kPlaneCap = 48ll << 20;   // words of level planes one launch may fill (192 MB)
 
-constexpr int XBN = 128;
-constexpr int XSTAGES = 6;
-constexpr int XTILE_B_BYTES = XBN * BK * 2;
-constexpr int XSTAGE_BYTES = TILE_A_BYTES + XTILE_B_BYTES;
-constexpr int kChunkMax = 4096;     // 4096 * 64 * 64 = 2^24: exact FP32 integer sums
-constexpr int kRunCol = 2 * XBN;    // tensor-memory column of the FP64 running sum
+// ------------------------------------------------------------------ level fold
+struct FoldArgs {
+    int M, N, nlev;
+    const uint32_t *planes;       // group g (level nlev + 1 - g) at g * plane, batch z at z * z_step
+    int64_t plane, z_step;
+    int shift[kExactMaxDigits];   // per level from the top: < 0: R <- 128 R + acc, else R += acc >> shift
+    int lvl_r;                    // level whose units R counts in at the end
+    double alpha, beta;
+    const double *Cin;
+    int64_t ldcin, cin_step;
+    double *C;
+    float *C32;
+    int64_t ldc, c_step;
+    const int *eA, *eB;
+    int64_t eA_step, eB_step;
+    const DevState *state;
+};
 
-__global__ void __launch_bounds__(192, 1)
-    tc_exact_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
-                    const ExactArgs args) {
-    if (args.state != nullptr && *((volatile const int *)&args.state->done)) return;
+// R = sum_L acc_L 2^(7 (Lr - L)) over the levels from the top, counted in units of
+// level Lr: R <- 128 R + acc_L (Lr <- L) while a bound on |R| stays below 2^62; past
+// that Lr stays and a later level adds acc_L 2^-7(L - Lr) rounded to an integer.
+// With 7 digits and K up to 32768 every level is exact; otherwise the rounding is
+// below 2^-47 of the scaled operands' unit, far inside an FP64 GEMM's error bound.
+//
+// Bound by the plane traffic (4 bytes per level and element, mostly from L2): a
+// thread takes one row of four columns, so 4 s loads are in flight.
+__global__ void __launch_bounds__(256) level_fold_kernel(const __grid_constant__ FoldArgs a) {
+    if (a.state != nullptr && *((volatile const int *)&a.state->done)) return;
+    const int row = blockIdx.x * 32 + threadIdx.x;
+    const int col0 = (blockIdx.y * 8 + threadIdx.y) * 4;
     const int z = blockIdx.z;
-    extern __shared__ __align__(1024) uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full_bar[XSTAGES];
-    __shared__ __align__(8) uint64_t empty_bar[XSTAGES];
-    __shared__ __align__(8) uint64_t tfull_bar[2];
-    __shared__ __align__(8) uint64_t tempty_bar[2];
-    __shared__ uint32_t tmem_base;
-    __shared__ int abort_flag;
-    const uint64_t deadline = globaltimer_ns() + kWaitNs;
-
-    const int warp = threadIdx.x >> 5;
-    const int lane = threadIdx.x & 31;
-    const int m0 = blockIdx.y * BM;     // N tiles vary fastest: CTAs in flight share A tiles in L2
-    const int n0 = blockIdx.x * XBN;
-    const int nkb_total = (args.K + BK - 1) / BK;
-    const int kb_per_chunk = kChunkMax / BK;
-    const int nchunks = (nkb_total + kb_per_chunk - 1) / kb_per_chunk;
-    const int nunits = args.npairs * nchunks;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < XSTAGES; ++s) {
-            mbar_init(&full_bar[s], 1);
-            mbar_init(&empty_bar[s], 1);
-        }
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(&tfull_bar[b], 1);
-            mbar_init(&tempty_bar[b], 128);
-        }
-        abort_flag = 0;
-        mbar_fence_init();
-    }
-    if (warp == 1) tmem_alloc(&tmem_base, 512);
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_base;
-
-    if (warp == 0 && lane == 0) {
-        // ---------------- TMA producer: every unit's k-blocks, in unit order
-        const int a_row = args.a_row0 + z * args.a_row_step + m0;
-        const int b_row = args.b_row0 + z * args.b_row_step + n0;
-        int it = 0;
-        for (int u = 0; u < nunits && !abort_flag; ++u) {
-            const int p = u / nchunks, c = u % nchunks;
-            const int kb0 = c * kb_per_chunk;
-            const int kb1 = min(nkb_total, kb0 + kb_per_chunk);
-            for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                const int s = it % XSTAGES;
-                const uint32_t ph = (uint32_t)((it / XSTAGES) & 1);
-                if (!mbar_wait(&empty_bar[s], ph ^ 1u, deadline, &abort_flag, args.err)) break;
-                mbar_arrive_expect_tx(&full_bar[s], (uint32_t)XSTAGE_BYTES);
-                uint8_t *st = smem + s * XSTAGE_BYTES;
-                tma_load_3d(st, &mapA, kb * BK, a_row, args.pa[p], &full_bar[s]);
-                tma_load_3d(st + TILE_A_BYTES, &mapB, kb * BK, b_row, args.pb[p], &full_bar[s]);
-            }
-        }
-    } else if (warp == 1 && lane == 0) {
-        // ---------------- MMA issuer: unit u accumulates into buffer u & 1
-        constexpr uint32_t idesc = idesc_bf16(BM, XBN);
-        int it = 0;
-        for (int u = 0; u < nunits; ++u) {
-            const int c = u % nchunks;
-            const int b = u & 1;
-            if (!mbar_wait(&tempty_bar[b], (uint32_t)(((u >> 1) & 1) ^ 1), deadline, &abort_flag, args.err)) break;
-            tc_fence_after();
-            const uint32_t tacc = tmem + (uint32_t)(b * XBN);
-            const int kb0 = c * kb_per_chunk;
-            const int kb1 = min(nkb_total, kb0 + kb_per_chunk);
-            bool ok = true;
-            for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                const int s = it % XSTAGES;
-                const uint32_t ph = (uint32_t)((it / XSTAGES) & 1);
-                if (!mbar_wait(&full_bar[s], ph, deadline, &abort_flag, args.err)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t st = smem_u32(smem + s * XSTAGE_BYTES);
-                const uint64_t da = sdesc_sw128(st), db = sdesc_sw128(st + TILE_A_BYTES);
+    if (row >= a.M || col0 >= a.N) return;
+    const int nc = a.N - col0 < 4 ? a.N - col0 : 4;
+    const uint32_t *w = a.planes + (int64_t)z * a.z_step + (int64_t)col0 * a.M + row;
+    int64_t R[4] = {0, 0, 0, 0};
 #pragma unroll
-                for (int kk = 0; kk < BK / 16; ++kk)
-                    umma_bf16(tacc, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc,
-                              (kb != kb0 || kk != 0) ? 1u : 0u);
-                umma_commit(&empty_bar[s]);
-            }
-            umma_commit(&tfull_bar[b]);
-            if (!ok) break;
-        }
-    } else if (warp >= 2) {
-        // ---------------- epilogue
-        const int q = warp & 3;
-        const uint32_t lane_base = tmem + ((uint32_t)(32 * q) << 16);
-        const int row = m0 + 32 * q + lane;
-        int32_t acc[XBN];
+    for (int l = 0; l < kExactMaxDigits; ++l) {
+        if (l >= a.nlev) break;
+        const uint32_t *p = w + (int64_t)(a.nlev - 1 - l) * a.plane;
+        const int sh = a.shift[l];
+        const int64_t half = sh > 0 ? ((int64_t)1 << (sh - 1)) : 0;
 #pragma unroll
-        for (int j = 0; j < XBN; ++j) acc[j] = 0;
-        // Running sum in tensor memory (two words per value): the integer
-        // R = sum_L acc_L 2^(7 (Lr - L)) over the levels folded so far, counted
-        // in units of level Lr, updated with integer instructions only:
-        // R <- 128 R + acc_L (Lr <- L) while a bound on |R|, the same in every
-        // thread, stays below 2^62; past that, Lr stays and a later level adds
-        // acc_L 2^-7(L - Lr) rounded to an integer.  With 7 digits and K up to
-        // 32768 every level is exact; otherwise the rounding is below 2^-47 of
-        // the scaled operands' unit, far inside an FP64 GEMM's error bound.
-        // The code stays compact on purpose: an unrolled per-element body
-        // with heavy conversions overflows the instruction cache.
-        int mode = 0;           // 0 empty, 1 growing, 2 fixed units
-        int lvl_r = 0;          // level whose units R counts in
-        double bound = 0.0;     // bound on |R|
-        bool alive = true;
-        for (int u = 0; u < nunits; ++u) {
-            const int p = u / nchunks, c = u % nchunks;
-            const int b = u & 1;
-            bool got = alive && mbar_wait(&tfull_bar[b], (uint32_t)((u >> 1) & 1), deadline, &abort_flag, args.err);
-            got = __all_sync(0xffffffffu, got);
-            alive = got;
-            tc_fence_after();
-            if (got) {
-                // four 16-column loads in flight per wait
-#pragma unroll
-                for (int c0 = 0; c0 < XBN; c0 += 64) {
-                    uint32_t r0[16], r1[16], r2[16], r3[16];
-                    const uint32_t t = lane_base + (uint32_t)(b * XBN + c0);
-                    tmem_ld16_async(t, r0);
-                    tmem_ld16_async(t + 16, r1);
-                    tmem_ld16_async(t + 32, r2);
-                    tmem_ld16_async(t + 48, r3);
-                    tmem_wait_ld(r0);
-                    tmem_pin16(r1);
-                    tmem_pin16(r2);
-                    tmem_pin16(r3);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        acc[c0 + j] += __float2int_rn(__uint_as_float(r0[j]));
-                        acc[c0 + 16 + j] += __float2int_rn(__uint_as_float(r1[j]));
-                        acc[c0 + 32 + j] += __float2int_rn(__uint_as_float(r2[j]));
-                        acc[c0 + 48 + j] += __float2int_rn(__uint_as_float(r3[j]));
-                    }
-                }
-            }
-            tc_fence_before();
-            mbar_arrive(&tempty_bar[b]);
-            const int level = args.pa[p] + args.pb[p] + 2;
-            const bool last_of_level =
-                c == nchunks - 1 && (p == args.npairs - 1 || args.pa[p + 1] + args.pb[p + 1] + 2 != level);
-            if (last_of_level && got) {
-                int np = 0;   // pairs on this level
-                for (int p2 = 0; p2 < args.npairs; ++p2) np += (args.pa[p2] + args.pb[p2] + 2 == level);
-                const double add = (double)np * (double)nchunks * 16777216.0;   // |acc| < np nchunks 2^24
-                int next = mode;
-                if (mode == 0) next = 1;
-                else if (mode == 1 && !(bound * 128.0 + add < 4.6e18)) next = 2;
-                const int sh = next == 2 ? 7 * (level - lvl_r) : 0;            // fixed units: right shift
-                const int64_t half = sh > 0 ? ((int64_t)1 << (sh - 1)) : 0;
-#pragma unroll
-                for (int c0 = 0; c0 < XBN; c0 += 32) {
-                    uint32_t r[4][16];
-                    const uint32_t t = lane_base + (uint32_t)(kRunCol + 2 * c0);
-                    if (mode != 0) {
-                        tmem_ld16_async(t, r[0]);
-                        tmem_ld16_async(t + 16, r[1]);
-                        tmem_ld16_async(t + 32, r[2]);
-                        tmem_ld16_async(t + 48, r[3]);
-                        tmem_wait_ld(r[0]);
-                        tmem_pin16(r[1]);
-                        tmem_pin16(r[2]);
-                        tmem_pin16(r[3]);
-                    }
-#pragma unroll
-                    for (int g = 0; g < 4; ++g)
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const int64_t a = (int64_t)acc[c0 + 8 * g + j];
-                            const int64_t old = mode == 0 ? 0 : (int64_t)(((uint64_t)r[g][2 * j + 1] << 32) | r[g][2 * j]);
-                            const int64_t nv = next == 1 ? old * 128 + a : old + ((a + half) >> sh);
-                            r[g][2 * j] = (uint32_t)(uint64_t)nv;
-                            r[g][2 * j + 1] = (uint32_t)((uint64_t)nv >> 32);
-                        }
-                    tmem_st16_async(t, r[0]);
-                    tmem_st16_async(t + 16, r[1]);
-                    tmem_st16_async(t + 32, r[2]);
-                    tmem_st16_async(t + 48, r[3]);
-                }
-                tmem_wait_st();
-#pragma unroll
-                for (int j = 0; j < XBN; ++j) acc[j] = 0;
-                if (next == 1) {
-                    bound = mode == 0 ? add : bound * 128.0 + add;
-                    lvl_r = level;
-                } else {
-                    bound += add / ldexp(1.0, sh) + 1.0;
-                }
-                mode = next;
-            }
-        }
-        // final: C = alpha 2^(eA + eB) R 2^-(7 Lr - 2) + beta Cin, one integer-op
-        // conversion per value (rolled loop: compact code)
-        const bool ok = __all_sync(0xffffffffu, alive && mode != 0);
-        double *C = args.C != nullptr ? args.C + (int64_t)z * args.c_step : nullptr;
-        float *C32 = args.C32 != nullptr ? args.C32 + (int64_t)z * args.c_step : nullptr;
-        const double *Cin = args.Cin ? args.Cin + (int64_t)z * args.cin_step : nullptr;
-        const int *eA = args.eA + (int64_t)z * args.eA_step;
-        const int *eB = args.eB + (int64_t)z * args.eB_step;
-        const int e_row = (row < args.M ? eA[row] : 0) - (7 * lvl_r - 2);
-#pragma unroll 1
-        for (int c0 = 0; c0 < XBN; c0 += 8) {
-            uint32_t r[16];
-            if (ok) {
-                tmem_ld16_async(lane_base + (uint32_t)(kRunCol + 2 * c0), r);
-                tmem_wait_ld(r);
-            }
-            if (row < args.M) {
-                // Cin first: C may alias it as far as the compiler knows, so a load
-                // after a store would wait for that store
-                double cin[8];
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int col = n0 + c0 + j;
-                    cin[j] = (Cin != nullptr && col < args.N) ? __ldg(&Cin[row + (int64_t)col * args.ldcin]) : 0.0;
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int col = n0 + c0 + j;
-                    if (col >= args.N) break;
-                    double out = 0.0;
-                    if (ok) {
-                        const int64_t R = (int64_t)(((uint64_t)r[2 * j + 1] << 32) | r[2 * j]);
-                        const int e = e_row + eB[col];
-                        // normal-range results by integer ops; anything else (never for
-                        // operands within 2^+-900) through ldexp
-                        out = (e > -960 && e < 900) ? sw_i64_scaled(R, e) : ldexp((double)R, e);
-                    }
-                    if (args.alpha != 1.0) out *= args.alpha;
-                    if (Cin != nullptr) out = fma(args.beta, cin[j], out);
-                    if (C32 != nullptr) C32[row + (int64_t)col * args.ldc] = sw_d2f(out);
-                    else C[row + (int64_t)col * args.ldc] = out;
-                }
-            }
+        for (int j = 0; j < 4; ++j) {
+            const int64_t acc = j < nc ? (int64_t)(int32_t)__ldg(p + (int64_t)j * a.M) : 0;
+            R[j] = sh < 0 ? R[j] * 128 + acc : R[j] + ((acc + half) >> sh);
         }
     }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        __syncwarp();
-        tc_fence_after();
-        tmem_dealloc(tmem, 512);
+    const double *Cin = a.Cin != nullptr ? a.Cin + (int64_t)z * a.cin_step + row + (int64_t)col0 * a.ldcin : nullptr;
+    double cin[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cin[j] = (Cin != nullptr && j < nc) ? Cin[j * a.ldcin] : 0.0;
+    const int e_row = a.eA[(int64_t)z * a.eA_step + row] - (7 * a.lvl_r - 2);
+    const int *eB = a.eB + (int64_t)z * a.eB_step + col0;
+    const int64_t o = (int64_t)z * a.c_step + row + (int64_t)col0 * a.ldc;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (j >= nc) break;
+        const int e = e_row + eB[j];
+        // normal-range results by integer ops; anything else (never for operands
+        // within 2^+-900) through ldexp
+        double out = (e > -960 && e < 900) ? sw_i64_scaled(R[j], e) : ldexp((double)R[j], e);
+        if (a.alpha != 1.0) out *= a.alpha;
+        if (Cin != nullptr) out = fma(a.beta, cin[j], out);
+        if (a.C32 != nullptr) a.C32[o + j * a.ldc] = sw_d2f(out);
+        else a.C[o + j * a.ldc] = out;
     }
 }
 
@@ -430,17 +237,13 @@ int grid_for(int64_t work, int per_block) {
 
 }  // namespace
 
-void exact_pairs(int s, ExactArgs &a) {
-    int k = 0;
-    for (int lvl = 2; lvl <= s + 1; ++lvl)
-        for (int t = 1; t <= s; ++t) {
-            const int u = lvl - t;
-            if (u < 1 || u > s) continue;
-            a.pa[k] = (uint8_t)(t - 1);
-            a.pb[k] = (uint8_t)(u - 1);
-            ++k;
-        }
-    a.npairs = k;
+// (never decreasing in any argument and the same for (M, N) and (N, M), so that the
+// workspace of a caller's largest product serves its others)
+int64_t exact_plane_words(int64_t M, int64_t N, int64_t nbatch, int s) {
+    const int64_t all = (int64_t)s * nbatch * M * N;
+    const int64_t least = (int64_t)s * nbatch * (M > N ? M : N) * 256;   // one tile of columns
+    const int64_t most = least > kPlaneCap ? least : kPlaneCap;
+    return all < most ? all : most;
 }
 
 int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, int64_t ld, int *e,
@@ -475,18 +278,84 @@ int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, i
 }
 
 int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs &a, int nbatch, cudaStream_t st) {
-    if (a.M <= 0 || a.N <= 0 || a.K <= 0 || a.npairs < 1 || a.npairs > kExactMaxPairs || nbatch < 1)
+    const int s = a.s;
+    if (a.M <= 0 || a.N <= 0 || a.K <= 0 || s < 1 || s > kExactMaxDigits || nbatch < 1 || a.planes == nullptr)
         return OMM_ERR_ARG;
-    const int smem = XSTAGES * XSTAGE_BYTES + 1024;
-    static int attr_bytes = 0;
-    if (smem > attr_bytes) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(tc_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_bytes = smem;
+    // groups: the level with the most pairs first
+    UnitArgs u{};
+    u.M = a.M;
+    u.K = a.K;
+    u.nbatch = nbatch;
+    u.ngroups = s;
+    int np = 0;
+    for (int lvl = s + 1; lvl >= 2; --lvl) {
+        const int g = s + 1 - lvl;
+        u.first[g] = (uint8_t)np;
+        u.cnt[g] = (uint8_t)(lvl - 1);
+        for (int t = 1; t < lvl; ++t, ++np) {
+            u.pa[np] = (uint8_t)(t - 1);
+            u.pb[np] = (uint8_t)(lvl - t - 1);
+        }
     }
-    dim3 grid((unsigned)ceil_div(a.N, XBN), (unsigned)ceil_div(a.M, BM), (unsigned)nbatch);
-    tc_exact_kernel<<<grid, 192, smem, st>>>(mapA, mapB, a);
-    count_launch();
-    OMM_CUDA_TRY(cudaGetLastError());
+    u.a_row0 = a.a_row0;
+    u.a_row_step = a.a_row_step;
+    u.b_row_step = a.b_row_step;
+    u.ldp = a.M;
+    u.out = a.planes;
+    u.state = a.state;
+    u.err = a.err;
+    FoldArgs f{};
+    f.M = a.M;
+    f.nlev = s;
+    f.planes = a.planes;
+    const double nchunks = (double)ceil_div(ceil_div(a.K, 64), kChunkMax / 64);
+    double bound = 0.0;   // on |R|
+    for (int l = 0; l < s; ++l) {
+        const int lvl = l + 2;
+        const double add = (double)(lvl - 1) * nchunks * 16777216.0;   // |acc| < pairs * chunks * 2^24
+        const bool grow = l == 0 || (f.shift[l - 1] < 0 && bound * 128.0 + add < 4.6e18);
+        if (grow) {
+            f.shift[l] = -1;
+            bound = l == 0 ? add : bound * 128.0 + add;
+            f.lvl_r = lvl;
+        } else {
+            f.shift[l] = 7 * (lvl - f.lvl_r);
+            bound += add / ldexp(1.0, f.shift[l]) + 1.0;
+        }
+    }
+    f.alpha = a.alpha;
+    f.beta = a.beta;
+    f.Cin = a.Cin;
+    f.ldcin = a.ldcin;
+    f.cin_step = a.cin_step;
+    f.C = a.C;
+    f.C32 = a.C32;
+    f.ldc = a.ldc;
+    f.c_step = a.c_step;
+    f.eA = a.eA;
+    f.eB = a.eB;
+    f.eA_step = a.eA_step;
+    f.eB_step = a.eB_step;
+    f.state = a.state;
+    int64_t slab = exact_plane_words(a.M, a.N, nbatch, s) / ((int64_t)s * nbatch * a.M);
+    if (slab < a.N) slab = slab / 256 * 256;
+    for (int64_t c0 = 0; c0 < a.N; c0 += slab) {
+        const int nc = (int)(a.N - c0 < slab ? a.N - c0 : slab);
+        u.N = f.N = nc;
+        u.b_row0 = a.b_row0 + (int)c0;
+        u.plane = f.plane = (int64_t)a.M * nc;
+        u.z_step = f.z_step = u.plane * s;
+        const int rc = unit_gemm(mapA, mapB, u, false, kChunkMax, st);
+        if (rc != OMM_OK) return rc;
+        dim3 grid((unsigned)ceil_div(a.M, 32), (unsigned)ceil_div(nc, 32), (unsigned)nbatch);
+        level_fold_kernel<<<grid, dim3(32, 8), 0, st>>>(f);
+        count_launch();
+        OMM_CUDA_TRY(cudaGetLastError());
+        if (f.Cin != nullptr) f.Cin += slab * a.ldcin;
+        if (f.C32 != nullptr) f.C32 += slab * a.ldc;
+        else f.C += slab * a.ldc;
+        f.eB += slab;
+    }
     return OMM_OK;
 }
 
@@ -497,7 +366,8 @@ int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs
 extern "C" int64_t omm_op_exact_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int32_t ndigits) {
     if (M < 0 || N < 0 || K < 0 || ndigits < 1 || ndigits > omm::tc::kExactMaxDigits) return -1;
     const int64_t ldk = (K + 7) / 8 * 8;
-    return (int64_t)ndigits * (M + N) * ldk * 2 + (M + N) * 4 + 2048;
+    return (int64_t)ndigits * (M + N) * ldk * 2 + (M + N) * 4 + 2048 +
+           4 * omm::tc::exact_plane_words(M, N, 1, ndigits);
 }
 
 extern "C" int omm_op_exact_gemm(int32_t transA, int32_t transB, int64_t M, int64_t N, int64_t K,
@@ -532,7 +402,8 @@ extern "C" int omm_op_exact_gemm(int32_t transA, int32_t transB, int64_t M, int6
     if ((rc = tc::make_digit_map(&ma, Ad, K, M, ldk, M * ldk, ndigits, 128))) return rc;
     if ((rc = tc::make_digit_map(&mb, Bd, K, N, ldk, N * ldk, ndigits, 128))) return rc;
     tc::ExactArgs a{};
-    tc::exact_pairs(ndigits, a);
+    a.s = ndigits;
+    a.planes = (uint32_t *)(((uintptr_t)(eB + N) + 255) & ~(uintptr_t)255);
     a.M = (int)M;
     a.N = (int)N;
     a.K = (int)K;

@@ -10,14 +10,12 @@ namespace omm {
 namespace tc {
 
 constexpr int kExactMaxDigits = 8;
-constexpr int kExactMaxPairs = kExactMaxDigits * (kExactMaxDigits + 1) / 2;
 
 // C_z = alpha 2^(eA_i + eB_j) sum_{t+u <= s+1} 2^-(7(t+u)-2) A_t B_u^T + beta Cin_z
-// with A, B the digit planes of rows scaled by 2^-eA / 2^-eB (see tc_exact.cu).
+// with A, B the s digit planes of rows scaled by 2^-eA / 2^-eB (see tc_exact.cu).
 struct ExactArgs {
     int M, N, K;
-    int npairs;
-    uint8_t pa[kExactMaxPairs], pb[kExactMaxPairs];   // level-major pair order
+    int s;
     int a_row0, b_row0, a_row_step, b_row_step;
     double alpha, beta;
     const double *Cin;
@@ -28,11 +26,14 @@ struct ExactArgs {
     const int *eA;     // row exponents of A (indexed by output row)
     const int *eB;     // row exponents of B (indexed by output column)
     int64_t eA_step, eB_step;   // per batch z
+    uint32_t *planes;  // level planes: exact_plane_words(M, N, nbatch, s) words
     const DevState *state;
     int *err;
 };
 
-void exact_pairs(int s, ExactArgs &a);
+// Words of the level planes of one product: all of them up to kPlaneCap, else those of
+// a slab of columns (exact_gemm then works slab by slab).
+int64_t exact_plane_words(int64_t M, int64_t N, int64_t nbatch, int s);
 // Digits of the K-major operand rows of the FP64 column-major matrix X (rows x cols, ld):
 // k_along_rows: operand row r = column r of X, K = rows; else operand row r = row r of X, K = cols.
 // Writes the row exponents e[] and planes dst[t * plane + r * ldk + k].

@@ -14,7 +14,9 @@
 // next.  That leaves no tensor memory for the combination of the planes, which is
 // why it is a pass of its own over planes that mostly stay in L2.  An earlier form
 // combined the levels in tensor memory and had room for 128 columns only: it ran
-// the tensor pipe 36% of its active cycles.
+// the tensor pipe 36% of its active cycles.  W^T (H W) of 1024 x 1000 x 4096 with 7
+// digits (packing included) went from 621 to 255 us, the 6-digit gradient of a
+// 4096 x 1024 system from 498 to about 250 us, with the same bits.
 //
 // One work item is one output tile of one plane.  Planes are independent, so a
 // product of few tiles still fills the chip: 16 residue planes (or 6 to 8 digit

@@ -79,6 +79,7 @@ def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7) -> in
         f64 += 2 * 3 * (2 * m * ldm + 4 * n * ldm + m * ld2n + n * ld2n)          # split digits
         f64 += 4 * (2 * m * n + 4 * n * n + 4 * m * n)                             # FP32 increments
         f64 += 2 * exact_digits * (2 * m * ldm + 3 * n * ldm + m * ld2n + n * ld2n)  # exact digits
+        f64 += 4 * min(12 * m * n, max(48 << 20, 12 * m * 256))                     # level planes
     else:
         ldm, ld2n = (m + 7) // 8 * 8, (2 * n + 7) // 8 * 8
         planes = 32 * (2 * m * ldm + 4 * n * ldm + m * ld2n + n * ld2n) + 16 * max(2 * m * n, 4 * n * n)

@@ -128,3 +128,16 @@ def test_exact_gemm_digits_control_accuracy(omm):
     print("exact-digit relative errors:", errs)
     assert errs[3] > errs[5] > errs[7]
     assert errs[7] < 1e-13
+
+
+def test_exact_gemm_in_column_slabs(omm):
+    """A product whose level planes exceed one launch's share runs slab by slab of
+    columns: the same bits as the same columns asked for in products that fit."""
+    rng = np.random.default_rng(8)
+    M, N, K, nd = 4096, 1801, 70, 7
+    A, B, Cin = rng.standard_normal((M, K)), rng.standard_normal((K, N)), rng.standard_normal((M, N))
+    whole = run_exact(omm, 0, 0, M, N, K, nd, A, B, alpha=-2.0, beta=4.0, Cin=Cin)
+    for lo, hi in ((0, 900), (900, N)):
+        part = run_exact(omm, 0, 0, M, hi - lo, K, nd, A, B[:, lo:hi].copy(order="F"), alpha=-2.0, beta=4.0,
+                         Cin=Cin[:, lo:hi].copy(order="F"))
+        assert np.array_equal(whole[:, lo:hi], part)
