@@ -19,9 +19,11 @@
 // 3e-16 .. 1e-15 to 4e-17 .. 7e-17 (m = 141 .. 1597, H alone and with a kinetic part).
 //
 // Reconstruction.  With q_i = (P / p_i)^-1 mod p_i folded into one operand's
-// residues, x / P = frac(sum_i y_i / p_i), y_i the residues of the product: a sum
-// of byte x 90-bit fractions in three 30-bit limbs, taken modulo 1 by letting the
-// 64-bit integers wrap, times P, rounded once.
+// residues, x / P = frac(sum_i y_i / p_i), y_i the residues of the product.  Two
+// moduli at a time, y_i / p_i + y_j / p_j = (y_i p_j + y_j p_i) / (p_i p_j): a sum of
+// 17-bit integers times 90-bit fractions in three 30-bit limbs (24 wide multiply-adds
+// in place of 48), taken modulo 1 by letting the 64-bit integers wrap, times P,
+// rounded once.
 //
 // A row with a NaN or an infinity gets the exponent kNonFinite, and every output of
 // that row is a NaN.
@@ -47,7 +49,7 @@ struct Tables {
     int p[kModuli];
     float pf[kModuli], inv[kModuli];
     float c[2][kModuli][4];        // 2^(16 j) mod p (centred); [1]: times q_i
-    int f2[kModuli], f1[kModuli], f0[kModuli];   // floor(2^90 / p) in 30-bit limbs
+    int f2[kModuli / 2], f1[kModuli / 2], f0[kModuli / 2];   // floor(2^90 / (p_2i p_2i+1)) in 30-bit limbs
     unsigned long long pm;         // P / 2^62
 };
 
@@ -74,13 +76,16 @@ constexpr Tables make_tables() {
             t.c[1][i][j] = (float)centred(pw * q % p[i], p[i]);
             pw = pw * (65536 % p[i]) % p[i];
         }
-        // 2^90 / p_i by long division, 30 bits at a time
+    }
+    for (int i = 0; i < kModuli / 2; ++i) {
+        // 2^90 / (p_2i p_2i+1) by long division, 30 bits at a time
+        const unsigned long long pp = (unsigned long long)p[2 * i] * p[2 * i + 1];
         unsigned long long rem = 1ull << 30;
-        t.f2[i] = (int)(rem / p[i]);
-        rem = (rem % p[i]) << 30;
-        t.f1[i] = (int)(rem / p[i]);
-        rem = (rem % p[i]) << 30;
-        t.f0[i] = (int)(rem / p[i]);
+        t.f2[i] = (int)(rem / pp);
+        rem = (rem % pp) << 30;
+        t.f1[i] = (int)(rem / pp);
+        rem = (rem % pp) << 30;
+        t.f0[i] = (int)(rem / pp);
     }
     return t;
 }
@@ -246,21 +251,13 @@ __global__ void __launch_bounds__(128) row_norm_kernel(int64_t R, int64_t K, con
     part[(int64_t)blockIdx.y * R + r] = make_float2(__int_as_float(be), S);
 }
 
-__device__ __forceinline__ int row_exponent(const float2 *part, int64_t R, int64_t r, int nslice) {
-    int be = 0;
-    for (int s = 0; s < nslice; ++s) {
-        const int b = __float_as_int(part[(int64_t)s * R + r].x);
-        be = b > be ? b : be;
-    }
-    if (be == 0x7FF) return kNonFinite;
-    if (be == 0) return 0;
-    float S = 0.f;
-    for (int s = 0; s < nslice; ++s) {
-        const float2 v = part[(int64_t)s * R + r];
-        const int d = 127 - 2 * (be - __float_as_int(v.x));
-        if (d > 0) S += v.y * __uint_as_float((uint32_t)d << 23);
-    }
-    return scale_exponent(be - 1022, S);
+// (X, S) pairs combined in the order of their index
+__device__ __forceinline__ void norm_join(int &be, float &S, int be2, float S2) {
+    const int top = be > be2 ? be : be2;
+    const int d1 = 127 - 2 * (top - be), d2 = 127 - 2 * (top - be2);
+    S = (d1 > 0 ? S * __uint_as_float((uint32_t)d1 << 23) : 0.f) +
+        (d2 > 0 ? S2 * __uint_as_float((uint32_t)d2 << 23) : 0.f);
+    be = top;
 }
 
 // 32 rows x 64 columns per CTA, turned through shared memory so that both the reads
@@ -271,24 +268,43 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(int64_t R, int64_t K, co
                                                         __nv_bfloat16 *dst, int64_t ldk, int64_t plane,
                                                         const DevState *state) {
     if (state != nullptr && *((volatile const int *)&state->done)) return;
-    __shared__ double tile[64][33];
+    __shared__ double tile[2][32][33];   // [k & 1][k / 2][row]: conflict-free both ways
+    __shared__ float2 ns[8][32];
     __shared__ int es[32];
     const int64_t r0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 64;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int i = warp; i < 64; i += 8) {
         const int64_t r = r0 + lane, k = k0 + i;
-        tile[i][lane] = (r < R && k < K) ? X[r + k * ld] : 0.0;
+        tile[i & 1][i >> 1][lane] = (r < R && k < K) ? X[r + k * ld] : 0.0;
     }
-    if (warp == 0 && r0 + lane < R) {
-        es[lane] = row_exponent(part, R, r0 + lane, nslice);
-        if (blockIdx.y == 0) e[r0 + lane] = es[lane];
+    {
+        // the rows' partial norms: warp w joins slices w, w + 8, ..., warp 0 the warps' results
+        float2 v[kRowSlices / 8];
+#pragma unroll
+        for (int q = 0; q < kRowSlices / 8; ++q)
+            v[q] = (warp + 8 * q < nslice && r0 + lane < R) ? part[(int64_t)(warp + 8 * q) * R + r0 + lane]
+                                                            : make_float2(0.f, 0.f);
+        int be = __float_as_int(v[0].x);
+        float S = v[0].y;
+#pragma unroll
+        for (int q = 1; q < kRowSlices / 8; ++q) norm_join(be, S, __float_as_int(v[q].x), v[q].y);
+        ns[warp][lane] = make_float2(__int_as_float(be), S);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int be = __float_as_int(ns[0][lane].x);
+        float S = ns[0][lane].y;
+#pragma unroll
+        for (int w = 1; w < 8; ++w) norm_join(be, S, __float_as_int(ns[w][lane].x), ns[w][lane].y);
+        es[lane] = be == 0x7FF ? kNonFinite : (be == 0 ? 0 : scale_exponent(be - 1022, S));
+        if (blockIdx.y == 0 && r0 + lane < R) e[r0 + lane] = es[lane];
     }
     __syncthreads();
     const int64_t k = k0 + 2 * lane;
     const int nv = K - k < 2 ? (int)(K - k) : 2;
     for (int i = warp; i < 32; i += 8) {
         if (r0 + i >= R || nv <= 0) break;
-        const int64_t F[2] = {to_fixed(tile[2 * lane][i], es[i]), to_fixed(tile[2 * lane + 1][i], es[i])};
+        const int64_t F[2] = {to_fixed(tile[0][lane][i], es[i]), to_fixed(tile[1][lane][i], es[i])};
         put_residues<INV, 2>(F, dst + (r0 + i) * ldk + k, plane, nv);
     }
 }
@@ -331,9 +347,11 @@ __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldA
         if (j >= nc) break;
         const int eb = a.eB[(int64_t)z * a.eB_step + 4 * c4 + j];
         int64_t s2 = 0, s1 = 0, s0 = 0;
+        const int lsh = 24 - 8 * j;   // byte j to the top, and back with its sign
 #pragma unroll
-        for (int i = 0; i < kModuli; ++i) {
-            const int v = (int)(y[i] << (24 - 8 * j)) >> 24;
+        for (int i = 0; i < kModuli / 2; ++i) {
+            const int v = ((int)(y[2 * i] << lsh) >> 24) * kT.p[2 * i + 1] +
+                          ((int)(y[2 * i + 1] << lsh) >> 24) * kT.p[2 * i];
             s2 += (int64_t)v * kT.f2[i];
             s1 += (int64_t)v * kT.f1[i];
             s0 += (int64_t)v * kT.f0[i];
@@ -348,9 +366,8 @@ __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldA
             out = __longlong_as_double(0x7FF8000000000000ll);
         } else {
             const int ex = ea + eb + 61;
-            const int64_t x = V < 0 ? -(int64_t)u : (int64_t)u;
             // normal results by integer operations; anything else through ldexp
-            out = (ex > -960 && ex < 900) ? sw_i64_scaled(x, ex) : ldexp((double)x, ex);
+            out = (ex > -960 && ex < 900) ? sw_u64_scaled(u, V < 0, ex) : ldexp(V < 0 ? -(double)u : (double)u, ex);
         }
         if (a.alpha != 1.0) out *= a.alpha;
         if (Cin != nullptr) out = fma(a.beta, cin[j], out);

@@ -10,7 +10,7 @@ namespace omm {
 namespace crt {
 
 constexpr int kModuli = 16;
-constexpr int kRowSlices = 16;   // partial row norms per operand row (pack_rows)
+constexpr int kRowSlices = 32;   // partial row norms per operand row (pack_rows)
 
 // C_z = alpha A B_z + beta Cin_z from packed operands (see crt.cu); column-major.
 struct Args {

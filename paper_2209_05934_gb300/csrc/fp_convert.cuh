@@ -76,6 +76,17 @@ __device__ __forceinline__ double sw_i64_scaled(int64_t v, int e2) {
     return __longlong_as_double((long long)(sign | ((uint64_t)(1023 + p + e2) << 52) | (q & 0xFFFFFFFFFFFFFull)));
 }
 
+// The same for a magnitude and a sign, without branches: the leading one to bit 63,
+// then one rounded shift whose carry runs into the exponent.
+__device__ __forceinline__ double sw_u64_scaled(uint64_t a, bool neg, int e2) {
+    const int lz = __clzll((long long)a);
+    const uint64_t n = a << (lz & 63);
+    const uint64_t t = n + (0x3FFull + ((n >> 11) & 1ull));    // ties to even
+    const uint64_t q = (t >> 11) + (t < n ? 1ull << 53 : 0ull);
+    const uint64_t b = ((uint64_t)(1085 - lz + e2) << 52) + q;  // q's leading one adds one to the exponent
+    return __longlong_as_double((long long)((a != 0 ? b : 0ull) | ((neg && a != 0) ? 1ull << 63 : 0ull)));
+}
+
 // x * 2^e by an exponent add when x and the result are normal; other cases
 // (zero, subnormal, overflow, non-finite) go through ldexp.
 __device__ __forceinline__ double sw_scale2(double x, int e) {

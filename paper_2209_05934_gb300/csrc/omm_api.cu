@@ -79,6 +79,7 @@ struct ExactBufs {
 // words: the residue planes of a product; part: partial row norms.
 struct CrtBufs {
     int64_t ldm = 0, ld2n = 0;
+    char *base = nullptr;   // one allocation holds them all
     __nv_bfloat16 *HSr = nullptr, *WDr = nullptr, *HDSDr = nullptr, *SWHWr = nullptr, *HSWr = nullptr;
     __nv_bfloat16 *Pr = nullptr, *Gr = nullptr;   // preconditioner: rows of P, columns of G
     int *e = nullptr;
@@ -177,9 +178,7 @@ int dalloc(T **p, size_t count) {
 }
 
 void crt_free(CrtBufs &c) {
-    for (void *p : {(void *)c.HSr, (void *)c.WDr, (void *)c.HDSDr, (void *)c.SWHWr, (void *)c.HSWr, (void *)c.Pr,
-                    (void *)c.Gr, (void *)c.e, (void *)c.part, (void *)c.words})
-        cudaFree(p);
+    cudaFree(c.base);
     c = CrtBufs{};
 }
 
@@ -514,20 +513,35 @@ int crt_alloc(omm_handle *h) {
     const int64_t w1 = 2 * omm::crt::words_of(m, n), w2 = omm::crt::words_of(2 * n, 2 * n);
     const int64_t words = w1 > w2 ? w1 : w2;
     const int64_t nP = pre ? L * m * c.ldm : 0, nG = pre ? L * n * c.ldm : 0;
-    const int64_t bytes = 2 * (nHS + 2 * nWD + nSWHW + nHSW + nP + nG) + 4 * words;
+    const int64_t nE = 2 * m + 4 * n + m + n + m + n, nPart = omm::crt::kRowSlices * m;
+    int64_t bytes = 0;
+    auto take = [&](int64_t size) {   // 256-byte aligned offsets
+        const int64_t at = bytes;
+        bytes += (size + 255) / 256 * 256;
+        return at;
+    };
+    const int64_t oHS = take(2 * nHS), oWD = take(2 * nWD), oHDSD = take(2 * nWD), oSWHW = take(2 * nSWHW),
+                  oHSW = take(2 * nHSW), oP = take(2 * nP), oG = take(2 * nG), oE = take(4 * nE), oPart = take(8 * nPart),
+                  oWords = take(4 * words);
     size_t free_b = 0, total_b = 0;
     OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
     if (bytes > (int64_t)(total_b / 8)) return OMM_OK;
-    int rc;
-    if ((rc = dalloc(&c.HSr, (size_t)nHS)) || (rc = dalloc(&c.WDr, (size_t)nWD)) ||
-        (rc = dalloc(&c.HDSDr, (size_t)nWD)) || (rc = dalloc(&c.SWHWr, (size_t)nSWHW)) ||
-        (rc = dalloc(&c.HSWr, (size_t)nHSW)) || (pre && (rc = dalloc(&c.Pr, (size_t)nP))) ||
-        (pre && (rc = dalloc(&c.Gr, (size_t)nG))) || (rc = dalloc(&c.e, (size_t)(2 * m + 4 * n + m + n + m + n))) ||
-        (rc = dalloc(&c.part, (size_t)(omm::crt::kRowSlices * m))) || (rc = dalloc(&c.words, (size_t)words))) {
+    if (cudaMalloc((void **)&c.base, (size_t)bytes) != cudaSuccess) {
         cudaGetLastError();   // the handle works without them
-        crt_free(c);
+        c = CrtBufs{};
         return OMM_OK;
     }
+    c.HSr = (__nv_bfloat16 *)(c.base + oHS);
+    c.WDr = (__nv_bfloat16 *)(c.base + oWD);
+    c.HDSDr = (__nv_bfloat16 *)(c.base + oHDSD);
+    c.SWHWr = (__nv_bfloat16 *)(c.base + oSWHW);
+    c.HSWr = (__nv_bfloat16 *)(c.base + oHSW);
+    c.Pr = (__nv_bfloat16 *)(c.base + oP);
+    c.Gr = (__nv_bfloat16 *)(c.base + oG);
+    c.e = (int *)(c.base + oE);
+    c.part = (float2 *)(c.base + oPart);
+    c.words = (uint32_t *)(c.base + oWords);
+    int rc;
     c.eHS = c.e;
     c.eWD = c.eHS + 2 * m;
     c.eHDSD = c.eWD + 2 * n;
