@@ -319,9 +319,9 @@ int omm_batch_solve(omm_handle **handles, int32_t count, const double *const *W0
  * for OMM solver use").  The first, split-precision phase of every system runs in
  * lock step: each CG step's three split products (H'D and SD, the contractions,
  * the gradient) are each ONE persistent grouped tensor-core launch over the tile
- * lists of all systems (longest K first), while each system's line minimum,
- * updates and direction run on its own stream in between; a chunk of 8 such steps
- * is captured once as a CUDA graph and replayed until every system has left the
+ * lists of all systems (longest K first), and the line minima, updates, dots and
+ * directions of all systems one grouped launch each in between; a chunk of 8 such
+ * steps is captured once as a CUDA graph and replayed until every system has left the
  * first phase.  The refinement then runs per system as in omm_batch_solve.
  * tile_mode: 0 one CTA per 128 x 256 tile, 1 CTA pairs (256 x 256 tiles,
  * tcgen05.mma.cta_group::2), -1 autotune: the first call for a group of this

@@ -120,13 +120,13 @@ __device__ void block_sum(double (&v)[NV], double *red, bool lane0_only = false)
 
 template <int NV>
 __device__ bool publish_and_collect(const double (&v)[NV], double *partials, unsigned int *counter,
-                                    double (&tot)[NV], double *red) {
+                                    double (&tot)[NV], double *red, unsigned blk, unsigned nblk) {
     __shared__ bool is_last;
     if (threadIdx.x == 0) {
 #pragma unroll
-        for (int q = 0; q < NV; ++q) partials[blockIdx.x * NV + q] = v[q];
+        for (int q = 0; q < NV; ++q) partials[blk * NV + q] = v[q];
         __threadfence();
-        is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
+        is_last = (atomicAdd(counter, 1u) == nblk - 1);
     }
     __syncthreads();
     if (!is_last) return false;
@@ -138,14 +138,14 @@ __device__ bool publish_and_collect(const double (&v)[NV], double *partials, uns
         double s = 0.0;
         // the lane's blocks in order, eight loads in flight at a time
         unsigned b = threadIdx.x & 31;
-        for (; b + 224 < gridDim.x; b += 256) {
+        for (; b + 224 < nblk; b += 256) {
             double p[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) p[k] = __ldcg(&partials[(b + 32 * k) * NV + q]);
 #pragma unroll
             for (int k = 0; k < 8; ++k) s += p[k];
         }
-        for (; b < gridDim.x; b += 32) s += __ldcg(&partials[b * NV + q]);
+        for (; b < nblk; b += 32) s += __ldcg(&partials[b * NV + q]);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
         if ((threadIdx.x & 31) == 0) red[q] = s;
@@ -162,14 +162,13 @@ __device__ bool publish_and_collect(const double (&v)[NV], double *partials, uns
 // partials: 0 tr h2, 1 <s0,h2>, 2 <Y,X>, 3 <Y,X^T>, 4 <s2,h0>, 5 <Y,h2>, 6 <s2,X>, 7 <s2,h2>
 constexpr int NC = 8;
 
-__global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__restrict__ h0,
-                                                        const double *__restrict__ s0, int64_t ldh,
-                                                        const float *__restrict__ Z, int64_t ldz,
-                                                        double *partials, unsigned int *counter,
-                                                        DevState *state, const double *__restrict__ slope,
-                                                        int nslope) {
+__device__ __forceinline__ void mx_coeffs_body(int n, const double *__restrict__ h0, const double *__restrict__ s0,
+                                               int64_t ldh, const float *__restrict__ Z, int64_t ldz,
+                                               double *partials, unsigned int *counter, DevState *state,
+                                               const double *__restrict__ slope, int nslope, unsigned blk,
+                                               unsigned nblk) {
     if (*((volatile int *)&state->done)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) state->done_upd = 1;
+        if (blk == 0 && threadIdx.x == 0) state->done_upd = 1;
         return;
     }
     __shared__ float Xt[TILE][TILE + 1];
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__re
     float f[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) f[q] = 0.f;
-    for (int t = blockIdx.x; t < T * T; t += gridDim.x) {
+    for (int t = blk; t < T * T; t += nblk) {
         const int ti = t % T, tj = t / T;
         // every load of the tile is issued before any is used (zero outside the
         // matrix instead of a branch), so a thread has ~30 loads in flight
@@ -222,7 +221,7 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__re
     to_f64<NC>(f, v);
     block_sum<NC>(v, red, true);
     double tot[NC] = {};
-    if (!publish_and_collect<NC>(v, partials, counter, tot, red)) return;
+    if (!publish_and_collect<NC>(v, partials, counter, tot, red, blk, nblk)) return;
     // the slope <G, D>: the direction kernel's per-block parts (one-digit
     // directions), else the dots kernel's value
     double gd[1] = {0.0};
@@ -255,13 +254,21 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__re
     state->done_upd = st != OMM_OK ? 1 : 0;
 }
 
+__global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__restrict__ h0,
+                                                       const double *__restrict__ s0, int64_t ldh,
+                                                       const float *__restrict__ Z, int64_t ldz, double *partials,
+                                                       unsigned int *counter, DevState *state,
+                                                       const double *__restrict__ slope, int nslope) {
+    mx_coeffs_body(n, h0, s0, ldh, Z, ldz, partials, counter, state, slope, nslope, blockIdx.x, gridDim.x);
+}
+
 // ---------------------------------------------------------------- H_W, S_W update
 // h0 += x (X + X^T) + x^2 sym(h2), s0 likewise (FP32 increments, FP64 sums);
 // ||s0 - I||_F^2 for the orthonormality test; digits of [H_W ; S_W] columns.
-__global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, double *s0, int64_t ldh,
-                                                           const float *__restrict__ Z, int64_t ldz,
-                                                           double *partials, unsigned int *counter,
-                                                           DevState *state, DigitOut hsw) {
+__device__ __forceinline__ void mx_nn_update_body(int n, double *h0, double *s0, int64_t ldh,
+                                                  const float *__restrict__ Z, int64_t ldz, double *partials,
+                                                  unsigned int *counter, DevState *state, DigitOut hsw, unsigned blk,
+                                                  unsigned nblk) {
     if (*((volatile int *)&state->done)) return;
     __shared__ float Tt[4][TILE][TILE + 1];
     __shared__ double red[(NT / 32)];
@@ -270,7 +277,7 @@ __global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, 
     const int T = (n + TILE - 1) / TILE;
     const float x = state->x_f;
     float orth = 0.f;
-    for (int t = blockIdx.x; t < T * T; t += gridDim.x) {
+    for (int t = blk; t < T * T; t += nblk) {
         const int ti = t % T, tj = t / T;
         // all loads of the tile first (zero outside the matrix), then the transposes
         // through shared memory, then the updates
@@ -326,7 +333,7 @@ __global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, 
     to_f64<1>(fo, v);
     block_sum<1>(v, red, true);
     double tot[1];
-    if (!publish_and_collect<1>(v, partials, counter, tot, red)) return;
+    if (!publish_and_collect<1>(v, partials, counter, tot, red, blk, nblk)) return;
     if (threadIdx.x != 0) return;
     const double E = state->E_next;
     state->orth2 = tot[0];
@@ -351,18 +358,25 @@ __global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, 
     }
 }
 
+__global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, double *s0, int64_t ldh,
+                                                             const float *__restrict__ Z, int64_t ldz,
+                                                             double *partials, unsigned int *counter,
+                                                             DevState *state, DigitOut hsw) {
+    mx_nn_update_body(n, h0, s0, ldh, Z, ldz, partials, counter, state, hsw, blockIdx.x, gridDim.x);
+}
+
 // ---------------------------------------------------------------- W, H'W, SW update
-__global__ void __launch_bounds__(NT) mx_update_kernel(int m, int n, double *W, const float *__restrict__ D,
-                                                        double *HW, const float *__restrict__ HD, double *SW,
-                                                        const float *__restrict__ SD, const DevState *state,
-                                                        DigitOut wd, DigitOut swhw) {
+__device__ __forceinline__ void mx_update_body(int m, int n, double *W, const float *__restrict__ D, double *HW,
+                                               const float *__restrict__ HD, double *SW,
+                                               const float *__restrict__ SD, const DevState *state, DigitOut wd,
+                                               DigitOut swhw, unsigned blk, unsigned nblk) {
     if (*((volatile const int *)&state->done_upd)) return;
     __shared__ float tH[TILE][TILE + 1];
     __shared__ float tS[TILE][TILE + 1];
     const float x = state->x_f;
     const int lx = threadIdx.x % TILE, ly = threadIdx.x / TILE;
     const int Tm = (m + TILE - 1) / TILE, Tn = (n + TILE - 1) / TILE;
-    for (int t = blockIdx.x; t < Tm * Tn; t += gridDim.x) {
+    for (int t = blk; t < Tm * Tn; t += nblk) {
         const int ti = t % Tm, tj = t / Tm;
         const int i = ti * TILE + lx;
 #pragma unroll
@@ -396,20 +410,27 @@ __global__ void __launch_bounds__(NT) mx_update_kernel(int m, int n, double *W, 
     }
 }
 
+__global__ void __launch_bounds__(NT) mx_update_kernel(int m, int n, double *W, const float *__restrict__ D,
+                                                       double *HW, const float *__restrict__ HD, double *SW,
+                                                       const float *__restrict__ SD, const DevState *state,
+                                                       DigitOut wd, DigitOut swhw) {
+    mx_update_body(m, n, W, D, HW, HD, SW, SD, state, wd, swhw, blockIdx.x, gridDim.x);
+}
+
 // Two consecutive rows per thread on 64 x 32 tiles (m even, 16-byte aligned
 // FP64 arrays): double2 / float2 accesses, paired digit conversions.
 constexpr int TI2 = 64;
-__global__ void __launch_bounds__(NT) mx_update2_kernel(int m, int n, double2 *W, const float2 *__restrict__ D,
-                                                         double2 *HW, const float2 *__restrict__ HD, double2 *SW,
-                                                         const float2 *__restrict__ SD, const DevState *state,
-                                                         DigitOut wd, DigitOut swhw) {
+__device__ __forceinline__ void mx_update2_body(int m, int n, double2 *W, const float2 *__restrict__ D, double2 *HW,
+                                                const float2 *__restrict__ HD, double2 *SW,
+                                                const float2 *__restrict__ SD, const DevState *state, DigitOut wd,
+                                                DigitOut swhw, unsigned blk, unsigned nblk) {
     if (*((volatile const int *)&state->done_upd)) return;
     __shared__ float tH[TILE][TI2 + 1];
     __shared__ float tS[TILE][TI2 + 1];
     const float x = state->x_f;
     const int lx = threadIdx.x % 32, ly = threadIdx.x / 32;
     const int Tm = (m + TI2 - 1) / TI2, Tn = (n + TILE - 1) / TILE;
-    for (int t = blockIdx.x; t < Tm * Tn; t += gridDim.x) {
+    for (int t = blk; t < Tm * Tn; t += nblk) {
         const int ti = t % Tm, tj = t / Tm;
         const int i = ti * TI2 + 2 * lx;
 #pragma unroll
@@ -450,23 +471,30 @@ __global__ void __launch_bounds__(NT) mx_update2_kernel(int m, int n, double2 *W
     }
 }
 
+__global__ void __launch_bounds__(NT) mx_update2_kernel(int m, int n, double2 *W, const float2 *__restrict__ D,
+                                                        double2 *HW, const float2 *__restrict__ HD, double2 *SW,
+                                                        const float2 *__restrict__ SD, const DevState *state,
+                                                        DigitOut wd, DigitOut swhw) {
+    mx_update2_body(m, n, W, D, HW, HD, SW, SD, state, wd, swhw, blockIdx.x, gridDim.x);
+}
+
 // ---------------------------------------------------------------- CG dots and direction
 // <Z,G>, <Z,Gp>, <G,D> with Z = P G (PRE) or Z = G
 constexpr int ND = 3;
 
 template <bool PRE>
-__global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__restrict__ G,
-                                                      const float *__restrict__ Zg, const float *__restrict__ Gp,
-                                                      const float *__restrict__ D, double *partials,
-                                                      unsigned int *counter, DevState *state, int first) {
+__device__ __forceinline__ void mx_dots_body(int64_t mn, const float *__restrict__ G, const float *__restrict__ Zg,
+                                             const float *__restrict__ Gp, const float *__restrict__ D,
+                                             double *partials, unsigned int *counter, DevState *state, int first,
+                                             unsigned blk, unsigned nblk) {
     if (*((volatile int *)&state->done)) return;
     __shared__ double red[(NT / 32) * ND];
     float f[ND] = {0.f, 0.f, 0.f};
-    const int64_t n4 = mn / 4, stride = (int64_t)gridDim.x * NT;
+    const int64_t n4 = mn / 4, stride = (int64_t)nblk * NT;
     const float4 *G4 = reinterpret_cast<const float4 *>(G), *Gp4 = reinterpret_cast<const float4 *>(Gp),
                  *D4 = reinterpret_cast<const float4 *>(D), *Z4 = reinterpret_cast<const float4 *>(Zg);
 #pragma unroll 4
-    for (int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x; k < n4; k += stride) {
+    for (int64_t k = (int64_t)blk * NT + threadIdx.x; k < n4; k += stride) {
         const float4 g = G4[k];
         const float4 z = PRE ? Z4[k] : g;
         f[0] = fmaf(z.x, g.x, fmaf(z.y, g.y, fmaf(z.z, g.z, fmaf(z.w, g.w, f[0]))));
@@ -476,7 +504,7 @@ __global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__
             f[2] = fmaf(g.x, d.x, fmaf(g.y, d.y, fmaf(g.z, d.z, fmaf(g.w, d.w, f[2]))));
         }
     }
-    for (int64_t i = 4 * n4 + (int64_t)blockIdx.x * NT + threadIdx.x; i < mn; i += stride) {   // tail
+    for (int64_t i = 4 * n4 + (int64_t)blk * NT + threadIdx.x; i < mn; i += stride) {   // tail
         const float g = G[i], z = PRE ? Zg[i] : g;
         f[0] = fmaf(z, g, f[0]);
         if (!first) {
@@ -488,7 +516,7 @@ __global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__
     to_f64<ND>(f, v);
     block_sum<ND>(v, red, true);
     double tot[ND];
-    if (!publish_and_collect<ND>(v, partials, counter, tot, red)) return;
+    if (!publish_and_collect<ND>(v, partials, counter, tot, red, blk, nblk)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;
@@ -514,33 +542,42 @@ __global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__
     state->gD = restart ? -gg : -gg + beta * tot[2];   // <G, D_new>
 }
 
+template <bool PRE>
+__global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__restrict__ G,
+                                                     const float *__restrict__ Zg, const float *__restrict__ Gp,
+                                                     const float *__restrict__ D, double *partials,
+                                                     unsigned int *counter, DevState *state, int first) {
+    mx_dots_body<PRE>(mn, G, Zg, Gp, D, partials, counter, state, first, blockIdx.x, gridDim.x);
+}
+
 // Df = -Z + beta Df (Df = -Z on a restart), Z = P G (Zg) or G; Gp <- G.  Df is
 // the direction of the CG recurrence.  ROUND1: the line search runs along D, Df
 // rounded to one BF16 digit (its digit planes past the first are zero), while
 // the recurrence keeps Df unrounded; each block leaves its part of the slope
-// <G, D> of the rounded direction in slope[blockIdx.x], which the coefficients
+// <G, D> of the rounded direction in slope[block], which the coefficients
 // kernel sums (c1 / 2 of the quartic; no serial tail here).  Without ROUND1, D
 // and Df are the same array.
 template <bool ROUND1>
-__device__ __forceinline__ void direction_slope(float gd, double *slope) {
+__device__ __forceinline__ void direction_slope(float gd, double *slope, unsigned blk) {
     if (!ROUND1) return;
     __shared__ double red[NT / 32];
     const float f[1] = {gd};
     double v[1];
     to_f64<1>(f, v);
     block_sum<1>(v, red, true);
-    if (threadIdx.x == 0) slope[blockIdx.x] = v[0];
+    if (threadIdx.x == 0) slope[blk] = v[0];
 }
 
 template <bool ROUND1>
-__global__ void __launch_bounds__(NT) mx_direction_kernel(int m, int64_t mn, const float *__restrict__ G,
-                                                           const float *__restrict__ Zg, float *Gp, float *Df,
-                                                           float *D, DevState *state, DigitOut dd, double *slope) {
+__device__ __forceinline__ void mx_direction_body(int m, int64_t mn, const float *__restrict__ G,
+                                                  const float *__restrict__ Zg, float *Gp, float *Df, float *D,
+                                                  DevState *state, DigitOut dd, double *slope, unsigned blk,
+                                                  unsigned nblk) {
     if (*((volatile const int *)&state->done)) return;
     const float beta = state->beta_f;
     const bool restart = state->restart != 0;
     float gd = 0.f;
-    for (int64_t o = (int64_t)blockIdx.x * NT + threadIdx.x; o < mn; o += (int64_t)gridDim.x * NT) {
+    for (int64_t o = (int64_t)blk * NT + threadIdx.x; o < mn; o += (int64_t)nblk * NT) {
         const float g = G[o], z = Zg != nullptr ? Zg[o] : g;
         const float d = restart ? -z : fmaf(beta, Df[o], -z);
         Df[o] = d;
@@ -561,21 +598,28 @@ __global__ void __launch_bounds__(NT) mx_direction_kernel(int m, int64_t mn, con
             put3f(dd, j * dd.ld + i, d);
         }
     }
-    direction_slope<ROUND1>(gd, slope);
+    direction_slope<ROUND1>(gd, slope, blk);
+}
+
+template <bool ROUND1>
+__global__ void __launch_bounds__(NT) mx_direction_kernel(int m, int64_t mn, const float *__restrict__ G,
+                                                          const float *__restrict__ Zg, float *Gp, float *Df,
+                                                          float *D, DevState *state, DigitOut dd, double *slope) {
+    mx_direction_body<ROUND1>(m, mn, G, Zg, Gp, Df, D, state, dd, slope, blockIdx.x, gridDim.x);
 }
 
 // four consecutive rows of one column per thread (m % 4 == 0, 16-byte aligned arrays)
 template <bool PRE, bool ROUND1>
-__global__ void __launch_bounds__(NT) mx_direction4_kernel(int m, int64_t mn, const float4 *__restrict__ G,
-                                                            const float4 *__restrict__ Zg, float4 *Gp, float4 *Df,
-                                                            float4 *D, DevState *state, DigitOut dd,
-                                                            double *slope) {
+__device__ __forceinline__ void mx_direction4_body(int m, int64_t mn, const float4 *__restrict__ G,
+                                                   const float4 *__restrict__ Zg, float4 *Gp, float4 *Df, float4 *D,
+                                                   DevState *state, DigitOut dd, double *slope, unsigned blk,
+                                                   unsigned nblk) {
     if (*((volatile const int *)&state->done)) return;
     const float beta = state->beta_f;
     const bool restart = state->restart != 0;
     const int64_t n4 = mn / 4;
     float gd = 0.f;
-    for (int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x; k < n4; k += (int64_t)gridDim.x * NT) {
+    for (int64_t k = (int64_t)blk * NT + threadIdx.x; k < n4; k += (int64_t)nblk * NT) {
         const float4 g = G[k];
         const float4 z = PRE ? Zg[k] : g;
         float4 d = Df[k];
@@ -609,7 +653,14 @@ __global__ void __launch_bounds__(NT) mx_direction4_kernel(int m, int64_t mn, co
             put3f4(dd, j * dd.ld + i, d);
         }
     }
-    direction_slope<ROUND1>(gd, slope);
+    direction_slope<ROUND1>(gd, slope, blk);
+}
+
+template <bool PRE, bool ROUND1>
+__global__ void __launch_bounds__(NT) mx_direction4_kernel(int m, int64_t mn, const float4 *__restrict__ G,
+                                                           const float4 *__restrict__ Zg, float4 *Gp, float4 *Df,
+                                                           float4 *D, DevState *state, DigitOut dd, double *slope) {
+    mx_direction4_body<PRE, ROUND1>(m, mn, G, Zg, Gp, Df, D, state, dd, slope, blockIdx.x, gridDim.x);
 }
 
 // Grid-wide barrier of a cooperative launch (every block of the grid is
@@ -662,10 +713,10 @@ __device__ __forceinline__ void grid_barrier(unsigned int *bar, int *err) {
 // Df are read twice, the second time mostly from L2.
 template <bool PRE, bool ROUND1>
 __global__ void __launch_bounds__(NT, 4) mx_dots_direction4_kernel(int m, int64_t mn, const float4 *__restrict__ G,
-                                                                 const float4 *__restrict__ Zg, float4 *Gp,
-                                                                 float4 *Df, float4 *D, DevState *state, DigitOut dd,
-                                                                 double *slope, double *partials,
-                                                                 unsigned int *bar, int first) {
+                                                                   const float4 *__restrict__ Zg, float4 *Gp,
+                                                                   float4 *Df, float4 *D, DevState *state,
+                                                                   DigitOut dd, double *slope, double *partials,
+                                                                   unsigned int *bar, int first) {
     if (*((volatile const int *)&state->done)) return;
     __shared__ double red[(NT / 32) * ND];
     __shared__ float s_beta;
@@ -783,12 +834,72 @@ __global__ void __launch_bounds__(NT, 4) mx_dots_direction4_kernel(int m, int64_
             put3f4(dd, j * dd.ld + i, d);
         }
     }
-    direction_slope<ROUND1>(gd, slope);
+    direction_slope<ROUND1>(gd, slope, blockIdx.x);
+}
+
+// ---------------------------------------------------------------- grouped glue
+// The same per-system blocks for many systems in one launch: block b of the grid is
+// block blks[b].y of system blks[b].x, and computes what that block of the system's
+// own launch computes, with the same partial-sum slots and block counts, so every
+// result keeps its bits.  One launch per kernel and step instead of one per system:
+// the systems' tails overlap, nothing waits for a fork and join of streams, and the
+// dots and the direction are two launches instead of a cooperative one, of which
+// only one could be resident at a time.
+__global__ void __launch_bounds__(NT) mx_group_coeffs_kernel(const GlueSys *__restrict__ sys,
+                                                             const int2 *__restrict__ blks) {
+    const int2 b = blks[blockIdx.x];
+    const GlueSys &g = sys[b.x];
+    mx_coeffs_body(g.n, g.h0, g.s0, 2 * g.n, g.Z, 2 * g.n, g.scr[0], g.ctr[0], g.state, g.slope, g.nslope, (unsigned)b.y,
+                   (unsigned)g.nn_blocks);
+}
+
+// H_W, S_W updates (b.y < nn_blocks) and, beside them, the W, H'W, SW updates
+__global__ void __launch_bounds__(NT, 4) mx_group_update_kernel(const GlueSys *__restrict__ sys,
+                                                                const int2 *__restrict__ blks) {
+    const int2 b = blks[blockIdx.x];
+    const GlueSys &g = sys[b.x];
+    if (b.y < g.nn_blocks) {
+        mx_nn_update_body(g.n, g.h0, g.s0, 2 * g.n, g.Z, 2 * g.n, g.scr[1], g.ctr[1], g.state, g.hsw, (unsigned)b.y,
+                          (unsigned)g.nn_blocks);
+        return;
+    }
+    const unsigned blk = (unsigned)(b.y - g.nn_blocks), nblk = (unsigned)g.up_blocks;
+    if (g.up2)
+        mx_update2_body(g.m, g.n, reinterpret_cast<double2 *>(g.W), reinterpret_cast<const float2 *>(g.D),
+                        reinterpret_cast<double2 *>(g.HW), reinterpret_cast<const float2 *>(g.HD),
+                        reinterpret_cast<double2 *>(g.SW), reinterpret_cast<const float2 *>(g.SD), g.state, g.wd, g.swhw,
+                        blk, nblk);
+    else
+        mx_update_body(g.m, g.n, g.W, g.D, g.HW, g.HD, g.SW, g.SD, g.state, g.wd, g.swhw, blk, nblk);
+}
+
+__global__ void __launch_bounds__(NT) mx_group_dots_kernel(const GlueSys *__restrict__ sys,
+                                                           const int2 *__restrict__ blks) {
+    const int2 b = blks[blockIdx.x];
+    const GlueSys &g = sys[b.x];
+    mx_dots_body<false>((int64_t)g.m * g.n, g.G, g.G, g.Gp, g.Df, g.scr[2], g.ctr[2], g.state, 0, (unsigned)b.y,
+                        (unsigned)g.dots_blocks);
+}
+
+template <bool ROUND1>
+__global__ void __launch_bounds__(NT) mx_group_direction_kernel(const GlueSys *__restrict__ sys,
+                                                                const int2 *__restrict__ blks) {
+    const int2 b = blks[blockIdx.x];
+    const GlueSys &g = sys[b.x];
+    const int64_t mn = (int64_t)g.m * g.n;
+    if (g.dir4)
+        mx_direction4_body<false, ROUND1>(g.m, mn, reinterpret_cast<const float4 *>(g.G),
+                                          reinterpret_cast<const float4 *>(g.G), reinterpret_cast<float4 *>(g.Gp),
+                                          reinterpret_cast<float4 *>(g.Df), reinterpret_cast<float4 *>(g.Dw), g.state,
+                                          g.dd, g.slope_out, (unsigned)b.y, (unsigned)g.dir_blocks);
+    else
+        mx_direction_body<ROUND1>(g.m, mn, g.G, nullptr, g.Gp, g.Df, g.Dw, g.state, g.dd, g.slope_out, (unsigned)b.y,
+                                  (unsigned)g.dir_blocks);
 }
 
 // Digits of four consecutive rows of one column per thread (m % 4 == 0)
 __global__ void __launch_bounds__(NT) mx_digits4_kernel(int m, int64_t mn, const float4 *__restrict__ A,
-                                                         const DevState *state, DigitOut dd) {
+                                                        const DevState *state, DigitOut dd) {
     if (*((volatile const int *)&state->done)) return;
     for (int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x; k < mn / 4; k += (int64_t)gridDim.x * NT) {
         const int64_t o = 4 * k, j = o / m, i = o - j * m;
@@ -815,6 +926,41 @@ int tiles_blocks(int64_t a, int64_t b) {
     return (int)(nb < 1 ? 1 : nb);
 }
 
+// two rows per thread in the m x n update: even m and aligned arrays
+bool update_by_two(int64_t m, const double *W, const float *D, const double *HW, const float *HD, const double *SW,
+                   const float *SD, const DigitOut &wd) {
+    return m % 2 == 0 && ((((uintptr_t)W) | ((uintptr_t)HW) | ((uintptr_t)SW)) & 15u) == 0 &&
+           ((((uintptr_t)D) | ((uintptr_t)HD) | ((uintptr_t)SD)) & 7u) == 0 &&
+           (wd.ptr == nullptr || ((((uintptr_t)wd.ptr) & 3u) == 0 && wd.ld % 2 == 0 && wd.plane % 2 == 0));
+}
+
+int64_t update_blocks(int64_t m, int64_t n, bool two) {
+    const int64_t nb = ceil_div(m, two ? TI2 : TILE) * ceil_div(n, TILE);
+    return nb > 152 * 8 ? 152 * 8 : nb;
+}
+
+// blocks of the dots: up to kRedBlocksMax (the partial-sum slots), enough warps per
+// SM to keep the three streams' loads in flight
+int64_t dots_blocks(int64_t mn) {
+    const int64_t nb = ceil_div(mn, (int64_t)NT * 8);
+    return nb > kRedBlocksMax ? kRedBlocksMax : nb;
+}
+
+// four rows per thread in the direction: m % 4 == 0 and aligned arrays
+bool direction_by_four(int64_t m, const float *G, const float *Zg, const float *Gp, const float *Df, const float *D,
+                       const DigitOut &dd) {
+    return m % 4 == 0 &&
+           ((((uintptr_t)G) | ((uintptr_t)Gp) | ((uintptr_t)Df) | ((uintptr_t)D) | ((uintptr_t)Zg)) & 15u) == 0 &&
+           (dd.ptr == nullptr || ((((uintptr_t)dd.ptr) & 7u) == 0 && dd.ld % 4 == 0 && dd.plane % 4 == 0));
+}
+
+// blocks of the direction kernel; with one-digit directions each leaves a slope part
+int64_t direction_blocks(int64_t mn, bool vec, bool round1) {
+    const int64_t cap = round1 ? kRedBlocksMax : 152 * 8;
+    const int64_t nb = vec ? ceil_div(mn / 4, (int64_t)NT * 4) : ceil_div(mn, (int64_t)NT * 4);
+    return nb > cap ? cap : (nb < 1 ? 1 : nb);
+}
+
 }  // namespace
 
 int mx_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh, const float *Z, int64_t ldz,
@@ -830,12 +976,9 @@ int mx_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh, co
 
 int mx_update(int64_t m, int64_t n, double *W, const float *D, double *HW, const float *HD, double *SW,
               const float *SD, const DevState *state, DigitOut wd, DigitOut swhw, cudaStream_t st) {
-    const bool aligned = ((((uintptr_t)W) | ((uintptr_t)HW) | ((uintptr_t)SW)) & 15u) == 0 &&
-                         ((((uintptr_t)D) | ((uintptr_t)HD) | ((uintptr_t)SD)) & 7u) == 0 &&
-                         (wd.ptr == nullptr || ((((uintptr_t)wd.ptr) & 3u) == 0 && wd.ld % 2 == 0 && wd.plane % 2 == 0));
-    if (m % 2 == 0 && aligned) {
-        int64_t nb = ceil_div(m, TI2) * ceil_div(n, TILE);
-        if (nb > 152 * 8) nb = 152 * 8;
+    const bool two = update_by_two(m, W, D, HW, HD, SW, SD, wd);
+    const int64_t nb = update_blocks(m, n, two);
+    if (two) {
         mx_update2_kernel<<<(unsigned)nb, NT, 0, st>>>(
             (int)m, (int)n, reinterpret_cast<double2 *>(W), reinterpret_cast<const float2 *>(D),
             reinterpret_cast<double2 *>(HW), reinterpret_cast<const float2 *>(HD), reinterpret_cast<double2 *>(SW),
@@ -844,8 +987,6 @@ int mx_update(int64_t m, int64_t n, double *W, const float *D, double *HW, const
         OMM_CUDA_TRY(cudaGetLastError());
         return OMM_OK;
     }
-    int64_t nb = ceil_div(m, TILE) * ceil_div(n, TILE);
-    if (nb > 152 * 8) nb = 152 * 8;
     mx_update_kernel<<<(unsigned)nb, NT, 0, st>>>((int)m, (int)n, W, D, HW, HD, SW, SD, state, wd, swhw);
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
@@ -863,10 +1004,7 @@ int mx_nn_update(int n, double *h0, double *s0, int64_t ldh, const float *Z, int
 int mx_dots_beta(int64_t mn, const float *G, const float *Zg, const float *Gp, const float *D, double *scratch,
                  unsigned int *counter, DevState *state, int first, cudaStream_t st) {
     if (((((uintptr_t)G) | ((uintptr_t)Gp) | ((uintptr_t)D) | ((uintptr_t)Zg)) & 15u) != 0) return OMM_ERR_ARG;
-    // up to kRedBlocksMax blocks (the partial-sum slots): enough warps per SM to
-    // keep the three streams' loads in flight
-    int64_t nb = ceil_div(mn, (int64_t)NT * 8);
-    if (nb > kRedBlocksMax) nb = kRedBlocksMax;
+    const int64_t nb = dots_blocks(mn);
     const unsigned grid = (unsigned)(nb < 1 ? 1 : nb);
     if (Zg != nullptr)
         mx_dots_kernel<true><<<grid, NT, 0, st>>>(mn, G, Zg, Gp, D, scratch, counter, state, first);
@@ -882,15 +1020,8 @@ int mx_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *G
     if (round1 && (slope == nullptr || D == nullptr || D == Df)) return OMM_ERR_ARG;
     if (!round1) D = Df;
     const int64_t mn = m * n;
-    const bool aligned =
-        ((((uintptr_t)G) | ((uintptr_t)Gp) | ((uintptr_t)Df) | ((uintptr_t)D) | ((uintptr_t)Zg)) & 15u) == 0 &&
-        (dd.ptr == nullptr || ((((uintptr_t)dd.ptr) & 7u) == 0 && dd.ld % 4 == 0 && dd.plane % 4 == 0));
-    // the rounding form leaves one slope partial per block: at most kRedBlocksMax
-    const int64_t cap = round1 ? kRedBlocksMax : 152 * 8;
-    const bool vec = m % 4 == 0 && aligned;
-    int64_t nb = vec ? ceil_div(mn / 4, (int64_t)NT * 4) : ceil_div(mn, (int64_t)NT * 4);
-    if (nb > cap) nb = cap;
-    const unsigned grid = (unsigned)(nb < 1 ? 1 : nb);
+    const bool vec = direction_by_four(m, G, Zg, Gp, Df, D, dd);
+    const unsigned grid = (unsigned)direction_blocks(mn, vec, round1);
     if (slope_blocks != nullptr) *slope_blocks = round1 ? (int)grid : 0;
     if (vec) {
         const float4 *G4 = reinterpret_cast<const float4 *>(G);
@@ -913,21 +1044,13 @@ int mx_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *G
     return OMM_OK;
 }
 
-int mx_dots_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *Gp, float *Df, float *D,
-                      DevState *state, DigitOut dd, bool round1, double *slope, int *slope_blocks, double *scratch,
-                      unsigned int *bar, int first, cudaStream_t st) {
-    if (round1 && (slope == nullptr || D == nullptr || D == Df)) return OMM_ERR_ARG;
-    if (!round1) D = Df;
-    const int64_t mn = m * n;
-    const bool aligned =
-        ((((uintptr_t)G) | ((uintptr_t)Gp) | ((uintptr_t)Df) | ((uintptr_t)D) | ((uintptr_t)Zg)) & 15u) == 0 &&
-        (dd.ptr == nullptr || ((((uintptr_t)dd.ptr) & 7u) == 0 && dd.ld % 4 == 0 && dd.plane % 4 == 0));
-    if (m % 4 != 0 || !aligned || bar == nullptr || (((uintptr_t)bar) & 7u) != 0) return OMM_ERR_UNSUPPORTED;
-    const int variant = (Zg != nullptr ? 2 : 0) + (round1 ? 1 : 0);
-    auto kern = Zg != nullptr
-                    ? (round1 ? mx_dots_direction4_kernel<true, true> : mx_dots_direction4_kernel<true, false>)
+namespace {
+// Grid of the cooperative dots + direction launch: every block must be resident at
+// once, so the blocks of the dots are capped by the occupancy.
+int coop_blocks(int64_t mn, bool pre, bool round1, int64_t *out) {
+    const int variant = (pre ? 2 : 0) + (round1 ? 1 : 0);
+    auto kern = pre ? (round1 ? mx_dots_direction4_kernel<true, true> : mx_dots_direction4_kernel<true, false>)
                     : (round1 ? mx_dots_direction4_kernel<false, true> : mx_dots_direction4_kernel<false, false>);
-    // every block must be resident at once: the grid is capped by the occupancy
     static int coop = -1, sms = 0;
     if (coop < 0) {
         int dev = 0, c = 0;
@@ -939,11 +1062,29 @@ int mx_dots_direction(int64_t m, int64_t n, const float *G, const float *Zg, flo
     }
     if (!coop) return OMM_ERR_UNSUPPORTED;
     static int occupancy[4] = {0, 0, 0, 0};
-    if (occupancy[variant] == 0) OMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occupancy[variant], kern, NT, 0));
-    const int per_sm = occupancy[variant];
-    int64_t nb = ceil_div(mn, (int64_t)NT * 8);
-    if (nb > kRedBlocksMax) nb = kRedBlocksMax;
-    if (nb > (int64_t)per_sm * sms) nb = (int64_t)per_sm * sms;
+    if (occupancy[variant] == 0)
+        OMM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occupancy[variant], kern, NT, 0));
+    int64_t nb = dots_blocks(mn);
+    if (nb > (int64_t)occupancy[variant] * sms) nb = (int64_t)occupancy[variant] * sms;
+    *out = nb;
+    return OMM_OK;
+}
+}  // namespace
+
+int mx_dots_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *Gp, float *Df, float *D,
+                      DevState *state, DigitOut dd, bool round1, double *slope, int *slope_blocks, double *scratch,
+                      unsigned int *bar, int first, cudaStream_t st) {
+    if (round1 && (slope == nullptr || D == nullptr || D == Df)) return OMM_ERR_ARG;
+    if (!round1) D = Df;
+    const int64_t mn = m * n;
+    if (!direction_by_four(m, G, Zg, Gp, Df, D, dd) || bar == nullptr || (((uintptr_t)bar) & 7u) != 0)
+        return OMM_ERR_UNSUPPORTED;
+    auto kern = Zg != nullptr
+                    ? (round1 ? mx_dots_direction4_kernel<true, true> : mx_dots_direction4_kernel<true, false>)
+                    : (round1 ? mx_dots_direction4_kernel<false, true> : mx_dots_direction4_kernel<false, false>);
+    int64_t nb = 0;
+    const int rc = coop_blocks(mn, Zg != nullptr, round1, &nb);
+    if (rc != OMM_OK) return rc;
     if (nb < 1) return OMM_ERR_UNSUPPORTED;
     if (slope_blocks != nullptr) *slope_blocks = round1 ? (int)nb : 0;
     const float4 *G4 = reinterpret_cast<const float4 *>(G);
@@ -987,6 +1128,43 @@ int mx_round(int64_t count, const double *src, float *dst, const DevState *state
     int64_t nb = ceil_div(count, 256 * 4);
     if (nb > 152 * 8) nb = 152 * 8;
     mx_round_kernel<<<(unsigned)(nb < 1 ? 1 : nb), 256, 0, st>>>(count, src, dst, state);
+    count_launch();
+    OMM_CUDA_TRY(cudaGetLastError());
+    return OMM_OK;
+}
+
+// ---------------------------------------------------------------- grouped launches
+int mx_group_prepare(GlueSys &g, bool round1) {
+    const int64_t m = g.m, n = g.n, mn = m * n;
+    if (((((uintptr_t)g.G) | ((uintptr_t)g.Gp) | ((uintptr_t)g.Df)) & 15u) != 0) return OMM_ERR_ARG;
+    g.nn_blocks = tiles_blocks(n, n);
+    g.up2 = update_by_two(m, g.W, g.D, g.HW, g.HD, g.SW, g.SD, g.wd) ? 1 : 0;
+    g.up_blocks = (int)update_blocks(m, n, g.up2 != 0);
+    g.dir4 = direction_by_four(m, g.G, nullptr, g.Gp, g.Df, g.Dw, g.dd) ? 1 : 0;
+    int64_t nb = 0;
+    // block counts of the system's own launches: the cooperative one where it applies
+    if (g.dir4 && coop_blocks(mn, false, round1, &nb) == OMM_OK && nb >= 1) {
+        g.dots_blocks = g.dir_blocks = (int)nb;
+    } else {
+        g.dots_blocks = (int)(dots_blocks(mn) < 1 ? 1 : dots_blocks(mn));
+        g.dir_blocks = (int)direction_blocks(mn, g.dir4 != 0, round1);
+    }
+    g.nslope = round1 ? g.dir_blocks : 0;
+    return OMM_OK;
+}
+
+int mx_group_launch(int which, const GlueSys *sys, const int2 *blks, int nblks, bool round1, cudaStream_t st) {
+    if (nblks <= 0) return OMM_OK;
+    switch (which) {
+        case GLUE_COEFFS: mx_group_coeffs_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
+        case GLUE_UPDATE: mx_group_update_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
+        case GLUE_DOTS: mx_group_dots_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
+        case GLUE_DIRECTION:
+            if (round1) mx_group_direction_kernel<true><<<nblks, NT, 0, st>>>(sys, blks);
+            else mx_group_direction_kernel<false><<<nblks, NT, 0, st>>>(sys, blks);
+            break;
+        default: return OMM_ERR_ARG;
+    }
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;

@@ -152,7 +152,6 @@ struct omm_handle {
     // second stream of the mixed form: H_W, S_W updates run beside the m x n updates
     cudaStream_t aux = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    bool grouped = false;     // inside omm_batch_solve_grouped's lock-step phase
     omm::sp::Host sh;   // linear-scaling form: patterns and gather lists (host)
     omm::sp::Dev sd;    // linear-scaling form: device arrays
     // optional per-stage device timing (omm_set_profiling)
@@ -1019,9 +1018,9 @@ int mixed_glue1(omm_handle *h, bool accurate_gradient) {
     { StageTimer t(h, OMM_STAGE_UPDATE);
       // the n x n update (H_W, S_W, energy, stop test) reads and writes nothing the
       // m x n update touches: for large systems it runs beside it on the handle's
-      // second stream (in a grouped batch, and for small systems, the extra fork
-      // and join cost more than the overlap gains)
-      const bool fork = !h->grouped && m * n >= ((int64_t)1 << 21) && st != cudaStreamLegacy &&
+      // second stream (for small systems the extra fork and join cost more than the
+      // overlap gains)
+      const bool fork = m * n >= ((int64_t)1 << 21) && st != cudaStreamLegacy &&
                         st != cudaStreamPerThread && st != nullptr;
       cudaStream_t sn = fork ? h->aux : st;
       if (fork) {
@@ -1995,29 +1994,95 @@ std::mutex g_tune_mu;
 std::vector<TuneEntry> g_tune;
 TuneEntry g_last_tune;
 
-// Fork every system's stream off the group stream, run fn(h) on each, join back.
-template <class F>
-int fork_join(omm_handle **hs, int count, cudaStream_t gs, cudaEvent_t ev_fork, cudaEvent_t *ev_join, F fn) {
-    OMM_CUDA_TRY(cudaEventRecord(ev_fork, gs));
-    for (int i = 0; i < count; ++i) {
-        OMM_CUDA_TRY(cudaStreamWaitEvent(hs[i]->stream, ev_fork, 0));
-        TRY(fn(hs[i]));
-        OMM_CUDA_TRY(cudaEventRecord(ev_join[i], hs[i]->stream));
-        OMM_CUDA_TRY(cudaStreamWaitEvent(gs, ev_join[i], 0));
+// The glue kernels of a group: every system's arguments and, per kernel, the list of
+// (system, block) pairs, larger systems first (one device allocation).
+struct GroupGlue {
+    char *mem = nullptr;
+    const omm::GlueSys *sys = nullptr;
+    const int2 *blks[omm::GLUE_KERNELS] = {};
+    int nblks[omm::GLUE_KERNELS] = {};
+    bool round1 = false;
+    void release() {
+        cudaFree(mem);
+        mem = nullptr;
     }
+};
+
+int build_group_glue(omm_handle **hs, int count, GroupGlue &G) {
+    G.round1 = hs[0]->opt.dir_digits == 1;
+    std::vector<omm::GlueSys> sys((size_t)count);
+    std::vector<int> order((size_t)count);
+    for (int i = 0; i < count; ++i) {
+        omm_handle *h = hs[i];
+        MixedBufs &x = h->mx;
+        const int64_t n = h->n, mn = h->m * n;
+        omm::GlueSys &g = sys[i];
+        g.m = (int)h->m;
+        g.n = (int)n;
+        g.h0 = h->h0s0;
+        g.s0 = h->h0s0 + n;
+        g.Z = x.Z32;
+        g.W = h->WD;
+        g.HW = h->SWHW + mn;
+        g.SW = h->SWHW;
+        g.D = x.D32;
+        g.HD = x.HDSD32;
+        g.SD = x.HDSD32 + mn;
+        g.G = x.G32;
+        g.Gp = x.Gp32;
+        g.Df = G.round1 ? x.Df32 : x.D32;
+        g.Dw = x.D32;
+        g.wd = dig_W(h);
+        g.swhw = dig_SWHW(h);
+        g.hsw = dig_HSW(h);
+        g.dd = dig_D(h);
+        for (int k = 0; k < 3; ++k) {
+            g.scr[k] = scr(h, k);
+            g.ctr[k] = ctr(h, k);
+        }
+        g.slope = g.slope_out = scr(h, 3);
+        g.state = h->dstate;
+        TRY(omm::mx_group_prepare(g, G.round1));
+        // the start's direction left its slope parts by the same rule
+        if (g.nslope != h->slope_blocks) return OMM_ERR_STATE;
+        order[i] = i;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return sys[a].m > sys[b].m; });
+    std::vector<int2> list[omm::GLUE_KERNELS];
+    for (int i : order) {
+        const omm::GlueSys &g = sys[i];
+        const int nb[omm::GLUE_KERNELS] = {g.nn_blocks, g.nn_blocks + g.up_blocks, g.dots_blocks, g.dir_blocks};
+        for (int k = 0; k < omm::GLUE_KERNELS; ++k)
+            for (int b = 0; b < nb[k]; ++b) list[k].push_back(int2{i, b});
+    }
+    size_t bytes = (sys.size() * sizeof(omm::GlueSys) + 255) / 256 * 256, off[omm::GLUE_KERNELS];
+    for (int k = 0; k < omm::GLUE_KERNELS; ++k) {
+        off[k] = bytes;
+        bytes += list[k].size() * sizeof(int2);
+        G.nblks[k] = (int)list[k].size();
+    }
+    std::vector<char> host(bytes);
+    memcpy(host.data(), sys.data(), sys.size() * sizeof(omm::GlueSys));
+    for (int k = 0; k < omm::GLUE_KERNELS; ++k) memcpy(host.data() + off[k], list[k].data(), list[k].size() * sizeof(int2));
+    OMM_CUDA_TRY(cudaMalloc((void **)&G.mem, bytes));
+    OMM_CUDA_TRY(cudaMemcpy(G.mem, host.data(), bytes, cudaMemcpyHostToDevice));
+    G.sys = (const omm::GlueSys *)G.mem;
+    for (int k = 0; k < omm::GLUE_KERNELS; ++k) G.blks[k] = (const int2 *)(G.mem + off[k]);
     return OMM_OK;
 }
 
-// One first-phase CG step of every system: the three split products as grouped
-// persistent launches on the group stream, the per-system line minimum, updates
-// and direction on the systems' own streams in between.
-int group_iteration(omm_handle **hs, int count, const GroupList *L, const int *mode, cudaStream_t gs,
-                    cudaEvent_t ev_fork, cudaEvent_t *ev_join) {
+// One first-phase CG step of every system on the group stream: the three split
+// products as grouped persistent launches, the line minima, updates and directions
+// as grouped glue launches between them.
+int group_iteration(omm_handle **hs, const GroupList *L, const int *mode, const GroupGlue &G, cudaStream_t gs) {
+    auto glue = [&](int k) { return omm::mx_group_launch(k, G.sys, G.blks[k], G.nblks[k], G.round1, gs); };
     TRY(run_group_list(L[0], mode[0], hs[0], gs));
     TRY(run_group_list(L[1], mode[1], hs[0], gs));
-    TRY(fork_join(hs, count, gs, ev_fork, ev_join, [](omm_handle *h) { return mixed_glue1(h, false); }));
+    TRY(glue(omm::GLUE_COEFFS));
+    TRY(glue(omm::GLUE_UPDATE));
     TRY(run_group_list(L[2], mode[2], hs[0], gs));
-    return fork_join(hs, count, gs, ev_fork, ev_join, [](omm_handle *h) { return mixed_direction(h, 0); });
+    TRY(glue(omm::GLUE_DOTS));
+    return glue(omm::GLUE_DIRECTION);
 }
 
 }  // namespace
@@ -2050,18 +2115,11 @@ int omm_batch_solve_grouped(omm_handle **handles, int32_t count, const double *c
     }
     // ---- phase 1 of every system in lock step
     for (int32_t i = 0; i < count; ++i) TRY(begin_setup(handles[i], W0 ? W0[i] : nullptr, W0_on_device, tol));
-    struct Ungroup {
-        omm_handle **hs;
-        int32_t count;
-        ~Ungroup() {
-            for (int32_t i = 0; i < count; ++i) hs[i]->grouped = false;
-        }
-    } ungroup{handles, count};
-    for (int32_t i = 0; i < count; ++i) handles[i]->grouped = true;
     cudaStream_t gs = nullptr;
     cudaEvent_t ev_fork = nullptr;
     std::vector<cudaEvent_t> ev_join((size_t)count, nullptr);
     GroupList lists[2][3];
+    GroupGlue glue;
     cudaGraphExec_t gexec = nullptr;
     int rc = OMM_OK;
     auto cleanup = [&]() {
@@ -2069,6 +2127,7 @@ int omm_batch_solve_grouped(omm_handle **handles, int32_t count, const double *c
         if (gexec) cudaGraphExecDestroy(gexec);
         for (auto &row : lists)
             for (auto &L : row) L.release();
+        glue.release();
         for (auto e : ev_join)
             if (e) cudaEventDestroy(e);
         if (ev_fork) cudaEventDestroy(ev_fork);
@@ -2148,13 +2207,14 @@ int omm_batch_solve_grouped(omm_handle **handles, int32_t count, const double *c
         for (int k = 0; k < 3; ++k) g_last_tune.mode[k] = mode[k];
     }
     GroupList use[3] = {lists[mode[0]][0], lists[mode[1]][1], lists[mode[2]][2]};
+    GTRY(build_group_glue(handles, count, glue));
     // ---- a chunk of first-phase steps, captured once, replayed until every system is done
     const int chunk = 8;
     const int64_t before = omm_kernel_launches();
     GCUDA(cudaStreamBeginCapture(gs, cudaStreamCaptureModeThreadLocal));
     int crc = OMM_OK;
     for (int c = 0; c < chunk && crc == OMM_OK; ++c)
-        crc = group_iteration(handles, count, use, mode, gs, ev_fork, ev_join.data());
+        crc = group_iteration(handles, use, mode, glue, gs);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(gs, &graph);
     if (crc != OMM_OK || ce != cudaSuccess) {
@@ -2186,7 +2246,6 @@ int omm_batch_solve_grouped(omm_handle **handles, int32_t count, const double *c
         if (all) break;
     }
     // ---- phase 2 (refinement) per system on its own stream, as omm_batch_solve
-    for (int32_t i = 0; i < count; ++i) handles[i]->grouped = false;
     GCUDA(cudaEventRecord(ev_fork, gs));
     for (int32_t i = 0; i < count; ++i) {
         GCUDA(cudaStreamWaitEvent(handles[i]->stream, ev_fork, 0));

@@ -155,6 +155,29 @@ int mx_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *G
 int mx_dots_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *Gp, float *Df, float *D,
                       DevState *state, DigitOut dd, bool round1, double *slope, int *slope_blocks, double *scratch,
                       unsigned int *bar, int first, cudaStream_t st);
+// The glue kernels of many systems' first-phase steps as grouped launches: each
+// system's arguments, and a list of (system, block) pairs per kernel.  mx_group_prepare
+// fills the block counts (those of the system's own launches, so that the partial
+// sums and their order are the same) and nslope.
+struct GlueSys {
+    int m, n;
+    double *h0, *s0;                 // ld 2n
+    const float *Z;                  // ld 2n
+    double *W, *HW, *SW;
+    const float *D, *HD, *SD;        // D: the search direction of this step
+    const float *G;
+    float *Gp, *Df, *Dw;             // Df: the recurrence's direction; Dw: where D is written
+    DigitOut wd, swhw, hsw, dd;
+    double *scr[3];                  // partial sums: coefficients, n x n update, dots
+    unsigned int *ctr[3];
+    const double *slope;             // the direction's per-block slope parts, read and written
+    double *slope_out;
+    DevState *state;
+    int nslope, nn_blocks, up_blocks, dots_blocks, dir_blocks, up2, dir4;
+};
+enum { GLUE_COEFFS = 0, GLUE_UPDATE = 1, GLUE_DOTS = 2, GLUE_DIRECTION = 3, GLUE_KERNELS = 4 };
+int mx_group_prepare(GlueSys &g, bool round1);
+int mx_group_launch(int which, const GlueSys *sys, const int2 *blks, int nblks, bool round1, cudaStream_t st);
 // digits of an FP32 m x n column-major array: column j -> row j of the planes
 int mx_digits(int64_t m, int64_t n, const float *A, const DevState *state, DigitOut dd, cudaStream_t st);
 int mx_round(int64_t count, const double *src, float *dst, const DevState *state, cudaStream_t st);
