@@ -27,10 +27,10 @@
 //
 // A row with a NaN or an infinity gets the exponent kNonFinite, and every output of
 // that row is a NaN.
-#include <limits.h>
 #include <math.h>
 
 #include "crt.cuh"
+#include "fixed.cuh"
 #include "fp_convert.cuh"
 #include "tc_units.cuh"
 
@@ -38,7 +38,6 @@ namespace omm {
 namespace crt {
 namespace {
 
-constexpr int kNonFinite = INT_MIN;
 constexpr int kNormBits = 62;         // ||F||_2 <= 2^62
 constexpr int kKmax = 1024;           // 1024 * 128 * 128 = 2^24
 constexpr float kMagic = 12582912.f;  // 1.5 * 2^23
@@ -91,37 +90,6 @@ constexpr Tables make_tables() {
 }
 constexpr Tables kTables = make_tables();
 __constant__ constexpr Tables kT = make_tables();
-
-// ------------------------------------------------------------------ scaling
-// Row scale from X (2^X > max |a| >= 2^(X-1)) and S = sum (a 2^-X)^2: the exponent e
-// with a = F 2^e.  ||a|| <= 2^X sqrt(1.001 S) <= 2^(X + L) (the 1.001 covers the FP32
-// rounding of S).
-__device__ __forceinline__ int scale_exponent(int X, float S) {
-    const float s = S * 1.001f;
-    const int k = (int)((__float_as_uint(s) >> 23) & 0xFF) - 126;   // s < 2^k
-    return X + ((k + 1) >> 1) - kNormBits;
-}
-
-// (a 2^-X)^2 in FP32, a's magnitude bits `b` (sign cleared)
-__device__ __forceinline__ float scaled_square(uint64_t b, int X) {
-    const int e = (int)(b >> 52) - 1023 - X + 127;
-    if (e <= 0) return 0.f;   // below 2^-126 of the largest: nothing of the sum
-    const float f = __uint_as_float(((uint32_t)e << 23) | (uint32_t)((b & 0xFFFFFFFFFFFFFull) >> 29));
-    return f * f;
-}
-
-// F = round(v 2^-e), |F| < 2^62
-__device__ __forceinline__ int64_t to_fixed(double v, int e) {
-    const uint64_t b = (uint64_t)__double_as_longlong(v);
-    const int be = (int)((b >> 52) & 0x7FF);
-    if (be == 0 || e == kNonFinite) return 0;
-    const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);   // v = mant 2^(be - 1075)
-    const int shift = be - 1075 - e;
-    int64_t F = 0;
-    if (shift >= 0) F = (int64_t)(mant << shift);
-    else if (shift > -64) F = (int64_t)((mant + (1ull << (-shift - 1))) >> (-shift));
-    return (b >> 63) ? -F : F;
-}
 
 // Residues of NV values, written as BF16 to dst[i * plane + 0..NV).  F in four
 // balanced 16-bit pieces f_j: sum_j f_j (2^(16 j) mod p) <= 4 * 2^15 * 2^7 = 2^24 is
@@ -196,23 +164,22 @@ __global__ void __launch_bounds__(256) pack_cols_kernel(int64_t K, int64_t R, co
         __syncthreads();
         for (int w = 0; w < nw; ++w) mx = smax[w] > mx ? smax[w] : mx;
         const int be = (int)(mx >> 52);
-        const int X2 = be - 1022;
         float S = 0.f;
         if (be != 0 && be != 0x7FF)
-            for (int64_t k = tid; k < K; k += blockDim.x) S += scaled_square(xb[k] & 0x7FFFFFFFFFFFFFFFull, X2);
+            for (int64_t k = tid; k < K; k += blockDim.x) S += fx_square(xb[k] & 0x7FFFFFFFFFFFFFFFull, be - 1022);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
         if (lane == 0) ssum[warp] = S;
         __syncthreads();
         S = 0.f;
         for (int w = 0; w < nw; ++w) S += ssum[w];
-        const int er = be == 0x7FF ? kNonFinite : (be == 0 ? 0 : scale_exponent(X2, S));
+        const int er = fx_exponent(be, S, kNormBits);
         if (tid == 0) e[r] = er;
         for (int64_t k = 4 * tid; k < K; k += 4 * blockDim.x) {
             const int nv = K - k < 4 ? (int)(K - k) : 4;
             int64_t F[4];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) F[v] = v < nv ? to_fixed(x[k + v], er) : 0;
+            for (int v = 0; v < 4; ++v) F[v] = v < nv ? fx_round(x[k + v], er) : 0;
             put_residues<INV, 4>(F, dst + r * ldk + k, plane, nv);
         }
         __syncthreads();
@@ -246,7 +213,7 @@ __global__ void __launch_bounds__(128) row_norm_kernel(int64_t R, int64_t K, con
             be = top;
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) S += scaled_square(a[u], be - 1022);
+        for (int u = 0; u < 8; ++u) S += fx_square(a[u], be - 1022);
     }
     part[(int64_t)blockIdx.y * R + r] = make_float2(__int_as_float(be), S);
 }
@@ -296,7 +263,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(int64_t R, int64_t K, co
         float S = ns[0][lane].y;
 #pragma unroll
         for (int w = 1; w < 8; ++w) norm_join(be, S, __float_as_int(ns[w][lane].x), ns[w][lane].y);
-        es[lane] = be == 0x7FF ? kNonFinite : (be == 0 ? 0 : scale_exponent(be - 1022, S));
+        es[lane] = fx_exponent(be, S, kNormBits);
         if (blockIdx.y == 0 && r0 + lane < R) e[r0 + lane] = es[lane];
     }
     __syncthreads();
@@ -304,7 +271,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(int64_t R, int64_t K, co
     const int nv = K - k < 2 ? (int)(K - k) : 2;
     for (int i = warp; i < 32; i += 8) {
         if (r0 + i >= R || nv <= 0) break;
-        const int64_t F[2] = {to_fixed(tile[0][lane][i], es[i]), to_fixed(tile[1][lane][i], es[i])};
+        const int64_t F[2] = {fx_round(tile[0][lane][i], es[i]), fx_round(tile[1][lane][i], es[i])};
         put_residues<INV, 2>(F, dst + (r0 + i) * ldk + k, plane, nv);
     }
 }

@@ -712,6 +712,41 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
     }
 }
 
+// X = W^T H'W and Y = W^T S W alone (D = W: the start and the density matrices have no
+// h2, s2 of their own): sixteen lanes per P_N block, two blocks per warp, the lanes and
+// the order of the sums those of contract_kernel's X and Y.
+template <int BM, int BN, typename T = double>
+__global__ void __launch_bounds__(NT) contract_xy_kernel(int64_t nnzN, const int64_t *__restrict__ Crp,
+                                                          const int32_t *__restrict__ Ca,
+                                                          const int32_t *__restrict__ Cb, const T *__restrict__ W,
+                                                          const T *__restrict__ HW, const T *__restrict__ SW, T *X,
+                                                          T *Y, const DevState *state) {
+    if (done(state)) return;
+    static_assert(BN == 2, "contraction lanes assume 2 orbitals per W block");
+    const int l16 = threadIdx.x & 15, v = l16 >> 1, half = l16 & 1;
+    const int mat = v >> 2, a = (v >> 1) & 1, b = v & 1;   // mat: 0 X, 1 Y
+    const T *R = mat == 0 ? HW : SW;
+    T *out = mat == 0 ? X : Y;
+    const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
+    for (int64_t qb = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * 2; qb < nnzN; qb += nwarps * 2) {
+        const int64_t q = qb + ((threadIdx.x >> 4) & 1);
+        T acc = T(0);
+        const int64_t t1 = q < nnzN ? Crp[q + 1] : 0;
+#pragma unroll 4
+        for (int64_t t = q < nnzN ? Crp[q] : 0; t < t1; ++t) {
+            const T *l = W + (int64_t)Ca[t] * BM * BN + a;
+            const T *rr = R + (int64_t)Cb[t] * BM * BN + b;
+#pragma unroll
+            for (int kk = 0; kk < BM / 2; ++kk) {
+                const int k = half * (BM / 2) + kk;
+                acc = fma(l[k * BN], rr[k * BN], acc);
+            }
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        if (half == 0 && q < nnzN) out[q * 4 + a * 2 + b] = acc;
+    }
+}
+
 // The FP32 contraction by P_N rows: a CTA takes row J (outputs (J, J2)); the
 // W and D blocks of W's column J (every triple of the row draws its left block
 // from them) are staged in shared memory once, so per triple only the H'D and
@@ -1393,6 +1428,7 @@ void release(Dev &d) {
                     d.Ndiag, d.HS, d.Hin, d.W, d.D, d.G, d.Gp, d.HW, d.SW, d.HD, d.SD, d.h0, d.s0, d.X,
                     d.Y, d.h2, d.s2, d.keep, d.nrm, d.fbuf, d.Nrp, d.WcolRp, d.WcolIdx, d.CaSlot};
     for (void *p : ptrs) cudaFree(p);
+    cudaFree(d.fx.base);
     d = Dev{};
 }
 
@@ -1412,6 +1448,10 @@ int set_HS(Dev &d, const double *H, const double *S, bool on_device, double eps,
     }
     shift_pack_kernel<<<blocks_for(d.nnzH * bb, 256), 256, 0, st>>>(d.nnzH, (int)bb, Hc, Sc, d.keep, state, d.HS);
     LAUNCHED();
+    if (d.fx.base != nullptr) {
+        const int rc = fx_set_HS(d, st);
+        if (rc != OMM_OK) return rc;
+    }
     return norms(d, NRM_HS, nullptr, st);
 }
 
@@ -1471,6 +1511,8 @@ int products(Dev &d, const double *Din, double *HDo, double *SDo, const double *
         DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, true><<<blocks_for(d.nnzHW * 32, NT), NT, 0, st>>>(
                                          d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS, Din, HDo, SDo, d.nHS, nDin,
                                          d.screen_eps2, state)));
+    } else if (d.fx.base != nullptr) {
+        return fx_products(d, Din, HDo, SDo, state, st);
     } else {
         DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, false><<<blocks_for(d.nnzHW * 32, NT), NT, 0, st>>>(
                                          d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS, Din, HDo, SDo, nullptr, nullptr, 0.0,
@@ -1492,12 +1534,21 @@ int contract(Dev &d, const double *Wl, const double *Dl, const double *HDr, cons
     }
     // without screening D^T H'D and D^T S D are formed on the upper triangle of P_N
     // and mirrored to the lower one (H' and S are symmetric); with D = W (the start,
-    // the density matrices) every block of every output is formed
+    // the density matrices) X and Y are all there is
     const bool sym = Dl != Wl;
-    DISPATCH_BLOCKS(d.bm, d.bn, (contract_kernel<BM, BN, false><<<blocks_for(d.nnzN * 32, NT), NT, 0, st>>>(
-                                     d.nnzN, d.Crp, d.Ca, d.Cb, Wl, Dl, HDr, SDr, Xo, Yo, h2o, s2o, nullptr,
-                                     nullptr, nullptr, nullptr, 0.0, sym ? d.Ntr : nullptr, state)));
-    LAUNCHED();
+    if (d.fx.base != nullptr) {
+        const int rc = fx_contract(d, Wl, Dl, HDr, SDr, Xo, Yo, h2o, s2o, d.Ntr, state, st);
+        if (rc != OMM_OK) return rc;
+    } else if (!sym) {
+        DISPATCH_BLOCKS(d.bm, d.bn, (contract_xy_kernel<BM, BN><<<blocks_for(d.nnzN * 16, NT), NT, 0, st>>>(
+                                         d.nnzN, d.Crp, d.Ca, d.Cb, Wl, HDr, SDr, Xo, Yo, state)));
+        LAUNCHED();
+    } else {
+        DISPATCH_BLOCKS(d.bm, d.bn, (contract_kernel<BM, BN, false><<<blocks_for(d.nnzN * 32, NT), NT, 0, st>>>(
+                                         d.nnzN, d.Crp, d.Ca, d.Cb, Wl, Dl, HDr, SDr, Xo, Yo, h2o, s2o, nullptr,
+                                         nullptr, nullptr, nullptr, 0.0, d.Ntr, state)));
+        LAUNCHED();
+    }
     if (sym) {
         mirror_kernel<double><<<blocks_for(d.nnzN * 4, 256), 256, 0, st>>>(d.nnzN, d.Ntr, h2o, s2o, state);
         LAUNCHED();
@@ -1549,6 +1600,8 @@ int gradient(Dev &d, const DevState *state, cudaStream_t st) {
         DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, true><<<blocks_for(d.nnzW * 16, NT), NT, 0, st>>>(
                                          d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW, d.SW, d.h0, d.s0, d.G, d.nHW,
                                          d.nSW, d.nh0, d.ns0, d.screen_eps2, state)));
+    } else if (d.fx.base != nullptr) {
+        return fx_gradient(d, state, st);
     } else {
         DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, false><<<blocks_for(d.nnzW * 16, NT), NT, 0, st>>>(
                                          d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW, d.SW, d.h0, d.s0, d.G, nullptr,
