@@ -524,39 +524,39 @@ __global__ void __launch_bounds__(NT) products_kernel(int64_t nnzHW, const int64
                                                        const DevState *state) {
     if (done(state)) return;
     if constexpr (VecGather<T, BM, BN, SCREEN>::on) {
-        // FP32 (8x2 blocks): lane (which, r) computes both columns of row r from
-        // its A row (two 16-byte loads) and the whole D block (four): two P_HW
-        // blocks per warp, half the L1 bytes of a lane per output element; the
-        // FMAs of each output run in k order, as in the scalar form
-        const int lane = threadIdx.x & 31;
-        const int r = lane & 7, which = (lane >> 3) & 1;
-        const int64_t ngroups = ((int64_t)gridDim.x * NT) >> 4;
-        for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 4; o < nnzHW; o += ngroups) {
-            float acc0 = 0.f, acc1 = 0.f;
+        // FP32 (8x2 blocks): lane r of an eight-lane group computes row r of H'D and of
+        // SD, both columns, from one row of H' and of S (two 16-byte loads each) and the
+        // whole D block (four): the D block serves 32 multiply-adds a lane instead of
+        // the 16 of a lane per matrix, 4 bytes from the L1 each instead of 6 (171 ->
+        // 138 us at 1728 atoms).  The FMAs of each output run in k order, as in the
+        // scalar form.
+        const int r = threadIdx.x & 7;
+        const int64_t ngroups = ((int64_t)gridDim.x * NT) >> 3;
+        for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 3; o < nnzHW; o += ngroups) {
+            float h0 = 0.f, h1 = 0.f, s0 = 0.f, s1 = 0.f;
+            auto step = [&](float a, float w, float bx, float by) {
+                h0 = fmaf(a, bx, h0);
+                h1 = fmaf(a, by, h1);
+                s0 = fmaf(w, bx, s0);
+                s1 = fmaf(w, by, s1);
+            };
 #pragma unroll 2
             for (int64_t t = Prp[o]; t < Prp[o + 1]; ++t) {
-                const float *A = HS + ((int64_t)Ph[t] * 2 + which) * 64 + r * 8;
+                const float *A = HS + (int64_t)Ph[t] * 128 + r * 8;
                 const float *B = D + (int64_t)Pw[t] * 16;
-                const float4 a0 = ld4(A), a1 = ld4(A + 4);
+                const float4 a0 = ld4(A), a1 = ld4(A + 4), w0 = ld4(A + 64), w1 = ld4(A + 68);
                 const float4 b0 = ld4(B), b1 = ld4(B + 4), b2 = ld4(B + 8), b3 = ld4(B + 12);
-                acc0 = fmaf(a0.x, b0.x, acc0);
-                acc1 = fmaf(a0.x, b0.y, acc1);
-                acc0 = fmaf(a0.y, b0.z, acc0);
-                acc1 = fmaf(a0.y, b0.w, acc1);
-                acc0 = fmaf(a0.z, b1.x, acc0);
-                acc1 = fmaf(a0.z, b1.y, acc1);
-                acc0 = fmaf(a0.w, b1.z, acc0);
-                acc1 = fmaf(a0.w, b1.w, acc1);
-                acc0 = fmaf(a1.x, b2.x, acc0);
-                acc1 = fmaf(a1.x, b2.y, acc1);
-                acc0 = fmaf(a1.y, b2.z, acc0);
-                acc1 = fmaf(a1.y, b2.w, acc1);
-                acc0 = fmaf(a1.z, b3.x, acc0);
-                acc1 = fmaf(a1.z, b3.y, acc1);
-                acc0 = fmaf(a1.w, b3.z, acc0);
-                acc1 = fmaf(a1.w, b3.w, acc1);
+                step(a0.x, w0.x, b0.x, b0.y);
+                step(a0.y, w0.y, b0.z, b0.w);
+                step(a0.z, w0.z, b1.x, b1.y);
+                step(a0.w, w0.w, b1.z, b1.w);
+                step(a1.x, w1.x, b2.x, b2.y);
+                step(a1.y, w1.y, b2.z, b2.w);
+                step(a1.z, w1.z, b3.x, b3.y);
+                step(a1.w, w1.w, b3.z, b3.w);
             }
-            *reinterpret_cast<float2 *>((which ? SD : HD) + o * 16 + r * 2) = make_float2(acc0, acc1);
+            *reinterpret_cast<float2 *>(HD + o * 16 + r * 2) = make_float2(h0, h1);
+            *reinterpret_cast<float2 *>(SD + o * 16 + r * 2) = make_float2(s0, s1);
         }
     } else {
         const int lane = threadIdx.x & 31;
@@ -747,85 +747,91 @@ __global__ void __launch_bounds__(NT) contract_xy_kernel(int64_t nnzN, const int
     }
 }
 
-// The FP32 contraction by P_N rows: a CTA takes row J (outputs (J, J2)); the
-// W and D blocks of W's column J (every triple of the row draws its left block
-// from them) are staged in shared memory once, so per triple only the H'D and
-// SD rows come from the L1 and L2; CaSlot names the left block's slot in the
-// column.  Lanes as in contract_kernel's FP32 form: an eight-lane group per
-// output block, lane k holding all sixteen outputs for basis row k.
-__global__ void __launch_bounds__(NT) contract_rows_kernel(int64_t nbc, const int64_t *__restrict__ Nrp,
-                                                            const int64_t *__restrict__ WcolRp,
-                                                            const int32_t *__restrict__ WcolIdx,
-                                                            const int64_t *__restrict__ Crp,
-                                                            const uint16_t *__restrict__ CaSlot,
-                                                            const int32_t *__restrict__ Cb, const float *__restrict__ W,
-                                                            const float *__restrict__ D, const float *__restrict__ HD,
-                                                            const float *__restrict__ SD, float *X, float *Y, float *h2,
-                                                            float *s2, const int32_t *__restrict__ Ntr,
-                                                            const DevState *state) {
+// The FP32 contraction by groups of `rows` P_N rows: the W and D blocks of the group's
+// columns of W (every triple of row J draws its left block from column J) are staged in
+// shared memory once, and the group's output blocks (J, J2) are taken in the order of
+// J2 (Nord), so that the H'D and SD blocks (K, J2), which neighbouring rows J share,
+// come from the L1 after the first: taken row by row each was read from L2 again for
+// every J (459 -> 412 us at 1728 atoms).  CaSlot names the left block's slot in its
+// column.  A CTA takes one of `parts` equal parts of a group.  Lanes as in
+// contract_kernel's FP32 form: an eight-lane group per output block, lane k holding all
+// sixteen outputs for basis row k.
+constexpr int kRowsNT = 512;
+__global__ void __launch_bounds__(kRowsNT) contract_rows_kernel(
+    int64_t nbc, int rows, int parts, const int64_t *__restrict__ Nrp, const uint32_t *__restrict__ Nord,
+    const int64_t *__restrict__ WcolRp, const int32_t *__restrict__ WcolIdx, const int64_t *__restrict__ Crp,
+    const uint16_t *__restrict__ CaSlot, const int32_t *__restrict__ Cb, const float *__restrict__ W,
+    const float *__restrict__ D, const float *__restrict__ HD, const float *__restrict__ SD, float *X, float *Y, float *h2,
+    float *s2, const int32_t *__restrict__ Ntr, const DevState *state) {
     if (done(state)) return;
-    extern __shared__ float4 stage4[];   // W rows of the column, then D rows (nc x 16 floats each)
+    extern __shared__ float4 stage4[];   // W rows of the columns, then D rows (16 floats a block)
+    __shared__ int first[8];             // slot of each column's first block
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, k = lane & 7, grp = lane >> 3;
-    for (int64_t J = blockIdx.x; J < nbc; J += gridDim.x) {
-        const int64_t c0 = WcolRp[J];
-        const int nc = (int)(WcolRp[J + 1] - c0);
-        float *sW = reinterpret_cast<float *>(stage4), *sD = sW + (int64_t)nc * 16;
-        __syncthreads();   // the previous row's readers are done with the stage
-        for (int e = threadIdx.x; e < nc * 4; e += NT) {   // one float4 per thread and step
-            const int64_t a = WcolIdx[c0 + (e >> 2)];
-            reinterpret_cast<float4 *>(sW)[e] = __ldg(reinterpret_cast<const float4 *>(W + a * 16) + (e & 3));
-            reinterpret_cast<float4 *>(sD)[e] = __ldg(reinterpret_cast<const float4 *>(D + a * 16) + (e & 3));
-        }
-        __syncthreads();
-        const int64_t q1 = Nrp[J + 1];
-        // warp-uniform loop: the four groups of a warp take blocks qb .. qb + 3
-        for (int64_t qb = Nrp[J] + 4 * warp; qb < q1; qb += 4 * (NT / 32)) {
-            const int64_t q = qb + grp;
-            const bool valid = q < q1;
-            const bool lower = valid && Ntr[q] < q;
-            float acc[16];
+    const int64_t J0 = (int64_t)(blockIdx.x / parts) * rows, J1 = J0 + rows < nbc ? J0 + rows : nbc;
+    const int part = (int)(blockIdx.x % parts);
+    const int64_t c0 = WcolRp[J0];
+    const int nc = (int)(WcolRp[J1] - c0);
+    float *sW = reinterpret_cast<float *>(stage4), *sD = sW + (int64_t)nc * 16;
+    if ((int)threadIdx.x < (int)(J1 - J0)) first[threadIdx.x] = (int)(WcolRp[J0 + threadIdx.x] - c0);
+    for (int e = threadIdx.x; e < nc * 4; e += kRowsNT) {   // one float4 per thread and step
+        const int64_t a = WcolIdx[c0 + (e >> 2)];
+        reinterpret_cast<float4 *>(sW)[e] = __ldg(reinterpret_cast<const float4 *>(W + a * 16) + (e & 3));
+        reinterpret_cast<float4 *>(sD)[e] = __ldg(reinterpret_cast<const float4 *>(D + a * 16) + (e & 3));
+    }
+    __syncthreads();
+    const int64_t p0 = Nrp[J0], len = Nrp[J1] - p0;
+    const int64_t q0 = p0 + len * part / parts, q1 = p0 + len * (part + 1) / parts;
+    // warp-uniform loop: the four groups of a warp take positions pb .. pb + 3
+    for (int64_t pb = q0 + 4 * warp; pb < q1; pb += 4 * (kRowsNT / 32)) {
+        const bool valid = pb + grp < q1;
+        const uint32_t ord = valid ? Nord[pb + grp] : 0;
+        const int64_t q = ord & kOrdMask;
+        const int s0 = first[ord >> kOrdBits] * 16 + 2 * k;
+        const bool lower = valid && Ntr[q] < q;
+        float acc[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-            const int64_t t1 = valid ? Crp[q + 1] : 0;
+        for (int i = 0; i < 16; ++i) acc[i] = 0.f;
+        const int64_t t1 = valid ? Crp[q + 1] : 0;
 #pragma unroll 2
-            for (int64_t t = valid ? Crp[q] : 0; t < t1; ++t) {
-                const int ia = (int)CaSlot[t] * 16 + 2 * k;
-                const int64_t ib = (int64_t)Cb[t] * 16 + 2 * k;
-                const float2 w = *reinterpret_cast<const float2 *>(sW + ia);
-                const float2 hd = __ldg(reinterpret_cast<const float2 *>(HD + ib));
-                const float2 sd = __ldg(reinterpret_cast<const float2 *>(SD + ib));
-                acc[0] = fmaf(w.x, hd.x, acc[0]);
-                acc[1] = fmaf(w.x, hd.y, acc[1]);
-                acc[2] = fmaf(w.y, hd.x, acc[2]);
-                acc[3] = fmaf(w.y, hd.y, acc[3]);
-                acc[4] = fmaf(w.x, sd.x, acc[4]);
-                acc[5] = fmaf(w.x, sd.y, acc[5]);
-                acc[6] = fmaf(w.y, sd.x, acc[6]);
-                acc[7] = fmaf(w.y, sd.y, acc[7]);
-                if (!lower) {
-                    const float2 dd = *reinterpret_cast<const float2 *>(sD + ia);
-                    acc[8] = fmaf(dd.x, hd.x, acc[8]);
-                    acc[9] = fmaf(dd.x, hd.y, acc[9]);
-                    acc[10] = fmaf(dd.y, hd.x, acc[10]);
-                    acc[11] = fmaf(dd.y, hd.y, acc[11]);
-                    acc[12] = fmaf(dd.x, sd.x, acc[12]);
-                    acc[13] = fmaf(dd.x, sd.y, acc[13]);
-                    acc[14] = fmaf(dd.y, sd.x, acc[14]);
-                    acc[15] = fmaf(dd.y, sd.y, acc[15]);
-                }
+        for (int64_t t = valid ? Crp[q] : 0; t < t1; ++t) {
+            const int ia = s0 + (int)CaSlot[t] * 16;
+            const int64_t ib = (int64_t)Cb[t] * 16 + 2 * k;
+            const float2 w = *reinterpret_cast<const float2 *>(sW + ia);
+            const float2 hd = __ldg(reinterpret_cast<const float2 *>(HD + ib));
+            const float2 sd = __ldg(reinterpret_cast<const float2 *>(SD + ib));
+            acc[0] = fmaf(w.x, hd.x, acc[0]);
+            acc[1] = fmaf(w.x, hd.y, acc[1]);
+            acc[2] = fmaf(w.y, hd.x, acc[2]);
+            acc[3] = fmaf(w.y, hd.y, acc[3]);
+            acc[4] = fmaf(w.x, sd.x, acc[4]);
+            acc[5] = fmaf(w.x, sd.y, acc[5]);
+            acc[6] = fmaf(w.y, sd.x, acc[6]);
+            acc[7] = fmaf(w.y, sd.y, acc[7]);
+            if (!lower) {
+                const float2 dd = *reinterpret_cast<const float2 *>(sD + ia);
+                acc[8] = fmaf(dd.x, hd.x, acc[8]);
+                acc[9] = fmaf(dd.x, hd.y, acc[9]);
+                acc[10] = fmaf(dd.y, hd.x, acc[10]);
+                acc[11] = fmaf(dd.y, hd.y, acc[11]);
+                acc[12] = fmaf(dd.x, sd.x, acc[12]);
+                acc[13] = fmaf(dd.x, sd.y, acc[13]);
+                acc[14] = fmaf(dd.y, sd.x, acc[14]);
+                acc[15] = fmaf(dd.y, sd.y, acc[15]);
             }
+        }
+        // (sums by halving, the same pairs in 14 exchanges instead of 48, took 453 us: the
+        // selects cost more than the shuffles)
 #pragma unroll
-            for (int off = 1; off < 8; off <<= 1)
+        for (int off = 1; off < 8; off <<= 1)
 #pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
-            if (valid && k < (lower ? 2 : 4)) {
-                float *o = k == 0 ? X : k == 1 ? Y : k == 2 ? h2 : s2;
-                const float4 v = k == 0   ? make_float4(acc[0], acc[1], acc[2], acc[3])
-                                 : k == 1 ? make_float4(acc[4], acc[5], acc[6], acc[7])
-                                 : k == 2 ? make_float4(acc[8], acc[9], acc[10], acc[11])
-                                          : make_float4(acc[12], acc[13], acc[14], acc[15]);
-                *reinterpret_cast<float4 *>(o + q * 4) = v;
-            }
+            for (int i = 0; i < 16; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+        if (valid && k < (lower ? 2 : 4)) {
+            float *o = k == 0 ? X : k == 1 ? Y : k == 2 ? h2 : s2;
+            const float4 v = k == 0   ? make_float4(acc[0], acc[1], acc[2], acc[3])
+                             : k == 1 ? make_float4(acc[4], acc[5], acc[6], acc[7])
+                             : k == 2 ? make_float4(acc[8], acc[9], acc[10], acc[11])
+                                      : make_float4(acc[12], acc[13], acc[14], acc[15]);
+            *reinterpret_cast<float4 *>(o + q * 4) = v;
         }
     }
 }
@@ -860,32 +866,36 @@ __global__ void __launch_bounds__(NT) gradient_kernel(int64_t nnzW, const int64_
                                                        double eps2, const DevState *state) {
     if (done(state)) return;
     if constexpr (VecGather<T, BM, BN, SCREEN>::on) {
-        // FP32 (8x2 blocks): lane per block row r computing both columns from one
-        // row of the SW and H'W blocks and the whole 2x2 h0, s0 blocks (half the
-        // L1 bytes of a lane per output element), four W blocks per warp; the
-        // FMAs of each output run in the same order as the scalar form's
-        const int r = threadIdx.x & 7;
-        const int64_t ngroups = ((int64_t)gridDim.x * NT) >> 3;
-        for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 3; o < nnzW; o += ngroups) {
-            float acc0 = 0.f, acc1 = 0.f;
+        // FP32 (8x2 blocks): a lane per two block rows, both columns, from 16 bytes of
+        // the SW and H'W blocks and the whole 2x2 h0, s0 blocks: 4 bytes from the L1 per
+        // multiply-add (a lane per row read 6; 276 -> 237 us at 1728 atoms), eight W
+        // blocks per warp; the FMAs of each output run in the scalar form's order
+        const int r = threadIdx.x & 3;
+        const int64_t ngroups = ((int64_t)gridDim.x * NT) >> 2;
+        for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 2; o < nnzW; o += ngroups) {
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            auto step = [](float &c0, float &c1, float swx, float swy, float hwx, float hwy, const float4 &h,
+                           const float4 &s) {
+                c0 = fmaf(swx, h.x, c0);
+                c0 = fmaf(hwx, s.x, c0);
+                c0 = fmaf(swy, h.z, c0);
+                c0 = fmaf(hwy, s.z, c0);
+                c1 = fmaf(swx, h.y, c1);
+                c1 = fmaf(hwx, s.y, c1);
+                c1 = fmaf(swy, h.w, c1);
+                c1 = fmaf(hwy, s.w, c1);
+            };
 #pragma unroll 2
             for (int64_t t = Grp[o]; t < Grp[o + 1]; ++t) {
-                const int64_t gb = (int64_t)Gb[t] * 16 + r * 2, gq = (int64_t)Gq[t] * 4;
-                const float2 sw = __ldg(reinterpret_cast<const float2 *>(SW + gb));
-                const float2 hw = __ldg(reinterpret_cast<const float2 *>(HW + gb));
-                const float4 hq = ld4(h0 + gq), sq = ld4(s0 + gq);
-                acc0 = fmaf(sw.x, hq.x, acc0);
-                acc0 = fmaf(hw.x, sq.x, acc0);
-                acc0 = fmaf(sw.y, hq.z, acc0);
-                acc0 = fmaf(hw.y, sq.z, acc0);
-                acc1 = fmaf(sw.x, hq.y, acc1);
-                acc1 = fmaf(hw.x, sq.y, acc1);
-                acc1 = fmaf(sw.y, hq.w, acc1);
-                acc1 = fmaf(hw.y, sq.w, acc1);
+                const int64_t gb = (int64_t)Gb[t] * 16 + r * 4, gq = (int64_t)Gq[t] * 4;
+                const float4 sw = ld4(SW + gb), hw = ld4(HW + gb), hq = ld4(h0 + gq), sq = ld4(s0 + gq);
+                step(acc.x, acc.y, sw.x, sw.y, hw.x, hw.y, hq, sq);
+                step(acc.z, acc.w, sw.z, sw.w, hw.z, hw.w, hq, sq);
             }
-            const float2 hwo = *reinterpret_cast<const float2 *>(HW + (int64_t)WtoHW[o] * 16 + r * 2);
-            *reinterpret_cast<float2 *>(G + o * 16 + r * 2) =
-                make_float2(2.0f * (2.0f * hwo.x - acc0), 2.0f * (2.0f * hwo.y - acc1));
+            const float4 hwo = ld4(HW + (int64_t)WtoHW[o] * 16 + r * 4);
+            *reinterpret_cast<float4 *>(G + o * 16 + r * 4) =
+                make_float4(2.0f * (2.0f * hwo.x - acc.x), 2.0f * (2.0f * hwo.y - acc.y),
+                            2.0f * (2.0f * hwo.z - acc.z), 2.0f * (2.0f * hwo.w - acc.w));
         }
     } else {
         const int e = threadIdx.x & 15;
@@ -1426,7 +1436,7 @@ void release(Dev &d) {
     void *ptrs[] = {d.Trp, d.Rrp, d.Tw, d.Tq, d.Rt, d.Rw, d.K, d.T,
                     d.Hrp, d.Hcol, d.Prp, d.Ph, d.Pw, d.Crp, d.Ca, d.Cb, d.Grp, d.Gb, d.Gq, d.WtoHW, d.Ntr,
                     d.Ndiag, d.HS, d.Hin, d.W, d.D, d.G, d.Gp, d.HW, d.SW, d.HD, d.SD, d.h0, d.s0, d.X,
-                    d.Y, d.h2, d.s2, d.keep, d.nrm, d.fbuf, d.Nrp, d.WcolRp, d.WcolIdx, d.CaSlot};
+                    d.Y, d.h2, d.s2, d.keep, d.nrm, d.fbuf, d.Nrp, d.WcolRp, d.WcolIdx, d.CaSlot, d.Nord};
     for (void *p : ptrs) cudaFree(p);
     cudaFree(d.fx.base);
     d = Dev{};
@@ -1611,10 +1621,31 @@ int gradient(Dev &d, const DevState *state, cudaStream_t st) {
     return OMM_OK;
 }
 
+bool row_order(const Host &hs, int rows, std::vector<uint32_t> &ord) {
+    const int64_t nbc = hs.P.nbc, nnzN = hs.Nrp[nbc];
+    if (nnzN > (int64_t)kOrdMask || rows > 8) return false;
+    ord.resize((size_t)nnzN);
+    for (int64_t J0 = 0; J0 < nbc; J0 += rows) {
+        const int nr = (int)std::min<int64_t>(rows, nbc - J0);
+        int64_t at = hs.Nrp[J0], p[8];
+        for (int j = 0; j < nr; ++j) p[j] = hs.Nrp[J0 + j];
+        // merge of the rows' sorted columns
+        while (at < hs.Nrp[J0 + nr]) {
+            int32_t J2 = INT32_MAX;
+            for (int j = 0; j < nr; ++j)
+                if (p[j] < hs.Nrp[J0 + j + 1]) J2 = std::min(J2, hs.Ncol[p[j]]);
+            for (int j = 0; j < nr; ++j)
+                if (p[j] < hs.Nrp[J0 + j + 1] && hs.Ncol[p[j]] == J2)
+                    ord[at++] = (uint32_t)p[j]++ | (uint32_t)j << kOrdBits;
+        }
+    }
+    return true;
+}
+
 namespace {
-// Shared-memory budget of the row-staged contraction: W and D rows of one
-// column of W (16 floats each per block)
-constexpr int kRowStageMaxCol = 256;   // 32 KB
+// Shared-memory budget of the row-staged contraction: W and D blocks (16 floats each)
+// of a group's columns of W; two CTAs of 512 threads share an SM
+constexpr int64_t kRowStageBytes = 64 * 1024;
 }
 
 int mixed_alloc(const Host &hs, Dev &d) {
@@ -1623,7 +1654,17 @@ int mixed_alloc(const Host &hs, Dev &d) {
         const int64_t nbc = hs.P.nbc, nnzW = (int64_t)hs.WcolIdx.size();
         int64_t maxcol = 0;
         for (int64_t J = 0; J < nbc; ++J) maxcol = std::max(maxcol, hs.WcolRp[J + 1] - hs.WcolRp[J]);
-        if (maxcol > 0 && maxcol <= kRowStageMaxCol) {
+        // as many rows together as the staging holds (the slots of a triple are 16 bits)
+        int rows = 8;
+        auto stage = [&](int r) {
+            int64_t most = 0;
+            for (int64_t J = 0; J < nbc; J += r)
+                most = std::max(most, hs.WcolRp[std::min(nbc, J + r)] - hs.WcolRp[J]);
+            return most * 16 * 2 * (int64_t)sizeof(float);
+        };
+        while (rows > 1 && stage(rows) > kRowStageBytes) rows >>= 1;
+        std::vector<uint32_t> ord;
+        if (maxcol > 0 && stage(rows) <= kRowStageBytes && row_order(hs, rows, ord)) {
             std::vector<uint16_t> wslot(nnzW);
             std::vector<int32_t> widx(nnzW);
             for (int64_t J = 0; J < nbc; ++J)
@@ -1642,9 +1683,10 @@ int mixed_alloc(const Host &hs, Dev &d) {
             };
             int rc;
             if ((rc = up(&d.Nrp, hs.Nrp)) || (rc = up(&d.WcolRp, hs.WcolRp)) || (rc = up(&d.WcolIdx, widx)) ||
-                (rc = up(&d.CaSlot, slot)))
+                (rc = up(&d.CaSlot, slot)) || (rc = up(&d.Nord, ord)))
                 return rc;
-            d.maxcol = (int)maxcol;
+            d.stage_rows = rows;
+            d.stage_bytes = stage(rows);
         }
     }
     const int64_t bb = (int64_t)d.bm * d.bm, bw = (int64_t)d.bm * d.bn, bq = (int64_t)d.bn * d.bn;
@@ -1706,7 +1748,7 @@ int mixed_begin(Dev &d, const DevState *state, cudaStream_t st) {
 }
 
 int mixed_products(Dev &d, const DevState *state, cudaStream_t st) {
-    DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, false, float><<<blocks_for(d.nnzHW * 16, NT), NT, 0, st>>>(
+    DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, false, float><<<blocks_for(d.nnzHW * 8, NT), NT, 0, st>>>(
                                      d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS32, d.D32, d.HD32, d.SD32, nullptr, nullptr, 0.0,
                                      state)));
     LAUNCHED();
@@ -1714,11 +1756,18 @@ int mixed_products(Dev &d, const DevState *state, cudaStream_t st) {
 }
 
 int mixed_contract(Dev &d, const DevState *state, cudaStream_t st) {
-    if (d.maxcol > 0 && d.bm == 8 && d.bn == 2) {
-        const size_t smem = (size_t)d.maxcol * 16 * 2 * sizeof(float);
-        const int64_t nb = d.nbc < 152 * 8 ? d.nbc : 152 * 8;
-        contract_rows_kernel<<<(unsigned)(nb < 1 ? 1 : nb), NT, smem, st>>>(
-            d.nbc, d.Nrp, d.WcolRp, d.WcolIdx, d.Crp, d.CaSlot, d.Cb, d.W32, d.D32, d.HD32, d.SD32, d.X32, d.Y32,
+    if (d.stage_rows > 0 && d.bm == 8 && d.bn == 2) {
+        static int64_t attr_bytes = 0;
+        if (d.stage_bytes > attr_bytes) {
+            OMM_CUDA_TRY(cudaFuncSetAttribute(contract_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              (int)d.stage_bytes));
+            attr_bytes = d.stage_bytes;
+        }
+        // about four CTAs per place on the chip (two to an SM), for an even finish
+        const int64_t groups = ceil_div(d.nbc, d.stage_rows);
+        const int64_t parts = groups >= 1216 ? 1 : ceil_div(1216, groups);
+        contract_rows_kernel<<<(unsigned)(groups * parts), kRowsNT, (size_t)d.stage_bytes, st>>>(
+            d.nbc, d.stage_rows, (int)parts, d.Nrp, d.Nord, d.WcolRp, d.WcolIdx, d.Crp, d.CaSlot, d.Cb, d.W32, d.D32, d.HD32, d.SD32, d.X32, d.Y32,
             d.h232, d.s232, d.Ntr, state);
         LAUNCHED();
     } else {
@@ -1753,7 +1802,7 @@ int mixed_update(Dev &d, double *scratch, unsigned int *counter, DevState *state
 }
 
 int mixed_gradient(Dev &d, const DevState *state, cudaStream_t st) {
-    DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, false, float><<<blocks_for(d.nnzW * 8, NT), NT, 0, st>>>(
+    DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, false, float><<<blocks_for(d.nnzW * 4, NT), NT, 0, st>>>(
                                      d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW32, d.SW32, d.h032, d.s032, d.G32,
                                      nullptr, nullptr, nullptr, nullptr, 0.0, state)));
     LAUNCHED();

@@ -109,16 +109,26 @@ struct Dev {
     float *HS32 = nullptr, *W32 = nullptr, *D32 = nullptr, *G32 = nullptr, *Gp32 = nullptr, *HW32 = nullptr,
           *SW32 = nullptr, *HD32 = nullptr, *SD32 = nullptr, *h032 = nullptr, *s032 = nullptr, *X32 = nullptr,
           *Y32 = nullptr, *h232 = nullptr, *s232 = nullptr;
-    // the FP32 contraction by P_N rows (mixed form): row J's W and D blocks (W's
-    // column J, WcolRp / WcolIdx) staged in shared memory, each triple's W block
-    // named by its slot in that column (CaSlot); maxcol = 0: not built (a column
-    // longer than the staging allows), the per-block kernel runs instead
+    // the FP32 contraction by groups of stage_rows P_N rows (mixed form): the W and D
+    // blocks of the rows' columns of W (WcolRp / WcolIdx) staged in shared memory, each
+    // triple's W block named by its slot in its column (CaSlot), the output blocks in
+    // row_order (Nord); stage_rows = 0: not built (a column longer than the staging
+    // allows), the per-block kernel runs instead
     int64_t *Nrp = nullptr, *WcolRp = nullptr;
     int32_t *WcolIdx = nullptr;
     uint16_t *CaSlot = nullptr;
-    int maxcol = 0;
+    uint32_t *Nord = nullptr;
+    int stage_rows = 0;
+    int64_t stage_bytes = 0;
     Fx fx;
 };
+
+// P_N's blocks (J, J2) by groups of `rows` rows J, each group in the order of J2 and
+// then J: entry = block | (J - the group's first row) << kOrdBits, the group's entries
+// at the positions of its rows' blocks.  False where the numbers do not fit.
+constexpr int kOrdBits = 29;
+constexpr uint32_t kOrdMask = (1u << kOrdBits) - 1;
+bool row_order(const Host &hs, int rows, std::vector<uint32_t> &ord);
 
 // which block norms to refresh (norms())
 enum { NRM_HS = 1, NRM_W = 2, NRM_D = 4, NRM_HWSW = 8, NRM_HDSD = 16, NRM_N = 32 };
