@@ -12,6 +12,7 @@
 
 #include "linemin.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 
 namespace omm {
 namespace {
@@ -118,6 +119,7 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int n, const double *__restr
                                                      double *partials, unsigned int *counter,
                                                      DevState *state, double *coeffs_out,
                                                      int do_linemin) {
+    pdl_wait();
     if (state != nullptr && *((volatile int *)&state->done)) return;
     __shared__ double Xt[TILE][TILE + 1];
     __shared__ double red[(NT / 32) * NC];
@@ -200,6 +202,7 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
                                                         int64_t ldz, double *partials,
                                                         unsigned int *counter, DevState *state,
                                                         int mode, DigitOut hsw) {
+    pdl_wait();
     if (*((volatile int *)&state->done)) return;
     __shared__ double Tt[4][TILE][TILE + 1];
     __shared__ double red[(NT / 32) * NE];
@@ -299,6 +302,7 @@ __global__ void __launch_bounds__(NT) update_kernel(int m, int n, double *W, con
                                                      double *HW, const double *__restrict__ HD, double *SW,
                                                      const double *__restrict__ SD, const DevState *state,
                                                      DigitOut wd, DigitOut swhw) {
+    pdl_wait();
     if (*((volatile const int *)&state->done)) return;
     __shared__ double tH[TILE][TILE + 1];
     __shared__ double tS[TILE][TILE + 1];
@@ -349,6 +353,7 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t mn, const double *__re
                                                    const double *__restrict__ D, double *partials,
                                                    unsigned int *counter, DevState *state,
                                                    int first) {
+    pdl_wait();
     if (*((volatile int *)&state->done)) return;
     __shared__ double red[(NT / 32) * ND];
     double v[ND] = {0.0, 0.0, 0.0};
@@ -390,6 +395,7 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t mn, const double *__re
 // D = -Z + beta D (D = -Z on a restart); Gp <- G
 __global__ void direction_kernel(int m, int n, const double *__restrict__ G, const double *__restrict__ Zg,
                                  double *Gp, double *D, const DevState *state, DigitOut dd) {
+    pdl_wait();
     if (*((volatile const int *)&state->done)) return;
     const double beta = state->beta;
     const bool restart = state->restart != 0;
@@ -534,8 +540,8 @@ int launch_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh
     const double *Y = Z + (int64_t)n * ldz;
     const double *h2 = Z + n;
     const double *s2 = Z + n + (int64_t)n * ldz;
-    coeffs_kernel<<<red_blocks_for_tiles(n), NT, 0, st>>>(n, h0, s0, ldh, X, Y, h2, s2, ldz, scratch,
-                                                          counter, state, coeffs_out, do_linemin ? 1 : 0);
+    OMM_CUDA_TRY(launch_pdl(coeffs_kernel, dim3(red_blocks_for_tiles(n)), dim3(NT), 0, st, n, h0, s0, ldh, X, Y, h2,
+                            s2, ldz, scratch, counter, state, coeffs_out, do_linemin ? 1 : 0));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -545,7 +551,8 @@ int launch_update(int64_t m, int64_t n, double *W, const double *D, double *HW, 
                   const double *SD, const DevState *state, DigitOut wd, DigitOut swhw, cudaStream_t st) {
     int64_t nb = ceil_div(m, TILE) * ceil_div(n, TILE);
     if (nb > 152 * 8) nb = 152 * 8;
-    update_kernel<<<(unsigned)nb, NT, 0, st>>>((int)m, (int)n, W, D, HW, HD, SW, SD, state, wd, swhw);
+    OMM_CUDA_TRY(launch_pdl(update_kernel, dim3((unsigned)nb), dim3(NT), 0, st, (int)m, (int)n, W, D, HW, HD, SW,
+                            SD, state, wd, swhw));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -558,8 +565,8 @@ int launch_nn_update_energy(int n, double *h0, double *s0, int64_t ldh, const do
     const double *Y = Z + (int64_t)n * ldz;
     const double *h2 = Z + n;
     const double *s2 = Z + n + (int64_t)n * ldz;
-    nn_update_kernel<<<red_blocks_for_tiles(n), NT, 0, st>>>(n, h0, s0, ldh, X, Y, h2, s2, ldz,
-                                                             scratch, counter, state, mode, hsw);
+    OMM_CUDA_TRY(launch_pdl(nn_update_kernel, dim3(red_blocks_for_tiles(n)), dim3(NT), 0, st, n, h0, s0, ldh, X, Y,
+                            h2, s2, ldz, scratch, counter, state, mode, hsw));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -568,7 +575,8 @@ int launch_nn_update_energy(int n, double *h0, double *s0, int64_t ldh, const do
 int launch_dots_beta(int64_t mn, const double *G, const double *Zg, const double *Gp, const double *D,
                      double *scratch, unsigned int *counter, DevState *state, int first,
                      cudaStream_t st) {
-    dots_kernel<<<red_blocks_for_len(mn), NT, 0, st>>>(mn, G, Zg, Gp, D, scratch, counter, state, first);
+    OMM_CUDA_TRY(launch_pdl(dots_kernel, dim3(red_blocks_for_len(mn)), dim3(NT), 0, st, mn, G, Zg, Gp, D, scratch,
+                            counter, state, first));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -577,7 +585,7 @@ int launch_dots_beta(int64_t mn, const double *G, const double *Zg, const double
 int launch_direction(int64_t m, int64_t n, const double *G, const double *Zg, double *Gp, double *D,
                      const DevState *state, cudaStream_t st, DigitOut dd) {
     dim3 grid((unsigned)ceil_div(m, NT), (unsigned)(n < 1024 ? n : 1024));
-    direction_kernel<<<grid, NT, 0, st>>>((int)m, (int)n, G, Zg, Gp, D, state, dd);
+    OMM_CUDA_TRY(launch_pdl(direction_kernel, grid, dim3(NT), 0, st, (int)m, (int)n, G, Zg, Gp, D, state, dd));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;

@@ -22,6 +22,7 @@
 
 #include "chol.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 
 namespace omm {
 namespace chol {
@@ -37,6 +38,7 @@ constexpr int kLeafSmem = (2 * kLeaf * (kLeaf + 1) + 4 * kLeaf) * (int)sizeof(do
 // triangles inside the block are zeroed.
 __global__ void __launch_bounds__(kLeafThreads) chol_leaf_kernel(double *A, double *Y, int64_t m, int64_t n0, int s,
                                                                  DevState *state) {
+    pdl_wait();
     extern __shared__ double sm[];
     double(*a)[kLeaf + 1] = (double(*)[kLeaf + 1])sm;
     double(*y)[kLeaf + 1] = (double(*)[kLeaf + 1])(sm + kLeaf * (kLeaf + 1));
@@ -154,7 +156,8 @@ int64_t split(int64_t s) { return ceil_div(ceil_div(s, 2), kLeaf) * kLeaf; }
 int chol_inv(double *A, double *Y, int64_t m, int64_t n0, int64_t s, const Work &w, DevState *state,
              cudaStream_t st) {
     if (s <= kLeaf) {
-        chol_leaf_kernel<<<1, kLeafThreads, kLeafSmem, st>>>(A, Y, m, n0, (int)s, state);
+        OMM_CUDA_TRY(launch_pdl(chol_leaf_kernel, dim3(1), dim3(kLeafThreads), kLeafSmem, st, A, Y, m, n0, (int)s,
+                                state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         return OMM_OK;

@@ -32,6 +32,7 @@
 #include "crt.cuh"
 #include "fixed.cuh"
 #include "fp_convert.cuh"
+#include "pdl.cuh"
 #include "tc_units.cuh"
 
 namespace omm {
@@ -143,6 +144,7 @@ template <bool INV>
 __global__ void __launch_bounds__(256) pack_cols_kernel(int64_t K, int64_t R, const double *__restrict__ X, int64_t ld,
                                                         int *e, __nv_bfloat16 *dst, int64_t ldk, int64_t plane,
                                                         const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     __shared__ unsigned long long smax[8];
     __shared__ float ssum[8];
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(256) pack_cols_kernel(int64_t K, int64_t R, co
 // (coalesced); S follows X up as larger elements come.
 __global__ void __launch_bounds__(128) row_norm_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld,
                                                        float2 *part, int64_t slice, const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     const int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= R) return;
@@ -234,6 +237,7 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(int64_t R, int64_t K, co
                                                         const float2 *__restrict__ part, int nslice, int *e,
                                                         __nv_bfloat16 *dst, int64_t ldk, int64_t plane,
                                                         const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     __shared__ double tile[2][32][33];   // [k & 1][k / 2][row]: conflict-free both ways
     __shared__ float2 ns[8][32];
@@ -293,6 +297,7 @@ struct FoldArgs {
 
 // A thread takes one row of four columns: 16 words of four residues, four outputs.
 __global__ void __launch_bounds__(256) fold_kernel(const __grid_constant__ FoldArgs a) {
+    pdl_wait();
     if (a.state != nullptr && *((volatile const int *)&a.state->done)) return;
     const int row = blockIdx.x * 32 + threadIdx.x;
     const int c4 = blockIdx.y * 8 + threadIdx.y;
@@ -349,8 +354,10 @@ int pack_cols(int64_t K, int64_t R, const double *X, int64_t ld, int *e, __nv_bf
     if (K <= 0 || R <= 0) return OMM_OK;
     const unsigned grid = (unsigned)(R < 65536 ? R : 65536);
     const int threads = K <= 256 ? 64 : (K <= 512 ? 128 : 256);
-    if (inverse) pack_cols_kernel<true><<<grid, threads, 0, st>>>(K, R, X, ld, e, dst, ldk, plane, state);
-    else pack_cols_kernel<false><<<grid, threads, 0, st>>>(K, R, X, ld, e, dst, ldk, plane, state);
+    if (inverse) OMM_CUDA_TRY(launch_pdl(pack_cols_kernel<true>, grid, dim3(threads), 0, st, K, R, X, ld, e, dst,
+                                         ldk, plane, state));
+    else OMM_CUDA_TRY(launch_pdl(pack_cols_kernel<false>, grid, dim3(threads), 0, st, K, R, X, ld, e, dst, ldk,
+                                 plane, state));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -362,12 +369,14 @@ int pack_rows(int64_t R, int64_t K, const double *X, int64_t ld, int *e, float2 
     int64_t slice = ceil_div(ceil_div(K, kRowSlices), 8) * 8;
     const int nslice = (int)ceil_div(K, slice);
     dim3 ng((unsigned)ceil_div(R, 128), (unsigned)nslice);
-    row_norm_kernel<<<ng, 128, 0, st>>>(R, K, X, ld, part, slice, state);
+    OMM_CUDA_TRY(launch_pdl(row_norm_kernel, ng, dim3(128), 0, st, R, K, X, ld, part, slice, state));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     dim3 grid((unsigned)ceil_div(R, 32), (unsigned)ceil_div(K, 64));
-    if (inverse) pack_rows_kernel<true><<<grid, 256, 0, st>>>(R, K, X, ld, part, nslice, e, dst, ldk, plane, state);
-    else pack_rows_kernel<false><<<grid, 256, 0, st>>>(R, K, X, ld, part, nslice, e, dst, ldk, plane, state);
+    if (inverse) OMM_CUDA_TRY(launch_pdl(pack_rows_kernel<true>, grid, dim3(256), 0, st, R, K, X, ld, part, nslice,
+                                         e, dst, ldk, plane, state));
+    else OMM_CUDA_TRY(launch_pdl(pack_rows_kernel<false>, grid, dim3(256), 0, st, R, K, X, ld, part, nslice, e, dst,
+                                 ldk, plane, state));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -418,7 +427,7 @@ int gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const Args &a, int nb
     f.eB_step = a.eB_step;
     f.state = a.state;
     dim3 grid((unsigned)ceil_div(a.M, 32), (unsigned)ceil_div(ceil_div(a.N, 4), 8), (unsigned)nbatch);
-    fold_kernel<<<grid, dim3(32, 8), 0, st>>>(f);
+    OMM_CUDA_TRY(launch_pdl(fold_kernel, grid, dim3(32, 8), 0, st, f));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;

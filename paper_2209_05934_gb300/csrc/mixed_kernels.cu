@@ -22,6 +22,7 @@
 #include "fp_convert.cuh"
 #include "linemin.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 
 namespace omm {
 namespace {
@@ -259,6 +260,7 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int n, const double *__re
                                                        const float *__restrict__ Z, int64_t ldz, double *partials,
                                                        unsigned int *counter, DevState *state,
                                                        const double *__restrict__ slope, int nslope) {
+    pdl_wait();
     mx_coeffs_body(n, h0, s0, ldh, Z, ldz, partials, counter, state, slope, nslope, blockIdx.x, gridDim.x);
 }
 
@@ -414,6 +416,7 @@ __global__ void __launch_bounds__(NT) mx_update_kernel(int m, int n, double *W, 
                                                        double *HW, const float *__restrict__ HD, double *SW,
                                                        const float *__restrict__ SD, const DevState *state,
                                                        DigitOut wd, DigitOut swhw) {
+    pdl_wait();
     mx_update_body(m, n, W, D, HW, HD, SW, SD, state, wd, swhw, blockIdx.x, gridDim.x);
 }
 
@@ -475,6 +478,7 @@ __global__ void __launch_bounds__(NT) mx_update2_kernel(int m, int n, double2 *W
                                                         double2 *HW, const float2 *__restrict__ HD, double2 *SW,
                                                         const float2 *__restrict__ SD, const DevState *state,
                                                         DigitOut wd, DigitOut swhw) {
+    pdl_wait();
     mx_update2_body(m, n, W, D, HW, HD, SW, SD, state, wd, swhw, blockIdx.x, gridDim.x);
 }
 
@@ -547,6 +551,7 @@ __global__ void __launch_bounds__(NT) mx_dots_kernel(int64_t mn, const float *__
                                                      const float *__restrict__ Zg, const float *__restrict__ Gp,
                                                      const float *__restrict__ D, double *partials,
                                                      unsigned int *counter, DevState *state, int first) {
+    pdl_wait();
     mx_dots_body<PRE>(mn, G, Zg, Gp, D, partials, counter, state, first, blockIdx.x, gridDim.x);
 }
 
@@ -605,6 +610,7 @@ template <bool ROUND1>
 __global__ void __launch_bounds__(NT) mx_direction_kernel(int m, int64_t mn, const float *__restrict__ G,
                                                           const float *__restrict__ Zg, float *Gp, float *Df,
                                                           float *D, DevState *state, DigitOut dd, double *slope) {
+    pdl_wait();
     mx_direction_body<ROUND1>(m, mn, G, Zg, Gp, Df, D, state, dd, slope, blockIdx.x, gridDim.x);
 }
 
@@ -660,6 +666,7 @@ template <bool PRE, bool ROUND1>
 __global__ void __launch_bounds__(NT) mx_direction4_kernel(int m, int64_t mn, const float4 *__restrict__ G,
                                                            const float4 *__restrict__ Zg, float4 *Gp, float4 *Df,
                                                            float4 *D, DevState *state, DigitOut dd, double *slope) {
+    pdl_wait();
     mx_direction4_body<PRE, ROUND1>(m, mn, G, Zg, Gp, Df, D, state, dd, slope, blockIdx.x, gridDim.x);
 }
 
@@ -847,6 +854,7 @@ __global__ void __launch_bounds__(NT, 4) mx_dots_direction4_kernel(int m, int64_
 // only one could be resident at a time.
 __global__ void __launch_bounds__(NT) mx_group_coeffs_kernel(const GlueSys *__restrict__ sys,
                                                              const int2 *__restrict__ blks) {
+    pdl_wait();
     const int2 b = blks[blockIdx.x];
     const GlueSys &g = sys[b.x];
     mx_coeffs_body(g.n, g.h0, g.s0, 2 * g.n, g.Z, 2 * g.n, g.scr[0], g.ctr[0], g.state, g.slope, g.nslope, (unsigned)b.y,
@@ -856,6 +864,7 @@ __global__ void __launch_bounds__(NT) mx_group_coeffs_kernel(const GlueSys *__re
 // H_W, S_W updates (b.y < nn_blocks) and, beside them, the W, H'W, SW updates
 __global__ void __launch_bounds__(NT, 4) mx_group_update_kernel(const GlueSys *__restrict__ sys,
                                                                 const int2 *__restrict__ blks) {
+    pdl_wait();
     const int2 b = blks[blockIdx.x];
     const GlueSys &g = sys[b.x];
     if (b.y < g.nn_blocks) {
@@ -875,6 +884,7 @@ __global__ void __launch_bounds__(NT, 4) mx_group_update_kernel(const GlueSys *_
 
 __global__ void __launch_bounds__(NT) mx_group_dots_kernel(const GlueSys *__restrict__ sys,
                                                            const int2 *__restrict__ blks) {
+    pdl_wait();
     const int2 b = blks[blockIdx.x];
     const GlueSys &g = sys[b.x];
     mx_dots_body<false>((int64_t)g.m * g.n, g.G, g.G, g.Gp, g.Df, g.scr[2], g.ctr[2], g.state, 0, (unsigned)b.y,
@@ -884,6 +894,7 @@ __global__ void __launch_bounds__(NT) mx_group_dots_kernel(const GlueSys *__rest
 template <bool ROUND1>
 __global__ void __launch_bounds__(NT) mx_group_direction_kernel(const GlueSys *__restrict__ sys,
                                                                 const int2 *__restrict__ blks) {
+    pdl_wait();
     const int2 b = blks[blockIdx.x];
     const GlueSys &g = sys[b.x];
     const int64_t mn = (int64_t)g.m * g.n;
@@ -900,6 +911,7 @@ __global__ void __launch_bounds__(NT) mx_group_direction_kernel(const GlueSys *_
 // Digits of four consecutive rows of one column per thread (m % 4 == 0)
 __global__ void __launch_bounds__(NT) mx_digits4_kernel(int m, int64_t mn, const float4 *__restrict__ A,
                                                         const DevState *state, DigitOut dd) {
+    pdl_wait();
     if (*((volatile const int *)&state->done)) return;
     for (int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x; k < mn / 4; k += (int64_t)gridDim.x * NT) {
         const int64_t o = 4 * k, j = o / m, i = o - j * m;
@@ -908,6 +920,7 @@ __global__ void __launch_bounds__(NT) mx_digits4_kernel(int m, int64_t mn, const
 }
 
 __global__ void mx_digits_kernel(int m, int n, const float *__restrict__ A, const DevState *state, DigitOut dd) {
+    pdl_wait();
     if (*((volatile const int *)&state->done)) return;
     for (int j = blockIdx.y; j < n; j += gridDim.y)
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < m; i += gridDim.x * blockDim.x)
@@ -967,8 +980,8 @@ int mx_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh, co
                       double *scratch, unsigned int *counter, DevState *state, const double *slope, int nslope,
                       cudaStream_t st) {
     if (nslope < 0 || nslope > kRedBlocksMax || (nslope > 0 && slope == nullptr)) return OMM_ERR_ARG;
-    mx_coeffs_kernel<<<tiles_blocks(n, n), NT, 0, st>>>(n, h0, s0, ldh, Z, ldz, scratch, counter, state, slope,
-                                                        nslope);
+    OMM_CUDA_TRY(launch_pdl(mx_coeffs_kernel, dim3(tiles_blocks(n, n)), dim3(NT), 0, st, n, h0, s0, ldh, Z, ldz,
+                            scratch, counter, state, slope, nslope));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -979,15 +992,17 @@ int mx_update(int64_t m, int64_t n, double *W, const float *D, double *HW, const
     const bool two = update_by_two(m, W, D, HW, HD, SW, SD, wd);
     const int64_t nb = update_blocks(m, n, two);
     if (two) {
-        mx_update2_kernel<<<(unsigned)nb, NT, 0, st>>>(
-            (int)m, (int)n, reinterpret_cast<double2 *>(W), reinterpret_cast<const float2 *>(D),
-            reinterpret_cast<double2 *>(HW), reinterpret_cast<const float2 *>(HD), reinterpret_cast<double2 *>(SW),
-            reinterpret_cast<const float2 *>(SD), state, wd, swhw);
+        OMM_CUDA_TRY(launch_pdl(mx_update2_kernel, dim3((unsigned)nb), dim3(NT), 0, st,  (int)m, (int)n,
+                                reinterpret_cast<double2 *>(W), reinterpret_cast<const float2 *>(D),
+                                reinterpret_cast<double2 *>(HW), reinterpret_cast<const float2 *>(HD),
+                                reinterpret_cast<double2 *>(SW), reinterpret_cast<const float2 *>(SD), state, wd,
+                                swhw));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         return OMM_OK;
     }
-    mx_update_kernel<<<(unsigned)nb, NT, 0, st>>>((int)m, (int)n, W, D, HW, HD, SW, SD, state, wd, swhw);
+    OMM_CUDA_TRY(launch_pdl(mx_update_kernel, dim3((unsigned)nb), dim3(NT), 0, st, (int)m, (int)n, W, D, HW, HD, SW,
+                            SD, state, wd, swhw));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -1007,9 +1022,11 @@ int mx_dots_beta(int64_t mn, const float *G, const float *Zg, const float *Gp, c
     const int64_t nb = dots_blocks(mn);
     const unsigned grid = (unsigned)(nb < 1 ? 1 : nb);
     if (Zg != nullptr)
-        mx_dots_kernel<true><<<grid, NT, 0, st>>>(mn, G, Zg, Gp, D, scratch, counter, state, first);
+        OMM_CUDA_TRY(launch_pdl(mx_dots_kernel<true>, grid, dim3(NT), 0, st, mn, G, Zg, Gp, D, scratch, counter,
+                                state, first));
     else
-        mx_dots_kernel<false><<<grid, NT, 0, st>>>(mn, G, G, Gp, D, scratch, counter, state, first);
+        OMM_CUDA_TRY(launch_pdl(mx_dots_kernel<false>, grid, dim3(NT), 0, st, mn, G, G, Gp, D, scratch, counter,
+                                state, first));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -1030,15 +1047,17 @@ int mx_direction(int64_t m, int64_t n, const float *G, const float *Zg, float *G
                *D4 = reinterpret_cast<float4 *>(D);
         auto kern = Zg != nullptr ? (round1 ? mx_direction4_kernel<true, true> : mx_direction4_kernel<true, false>)
                                   : (round1 ? mx_direction4_kernel<false, true> : mx_direction4_kernel<false, false>);
-        kern<<<grid, NT, 0, st>>>((int)m, mn, G4, Z4, Gp4, Df4, D4, state, dd, slope);
+        OMM_CUDA_TRY(launch_pdl(kern, dim3(grid), dim3(NT), 0, st, (int)m, mn, G4, Z4, Gp4, Df4, D4, state, dd, slope));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         return OMM_OK;
     }
     if (round1)
-        mx_direction_kernel<true><<<grid, NT, 0, st>>>((int)m, mn, G, Zg, Gp, Df, D, state, dd, slope);
+        OMM_CUDA_TRY(launch_pdl(mx_direction_kernel<true>, grid, dim3(NT), 0, st, (int)m, mn, G, Zg, Gp, Df, D,
+                                state, dd, slope));
     else
-        mx_direction_kernel<false><<<grid, NT, 0, st>>>((int)m, mn, G, Zg, Gp, Df, D, state, dd, slope);
+        OMM_CUDA_TRY(launch_pdl(mx_direction_kernel<false>, grid, dim3(NT), 0, st, (int)m, mn, G, Zg, Gp, Df, D,
+                                state, dd, slope));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -1113,11 +1132,11 @@ int mx_digits(int64_t m, int64_t n, const float *A, const DevState *state, Digit
     if (m % 4 == 0 && aligned) {
         int64_t nb = ceil_div(m * n / 4, (int64_t)NT * 4);
         if (nb > 152 * 8) nb = 152 * 8;
-        mx_digits4_kernel<<<(unsigned)(nb < 1 ? 1 : nb), NT, 0, st>>>((int)m, m * n,
-                                                                       reinterpret_cast<const float4 *>(A), state, dd);
+        OMM_CUDA_TRY(launch_pdl(mx_digits4_kernel, dim3((unsigned)(nb < 1 ? 1 : nb)), dim3(NT), 0, st, (int)m,
+                                m * n, reinterpret_cast<const float4 *>(A), state, dd));
     } else {
         dim3 grid((unsigned)ceil_div(m, NT), (unsigned)(n < 1024 ? n : 1024));
-        mx_digits_kernel<<<grid, NT, 0, st>>>((int)m, (int)n, A, state, dd);
+        OMM_CUDA_TRY(launch_pdl(mx_digits_kernel, grid, dim3(NT), 0, st, (int)m, (int)n, A, state, dd));
     }
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
@@ -1155,18 +1174,16 @@ int mx_group_prepare(GlueSys &g, bool round1) {
 
 int mx_group_launch(int which, const GlueSys *sys, const int2 *blks, int nblks, bool round1, cudaStream_t st) {
     if (nblks <= 0) return OMM_OK;
+    void (*kern)(const GlueSys *, const int2 *) = nullptr;
     switch (which) {
-        case GLUE_COEFFS: mx_group_coeffs_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
-        case GLUE_UPDATE: mx_group_update_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
-        case GLUE_DOTS: mx_group_dots_kernel<<<nblks, NT, 0, st>>>(sys, blks); break;
-        case GLUE_DIRECTION:
-            if (round1) mx_group_direction_kernel<true><<<nblks, NT, 0, st>>>(sys, blks);
-            else mx_group_direction_kernel<false><<<nblks, NT, 0, st>>>(sys, blks);
-            break;
+        case GLUE_COEFFS: kern = mx_group_coeffs_kernel; break;
+        case GLUE_UPDATE: kern = mx_group_update_kernel; break;
+        case GLUE_DOTS: kern = mx_group_dots_kernel; break;
+        case GLUE_DIRECTION: kern = round1 ? mx_group_direction_kernel<true> : mx_group_direction_kernel<false>; break;
         default: return OMM_ERR_ARG;
     }
+    OMM_CUDA_TRY(launch_pdl(kern, dim3(nblks), dim3(NT), 0, st, sys, blks));
     count_launch();
-    OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
 }
 

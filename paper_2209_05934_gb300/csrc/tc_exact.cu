@@ -21,6 +21,7 @@
 
 #include "fp_convert.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 #include "tc_exact.cuh"
 #include "tc_gemm.cuh"
 #include "tc_units.cuh"
@@ -62,6 +63,7 @@ struct FoldArgs {
 // 1024 x 1000 outputs of 7 levels from 31 to 14 us.
 template <int NLEV>
 __global__ void __launch_bounds__(256) level_fold_kernel(const __grid_constant__ FoldArgs a) {
+    pdl_wait();
     if (a.state != nullptr && *((volatile const int *)&a.state->done)) return;
     const int row = blockIdx.x * 32 + threadIdx.x;
     const int col0 = (blockIdx.y * 8 + threadIdx.y) * 4;
@@ -157,6 +159,7 @@ __device__ __forceinline__ void put_digits(double v, int e, int s, __nv_bfloat16
 // K along the source's rows: operand row r is source column r (warp per column).
 __global__ void exp_cm_kernel(int64_t K, int64_t R, const double *__restrict__ X, int64_t ld, int *e,
                               const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     const int lane = threadIdx.x & 31;
     const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -195,6 +198,7 @@ __global__ void exp_cm_kernel(int64_t K, int64_t R, const double *__restrict__ X
 // atomic max (be zeroed first); exp_finish_kernel turns be into exponents.
 __global__ void exp_t_split_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld, int *be,
                                    int64_t kslice, const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
     const int64_t r = (int64_t)blockIdx.x * 32 + lx;
@@ -210,6 +214,7 @@ __global__ void exp_t_split_kernel(int64_t R, int64_t K, const double *__restric
 }
 
 __global__ void exp_finish_kernel(int64_t R, int *e, const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R; r += (int64_t)gridDim.x * blockDim.x)
         e[r] = exponent_from_maxbits((uint64_t)e[r] << 52);
@@ -218,6 +223,7 @@ __global__ void exp_finish_kernel(int64_t R, int *e, const DevState *state) {
 __global__ void digits_cm_kernel(int64_t K, int64_t R, const double *__restrict__ X, int64_t ld,
                                  const int *__restrict__ e, __nv_bfloat16 *dst, int64_t ldk, int64_t plane,
                                  int s, const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
         const int er = e[r];
@@ -229,6 +235,7 @@ __global__ void digits_cm_kernel(int64_t K, int64_t R, const double *__restrict_
 __global__ void digits_t_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld,
                                 const int *__restrict__ e, __nv_bfloat16 *dst, int64_t ldk, int64_t plane, int s,
                                 const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     __shared__ double tile[32][33];
     const int64_t tr = (int64_t)blockIdx.x * 32, tk = (int64_t)blockIdx.y * 32;
@@ -266,11 +273,13 @@ int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, i
     if (rows <= 0 || cols <= 0) return OMM_OK;
     if (s < 1 || s > kExactMaxDigits) return OMM_ERR_ARG;
     if (k_along_rows) {   // K = rows, operand rows = cols
-        exp_cm_kernel<<<grid_for(cols * 32, 256), 256, 0, st>>>(rows, cols, X, ld, e, state);
+        OMM_CUDA_TRY(launch_pdl(exp_cm_kernel, dim3(grid_for(cols * 32, 256)), dim3(256), 0, st, rows, cols, X, ld,
+                                e, state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         dim3 grid((unsigned)ceil_div(rows, 256 * 2), (unsigned)(cols < 8192 ? cols : 8192));
-        digits_cm_kernel<<<grid, 256, 0, st>>>(rows, cols, X, ld, e, dst, ldk, plane, s, state);
+        OMM_CUDA_TRY(launch_pdl(digits_cm_kernel, grid, dim3(256), 0, st, rows, cols, X, ld, e, dst, ldk, plane, s,
+                                state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
     } else {              // K = cols, operand rows = rows
@@ -278,14 +287,15 @@ int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, i
         OMM_CUDA_TRY(cudaMemsetAsync(e, 0, (size_t)rows * sizeof(int), st));
         const int64_t kslice = 256;
         dim3 eg((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, kslice));
-        exp_t_split_kernel<<<eg, 256, 0, st>>>(rows, cols, X, ld, e, kslice, state);
+        OMM_CUDA_TRY(launch_pdl(exp_t_split_kernel, eg, dim3(256), 0, st, rows, cols, X, ld, e, kslice, state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
-        exp_finish_kernel<<<grid_for(rows, 256), 256, 0, st>>>(rows, e, state);
+        OMM_CUDA_TRY(launch_pdl(exp_finish_kernel, dim3(grid_for(rows, 256)), dim3(256), 0, st, rows, e, state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         dim3 grid((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, 32));
-        digits_t_kernel<<<grid, 256, 0, st>>>(rows, cols, X, ld, e, dst, ldk, plane, s, state);
+        OMM_CUDA_TRY(launch_pdl(digits_t_kernel, grid, dim3(256), 0, st, rows, cols, X, ld, e, dst, ldk, plane, s,
+                                state));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
     }
@@ -364,7 +374,7 @@ int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs
         if (rc != OMM_OK) return rc;
         dim3 grid((unsigned)ceil_div(a.M, 32), (unsigned)ceil_div(nc, 32), (unsigned)nbatch);
         auto fold = s == 6 ? level_fold_kernel<6> : s == 7 ? level_fold_kernel<7> : level_fold_kernel<0>;
-        fold<<<grid, dim3(32, 8), 0, st>>>(f);
+        OMM_CUDA_TRY(launch_pdl(fold, grid, dim3(32, 8), 0, st, f));
         count_launch();
         OMM_CUDA_TRY(cudaGetLastError());
         if (f.Cin != nullptr) f.Cin += slab * a.ldcin;

@@ -29,6 +29,7 @@
 
 #include "fp_convert.cuh"
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 #include "tc_ptx.cuh"
 
@@ -328,6 +329,7 @@ template <int BN, int STAGES, int BKT>
 __global__ void __launch_bounds__(192, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                    const TcArgs args) {
+    pdl_wait();
     if (args.state != nullptr && *((volatile const int *)&args.state->done)) return;
     const int z = blockIdx.z;
     const int nA = args.nA, nB = args.nB;
@@ -456,6 +458,7 @@ template <int STAGES, int BKT>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                         const TcArgs args) {
+    pdl_wait();
     // state->done only changes between launches, so both CTAs of a pair return here together
     if (args.state != nullptr && *((volatile const int *)&args.state->done)) return;
     constexpr int BN = 256, BNH = 128;
@@ -609,6 +612,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
 template <bool PAIR, int STAGES, int BKT>
 __global__ void __launch_bounds__(192, 1)
     tc_gemm_list_kernel(const TileProblem *__restrict__ probs, const TileRef *__restrict__ tiles, int ntiles) {
+    pdl_wait();
     constexpr int BN = 256;                        // accumulator columns per pair class
     constexpr int BNC = PAIR ? 128 : 256;          // most B rows per CTA (a problem's tiles may be narrower)
     constexpr int TILE_A = BM * BKT * 2;
@@ -814,6 +818,7 @@ __global__ void wait_probe_kernel(uint64_t limit_ns, int *err, int *status) {
 __global__ void pack_cm_kernel(int64_t rows, int64_t cols, const double *__restrict__ src, int64_t ld_src,
                                __nv_bfloat16 *dst, int64_t ldd, int64_t plane, int ndig,
                                const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     for (int64_t j = blockIdx.y; j < cols; j += gridDim.y)
         for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < rows;
@@ -832,6 +837,7 @@ __global__ void pack_cm_kernel(int64_t rows, int64_t cols, const double *__restr
 __global__ void pack_t_kernel(int64_t rows, int64_t cols, const double *__restrict__ src, int64_t ld_src,
                               __nv_bfloat16 *dst, int64_t ldd, int64_t plane, int ndig,
                               const DevState *state) {
+    pdl_wait();
     if (state != nullptr && *((volatile const int *)&state->done)) return;
     __shared__ double tile[32][33];
     const int64_t ti = (int64_t)blockIdx.x * 32, tj = (int64_t)blockIdx.y * 32;
@@ -891,7 +897,7 @@ int launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, const TcArgs &a, int
     while (kacc > 1 && kacc > nkb) kacc >>= 1;
     b.kacc = kacc;
     dim3 grid((unsigned)ceil_div(a.N, BN), (unsigned)ceil_div(a.M, BM), (unsigned)nbatch);
-    tc_gemm_kernel<BN, STAGES, BKT><<<grid, 192, smem, st>>>(ma, mb, b);
+    OMM_CUDA_TRY(launch_pdl(tc_gemm_kernel<BN, STAGES, BKT>, grid, dim3(192), smem, st, ma, mb, b));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -918,7 +924,7 @@ int launch_tc_pair(const CUtensorMap &ma, const CUtensorMap &mb_half, const TcAr
     while (kacc > 1 && kacc > nkb) kacc >>= 1;
     b.kacc = kacc;
     dim3 grid((unsigned)(2 * ceil_div(a.N, 256)), (unsigned)ceil_div(a.M, 2 * BM), (unsigned)nbatch);
-    tc_gemm_pair_kernel<STAGES, BKT><<<grid, kPairThreads, smem, st>>>(ma, mb_half, b);
+    OMM_CUDA_TRY(launch_pdl(tc_gemm_pair_kernel<STAGES, BKT>, grid, dim3(kPairThreads), smem, st, ma, mb_half, b));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -944,13 +950,15 @@ int launch_list(const TileProblem *probs, const TileRef *tiles, int ntiles, int 
     cfg.blockDim = dim3(192, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr_c[1];
+    cudaLaunchAttribute attr_c[2];
     attr_c[0].id = cudaLaunchAttributeClusterDimension;
     attr_c[0].val.clusterDim.x = PAIR ? 2 : 1;
     attr_c[0].val.clusterDim.y = 1;
     attr_c[0].val.clusterDim.z = 1;
+    attr_c[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr_c[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr_c;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, probs, tiles, ntiles));
     count_launch();
     return OMM_OK;
@@ -1048,7 +1056,8 @@ int pack_cm(int64_t rows, int64_t cols, const double *src, int64_t ld_src, __nv_
             int64_t plane, int ndig, const DevState *state, cudaStream_t st) {
     if (rows <= 0 || cols <= 0) return OMM_OK;
     dim3 grid((unsigned)ceil_div(rows, 256 * 2), (unsigned)(cols < 8192 ? cols : 8192));
-    pack_cm_kernel<<<grid, 256, 0, st>>>(rows, cols, src, ld_src, dst, ldd, plane, ndig, state);
+    OMM_CUDA_TRY(launch_pdl(pack_cm_kernel, grid, dim3(256), 0, st, rows, cols, src, ld_src, dst, ldd, plane, ndig,
+                            state));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;
@@ -1058,7 +1067,8 @@ int pack_t(int64_t rows, int64_t cols, const double *src, int64_t ld_src, __nv_b
            int64_t plane, int ndig, const DevState *state, cudaStream_t st) {
     if (rows <= 0 || cols <= 0) return OMM_OK;
     dim3 grid((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, 32));
-    pack_t_kernel<<<grid, 256, 0, st>>>(rows, cols, src, ld_src, dst, ldd, plane, ndig, state);
+    OMM_CUDA_TRY(launch_pdl(pack_t_kernel, grid, dim3(256), 0, st, rows, cols, src, ld_src, dst, ldd, plane, ndig,
+                            state));
     count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;

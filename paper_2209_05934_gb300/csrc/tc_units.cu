@@ -33,6 +33,7 @@
 #include <cuda_bf16.h>
 
 #include "omm_internal.cuh"
+#include "pdl.cuh"
 #include "tc_ptx.cuh"
 #include "tc_units.cuh"
 
@@ -69,14 +70,11 @@ template <bool PAIR, bool CRT>
 __global__ void __launch_bounds__(kUnitThreads, 1)
     tc_unit_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                    const __grid_constant__ UnitArgs args) {
-    // state->done only changes between launches, so every CTA returns here together
-    if (args.state != nullptr && *((volatile const int *)&args.state->done)) return;
     constexpr int STAGES = PAIR ? 6 : 4;
     constexpr int STAGE_BYTES = PAIR ? 2 * kBox : 3 * kBox;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
     const int group = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
     const int ngroups = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-    const int nitems = args.ngroups * args.nbatch * args.tiles_m * args.tiles_n;
     const int bn = args.bn;
     const int nkb = (args.K + BK - 1) / BK;
     const int kb_chunk = args.kchunk / BK;
@@ -117,6 +115,10 @@ __global__ void __launch_bounds__(kUnitThreads, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_base;
     int issued = 0;
+    pdl_wait();   // the operands and the state are the work of earlier launches
+    // state->done only changes between launches: every CTA of a finished solve has no items
+    const bool live = args.state == nullptr || !*((volatile const int *)&args.state->done);
+    const int nitems = live ? args.ngroups * args.nbatch * args.tiles_m * args.tiles_n : 0;
 
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer: the ring runs on across units and items
@@ -328,13 +330,15 @@ int launch_unit(const CUtensorMap &ma, const CUtensorMap &mb, const UnitArgs &a,
     cfg.blockDim = dim3(kUnitThreads, 1, 1);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = PAIR ? 2 : 1;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     OMM_CUDA_TRY(cudaLaunchKernelEx(&cfg, tc_unit_kernel<PAIR, CRT>, ma, mb, a));
     count_launch();
     return OMM_OK;
