@@ -64,7 +64,8 @@ struct ExactBufs {
     int s = 0;
     __nv_bfloat16 *HSx = nullptr, *Wx = nullptr, *HWSWx = nullptr, *SWHWx = nullptr, *HSWx = nullptr;
     uint32_t *planes = nullptr;   // level planes of a product
-    int *e = nullptr;   // exponents: [2m HS | n W | 2n HWSW | m SWHW | n HSW]
+    int *e = nullptr;   // exponents: [2m HS | n W | 2n HWSW | m SWHW | n HSW], then part
+    int *part = nullptr;   // row maxima of SWHW
     int *eHS = nullptr, *eW = nullptr, *eHWSW = nullptr, *eSWHW = nullptr, *eHSW = nullptr;
     CUtensorMap mapHS_A, mapW, mapHWSW_B, mapSWHW_A, mapHSW_B;
 };
@@ -833,7 +834,7 @@ int exact_alloc(omm_handle *h) {
     TRY(dalloc(&e.HWSWx, (size_t)(s * 2 * n * x.ldm)));
     TRY(dalloc(&e.SWHWx, (size_t)(s * m * x.ld2n)));
     TRY(dalloc(&e.HSWx, (size_t)(s * n * x.ld2n)));
-    TRY(dalloc(&e.e, (size_t)(2 * m + n + 2 * n + m + n)));
+    TRY(dalloc(&e.e, (size_t)(2 * m + n + 2 * n + m + n + omm::tc::kDigitSlices * m)));
     // the anchor's [H';S] W is the largest product; both it and the gradient take six digits
     TRY(dalloc(&e.planes, (size_t)omm::tc::exact_plane_words(m, n, 2, s < 6 ? s : 6)));
     e.eHS = e.e;
@@ -841,6 +842,7 @@ int exact_alloc(omm_handle *h) {
     e.eHWSW = e.eW + n;
     e.eSWHW = e.eHWSW + 2 * n;
     e.eHSW = e.eSWHW + m;
+    e.part = e.eHSW + n;
     TRY(omm::tc::make_digit_map(&e.mapHS_A, e.HSx, m, 2 * m, x.ldm, 2 * m * x.ldm, s, 128));
     TRY(omm::tc::make_digit_map(&e.mapW, e.Wx, m, n, x.ldm, n * x.ldm, s, 128));
     TRY(omm::tc::make_digit_map(&e.mapHWSW_B, e.HWSWx, m, 2 * n, x.ldm, 2 * n * x.ldm, s, 128));
@@ -877,8 +879,9 @@ int exact_gradient(omm_handle *h) {
     const int sg = e.s < 6 ? e.s : 6;
     {
         StageTimer t(h, OMM_STAGE_PACK);
-        TRY(omm::tc::exact_pack(false, m, 2 * n, h->SWHW, m, e.eSWHW, e.SWHWx, x.ld2n, m * x.ld2n, sg, h->dstate, st));
-        TRY(omm::tc::exact_pack(true, 2 * n, n, h->h0s0, 2 * n, e.eHSW, e.HSWx, x.ld2n, n * x.ld2n, sg, h->dstate, st));
+        const omm::tc::PackJob pa{false, m, 2 * n, h->SWHW, m, e.eSWHW, e.SWHWx, x.ld2n, m * x.ld2n, e.part};
+        const omm::tc::PackJob pb{true, 2 * n, n, h->h0s0, 2 * n, e.eHSW, e.HSWx, x.ld2n, n * x.ld2n, nullptr};
+        TRY(omm::tc::exact_pack(pa, &pb, sg, h->dstate, st));
     }
     StageTimer t(h, OMM_STAGE_GRADIENT);
     omm::tc::ExactArgs a = exact_args(h, (int)m, (int)n, (int)(2 * n));
@@ -907,7 +910,8 @@ int exact_anchor(omm_handle *h) {
     const int sa = e.s < 6 ? e.s : 6;
     {
         StageTimer t(h, OMM_STAGE_ANCHOR);
-        TRY(omm::tc::exact_pack(true, m, n, h->WD, m, e.eW, e.Wx, x.ldm, n * x.ldm, sa, s, st));
+        const omm::tc::PackJob pw{true, m, n, h->WD, m, e.eW, e.Wx, x.ldm, n * x.ldm, nullptr};
+        TRY(omm::tc::exact_pack(pw, nullptr, sa, s, st));
         // z = 0: H'W -> SWHW + mn;  z = 1: SW -> SWHW
         omm::tc::ExactArgs a = exact_args(h, (int)m, (int)n, (int)m);
         a.s = sa;
@@ -921,9 +925,10 @@ int exact_anchor(omm_handle *h) {
         TRY(omm::tc::exact_gemm(e.mapHS_A, e.mapW, a, s_identity(h) ? 1 : 2, st));
         if (s_identity(h))
             OMM_CUDA_TRY(cudaMemcpyAsync(h->SWHW, h->WD, mn * sizeof(double), cudaMemcpyDeviceToDevice, st));
-        TRY(omm::tc::exact_pack(true, m, n, h->SWHW + mn, m, e.eHWSW, e.HWSWx, x.ldm, 2 * n * x.ldm, sa, s, st));
-        TRY(omm::tc::exact_pack(true, m, n, h->SWHW, m, e.eHWSW + n, e.HWSWx + n * x.ldm, x.ldm, 2 * n * x.ldm, sa,
-                                s, st));
+        const omm::tc::PackJob ph{true, m, n, h->SWHW + mn, m, e.eHWSW, e.HWSWx, x.ldm, 2 * n * x.ldm, nullptr};
+        const omm::tc::PackJob ps{true, m, n, h->SWHW, m, e.eHWSW + n, e.HWSWx + n * x.ldm, x.ldm, 2 * n * x.ldm,
+                                  nullptr};
+        TRY(omm::tc::exact_pack(ph, &ps, sa, s, st));
         // z = 0: H_W = W^T H'W -> rows [0, n) of h0s0;  z = 1: S_W -> rows [n, 2n)
         omm::tc::ExactArgs b = exact_args(h, (int)n, (int)n, (int)m);
         b.s = sa;
@@ -1305,9 +1310,10 @@ int dense_set(omm_handle *h, const double *H, const double *S, bool on_device) {
         TRY(omm::tc::pack_cm(m, cols, h->HS, m, h->mx.HSd, h->mx.ldm, 2 * m * h->mx.ldm, h->opt.split_digits, nullptr,
                              st));
         // the re-anchor reads six digits of H' and S (see exact_anchor)
-        if (h->opt.refine == OMM_REFINE_EXACT)
-            TRY(omm::tc::exact_pack(true, m, cols, h->HS, m, h->ex.eHS, h->ex.HSx, h->mx.ldm, 2 * m * h->mx.ldm,
-                                    h->ex.s < 6 ? h->ex.s : 6, nullptr, st));
+        if (h->opt.refine == OMM_REFINE_EXACT) {
+            const omm::tc::PackJob p{true, m, cols, h->HS, m, h->ex.eHS, h->ex.HSx, h->mx.ldm, 2 * m * h->mx.ldm, nullptr};
+            TRY(omm::tc::exact_pack(p, nullptr, h->ex.s < 6 ? h->ex.s : 6, nullptr, st));
+        }
     }
     if (crt_on(h)) {
         // rows of H' and S; omm_set_H and the Cholesky variant's S = I repack H' only

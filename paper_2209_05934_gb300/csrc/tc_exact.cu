@@ -131,130 +131,168 @@ __device__ __forceinline__ int exponent_from_maxbits(uint64_t mb) {
     return e < -1000 ? -1000 : (e > 1000 ? 1000 : e);
 }
 
-// Digits of a = v 2^-e: F = round(v 2^(B-e)) with B = 6 + 7(s-1), then balanced
-// base-128 digits from the bottom: F = sum_t d_t 128^(s-t), d_t in [-64, 64].
-// d_t then carries the weight 2^-(7t-1) of the fixed-point splitting.
-__device__ __forceinline__ void put_digits(double v, int e, int s, __nv_bfloat16 *dst, int64_t o, int64_t plane) {
-    const uint64_t b = (uint64_t)__double_as_longlong(v);
-    const int be = (int)((b >> 52) & 0x7FF);
-    int64_t F = 0;
-    if (be != 0) {
-        const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);   // v = mant 2^(be - 1075)
-        const int shift = be - 1075 + (6 + 7 * (s - 1)) - e;
-        if (shift >= 0) {
-            F = (int64_t)(mant << shift);             // |F| < 2^(6 + 7(s-1)) <= 2^55
-        } else if (shift > -64) {
-            F = (int64_t)((mant + (1ull << (-shift - 1))) >> (-shift));
-        }
-        if (b >> 63) F = -F;
-    }
-    for (int t = s - 1; t >= 1; --t) {
-        const int64_t r = ((F + 64) & 127) - 64;      // in [-64, 63]
-        dst[t * plane + o] = __float2bfloat16_rn((float)(int)r);   // small integers: exact, 32-bit convert
-        F = (F - r) >> 7;
-    }
-    dst[o] = __float2bfloat16_rn((float)(int)F);      // |F| <= 64
-}
-
-// K along the source's rows: operand row r is source column r (warp per column).
-__global__ void exp_cm_kernel(int64_t K, int64_t R, const double *__restrict__ X, int64_t ld, int *e,
-                              const DevState *state) {
-    pdl_wait();
-    if (state != nullptr && *((volatile const int *)&state->done)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const uint64_t *Xb = (const uint64_t *)X;
-    for (int64_t r = w; r < R; r += nw) {
-        // four independent maxima: four loads of each lane in flight (with one warp
-        // per column the grid holds few warps, so each must keep several loads going)
-        unsigned long long m4[4] = {0, 0, 0, 0};
-        int64_t k = lane;
-        for (; k + 96 < K; k += 128)
+// Digits of NV values a = v 2^-e, stored side by side: F = round(v 2^(B-e)) with
+// B = 6 + 7(s-1), then balanced base-128 digits F = sum_t d_t 128^(s-t), d_t in
+// [-64, 64] (all but the leading one in [-64, 63]: adding 64 to each turns them into
+// plain base-128 digits).  d_t then carries the weight 2^-(7t-1) of the fixed-point
+// splitting.  A small integer has its BF16 form in the upper half of its float.
+template <int NV>
+__device__ __forceinline__ void put_digits(const double (&v)[NV], int e, int s, __nv_bfloat16 *dst, int64_t plane, int nv) {
+    int64_t G[NV];
+    int64_t bias = 0;
+    for (int i = 0; i < s - 1; ++i) bias = bias * 128 + 64;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const unsigned long long a = Xb[k + 32 * u + r * ld] & 0x7FFFFFFFFFFFFFFFull;
-                m4[u] = a > m4[u] ? a : m4[u];
+    for (int j = 0; j < NV; ++j) {
+        const uint64_t b = (uint64_t)__double_as_longlong(v[j]);
+        const int be = (int)((b >> 52) & 0x7FF);
+        int64_t F = 0;
+        if (be != 0) {
+            const uint64_t mant = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);   // v = mant 2^(be - 1075)
+            const int shift = be - 1075 + (6 + 7 * (s - 1)) - e;
+            if (shift >= 0) {
+                F = (int64_t)(mant << shift);             // |F| < 2^(6 + 7(s-1)) <= 2^55
+            } else if (shift > -64) {
+                F = (int64_t)((mant + (1ull << (-shift - 1))) >> (-shift));
             }
-        for (; k < K; k += 32) {
-            const unsigned long long a = Xb[k + r * ld] & 0x7FFFFFFFFFFFFFFFull;
-            m4[0] = a > m4[0] ? a : m4[0];
+            if (b >> 63) F = -F;
         }
-        unsigned long long mx = m4[0] > m4[1] ? m4[0] : m4[1];
-        const unsigned long long m23 = m4[2] > m4[3] ? m4[2] : m4[3];
-        mx = m23 > mx ? m23 : mx;
+        G[j] = F + bias;
+    }
+    for (int t = s - 1; t >= 0; --t) {
+        uint32_t w[NV];
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const unsigned long long o = __shfl_xor_sync(0xffffffffu, mx, off);
-            mx = o > mx ? o : mx;
+        for (int j = 0; j < NV; ++j) {
+            const int d = t > 0 ? (int)((uint32_t)G[j] & 127u) - 64 : (int)G[j];
+            w[j] = __float_as_uint(__uint_as_float((uint32_t)(0x4B400000 + d)) - 12582912.f);
+            G[j] >>= 7;
         }
-        if (lane == 0) e[r] = exponent_from_maxbits(mx);
+        __nv_bfloat16 *o = dst + t * plane;
+        if (NV == 4 && nv == 4)
+            *reinterpret_cast<uint2 *>(o) = make_uint2(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[NV - 1], 0x7632));
+        else if (NV == 2 && nv == 2)
+            *reinterpret_cast<uint32_t *>(o) = __byte_perm(w[0], w[1], 0x7632);
+        else
+#pragma unroll
+            for (int j = 0; j < NV; ++j)
+                if (j < nv) reinterpret_cast<uint16_t *>(o)[j] = (uint16_t)(w[j] >> 16);
     }
 }
 
-// Row exponents when K runs along the source's columns, split over K: each warp
-// takes 32 rows (one per lane, coalesced) and a slice of the columns, and folds
-// the biased exponent of its largest magnitude into be[r] with an integer
-// atomic max (be zeroed first); exp_finish_kernel turns be into exponents.
-__global__ void exp_t_split_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld, int *be,
-                                   int64_t kslice, const DevState *state) {
-    pdl_wait();
-    if (state != nullptr && *((volatile const int *)&state->done)) return;
-    const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
-    const int64_t r = (int64_t)blockIdx.x * 32 + lx;
-    const int64_t k0 = (int64_t)blockIdx.y * kslice, k1 = k0 + kslice < K ? k0 + kslice : K;
-    const uint64_t *Xb = (const uint64_t *)X;
-    unsigned long long mx = 0;
-    if (r < R)
-        for (int64_t k = k0 + ly; k < k1; k += 8) {
-            const unsigned long long a = Xb[r + k * ld] & 0x7FFFFFFFFFFFFFFFull;
-            mx = a > mx ? a : mx;
-        }
-    if (r < R && mx != 0) atomicMax(&be[r], (int)(mx >> 52));
-}
+// One operand of a launch, with its share of the blocks of both kernels.
+struct PackBlocks {
+    PackJob j;
+    int64_t R, K;            // operand rows and their length
+    int nslice, tiles;       // columns in nslice slices; 32-row tiles (rows of the source)
+    int64_t slice;
+    int blocks_max, blocks;  // blocks of the maxima kernel, of the digits kernel
+};
+struct PackArgs {
+    PackBlocks p[2];
+    int s;
+    const DevState *state;
+};
 
-__global__ void exp_finish_kernel(int64_t R, int *e, const DevState *state) {
+// Largest biased exponent of every operand row over a slice of its columns, for
+// operands whose K runs along the source's columns: a thread per row, coalesced.
+__global__ void __launch_bounds__(128) row_max_kernel(const __grid_constant__ PackArgs a) {
     pdl_wait();
-    if (state != nullptr && *((volatile const int *)&state->done)) return;
-    for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < R; r += (int64_t)gridDim.x * blockDim.x)
-        e[r] = exponent_from_maxbits((uint64_t)e[r] << 52);
-}
-
-__global__ void digits_cm_kernel(int64_t K, int64_t R, const double *__restrict__ X, int64_t ld,
-                                 const int *__restrict__ e, __nv_bfloat16 *dst, int64_t ldk, int64_t plane,
-                                 int s, const DevState *state) {
-    pdl_wait();
-    if (state != nullptr && *((volatile const int *)&state->done)) return;
-    for (int64_t r = blockIdx.y; r < R; r += gridDim.y) {
-        const int er = e[r];
-        for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < K; k += (int64_t)gridDim.x * blockDim.x)
-            put_digits(X[k + r * ld], er, s, dst, r * ldk + k, plane);
+    if (a.state != nullptr && *((volatile const int *)&a.state->done)) return;
+    const int second = (int)blockIdx.x >= a.p[0].blocks_max ? 1 : 0;
+    const PackBlocks &p = a.p[second];
+    const int b = (int)blockIdx.x - (second ? a.p[0].blocks_max : 0);
+    const int sl = b % p.nslice;
+    const int64_t r = (int64_t)(b / p.nslice) * 128 + threadIdx.x;
+    if (r >= p.R) return;
+    const int64_t k0 = sl * p.slice, k1 = k0 + p.slice < p.K ? k0 + p.slice : p.K;
+    const uint64_t *x = reinterpret_cast<const uint64_t *>(p.j.X) + r;
+    uint64_t mx = 0;
+    for (int64_t k = k0; k < k1; k += 8) {
+        uint64_t v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = k + u < k1 ? x[(k + u) * p.j.ld] & 0x7FFFFFFFFFFFFFFFull : 0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mx = v[u] > mx ? v[u] : mx;
     }
+    p.j.part[(int64_t)sl * p.R + r] = (int)(mx >> 52);
 }
 
-__global__ void digits_t_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld,
-                                const int *__restrict__ e, __nv_bfloat16 *dst, int64_t ldk, int64_t plane, int s,
-                                const DevState *state) {
+// Digits and exponents of one or two operands.  K along the source's rows: a warp per
+// operand row (K <= kWarpK) or a CTA, which finds the maximum and then the digits, the
+// second read from L1; else 32-row tiles of 64 columns turned through shared memory,
+// with the exponents from row_max_kernel's slices.  Writes are 4 to 8 bytes a thread
+// and whole lines a warp.  One launch (two with row maxima) for both operands of a
+// product where there were up to eight: the recursion of the Cholesky factor runs 150
+// products a solve, most of them small.
+constexpr int64_t kWarpK = 1024;
+__global__ void __launch_bounds__(256) digit_pack_kernel(const __grid_constant__ PackArgs a) {
     pdl_wait();
-    if (state != nullptr && *((volatile const int *)&state->done)) return;
-    __shared__ double tile[32][33];
-    const int64_t tr = (int64_t)blockIdx.x * 32, tk = (int64_t)blockIdx.y * 32;
-    const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;
-    for (int i = ly; i < 32; i += 8) {
-        const int64_t r = tr + lx, k = tk + i;
-        tile[i][lx] = (r < R && k < K) ? X[r + k * ld] : 0.0;
+    if (a.state != nullptr && *((volatile const int *)&a.state->done)) return;
+    const int second = (int)blockIdx.x >= a.p[0].blocks ? 1 : 0;
+    const PackBlocks &p = a.p[second];
+    const PackJob &j = p.j;
+    const int64_t b = (int64_t)blockIdx.x - (second ? a.p[0].blocks : 0);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ double tile[2][32][33];
+    __shared__ unsigned long long smax[8];
+    __shared__ int part[8][32], es[32];
+    if (j.k_along_rows) {
+        const bool by_warp = p.K <= kWarpK;
+        const int64_t r = by_warp ? b * 8 + warp : b;
+        const int at = by_warp ? lane : tid, step = by_warp ? 32 : 256;
+        const double *x = j.X + r * j.ld;
+        unsigned long long mx = 0;
+        if (r < p.R)
+            for (int64_t k = at; k < p.K; k += step) {
+                const unsigned long long v = reinterpret_cast<const uint64_t *>(x)[k] & 0x7FFFFFFFFFFFFFFFull;
+                mx = v > mx ? v : mx;
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long v = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = v > mx ? v : mx;
+        }
+        if (!by_warp) {
+            if (lane == 0) smax[warp] = mx;
+            __syncthreads();
+            for (int w = 0; w < 8; ++w) mx = smax[w] > mx ? smax[w] : mx;
+        }
+        if (r >= p.R) return;
+        const int e = exponent_from_maxbits(mx);
+        if (at == 0) j.e[r] = e;
+        for (int64_t k = 4 * at; k < p.K; k += 4 * step) {
+            const int nv = p.K - k < 4 ? (int)(p.K - k) : 4;
+            double v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = u < nv ? x[k + u] : 0.0;
+            put_digits(v, e, a.s, j.dst + r * j.ldk + k, j.plane, nv);
+        }
+        return;
+    }
+    const int64_t r0 = (b % p.tiles) * 32, k0 = (b / p.tiles) * 64;
+    for (int i = warp; i < 64; i += 8) {
+        const int64_t r = r0 + lane, k = k0 + i;
+        tile[i & 1][i >> 1][lane] = (r < p.R && k < p.K) ? j.X[r + k * j.ld] : 0.0;
+    }
+    int be = 0;
+    for (int sl = warp; sl < p.nslice; sl += 8) {
+        const int v = r0 + lane < p.R ? j.part[(int64_t)sl * p.R + r0 + lane] : 0;
+        be = v > be ? v : be;
+    }
+    part[warp][lane] = be;
+    __syncthreads();
+    if (warp == 0) {
+        for (int w = 1; w < 8; ++w) be = part[w][lane] > be ? part[w][lane] : be;
+        es[lane] = exponent_from_maxbits((uint64_t)be << 52);
+        if (k0 == 0 && r0 + lane < p.R) j.e[r0 + lane] = es[lane];
     }
     __syncthreads();
-    for (int i = ly; i < 32; i += 8) {
-        const int64_t r = tr + i, k = tk + lx;
-        if (r < R && k < K) put_digits(tile[lx][i], e[r], s, dst, r * ldk + k, plane);
+    const int64_t k = k0 + 2 * lane;
+    const int nv = p.K - k < 2 ? (int)(p.K - k) : 2;
+    for (int i = warp; i < 32; i += 8) {
+        if (r0 + i >= p.R || nv <= 0) break;
+        const double v[2] = {tile[0][lane][i], tile[1][lane][i]};
+        put_digits(v, es[i], a.s, j.dst + (r0 + i) * j.ldk + k, j.plane, nv);
     }
-}
-
-int grid_for(int64_t work, int per_block) {
-    int64_t nb = ceil_div(work, per_block);
-    if (nb > 152 * 16) nb = 152 * 16;
-    return (int)(nb < 1 ? 1 : nb);
 }
 
 }  // namespace
@@ -268,37 +306,43 @@ int64_t exact_plane_words(int64_t M, int64_t N, int64_t nbatch, int s) {
     return all < most ? all : most;
 }
 
-int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, int64_t ld, int *e,
-               __nv_bfloat16 *dst, int64_t ldk, int64_t plane, int s, const DevState *state, cudaStream_t st) {
-    if (rows <= 0 || cols <= 0) return OMM_OK;
+int exact_pack(const PackJob &A, const PackJob *B, int s, const DevState *state, cudaStream_t st) {
     if (s < 1 || s > kExactMaxDigits) return OMM_ERR_ARG;
-    if (k_along_rows) {   // K = rows, operand rows = cols
-        OMM_CUDA_TRY(launch_pdl(exp_cm_kernel, dim3(grid_for(cols * 32, 256)), dim3(256), 0, st, rows, cols, X, ld,
-                                e, state));
-        count_launch();
-        OMM_CUDA_TRY(cudaGetLastError());
-        dim3 grid((unsigned)ceil_div(rows, 256 * 2), (unsigned)(cols < 8192 ? cols : 8192));
-        OMM_CUDA_TRY(launch_pdl(digits_cm_kernel, grid, dim3(256), 0, st, rows, cols, X, ld, e, dst, ldk, plane, s,
-                                state));
-        count_launch();
-        OMM_CUDA_TRY(cudaGetLastError());
-    } else {              // K = cols, operand rows = rows
-        // biased exponents by an atomic max over K slices of 256 columns, then exponents
-        OMM_CUDA_TRY(cudaMemsetAsync(e, 0, (size_t)rows * sizeof(int), st));
-        const int64_t kslice = 256;
-        dim3 eg((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, kslice));
-        OMM_CUDA_TRY(launch_pdl(exp_t_split_kernel, eg, dim3(256), 0, st, rows, cols, X, ld, e, kslice, state));
-        count_launch();
-        OMM_CUDA_TRY(cudaGetLastError());
-        OMM_CUDA_TRY(launch_pdl(exp_finish_kernel, dim3(grid_for(rows, 256)), dim3(256), 0, st, rows, e, state));
-        count_launch();
-        OMM_CUDA_TRY(cudaGetLastError());
-        dim3 grid((unsigned)ceil_div(rows, 32), (unsigned)ceil_div(cols, 32));
-        OMM_CUDA_TRY(launch_pdl(digits_t_kernel, grid, dim3(256), 0, st, rows, cols, X, ld, e, dst, ldk, plane, s,
-                                state));
-        count_launch();
-        OMM_CUDA_TRY(cudaGetLastError());
+    PackArgs a{};
+    a.s = s;
+    a.state = state;
+    int64_t bmax = 0, bdig = 0;
+    const PackJob *jobs[2] = {&A, B};
+    for (int i = 0; i < 2; ++i) {
+        if (jobs[i] == nullptr) continue;
+        PackBlocks &p = a.p[i];
+        p.j = *jobs[i];
+        p.R = p.j.k_along_rows ? p.j.cols : p.j.rows;
+        p.K = p.j.k_along_rows ? p.j.rows : p.j.cols;
+        if (p.R <= 0 || p.K <= 0) continue;
+        int64_t nb, nm = 0;
+        if (p.j.k_along_rows) {
+            nb = p.K <= kWarpK ? ceil_div(p.R, 8) : p.R;
+        } else {
+            p.slice = ceil_div(ceil_div(p.K, kDigitSlices), 8) * 8;
+            p.nslice = (int)ceil_div(p.K, p.slice);
+            nm = ceil_div(p.R, 128) * p.nslice;
+            p.tiles = (int)ceil_div(p.R, 32);
+            nb = p.tiles * ceil_div(p.K, 64);
+        }
+        bmax += nm;
+        bdig += nb;
+        if (bdig > 2147483647) return OMM_ERR_ARG;
+        p.blocks_max = (int)nm;
+        p.blocks = (int)nb;
     }
+    if (bdig == 0) return OMM_OK;
+    if (bmax > 0) {
+        OMM_CUDA_TRY(launch_pdl(row_max_kernel, dim3((unsigned)bmax), dim3(128), 0, st, a));
+        count_launch();
+    }
+    OMM_CUDA_TRY(launch_pdl(digit_pack_kernel, dim3((unsigned)bdig), dim3(256), 0, st, a));
+    count_launch();
     return OMM_OK;
 }
 
@@ -392,7 +436,7 @@ int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs
 extern "C" int64_t omm_op_exact_gemm_workspace_bytes(int64_t M, int64_t N, int64_t K, int32_t ndigits) {
     if (M < 0 || N < 0 || K < 0 || ndigits < 1 || ndigits > omm::tc::kExactMaxDigits) return -1;
     const int64_t ldk = (K + 7) / 8 * 8;
-    return (int64_t)ndigits * (M + N) * ldk * 2 + (M + N) * 4 + 2048 +
+    return (int64_t)ndigits * (M + N) * ldk * 2 + (1 + omm::tc::kDigitSlices) * (M + N) * 4 + 2048 +
            4 * omm::tc::exact_plane_words(M, N, 1, ndigits);
 }
 
@@ -415,21 +459,19 @@ extern "C" int omm_op_exact_gemm(int32_t transA, int32_t transB, int64_t M, int6
     __nv_bfloat16 *Bd = Ad + (int64_t)ndigits * M * ldk;
     int *eA = (int *)(Bd + (int64_t)ndigits * N * ldk);
     int *eB = eA + M;
+    int *part = eB + N;   // row maxima of an operand whose K runs along its columns
     int rc;
-    // op(A) M x K: rows of op(A) are K-major operand rows
-    if ((rc = tc::exact_pack(transA != 0, transA ? K : M, transA ? M : K, A, lda, eA, Ad, ldk, M * ldk, ndigits,
-                             nullptr, st)))
-        return rc;
-    // op(B) K x N: columns of op(B) are K-major operand rows
-    if ((rc = tc::exact_pack(transB == 0, transB ? N : K, transB ? K : N, B, ldb, eB, Bd, ldk, N * ldk, ndigits,
-                             nullptr, st)))
-        return rc;
+    // op(A) M x K: rows of op(A) are K-major operand rows; op(B) K x N: columns of op(B)
+    const tc::PackJob pa{transA != 0, transA ? K : M, transA ? M : K, A, lda, eA, Ad, ldk, M * ldk, part};
+    const tc::PackJob pb{transB == 0, transB ? N : K, transB ? K : N, B, ldb, eB, Bd, ldk, N * ldk,
+                         part + tc::kDigitSlices * M};
+    if ((rc = tc::exact_pack(pa, &pb, ndigits, nullptr, st))) return rc;
     CUtensorMap ma, mb;
     if ((rc = tc::make_digit_map(&ma, Ad, K, M, ldk, M * ldk, ndigits, 128))) return rc;
     if ((rc = tc::make_digit_map(&mb, Bd, K, N, ldk, N * ldk, ndigits, 128))) return rc;
     tc::ExactArgs a{};
     a.s = ndigits;
-    a.planes = (uint32_t *)(((uintptr_t)(eB + N) + 255) & ~(uintptr_t)255);
+    a.planes = (uint32_t *)(((uintptr_t)(part + tc::kDigitSlices * (M + N)) + 255) & ~(uintptr_t)255);
     a.M = (int)M;
     a.N = (int)N;
     a.K = (int)K;

@@ -35,10 +35,22 @@ struct ExactArgs {
 // a slab of columns (exact_gemm then works slab by slab).
 int64_t exact_plane_words(int64_t M, int64_t N, int64_t nbatch, int s);
 // Digits of the K-major operand rows of the FP64 column-major matrix X (rows x cols, ld):
-// k_along_rows: operand row r = column r of X, K = rows; else operand row r = row r of X, K = cols.
+// k_along_rows: operand row r = column r of X, K = rows; else operand row r = row r of X,
+// K = cols, and part holds kDigitSlices ints per row.
 // Writes the row exponents e[] and planes dst[t * plane + r * ldk + k].
-int exact_pack(bool k_along_rows, int64_t rows, int64_t cols, const double *X, int64_t ld, int *e,
-               __nv_bfloat16 *dst, int64_t ldk, int64_t plane, int s, const DevState *state, cudaStream_t st);
+constexpr int kDigitSlices = 16;
+struct PackJob {
+    bool k_along_rows;
+    int64_t rows, cols;
+    const double *X;
+    int64_t ld;
+    int *e;
+    __nv_bfloat16 *dst;
+    int64_t ldk, plane;
+    int *part;
+};
+// one or two operands (B nullable) with s digits
+int exact_pack(const PackJob &A, const PackJob *B, int s, const DevState *state, cudaStream_t st);
 int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs &a, int nbatch, cudaStream_t st);
 
 }  // namespace tc
