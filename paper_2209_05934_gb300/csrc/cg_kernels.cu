@@ -13,82 +13,13 @@
 #include "linemin.cuh"
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "reduce.cuh"
 
 namespace omm {
 namespace {
 
 constexpr int NT = 256;
 constexpr int TILE = 32;
-
-template <int NV>
-__device__ void block_sum(double (&v)[NV], double *red /* smem NV*8 */) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double s = v[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        v[q] = s;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < NV; ++q) red[warp * NV + q] = v[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = 0.0;
-            for (int w = 0; w < NT / 32; ++w) s += red[w * NV + q];
-            v[q] = s;
-        }
-    }
-    __syncthreads();
-}
-
-// Publish this block's NV partials; returns true in the last block to finish,
-// whose threads then all hold the totals in `tot`.  The last block sums the
-// partials in a fixed order (warp per value, lane-strided blocks, shuffle tree),
-// so the result does not depend on which block finished last.
-template <int NV>
-__device__ bool publish_and_collect(const double (&v)[NV], double *partials, unsigned int *counter,
-                                    double (&tot)[NV], double *red) {
-    __shared__ bool is_last;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) partials[blockIdx.x * NV + q] = v[q];
-        __threadfence();
-        const unsigned prev = atomicAdd(counter, 1u);
-        is_last = (prev == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    // warp w sums values w, w + NT/32, ...: its lanes take blocks lane, lane + 32,
-    // ... in order, then a fixed shuffle tree (one dependent chain per value on
-    // the long-latency FP64 unit, instead of a block-wide tree per value)
-    for (int q = threadIdx.x >> 5; q < NV; q += NT / 32) {
-        double s = 0.0;
-        // the lane's blocks in order, eight loads in flight at a time
-        unsigned b = threadIdx.x & 31;
-        for (; b + 224 < gridDim.x; b += 256) {
-            double p[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) p[k] = __ldcg(&partials[(b + 32 * k) * NV + q]);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s += p[k];
-        }
-        for (; b < gridDim.x; b += 32) s += __ldcg(&partials[b * NV + q]);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if ((threadIdx.x & 31) == 0) red[q] = s;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NV; ++q) tot[q] = red[q];
-    if (threadIdx.x == 0) *counter = 0u;
-    __syncthreads();   // red is free again for the caller
-    return true;
-}
 
 __device__ inline bool finite(double x) { return isfinite(x); }
 
@@ -122,7 +53,7 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int n, const double *__restr
     pdl_wait();
     if (state != nullptr && *((volatile int *)&state->done)) return;
     __shared__ double Xt[TILE][TILE + 1];
-    __shared__ double red[(NT / 32) * NC];
+    __shared__ double red[(NT / 32) * 16];
     const int lx = threadIdx.x % TILE, ly = threadIdx.x / TILE;
     const int T = (n + TILE - 1) / TILE;
     const int64_t ntiles = (int64_t)T * T;
@@ -160,9 +91,9 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int n, const double *__restr
             v[12] = fma(vs2, vh2, v[12]);
         }
     }
-    block_sum<NC>(v, red);
+    const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_and_collect<NC>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x >= 32) return;   // warp 0: the line minimum
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -205,7 +136,7 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
     pdl_wait();
     if (*((volatile int *)&state->done)) return;
     __shared__ double Tt[4][TILE][TILE + 1];
-    __shared__ double red[(NT / 32) * NE];
+    __shared__ double red[(NT / 32) * 4];
     const int lx = threadIdx.x % TILE, ly = threadIdx.x / TILE;
     const int T = (n + TILE - 1) / TILE;
     const int64_t ntiles = (int64_t)T * T;
@@ -253,9 +184,9 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
             v[2] = fma(e, e, v[2]);
         }
     }
-    block_sum<NE>(v, red);
+    const double sum = block_totals<NE>(v, red);
     double tot[NE];
-    if (!publish_and_collect<NE>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NE>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->trh0 = tot[0];
@@ -355,7 +286,7 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t mn, const double *__re
                                                    int first) {
     pdl_wait();
     if (*((volatile int *)&state->done)) return;
-    __shared__ double red[(NT / 32) * ND];
+    __shared__ double red[(NT / 32) * 4];
     double v[ND] = {0.0, 0.0, 0.0};
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < mn; i += (int64_t)gridDim.x * NT) {
         const double g = G[i], z = Zg[i];
@@ -365,9 +296,9 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t mn, const double *__re
             v[2] = fma(g, D[i], v[2]);
         }
     }
-    block_sum<ND>(v, red);
+    const double sum = block_totals<ND>(v, red);
     double tot[ND];
-    if (!publish_and_collect<ND>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<ND>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;

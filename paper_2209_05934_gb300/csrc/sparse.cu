@@ -25,6 +25,7 @@
 #include "fp_convert.cuh"
 #include "linemin.cuh"
 #include "omm_internal.cuh"
+#include "reduce.cuh"
 #include "sparse.cuh"
 
 namespace omm {
@@ -941,7 +942,7 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int64_t nnzN, const int32_t 
                                                      const double *__restrict__ h2, const double *__restrict__ s2,
                                                      double *partials, unsigned int *counter, DevState *state) {
     if (done(state)) return;
-    __shared__ double red[(NT / 32) * NC];
+    __shared__ double red[(NT / 32) * 16];
     double v[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) v[q] = 0.0;
@@ -963,9 +964,9 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int64_t nnzN, const int32_t 
         v[11] = fma(vs2, vx, v[11]);
         v[12] = fma(vs2, vh2, v[12]);
     }
-    block_sum<NC>(v, red);
+    const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_and_collect<NC>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x >= 32) return;   // warp 0: the line minimum
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -996,7 +997,7 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int64_t nnzN, const int32
                                                         int64_t n, double *partials, unsigned int *counter,
                                                         DevState *state, int mode) {
     if (done(state)) return;
-    __shared__ double red[(NT / 32) * NE3];
+    __shared__ double red[(NT / 32) * 4];
     const double x = state->x;
     double v[NE3] = {0.0, 0.0, 0.0};
     const int64_t total = nnzN * 4;
@@ -1017,9 +1018,9 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int64_t nnzN, const int32
         const double ee = vs - (dg ? 1.0 : 0.0);
         v[2] = fma(ee, ee, v[2]);
     }
-    block_sum<NE3>(v, red);
+    const double sum = block_totals<NE3>(v, red);
     double tot[NE3];
-    if (!publish_and_collect<NE3>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NE3>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->orth2 = tot[2];
