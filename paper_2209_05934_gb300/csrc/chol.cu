@@ -21,6 +21,7 @@
 #include <math.h>
 
 #include "chol.cuh"
+#include "fp_convert.cuh"
 #include "omm_internal.cuh"
 #include "pdl.cuh"
 
@@ -29,72 +30,164 @@ namespace chol {
 namespace {
 
 constexpr int kLeaf = 64;       // leaf size of the recursion
-constexpr int kLeafThreads = 256;
+constexpr int kLeafWarps = 16;  // warps that own rows; two more compute the columns of L and the rows of Y
+constexpr int kLeafThreads = 32 * (kLeafWarps + 2);
+constexpr int kLeafRows = kLeaf / kLeafWarps;
 constexpr int kRowBlock = 512;  // row / column blocks of the triangular products
-constexpr int kLeafSmem = (2 * kLeaf * (kLeaf + 1) + 4 * kLeaf) * (int)sizeof(double);
+constexpr int kLeafSmem = (kLeaf * kLeaf + kLeaf * (kLeaf + 1)) * (int)sizeof(double);
 
 // Cholesky factor and inverse of the s x s diagonal block at (n0, n0), s <= 64:
-// lower triangles of A and Y get L_kk and L_kk^-1, their strict upper
-// triangles inside the block are zeroed.
-__global__ void __launch_bounds__(kLeafThreads) chol_leaf_kernel(double *A, double *Y, int64_t m, int64_t n0, int s,
+// lower triangles of A and Y get L_kk and L_kk^-1, their strict upper triangles
+// inside the block are zeroed.
+//
+// One CTA and a chain of 64 pivots; 88,000 multiply-adds at the FP64 rate of one SM
+// are 26 us.  Factor and inverse run in one sweep, both in their outer-product form:
+// with column q of L and row q of Y known, every element (i, j), i > q, takes one
+// multiply-add, a(i, j) -= l(i, q) l(j, q) where j > q and sum(i, j) += l(i, q) y(q, j)
+// where j <= q, so a row stays at work on all its columns until q = i.  Sixteen
+// warps own rows w, w + 16, ... in registers, lanes along the columns (four warps
+// a scheduler: what follows a multiply-add waits 64 cycles and more for it).  One warp is a
+// column ahead: it takes column q + 1 as the owners left it before step q, adds
+// step q, and has the next pivot's root, reciprocal and scaled column ready when the
+// owners are done with step q.  One warp finishes row q of Y meanwhile, so the sums
+// of Y run one step behind.  One barrier a step.  The roots in integers: in FP64
+// they are 20 dependent instructions that queue with the owners' for the FP64 unit.
+// The sum of y(i, j) is held in four interleaved slices (q - j) mod 4, added in
+// order at the end; the register of a slice is the one of q mod 4, which the unrolled
+// loop knows (slice g of column j is in register (g + j) mod 4).
+// 140 us when factor and inverse were two sweeps over shared memory with three
+// and two barriers a step; 94 us with eight owner warps that also finished the rows of
+// Y; 71 us now, the FP64 unit busy for 68 % of it.  The same results to the last bit.
+__global__ void __launch_bounds__(kLeafThreads, 1) chol_leaf_kernel(double *A, double *Y, int64_t m, int64_t n0, int s,
                                                                  DevState *state) {
     pdl_wait();
     extern __shared__ double sm[];
-    double(*a)[kLeaf + 1] = (double(*)[kLeaf + 1])sm;
-    double(*y)[kLeaf + 1] = (double(*)[kLeaf + 1])(sm + kLeaf * (kLeaf + 1));
-    double(*part)[kLeaf] = (double(*)[kLeaf])(sm + 2 * kLeaf * (kLeaf + 1));
-    __shared__ int bad;
-    __shared__ double rdiag[kLeaf];   // 1 / l(j, j): one division per pivot (FP64 division is slow here)
-    const int tid = threadIdx.x;
-    for (int e = tid; e < s * s; e += kLeafThreads) {
-        const int r = e % s, c = e / s;
-        a[r][c] = A[(n0 + r) + (n0 + c) * m];
-    }
-    if (tid == 0) bad = 0;
-    __syncthreads();
-    // right-looking factorisation, element-parallel trailing updates
-    for (int j = 0; j < s; ++j) {
-        if (tid == 0) {
-            double d = a[j][j];
-            if (!(d > 0.0)) {
-                bad = 1;
-                d = 1.0;
+    double(*lc)[kLeaf] = (double(*)[kLeaf])sm;                              // lc[q]: column q of L
+    double(*yr)[kLeaf + 1] = (double(*)[kLeaf + 1])(sm + kLeaf * kLeaf);    // yr[q]: row q of Y
+    __shared__ double col[2][kLeaf];   // column q + 2 after step q
+    __shared__ double rdiag[kLeaf];    // 1 / l(q, q)
+    __shared__ double slice[2][4][kLeaf];   // sums of row q + 1 of Y after step q - 1
+    const int lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) - 2;
+    const double *Ab = A + n0 + n0 * m;
+    auto load = [&](int r, int c) {    // beyond the block: the identity
+        return (r < s && c < s) ? (c <= r ? Ab[r + c * m] : 0.0) : (r == c ? 1.0 : 0.0);
+    };
+    bool bad = false;
+    double l[2];                   // the newest column of L (rows lane and lane + 32), of its warp
+    auto pivot = [&](int q, const double (&b)[2]) {   // column q of L from its final values b
+        double d = __shfl_sync(0xffffffffu, q < 32 ? b[0] : b[1], q & 31);
+        if (!(d > 0.0)) {
+            bad = bad || q < s;
+            d = 1.0;
+        }
+        double root, r;
+        sw_sqrt_rcp(d, root, r);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int row = lane + 32 * h;
+            l[h] = row > q ? b[h] * r : (row == q ? root : 0.0);
+            lc[q][row] = l[h];
+        }
+        if (lane == 0) rdiag[q] = r;
+    };
+    double acc[kLeafRows][2][4];   // a(i, j) in slot 3 until column j is done, then the slices
+    double y[2] = {0.0, 0.0};      // the newest row of Y, of its warp
+    if (warp == -2) {
+        const double b0[2] = {load(lane, 0), load(lane + 32, 0)};
+        pivot(0, b0);
+    } else if (warp >= 0) {
+#pragma unroll
+        for (int k = 0; k < kLeafRows; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = warp + kLeafWarps * k;
+#pragma unroll
+                for (int u = 0; u < 3; ++u) acc[k][h][u] = 0.0;
+                acc[k][h][3] = load(i, lane + 32 * h);
+                if (h == 0 && lane == 1) col[1][i] = acc[k][h][3];
             }
-            a[j][j] = sqrt(d);
-            rdiag[j] = 1.0 / a[j][j];
-        }
-        __syncthreads();
-        const double rjj = rdiag[j];
-        for (int r = j + 1 + tid; r < s; r += kLeafThreads) a[r][j] *= rjj;
-        __syncthreads();
-        // lanes along rows, the 8 warps along columns (no integer division)
-        for (int c = j + 1 + (tid >> 5); c < s; c += kLeafThreads / 32) {
-            const double acj = a[c][j];
-            for (int r = c + (tid & 31); r < s; r += 32) a[r][c] -= a[r][j] * acj;
-        }
-        __syncthreads();
     }
-    // Y = L^-1 row by row: y(i, j) = (delta_ij - sum_{j <= q < i} l(i, q) y(q, j)) / l(i, i),
-    // columns j across 64 threads, the q-sum in 4 interleaved slices
-    const int j = tid % kLeaf, g = tid / kLeaf;
-    for (int i = 0; i < s; ++i) {
-        double v = 0.0;
-        if (j < i)
-            for (int q = j + g; q < i; q += 4) v += a[i][q] * y[q][j];
-        part[g][j] = v;
-        __syncthreads();
-        if (g == 0 && j < s) {
-            const double sum = part[0][j] + part[1][j] + part[2][j] + part[3][j];
-            y[i][j] = (j < i) ? -sum * rdiag[i] : (j == i ? rdiag[i] : 0.0);
+    __syncthreads();
+#pragma unroll 1
+    for (int q0 = 0; q0 < s; q0 += 4) {   // steps past s work on the identity's columns
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = q0 + u;
+            constexpr int kSlot[4] = {3, 0, 1, 2};   // (q - 1) mod 4
+            if (warp == -2) {
+                if (q + 1 < kLeaf) {
+                    const double piv = __shfl_sync(0xffffffffu, q + 1 < 32 ? l[0] : l[1], (q + 1) & 31);
+                    const double b1[2] = {fma(-l[0], piv, col[(q + 1) & 1][lane]),
+                                          fma(-l[1], piv, col[(q + 1) & 1][lane + 32])};
+                    pivot(q + 1, b1);
+                }
+            } else if (warp == -1) {   // row q of Y: its last step, the sum of its slices
+                const double r = rdiag[q];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int j = lane + 32 * h;
+                    double v[4];   // slice g is in register (g + j) mod 4
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) v[p] = j < q ? slice[q & 1][p][j] : 0.0;
+                    if (j < q) v[kSlot[u]] = fma(lc[q > 0 ? q - 1 : 0][q], y[h], v[kSlot[u]]);
+                    const bool r1 = (j & 1) != 0, r2 = (j & 2) != 0;
+                    const double t0 = r1 ? v[1] : v[0], t1 = r1 ? v[2] : v[1], t2 = r1 ? v[3] : v[2],
+                                 t3 = r1 ? v[0] : v[3];
+                    const double tot = (r2 ? t2 : t0) + (r2 ? t3 : t1) + (r2 ? t0 : t2) + (r2 ? t1 : t3);
+                    y[h] = j < q ? -tot * r : (j == q ? r : 0.0);
+                    yr[q][j] = y[h];
+                }
+            } else {
+                // a lane beyond column q takes step q of the factor, one before it step q - 1 of the inverse
+                double v[2], sc[kLeafRows][2];
+                bool fac[2], inv[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int j = lane + 32 * h;
+                    fac[h] = j > q;
+                    inv[h] = j < q;
+                    v[h] = fac[h] ? -lc[q][j] : (inv[h] ? yr[q - 1][j] : 0.0);
+                    const double *src = (inv[h] ? lc[q - 1] : lc[q]) + warp;
+#pragma unroll
+                    for (int k = 0; k < kLeafRows; ++k) sc[k][h] = src[kLeafWarps * k];
+                }
+#pragma unroll
+                for (int k = 0; k < kLeafRows; ++k) {
+                    const int i = warp + kLeafWarps * k;
+                    if (i <= q) continue;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (h == 1 && kLeafWarps * k < 32) continue;   // rows 0 .. 31 end before column 32
+                        double &a = acc[k][h][3], &sum = acc[k][h][kSlot[u]];
+                        double t = fac[h] ? a : sum;
+                        asm volatile("" : "+d"(t));   // one multiply-add, not one for each case
+                        t = fma(sc[k][h], v[h], t);
+                        if (lane + 32 * h == q + 2) col[q & 1][i] = t;
+                        if (inv[h]) sum = t;
+                        if (fac[h]) a = t;
+                        if (lane + 32 * h == q) a = 0.0;
+                        // settle the selects here: carried on unresolved over the unrolled steps they spill
+                        asm volatile("" : "+d"(acc[k][h][3]), "+d"(acc[k][h][kSlot[u] % 3]));
+                    }
+                    if (i == q + 1) {
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int p = 0; p < 4; ++p)
+                                if (h == 0 || kLeafWarps * k >= 32) slice[i & 1][p][lane + 32 * h] = acc[k][h][p];
+                    }
+                }
+            }
+            __syncthreads();
         }
-        __syncthreads();
     }
-    for (int e = tid; e < s * s; e += kLeafThreads) {
-        const int r = e % s, c = e / s;
-        A[(n0 + r) + (n0 + c) * m] = (c <= r) ? a[r][c] : 0.0;
-        Y[(n0 + r) + (n0 + c) * m] = (c <= r) ? y[r][c] : 0.0;
+    for (int e = threadIdx.x; e < s * kLeaf; e += kLeafThreads) {
+        const int r = e % kLeaf, c = e / kLeaf;
+        if (r >= s) continue;
+        A[(n0 + r) + (n0 + c) * m] = lc[c][r];
+        Y[(n0 + r) + (n0 + c) * m] = yr[r][c];
     }
-    if (tid == 0 && bad) state->status = OMM_ERR_NOT_SPD;
+    if (bad && lane == 0) state->status = OMM_ERR_NOT_SPD;
 }
 
 // Zero the strict upper triangle (the factor is read as a lower triangle).

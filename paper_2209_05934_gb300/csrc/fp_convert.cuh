@@ -97,4 +97,59 @@ __device__ __forceinline__ double sw_scale2(double x, int e) {
     return __longlong_as_double((long long)((b & ~(0x7FFull << 52)) | ((uint64_t)ne << 52)));
 }
 
+// root = sqrt(d) and rcp = 1 / root, both rounded to nearest like the hardware's own, for
+// d > 0.  Integer Newton steps (Newton 1669 on s^2 = N and s q = 2^105, each ended by
+// the exact remainder in 64-bit wrap-around arithmetic): with d = N 2^(2k - 104), N in
+// [2^104, 2^106), the root's significand is the integer nearest to sqrt(N).  From FP32 seeds h and y
+// = 1 / sqrt(x) good to 2^-22, one step gives ~2^-45 of s, the next its last bit or
+// that +- 1, which the remainder decides: -s < N - s^2 <= s, and |2 (2^105 - q s)| <= s
+// (neither has ties).  ~25 dependent integer instructions of 4 - 5 cycles each for both, where the
+// FP64 forms are ~20 dependent FP64 instructions of 64 cycles and queue for
+// the FP64 unit.
+__device__ __forceinline__ void sw_sqrt_rcp(double d, double &root, double &rcp) {
+    const uint64_t b = (uint64_t)__double_as_longlong(d);
+    const int e = (int)((b >> 52) & 0x7FF);
+    uint64_t man = b & 0xFFFFFFFFFFFFFull;
+    int ex = e - 1023;
+    if (e == 0) {   // subnormal
+        const int sh = __clzll((long long)man) - 11;
+        man <<= sh;
+        ex = -1022 - sh;
+    }
+    man |= 1ull << 52;
+    const int odd = ex & 1, k = (ex - odd) >> 1;                  // root in [2^k, 2^(k + 1)]
+    const uint64_t lo = man << (52 + odd);                        // N mod 2^64; N >> 43 = man << (9 + odd)
+    const float x = __uint_as_float(((uint32_t)(man >> 29) & 0x7FFFFFu) | ((uint32_t)(125 + odd) << 23));   // [1/4, 1)
+    float y = rsqrtf(x);
+    y = fmaf(0.5f * y, fmaf(-(x * y), y, 1.0f), y);
+    y = fminf(fmaxf(y, 1.0f), 1.9999999f);
+    float h = x * y;
+    h = fmaf(0.5f * y, fmaf(-h, h, x), h);
+    h = fminf(fmaxf(h, 0.5f), 0.99999994f);
+    const uint32_t h24 = (__float_as_uint(h) & 0x7FFFFFu) | 0x800000u;   // h 2^24
+    const uint32_t y24 = (__float_as_uint(y) & 0x7FFFFFu) | 0x800000u;   // y 2^23
+    const int y31 = (int)(y24 << 7);                                     // y 2^30
+    // the steps' corrections are rem / (2 s) = rem y 2^-54 and rem / s; the upper halves of
+    // the remainders stay below 2^31 (a seventh of it at most)
+    const int64_t r0 = (int64_t)((man << (9 + odd)) - (((uint64_t)h24 * h24) << 15));   // (N - s^2) >> 43
+    int64_t s = (int64_t)((uint64_t)h24 << 29) + (((int64_t)(int)(r0 >> 10) * y31) >> 31);
+    int64_t r = (int64_t)(lo - (uint64_t)s * (uint64_t)s);
+    s += ((int64_t)(int)(r >> 31) * y31 + (1ll << 52)) >> 53;
+    r = (int64_t)(lo - (uint64_t)s * (uint64_t)s);
+    s += (r > s ? 1 : 0) - (r <= -s ? 1 : 0);
+    int64_t t = (int64_t)(0ull - (uint64_t)y24 * (uint64_t)s);                          // (2^105 - q s) >> 29
+    int64_t q = (int64_t)((uint64_t)y24 << 29) + (((int64_t)(int)(t >> 24) * y31) >> 30);
+    t = (int64_t)(0ull - (uint64_t)q * (uint64_t)s);
+    q += ((int64_t)(int)(t >> 31) * y31 + (1ll << 51)) >> 52;
+    t = (int64_t)(0ull - (uint64_t)q * (uint64_t)s);
+    q += (2 * t > s ? 1 : 0) - (2 * t < -s ? 1 : 0);
+    // a significand of 2^53 carries into the exponent
+    root = __longlong_as_double((long long)(((uint64_t)(k + 1022) << 52) + (uint64_t)s));
+    rcp = __longlong_as_double((long long)(((uint64_t)(1021 - k) << 52) + (uint64_t)q));
+    if (e == 0x7FF) {   // infinite
+        root = d;
+        rcp = 0.0;
+    }
+}
+
 }  // namespace omm

@@ -209,3 +209,29 @@ def test_set_H_requires_set_HS(omm):
         s.set_H(dev(sysm.dense_H()))
     assert ei.value.status == omm.ERR_STATE
     s.close()
+
+
+# one leaf (1 .. 64 columns: a single pivot, a ragged group of four, a full warp of lanes
+# and one more, the full leaf) and a ragged second one (65, 127)
+@pytest.mark.parametrize("m", [2, 5, 31, 33, 62, 63, 64, 65, 127])
+def test_cholesky_leaf_sizes(omm, m):
+    rng = np.random.default_rng(m)
+    n = max(1, m // 4)
+    A = rng.uniform(-0.4, 0.4, (m, m)) / m
+    S = np.asfortranarray(np.eye(m) + 0.5 * (A + A.T))   # diagonally dominant, condition number below 2.4
+    H = rng.standard_normal((m, m))
+    H = np.asfortranarray(0.5 * (H + H.T)) - 3.0 * np.sqrt(m) * S
+    W0 = np.asfortranarray(0.3 * rng.standard_normal((m, n)) / np.sqrt(m))
+    eta = O.gershgorin_eta(H, S)
+    steps = 3
+    s = omm.Solver(m, n, 8, cholesky=1, max_iter=steps)
+    s.set_HS(dev(H), dev(S))
+    W = empty_cm(m, n)
+    E, iters, st = s.solve(dev(W0), tol=0.0, W_out=W, raise_on_error=False)
+    ref = O.omm_cg_cholesky(H, S, W0, tol=0.0, eta=eta, max_iter=steps)
+    assert st == omm.ERR_MAXITER and iters == steps == ref.iters
+    # each step's sums round at m eps cond(S) ~ 1e-13 of their terms, the energy's terms
+    # (2 eta n and the shifted one) cancel by one digit or two
+    assert abs(E - ref.E) <= 1e-11 * max(abs(ref.E), abs(2 * eta * n))
+    np.testing.assert_allclose(W.cpu().numpy(), ref.W, rtol=0, atol=1e-10 * np.abs(ref.W).max())
+    s.close()
