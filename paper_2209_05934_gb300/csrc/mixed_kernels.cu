@@ -92,8 +92,11 @@ __device__ __forceinline__ void to_f64(const float (&f)[NV], double (&v)[NV]) {
     }
 }
 
+// Sums of NV values over the block, value t in lane t of warp 0: the warps' sums added
+// in order, a lane per value (one thread for all of them took 8 NV additions, at ~18
+// cycles each for the SM's FP64 unit and three blocks an SM).
 template <int NV>
-__device__ void block_sum(double (&v)[NV], double *red, bool lane0_only = false) {
+__device__ __forceinline__ double block_sum(double (&v)[NV], double *red, bool lane0_only = false) {
     if (!lane0_only) {
 #pragma unroll
         for (int q = 0; q < NV; ++q) {
@@ -108,26 +111,24 @@ __device__ void block_sum(double (&v)[NV], double *red, bool lane0_only = false)
 #pragma unroll
         for (int q = 0; q < NV; ++q) red[warp * NV + q] = v[q];
     __syncthreads();
-    if (threadIdx.x == 0) {
+    double s = 0.0;
+    if (threadIdx.x < NV)
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = 0.0;
-            for (int w = 0; w < NT / 32; ++w) s += red[w * NV + q];
-            v[q] = s;
-        }
-    }
+        for (int w = 0; w < NT / 32; ++w) s += red[w * NV + threadIdx.x];
     __syncthreads();
+    return s;
 }
 
+// v: value t in lane t of warp 0
 template <int NV>
-__device__ bool publish_and_collect(const double (&v)[NV], double *partials, unsigned int *counter,
-                                    double (&tot)[NV], double *red, unsigned blk, unsigned nblk) {
+__device__ __forceinline__ bool publish_and_collect(double v, double *partials, unsigned int *counter,
+                                                    double (&tot)[NV], double *red, unsigned blk, unsigned nblk) {
     __shared__ bool is_last;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) partials[blk * NV + q] = v[q];
+    if (threadIdx.x < 32) {
+        if (threadIdx.x < NV) partials[blk * NV + threadIdx.x] = v;
         __threadfence();
-        is_last = (atomicAdd(counter, 1u) == nblk - 1);
+        __syncwarp();
+        if (threadIdx.x == 0) is_last = (atomicAdd(counter, 1u) == nblk - 1);
     }
     __syncthreads();
     if (!is_last) return false;
@@ -220,15 +221,15 @@ __device__ __forceinline__ void mx_coeffs_body(int n, const double *__restrict__
     }
     double v[NC];
     to_f64<NC>(f, v);
-    block_sum<NC>(v, red, true);
+    const double sum = block_sum<NC>(v, red, true);
     double tot[NC] = {};
-    if (!publish_and_collect<NC>(v, partials, counter, tot, red, blk, nblk)) return;
+    if (!publish_and_collect<NC>(sum, partials, counter, tot, red, blk, nblk)) return;
     // the slope <G, D>: the direction kernel's per-block parts (one-digit
     // directions), else the dots kernel's value
     double gd[1] = {0.0};
     if (nslope > 0) {
         for (int b = threadIdx.x; b < nslope; b += NT) gd[0] += __ldcg(&slope[b]);
-        block_sum<1>(gd, red);
+        gd[0] = block_sum<1>(gd, red);
     }
     if (threadIdx.x >= 32) return;   // warp 0: the line minimum
 #pragma unroll
@@ -333,9 +334,9 @@ __device__ __forceinline__ void mx_nn_update_body(int n, double *h0, double *s0,
     const float fo[1] = {orth};
     double v[1];
     to_f64<1>(fo, v);
-    block_sum<1>(v, red, true);
+    const double sum = block_sum<1>(v, red, true);
     double tot[1];
-    if (!publish_and_collect<1>(v, partials, counter, tot, red, blk, nblk)) return;
+    if (!publish_and_collect<1>(sum, partials, counter, tot, red, blk, nblk)) return;
     if (threadIdx.x != 0) return;
     const double E = state->E_next;
     state->orth2 = tot[0];
@@ -350,7 +351,10 @@ __device__ __forceinline__ void mx_nn_update_body(int n, double *h0, double *s0,
     state->E = E;
     state->rel = rel;
     state->k += 1;
-    const bool orth_ok = !(state->orth_tol > 0.0) || sqrt(tot[0]) < state->orth_tol;
+    // the root in integers where it has one (a zero or a NaN passes through)
+    double root = tot[0], rcp;
+    if (root > 0.0) sw_sqrt_rcp(tot[0], root, rcp);
+    const bool orth_ok = !(state->orth_tol > 0.0) || root < state->orth_tol;
     if (rel < state->tol && orth_ok) {
         state->status = OMM_OK;
         state->done = 1;
@@ -557,9 +561,9 @@ __device__ __forceinline__ void mx_dots_body(int64_t mn, const float *__restrict
     }
     double v[ND];
     to_f64<ND>(f, v);
-    block_sum<ND>(v, red, true);
+    const double sum = block_sum<ND>(v, red, true);
     double tot[ND];
-    if (!publish_and_collect<ND>(v, partials, counter, tot, red, blk, nblk)) return;
+    if (!publish_and_collect<ND>(sum, partials, counter, tot, red, blk, nblk)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;
@@ -608,8 +612,8 @@ __device__ __forceinline__ void direction_slope(float gd, double *slope, unsigne
     const float f[1] = {gd};
     double v[1];
     to_f64<1>(f, v);
-    block_sum<1>(v, red, true);
-    if (threadIdx.x == 0) slope[blk] = v[0];
+    const double sum = block_sum<1>(v, red, true);
+    if (threadIdx.x == 0) slope[blk] = sum;
 }
 
 template <bool ROUND1>
@@ -813,11 +817,8 @@ __global__ void __launch_bounds__(NT, 4) mx_dots_direction4_kernel(int m, int64_
         }
         double v[ND];
         to_f64<ND>(f, v);
-        block_sum<ND>(v, red, true);
-        if (threadIdx.x == 0) {
-#pragma unroll
-            for (int q = 0; q < ND; ++q) partials[blockIdx.x * ND + q] = v[q];
-        }
+        const double sum = block_sum<ND>(v, red, true);
+        if (threadIdx.x < ND) partials[blockIdx.x * ND + threadIdx.x] = sum;
     }
     grid_barrier(bar, &state->wait_timeout);
     // the totals, warp q for value q, lanes over the blocks in order (as the
