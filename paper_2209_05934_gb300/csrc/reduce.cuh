@@ -9,30 +9,31 @@ namespace omm {
 constexpr int kRedThreads = 256;
 
 // Sums of NV (at most 16) values over the block, value t in lane t of warp 0.  The
-// lanes of a warp halve the values between them (16 + 15 additions for 13 values where a
-// tree per value takes 65: an FP64 instruction occupies this part's FP64 unit for ~18
-// cycles, and eight warps of such trees took 5 us), then warp 0 adds the warps' values
-// in order.
+// lanes of a warp halve the values between them (16 additions for 16 values where a
+// tree per value takes 80: an FP64 instruction occupies this part's FP64 unit for ~18
+// cycles, and eight warps of such trees took 5 us); the partners are the tree's, so the sums
+// are too.  Then a lane per value adds the warps' sums in order.
 template <int NV>
-__device__ __forceinline__ double block_totals(const double (&v)[NV], double *red /* smem NV*8, NV rounded up to 4 or 16 */) {
+__device__ __forceinline__ double block_totals(const double (&v)[NV], double *red /* smem 8 P, P = 4 or 16 */) {
     constexpr int P = NV <= 4 ? 4 : 16;
     static_assert(NV <= 16, "one lane per value");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double w[P];
 #pragma unroll
     for (int q = 0; q < P; ++q) w[q] = q < NV ? v[q < NV ? q : 0] : 0.0;
+    // after the step with partner lane ^ off a lane holds half as many values
 #pragma unroll
-    for (int n = P / 2; n > 0; n >>= 1) {
-        const bool up = (lane & n) != 0;
+    for (int n = P / 2, off = 16; n > 0; n >>= 1, off >>= 1) {
+        const bool up = (lane & off) != 0;
 #pragma unroll
         for (int i = 0; i < n; ++i) {
             const double give = up ? w[i] : w[i + n], keep = up ? w[i + n] : w[i];
-            w[i] = keep + __shfl_xor_sync(0xffffffffu, give, n);
+            w[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
         }
     }
 #pragma unroll
-    for (int off = P; off < 32; off <<= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], off);
-    if (lane < P) red[warp * P + lane] = w[0];
+    for (int off = 16 / P; off > 0; off >>= 1) w[0] += __shfl_xor_sync(0xffffffffu, w[0], off);
+    if (lane % (32 / P) == 0) red[warp * P + lane / (32 / P)] = w[0];
     __syncthreads();
     double s = 0.0;
     if (warp == 0 && lane < NV)

@@ -338,72 +338,6 @@ namespace {
 
 constexpr int NT = 256;
 
-// Block sum / last-block combination (fixed order; same scheme as the dense kernels)
-template <int NV>
-__device__ void block_sum(double (&v)[NV], double *red) {
-#pragma unroll
-    for (int q = 0; q < NV; ++q) {
-        double s = v[q];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        v[q] = s;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < NV; ++q) red[warp * NV + q] = v[q];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-            double s = 0.0;
-            for (int w = 0; w < NT / 32; ++w) s += red[w * NV + q];
-            v[q] = s;
-        }
-    }
-    __syncthreads();
-}
-
-template <int NV>
-__device__ bool publish_and_collect(const double (&v)[NV], double *partials, unsigned int *counter,
-                                    double (&tot)[NV], double *red) {
-    __shared__ bool is_last;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NV; ++q) partials[blockIdx.x * NV + q] = v[q];
-        __threadfence();
-        is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return false;
-    __threadfence();
-    // warp w sums values w, w + NT/32, ...: its lanes take blocks lane, lane + 32,
-    // ... in order, then a fixed shuffle tree (one dependent chain per value on
-    // the long-latency FP64 unit, instead of a block-wide tree per value)
-    for (int q = threadIdx.x >> 5; q < NV; q += NT / 32) {
-        double s = 0.0;
-        // the lane's blocks in order, eight loads in flight at a time
-        unsigned b = threadIdx.x & 31;
-        for (; b + 224 < gridDim.x; b += 256) {
-            double p[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) p[k] = __ldcg(&partials[(b + 32 * k) * NV + q]);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) s += p[k];
-        }
-        for (; b < gridDim.x; b += 32) s += __ldcg(&partials[b * NV + q]);
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
-        if ((threadIdx.x & 31) == 0) red[q] = s;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NV; ++q) tot[q] = red[q];
-    if (threadIdx.x == 0) *counter = 0u;
-    __syncthreads();   // red is free again for the caller
-    return true;
-}
-
 __device__ __forceinline__ bool done(const DevState *s) { return s != nullptr && *((volatile const int *)&s->done); }
 
 // ---- block filtering: keep[b] = ||H_b||^2 >= eps^2 or ||S_b||^2 >= eps^2, squares
@@ -1069,25 +1003,29 @@ __global__ void axpy_kernel(int64_t nW, double *W, const double *__restrict__ D,
     }
 }
 
+// FP32 to FP64 on the integer pipe (the conversion unit takes ~160 cycles a warp)
+__device__ __forceinline__ double wide(float x) { return sw_f2d(x); }
+__device__ __forceinline__ double wide(double x) { return x; }
+
 constexpr int ND = 3;
 template <typename T>
 __global__ void __launch_bounds__(NT) dots_kernel(int64_t len, const T *__restrict__ G,
                                                    const T *__restrict__ Gp, const T *__restrict__ D,
                                                    double *partials, unsigned int *counter, DevState *state, int first) {
     if (done(state)) return;
-    __shared__ double red[(NT / 32) * ND];
+    __shared__ double red[(NT / 32) * 4];
     double v[ND] = {0.0, 0.0, 0.0};
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < len; i += (int64_t)gridDim.x * NT) {
-        const double g = G[i];
+        const double g = wide(G[i]);
         v[0] = fma(g, g, v[0]);
         if (!first) {
-            v[1] = fma(g, Gp[i], v[1]);
-            v[2] = fma(g, D[i], v[2]);
+            v[1] = fma(g, wide(Gp[i]), v[1]);
+            v[2] = fma(g, wide(D[i]), v[2]);
         }
     }
-    block_sum<ND>(v, red);
+    const double sum = block_totals<ND>(v, red);
     double tot[ND];
-    if (!publish_and_collect<ND>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<ND>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;
@@ -1155,7 +1093,7 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int64_t nnzN, const int32
                                                         const float *__restrict__ h2, const float *__restrict__ s2,
                                                         double *partials, unsigned int *counter, DevState *state) {
     if (done(state)) return;
-    __shared__ double red[(NT / 32) * NC];
+    __shared__ double red[(NT / 32) * 16];
     float f[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) f[q] = 0.f;
@@ -1180,9 +1118,9 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int64_t nnzN, const int32
     double v[NC];
 #pragma unroll
     for (int q = 0; q < NC; ++q) v[q] = sw_f2d(f[q]);
-    block_sum<NC>(v, red);
+    const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_and_collect<NC>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x >= 32) return;
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -1235,7 +1173,7 @@ __global__ void __launch_bounds__(NT) mx_nn_update_kernel(int64_t nnzN, const in
                                                            const float *__restrict__ s2, float *h0s, float *s0s,
                                                            double *partials, unsigned int *counter, DevState *state) {
     if (done(state)) return;
-    __shared__ double red[(NT / 32) * NE3];
+    __shared__ double red[(NT / 32) * 4];
     const double x = state->x;
     double v[NE3] = {0.0, 0.0, 0.0};
     const int64_t total = nnzN * 4;
@@ -1251,15 +1189,18 @@ __global__ void __launch_bounds__(NT) mx_nn_update_kernel(int64_t nnzN, const in
         s0[t] = vs;
         h0s[t] = sw_d2f(vh);
         s0s[t] = sw_d2f(vs);
-        const bool dg = Ndiag[q] && a == b;
-        if (dg) v[0] += vh;
+        double ee = vs;
+        if (__any_sync(__activemask(), Ndiag[q])) {   // few warps: nothing for the FP64 unit in the others
+            const bool dg = Ndiag[q] && a == b;
+            if (dg) v[0] += vh;
+            ee = vs - (dg ? 1.0 : 0.0);
+        }
         v[1] = fma(vs, vh, v[1]);
-        const double ee = vs - (dg ? 1.0 : 0.0);
         v[2] = fma(ee, ee, v[2]);
     }
-    block_sum<NE3>(v, red);
+    const double sum = block_totals<NE3>(v, red);
     double tot[NE3];
-    if (!publish_and_collect<NE3>(v, partials, counter, tot, red)) return;
+    if (!publish_totals<NE3>(sum, partials, counter, tot, red)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->orth2 = tot[2];
