@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <new>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "chol.cuh"
@@ -62,6 +63,7 @@ struct MixedBufs {
 //   HSWx  [s][n][ld2n]  columns of [H_W ; S_W]  B of the gradient
 struct ExactBufs {
     int s = 0;
+    char *base = nullptr;   // one allocation holds them all (seven of them took 0.4 ms more to create a handle)
     __nv_bfloat16 *HSx = nullptr, *Wx = nullptr, *HWSWx = nullptr, *SWHWx = nullptr, *HSWx = nullptr;
     uint32_t *planes = nullptr;   // level planes of a product
     int *e = nullptr;   // exponents: [2m HS | n W | 2n HWSW | m SWHW | n HSW], then part
@@ -211,13 +213,7 @@ void free_handle(omm_handle *h) {
     cudaFree(h->mx.Gp32);
     cudaFree(h->mx.D32);
     cudaFree(h->mx.Df32);
-    cudaFree(h->ex.HSx);
-    cudaFree(h->ex.Wx);
-    cudaFree(h->ex.HWSWx);
-    cudaFree(h->ex.SWHWx);
-    cudaFree(h->ex.HSWx);
-    cudaFree(h->ex.planes);
-    cudaFree(h->ex.e);
+    cudaFree(h->ex.base);
     crt_free(h->cr);
     cudaFree(h->L);
     cudaFree(h->Wsave);
@@ -829,14 +825,24 @@ int exact_alloc(omm_handle *h) {
     ExactBufs &e = h->ex;
     e.s = h->opt.exact_digits;
     const int s = e.s;
-    TRY(dalloc(&e.HSx, (size_t)(s * 2 * m * x.ldm)));
-    TRY(dalloc(&e.Wx, (size_t)(s * n * x.ldm)));
-    TRY(dalloc(&e.HWSWx, (size_t)(s * 2 * n * x.ldm)));
-    TRY(dalloc(&e.SWHWx, (size_t)(s * m * x.ld2n)));
-    TRY(dalloc(&e.HSWx, (size_t)(s * n * x.ld2n)));
-    TRY(dalloc(&e.e, (size_t)(2 * m + n + 2 * n + m + n + omm::tc::kDigitSlices * m)));
     // the anchor's [H';S] W is the largest product; both it and the gradient take six digits
-    TRY(dalloc(&e.planes, (size_t)omm::tc::exact_plane_words(m, n, 2, s < 6 ? s : 6)));
+    const int64_t planes = omm::tc::exact_plane_words(m, n, 2, s < 6 ? s : 6);
+    const int64_t ints = 2 * m + n + 2 * n + m + n + omm::tc::kDigitSlices * m;
+    for (int pass = 0; pass < 2; ++pass) {   // sizes, then addresses; each part on 256 bytes
+        int64_t at = 0;
+        auto part = [&](auto *&p, int64_t count) {
+            if (pass == 1) p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(e.base + at);
+            at += (count * (int64_t)sizeof(*p) + 255) / 256 * 256;
+        };
+        part(e.HSx, s * 2 * m * x.ldm);
+        part(e.Wx, s * n * x.ldm);
+        part(e.HWSWx, s * 2 * n * x.ldm);
+        part(e.SWHWx, s * m * x.ld2n);
+        part(e.HSWx, s * n * x.ld2n);
+        part(e.e, ints);
+        part(e.planes, planes);
+        if (pass == 0) TRY(dalloc(&e.base, (size_t)at));
+    }
     e.eHS = e.e;
     e.eW = e.eHS + 2 * m;
     e.eHWSW = e.eW + n;
