@@ -328,7 +328,7 @@ def run_omm(args):
         torch.cuda.synchronize()
         ms64 = f0.elapsed_time(f1)
         d64 = s64.diag()
-        fp64_beside = {"form": "plain FP64 on CUDA cores (DFMA GEMMs), same handle API", "ms_per_solve": ms64,
+        fp64_beside = {"form": "FP64, products through residues on the BF16 tensor cores, same handle API", "ms_per_solve": ms64,
                        "solves_per_s": 1e3 / ms64, "E": E64, "status": int(st64), "iters": int(it64),
                        "orth": d64.orth, "tol": TOL["fp64"]["tol"],
                        "rel_err": abs(E64 - e_exact) / abs(e_exact) if e_exact else None,
@@ -640,7 +640,7 @@ def run_c3(args, quiet=False):
             else:
                 roof[name] = {"ms_per_launch": per, "fp64_tflops": tf, "frac_fp64": tf / fp64_peak,
                               "hbm_gbs": rows[name]["bytes"] / (per * 1e-3) / 1e9,
-                              "bound": "alu (FP64 pipe; peak: cuBLAS DGEMM measured in this run)"}
+                              "bound": "alu (wide integer multiplies of the fixed-point gathers; frac: against cuBLAS DGEMM in this run)"}
     line = {"metric": "OMM solves/s & time-to-converge, linear-scaling form", "value": 1e3 / t_ms,
             "unit": "solves/s", "n_gpus": 1, "steps": args.steps, "warmup": 1, "ms_per_step": t_ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
