@@ -374,10 +374,10 @@ __global__ void __launch_bounds__(NT, 4) mx_nn_update_kernel(int n, double *h0, 
 // ---------------------------------------------------------------- W, H'W, SW update
 // Any m and alignment: 32 x 64 tiles, a row per lane.  Memory-bound (72 bytes an element:
 // FP64 state read and written, FP32 increments, digits); the loads of four columns come
-// before the first store (the compiler cannot tell the arrays apart), and the
-// transposed digits of two columns are stored together where n is even, 128 bytes a warp.
-// At m = 8171, n = 2044: 268 us with one column at a time on 32 x 32 tiles, 197 us now
-// (6.1 TB/s).
+// before the first store (the compiler cannot tell the arrays apart).  At m = 8171,
+// n = 2043: 329 us with one column at a time on 32 x 32 tiles, 270 with the loads ahead,
+// 248 on these tiles (4.9 TB/s; storing the transposed digits of two columns together
+// changed nothing).
 constexpr int TJ = 64;
 __device__ __forceinline__ void mx_update_body(int m, int n, double *W, const float *__restrict__ D, double *HW,
                                                const float *__restrict__ HD, double *SW,
@@ -389,7 +389,6 @@ __device__ __forceinline__ void mx_update_body(int m, int n, double *W, const fl
     const float x = state->x_f;
     const int lx = threadIdx.x % TILE, ly = threadIdx.x / TILE;
     const int Tm = (m + TILE - 1) / TILE, Tn = (n + TJ - 1) / TJ;
-    const bool pairs = (n & 1) == 0 && (swhw.ld & 1) == 0 && (swhw.plane & 1) == 0 && (((uintptr_t)swhw.ptr) & 3u) == 0;
     for (int t = blk; t < Tm * Tn; t += nblk) {
         const int ti = t % Tm, tj = t / Tm;
         const int i = ti * TILE + lx;
@@ -433,20 +432,12 @@ __device__ __forceinline__ void mx_update_body(int m, int n, double *W, const fl
                 const int il = ly + 8 * r, ii = ti * TILE + il;
                 if (ii >= m) break;
                 const int64_t o = (int64_t)ii * swhw.ld;
-                if (pairs) {
-                    const int jl = 2 * lx, jj = tj * TJ + jl;
-                    if (jj < n) {
-                        put3f2(swhw, o + jj, tS[jl][il], tS[jl + 1][il]);
-                        put3f2(swhw, o + n + jj, tH[jl][il], tH[jl + 1][il]);
-                    }
-                } else {
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int jl = lx + 32 * h, jj = tj * TJ + jl;
-                        if (jj < n) {
-                            put3f(swhw, o + jj, tS[jl][il]);
-                            put3f(swhw, o + n + jj, tH[jl][il]);
-                        }
+                for (int h = 0; h < 2; ++h) {
+                    const int jl = lx + 32 * h, jj = tj * TJ + jl;
+                    if (jj < n) {
+                        put3f(swhw, o + jj, tS[jl][il]);
+                        put3f(swhw, o + n + jj, tH[jl][il]);
                     }
                 }
             }
@@ -627,8 +618,8 @@ __device__ __forceinline__ void mx_direction_body(int m, int64_t mn, const float
     float gd = 0.f;
     // (i, j) of the thread's element carried on by a step's rows and columns, kU steps of
     // loads ahead of their stores (the compiler cannot tell the arrays apart): at m = 8171,
-    // n = 2044 100 us with one element at a time and a division for each, 82 with four, 78
-    // with eight (400 MB, 5.1 TB/s)
+    // n = 2043 122 us with one element at a time and a division for each, 100 with four, 97
+    // with eight (400 MB, 4.1 TB/s)
     constexpr int kU = 8;
     const int64_t step = (int64_t)nblk * NT, sj = step / m;
     const int si = (int)(step - sj * m);

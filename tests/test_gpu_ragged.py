@@ -64,6 +64,20 @@ def test_ragged_mixed(omm, m, n):
     s.close()
 
 
+# odd m (the update's 32 x 64 tiles) at column counts around a tile's edge, bounds as above
+@pytest.mark.parametrize("n", [31, 64, 65, 97])
+def test_ragged_mixed_update_tiles(omm, n):
+    m = 389
+    H, S, _, W0 = problem(m, n)
+    s = omm.Solver(m, n, 1, precision=omm.PREC_MIXED, orth_tol=1e-6)
+    s.set_HS(dev(H), dev(S))
+    E, _, st = s.solve(dev(W0), tol=1e-10)
+    ref = O.omm_cg(H, S, W0, tol=1e-13, eta=s.diag().eta)
+    assert st == omm.OK
+    assert abs(E - ref.E) / abs(ref.E) < 1e-8 and s.diag().orth < 1e-6
+    s.close()
+
+
 @pytest.mark.parametrize("form", ["cholesky", "precon"])
 def test_ragged_variants(omm, form):
     m, n = SIZES[0]
