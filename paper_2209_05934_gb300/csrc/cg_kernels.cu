@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int n, const double *__restr
     }
     const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x >= 32) return;   // warp 0: the line minimum
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -121,7 +121,12 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int n, const double *__restr
     }
 }
 
-// ---------------------------------------------------------------- n x n update + energy
+// ---------------------------------------------------------------- state update + energy
+// Blocks from nn_blocks on: W += x D, H'W += x H'D, SW += x SD, element by element (mn = 0:
+// none).  The first nn_blocks: the n x n update and the energy, whose last step waits for
+// every block of the launch, so none of them sees the `done` that it sets.  Two launches
+// took one dependent launch and the shorter of the two longer: 93.8 -> 91.0 us a step at
+// m = 144, 388 -> 380 us at m = 1996.
 // partials: 0 tr h0, 1 <s0,h0>, 2 ||s0 - I||^2
 constexpr int NE = 3;
 
@@ -132,7 +137,10 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
                                                         const double *__restrict__ s2,
                                                         int64_t ldz, double *partials,
                                                         unsigned int *counter, DevState *state,
-                                                        int mode, DigitOut hsw) {
+                                                        int mode, DigitOut hsw, int nn_blocks, int64_t mn, double *W,
+                                                        const double *__restrict__ D, double *HW,
+                                                        const double *__restrict__ HD, double *SW,
+                                                        const double *__restrict__ SD) {
     pdl_wait();
     if (*((volatile int *)&state->done)) return;
     __shared__ double Tt[4][TILE][TILE + 1];
@@ -142,7 +150,33 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
     const int64_t ntiles = (int64_t)T * T;
     const double x = state->x;
     double v[NE] = {0.0, 0.0, 0.0};
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    if ((int)blockIdx.x >= nn_blocks) {
+        constexpr int kU = 4;   // every load of a block's 4 NT elements before its first store
+        const int64_t step = (int64_t)(gridDim.x - nn_blocks) * NT * kU;
+        for (int64_t o0 = (int64_t)((int)blockIdx.x - nn_blocks) * NT * kU + threadIdx.x; o0 < mn; o0 += step) {
+            double w[kU], hw[kU], sw[kU], d[kU], hd[kU], sd[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int64_t o = o0 + u * NT;
+                const bool in = o < mn;
+                w[u] = in ? W[o] : 0.0;
+                hw[u] = in ? HW[o] : 0.0;
+                sw[u] = in ? SW[o] : 0.0;
+                d[u] = in ? D[o] : 0.0;
+                hd[u] = in ? HD[o] : 0.0;
+                sd[u] = in ? SD[o] : 0.0;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                const int64_t o = o0 + u * NT;
+                if (o >= mn) break;
+                W[o] = fma(x, d[u], w[u]);
+                HW[o] = fma(x, hd[u], hw[u]);
+                SW[o] = fma(x, sd[u], sw[u]);
+            }
+        }
+    }
+    for (int64_t t = (int)blockIdx.x < nn_blocks ? blockIdx.x : ntiles; t < ntiles; t += nn_blocks) {
         const int ti = (int)(t % T), tj = (int)(t / T);
         if (mode == 0) {
             __syncthreads();
@@ -184,9 +218,9 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
             v[2] = fma(e, e, v[2]);
         }
     }
-    const double sum = block_totals<NE>(v, red);
+    const double sum = (int)blockIdx.x < nn_blocks ? block_totals<NE>(v, red) : 0.0;
     double tot[NE];
-    if (!publish_totals<NE>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NE>(sum, partials, counter, tot, red, (unsigned)nn_blocks)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->trh0 = tot[0];
@@ -225,55 +259,6 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int n, double *h0, double
 }
 
 // ---------------------------------------------------------------- m x n kernels
-// W += x D, H'W += x H'D, SW += x SD over 32 x 32 tiles of the m x n arrays
-// (column-major, ld = m); optionally writes the digits of the new W (column
-// j = digit row j) and of the rows of [SW | H'W] (digit row i, K index j and
-// n + j) through a shared-memory transpose.
-__global__ void __launch_bounds__(NT) update_kernel(int m, int n, double *W, const double *__restrict__ D,
-                                                     double *HW, const double *__restrict__ HD, double *SW,
-                                                     const double *__restrict__ SD, const DevState *state,
-                                                     DigitOut wd, DigitOut swhw) {
-    pdl_wait();
-    if (*((volatile const int *)&state->done)) return;
-    __shared__ double tH[TILE][TILE + 1];
-    __shared__ double tS[TILE][TILE + 1];
-    const double x = state->x;
-    const int lx = threadIdx.x % TILE, ly = threadIdx.x / TILE;
-    const int Tm = (m + TILE - 1) / TILE, Tn = (n + TILE - 1) / TILE;
-    for (int t = blockIdx.x; t < Tm * Tn; t += gridDim.x) {
-        const int ti = t % Tm, tj = t / Tm;
-        const int i = ti * TILE + lx;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int jl = ly + 8 * r, j = tj * TILE + jl;
-            if (i < m && j < n) {
-                const int64_t o = (int64_t)j * m + i;
-                const double w = fma(x, D[o], W[o]);
-                const double hw = fma(x, HD[o], HW[o]);
-                const double sw = fma(x, SD[o], SW[o]);
-                W[o] = w;
-                HW[o] = hw;
-                SW[o] = sw;
-                if (wd.ptr != nullptr) put3(wd, (int64_t)j * wd.ld + i, w);
-                tH[jl][lx] = hw;
-                tS[jl][lx] = sw;
-            }
-        }
-        if (swhw.ptr != nullptr) {
-            __syncthreads();
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const int il = ly + 8 * r, ii = ti * TILE + il, jj = tj * TILE + lx;
-                if (ii < m && jj < n) {
-                    put3(swhw, (int64_t)ii * swhw.ld + jj, tS[lx][il]);
-                    put3(swhw, (int64_t)ii * swhw.ld + n + jj, tH[lx][il]);
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
 // <Z,G>, <Z,Gp>, <G,D> with Z = P G the preconditioned gradient (Z = G without
 // preconditioning: then <G,G>, <G,Gp>, <G,D>)
 constexpr int ND = 3;
@@ -298,7 +283,7 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t mn, const double *__re
     }
     const double sum = block_totals<ND>(v, red);
     double tot[ND];
-    if (!publish_totals<ND>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<ND>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;
@@ -478,26 +463,19 @@ int launch_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh
     return OMM_OK;
 }
 
-int launch_update(int64_t m, int64_t n, double *W, const double *D, double *HW, const double *HD, double *SW,
-                  const double *SD, const DevState *state, DigitOut wd, DigitOut swhw, cudaStream_t st) {
-    int64_t nb = ceil_div(m, TILE) * ceil_div(n, TILE);
-    if (nb > 152 * 8) nb = 152 * 8;
-    OMM_CUDA_TRY(launch_pdl(update_kernel, dim3((unsigned)nb), dim3(NT), 0, st, (int)m, (int)n, W, D, HW, HD, SW,
-                            SD, state, wd, swhw));
-    omm::count_launch();
-    OMM_CUDA_TRY(cudaGetLastError());
-    return OMM_OK;
-}
-
 int launch_nn_update_energy(int n, double *h0, double *s0, int64_t ldh, const double *Z,
                             int64_t ldz, double *scratch, unsigned int *counter, DevState *state,
-                            int mode, cudaStream_t st, DigitOut hsw) {
+                            int mode, cudaStream_t st, DigitOut hsw, const StateUpdate &u) {
     const double *X = Z;
     const double *Y = Z + (int64_t)n * ldz;
     const double *h2 = Z + n;
     const double *s2 = Z + n + (int64_t)n * ldz;
-    OMM_CUDA_TRY(launch_pdl(nn_update_kernel, dim3(red_blocks_for_tiles(n)), dim3(NT), 0, st, n, h0, s0, ldh, X, Y,
-                            h2, s2, ldz, scratch, counter, state, mode, hsw));
+    const int nn_blocks = red_blocks_for_tiles(n);
+    int64_t ub = ceil_div(u.mn, 4 * NT);
+    if (ub > 152 * 6) ub = 152 * 6;
+    OMM_CUDA_TRY(launch_pdl(nn_update_kernel, dim3((unsigned)(nn_blocks + ub)), dim3(NT), 0, st, n, h0, s0, ldh, X, Y,
+                            h2, s2, ldz, scratch, counter, state, mode, hsw, nn_blocks, u.mn, u.W, u.D, u.HW, u.HD,
+                            u.SW, u.SD));
     omm::count_launch();
     OMM_CUDA_TRY(cudaGetLastError());
     return OMM_OK;

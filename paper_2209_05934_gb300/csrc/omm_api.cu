@@ -439,12 +439,11 @@ int dense_iteration(omm_handle *h) {
     { StageTimer t(h, OMM_STAGE_LINESEARCH);
       TRY(omm::launch_coeffs_linemin((int)n, h->h0s0, h->h0s0 + n, 2 * n, h->Z, 2 * n, scr(h, 0),
                                      ctr(h, 0), s, nullptr, st, true)); }
-    // W += x D, H'W += x H'D, SW += x SD; then H_W, S_W update, energy, RelTol test
+    // W += x D, H'W += x H'D, SW += x SD, beside the H_W, S_W update, energy, RelTol test
     { StageTimer t(h, OMM_STAGE_UPDATE);
-      TRY(omm::launch_update(m, n, h->WD, h->WD + mn, h->SWHW + mn, h->HDSD, h->SWHW, h->HDSD + mn, s,
-                             omm::DigitOut{nullptr, 0, 0}, omm::DigitOut{nullptr, 0, 0}, st));
+      const omm::StateUpdate u{mn, h->WD, h->WD + mn, h->SWHW + mn, h->HDSD, h->SWHW, h->HDSD + mn};
       TRY(omm::launch_nn_update_energy((int)n, h->h0s0, h->h0s0 + n, 2 * n, h->Z, 2 * n, scr(h, 1),
-                                       ctr(h, 1), s, 0, st)); }
+                                       ctr(h, 1), s, 0, st, omm::DigitOut{nullptr, 0, 0}, u)); }
     // G = 4 H'W - 2 [SW H'W][H_W ; S_W]
     { StageTimer t(h, OMM_STAGE_GRADIENT); TRY(dense_gradient(h)); }
     return dense_direction(h, 0);

@@ -90,16 +90,23 @@ struct DigitOut {
     int nd = 3;   // planes written (the consumer's digit count, 2 or 3)
 };
 
-// W += x D, HW += x HD, SW += x SD  (three m x n arrays, ld = m), optionally
-// writing the digits of W (columns) and of the rows of [SW | HW]
-int launch_update(int64_t m, int64_t n, double *W, const double *D, double *HW, const double *HD, double *SW,
-                  const double *SD, const DevState *state, DigitOut wd, DigitOut swhw, cudaStream_t st);
+// W += x D, HW += x HD, SW += x SD: three arrays of mn elements
+struct StateUpdate {
+    int64_t mn = 0;
+    double *W = nullptr;
+    const double *D = nullptr;
+    double *HW = nullptr;
+    const double *HD = nullptr;
+    double *SW = nullptr;
+    const double *SD = nullptr;
+};
 
 // h0 += x (X + X^T) + x^2 sym(h2); s0 likewise; then energy, orthonormality,
 // convergence test (mode 0), or initial symmetrisation + energy (mode 1).
 int launch_nn_update_energy(int n, double *h0, double *s0, int64_t ldh, const double *Z,
                             int64_t ldz, double *scratch, unsigned int *counter, DevState *state,
-                            int mode, cudaStream_t st, DigitOut hsw = DigitOut{nullptr, 0, 0});
+                            int mode, cudaStream_t st, DigitOut hsw = DigitOut{nullptr, 0, 0},
+                            const StateUpdate &u = StateUpdate{});
 
 // <Z,G>, <Z,Gp>, <G,D> then beta (PR+) and the restart decision; Z = P G is the
 // preconditioned gradient (Z = G without preconditioning)

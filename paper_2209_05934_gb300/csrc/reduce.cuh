@@ -46,12 +46,14 @@ __device__ __forceinline__ double block_totals(const double (&v)[NV], double *re
 // Publish this block's NV partials (value t in lane t of warp 0); returns true in the
 // last block to finish, whose threads then all hold the totals in `tot`.  The last
 // block sums the partials in a fixed order (warp per value, lane-strided blocks, shuffle
-// tree), so the result does not depend on which block finished last.
+// tree), so the result does not depend on which block finished last.  Blocks from `parts`
+// on hold no partials and only count.
 template <int NV>
-__device__ __forceinline__ bool publish_totals(double v, double *partials, unsigned int *counter, double (&tot)[NV], double *red) {
+__device__ __forceinline__ bool publish_totals(double v, double *partials, unsigned int *counter, double (&tot)[NV],
+                                               double *red, unsigned parts) {
     __shared__ bool is_last;
     if (threadIdx.x < 32) {
-        if (threadIdx.x < NV) partials[blockIdx.x * NV + threadIdx.x] = v;
+        if (threadIdx.x < NV && blockIdx.x < parts) partials[blockIdx.x * NV + threadIdx.x] = v;
         __threadfence();
         __syncwarp();
         if (threadIdx.x == 0) is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
@@ -66,14 +68,14 @@ __device__ __forceinline__ bool publish_totals(double v, double *partials, unsig
         double s = 0.0;
         // the lane's blocks in order, eight loads in flight at a time
         unsigned b = threadIdx.x & 31;
-        for (; b + 224 < gridDim.x; b += 256) {
+        for (; b + 224 < parts; b += 256) {
             double p[8];
 #pragma unroll
             for (int k = 0; k < 8; ++k) p[k] = __ldcg(&partials[(b + 32 * k) * NV + q]);
 #pragma unroll
             for (int k = 0; k < 8; ++k) s += p[k];
         }
-        for (; b < gridDim.x; b += 32) s += __ldcg(&partials[b * NV + q]);
+        for (; b < parts; b += 32) s += __ldcg(&partials[b * NV + q]);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
         if ((threadIdx.x & 31) == 0) red[q] = s;

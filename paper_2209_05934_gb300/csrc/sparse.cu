@@ -900,7 +900,7 @@ __global__ void __launch_bounds__(NT) coeffs_kernel(int64_t nnzN, const int32_t 
     }
     const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x >= 32) return;   // warp 0: the line minimum
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -954,7 +954,7 @@ __global__ void __launch_bounds__(NT) nn_update_kernel(int64_t nnzN, const int32
     }
     const double sum = block_totals<NE3>(v, red);
     double tot[NE3];
-    if (!publish_totals<NE3>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NE3>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->orth2 = tot[2];
@@ -1025,7 +1025,7 @@ __global__ void __launch_bounds__(NT) dots_kernel(int64_t len, const T *__restri
     }
     const double sum = block_totals<ND>(v, red);
     double tot[ND];
-    if (!publish_totals<ND>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<ND>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x != 0) return;
     const double gg = tot[0];
     double beta = 0.0;
@@ -1120,7 +1120,7 @@ __global__ void __launch_bounds__(NT) mx_coeffs_kernel(int64_t nnzN, const int32
     for (int q = 0; q < NC; ++q) v[q] = sw_f2d(f[q]);
     const double sum = block_totals<NC>(v, red);
     double tot[NC] = {};
-    if (!publish_totals<NC>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NC>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x >= 32) return;
 #pragma unroll
     for (int q = 0; q < NC; ++q) tot[q] = __shfl_sync(0xffffffffu, tot[q], 0);
@@ -1200,7 +1200,7 @@ __global__ void __launch_bounds__(NT) mx_nn_update_kernel(int64_t nnzN, const in
     }
     const double sum = block_totals<NE3>(v, red);
     double tot[NE3];
-    if (!publish_totals<NE3>(sum, partials, counter, tot, red)) return;
+    if (!publish_totals<NE3>(sum, partials, counter, tot, red, gridDim.x)) return;
     if (threadIdx.x != 0) return;
     const double E = 2.0 * (2.0 * tot[0] - tot[1]) + state->e_shift;
     state->orth2 = tot[2];
