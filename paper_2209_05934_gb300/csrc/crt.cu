@@ -14,8 +14,8 @@
 // 2^-57 .. 2^-54 on the operands of the solver.  16 products at the BF16 rate
 // against one at the FP64 rate (1/1500 of it) is why this is the FP64 form's
 // product: digits of a fixed-point split (tc_exact.cu) would take 45 pairs for it.
-// A converged FP64 solve went from 18.4 to 4.6 ms at m = 144, 60 to 5.7 ms at m = 512
-// and 786 to 24.1 ms at m = 1996; S W and W^T H'W against quad precision went from
+// With the step's other kernels as they are, a converged FP64 solve went from 18.9 to
+// 4.0 ms at m = 144, 69 to 5.5 ms at m = 512 and 758 to 21.0 ms at m = 1996; S W and W^T H'W against quad precision went from
 // 3e-16 .. 1e-15 to 4e-17 .. 7e-17 (m = 141 .. 1597, H alone and with a kinetic part).
 //
 // Reconstruction.  With q_i = (P / p_i)^-1 mod p_i folded into one operand's
