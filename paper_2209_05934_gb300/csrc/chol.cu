@@ -24,6 +24,7 @@
 #include "fp_convert.cuh"
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "smem_optin.cuh"
 
 namespace omm {
 namespace chol {
@@ -292,11 +293,8 @@ int64_t work_bytes(int64_t m, int64_t n, int s) {
 int64_t linv_elems(int64_t m) { return m * m; }
 
 int cholesky(double *A, int64_t m, const Work &w, DevState *state, cudaStream_t st) {
-    static int attr = 0;
-    if (attr < kLeafSmem) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(chol_leaf_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kLeafSmem));
-        attr = kLeafSmem;
-    }
+    static SmemOptIn opt_in;
+    OMM_CUDA_TRY(opt_in(chol_leaf_kernel));
     OMM_CUDA_TRY(cudaMemsetAsync(w.Linv, 0, (size_t)(m * m) * sizeof(double), st));
     int rc = chol_inv(A, w.Linv, m, 0, m, w, state, st);
     if (rc != OMM_OK) return rc;

@@ -26,6 +26,7 @@
 #include "linemin.cuh"
 #include "omm_internal.cuh"
 #include "reduce.cuh"
+#include "smem_optin.cuh"
 #include "sparse.cuh"
 
 namespace omm {
@@ -1699,12 +1700,8 @@ int mixed_products(Dev &d, const DevState *state, cudaStream_t st) {
 
 int mixed_contract(Dev &d, const DevState *state, cudaStream_t st) {
     if (d.stage_rows > 0 && d.bm == 8 && d.bn == 2) {
-        static int64_t attr_bytes = 0;
-        if (d.stage_bytes > attr_bytes) {
-            OMM_CUDA_TRY(cudaFuncSetAttribute(contract_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                              (int)d.stage_bytes));
-            attr_bytes = d.stage_bytes;
-        }
+        static SmemOptIn opt_in;
+        OMM_CUDA_TRY(opt_in(contract_rows_kernel));
         // about four CTAs per place on the chip (two to an SM), for an even finish
         const int64_t groups = ceil_div(d.nbc, d.stage_rows);
         const int64_t parts = groups >= 1216 ? 1 : ceil_div(1216, groups);

@@ -30,6 +30,7 @@
 #include "fp_convert.cuh"
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "smem_optin.cuh"
 #include "tc_gemm.cuh"
 #include "tc_ptx.cuh"
 
@@ -880,12 +881,8 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 template <int BN, int STAGES, int BKT>
 int launch_tc(const CUtensorMap &ma, const CUtensorMap &mb, const TcArgs &a, int nbatch, cudaStream_t st) {
     const int smem = STAGES * (a.nA * BM * BKT * 2 + a.nB * BN * BKT * 2) + 1024;
-    static int attr_bytes = 0;
-    if (smem > attr_bytes) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_kernel<BN, STAGES, BKT>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_bytes = smem;
-    }
+    static SmemOptIn opt_in;
+    OMM_CUDA_TRY(opt_in(tc_gemm_kernel<BN, STAGES, BKT>));
     TcArgs b = a;
     const int nkb = (a.K + BKT - 1) / BKT;
     bool has_main = false, has_small = false;
@@ -907,12 +904,8 @@ template <int STAGES, int BKT>
 int launch_tc_pair(const CUtensorMap &ma, const CUtensorMap &mb_half, const TcArgs &a, int nbatch,
                    cudaStream_t st) {
     const int smem = STAGES * (a.nA * BM * BKT * 2 + a.nB * 128 * BKT * 2) + 1024;
-    static int attr_bytes = 0;
-    if (smem > attr_bytes) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(tc_gemm_pair_kernel<STAGES, BKT>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_bytes = smem;
-    }
+    static SmemOptIn opt_in;
+    OMM_CUDA_TRY(opt_in(tc_gemm_pair_kernel<STAGES, BKT>));
     TcArgs b = a;
     const int nkb = (a.K + BKT - 1) / BKT;
     bool has_main = false, has_small = false;
@@ -939,12 +932,8 @@ int launch_list(const TileProblem *probs, const TileRef *tiles, int ntiles, int 
     const int stages = (220 * 1024) / stage >= 3 ? 3 : 2;
     const int smem = stages * stage + 1024;
     auto kern = stages == 3 ? tc_gemm_list_kernel<PAIR, 3, BKT> : tc_gemm_list_kernel<PAIR, 2, BKT>;
-    static int attr3 = 0, attr2 = 0;
-    int &attr = stages == 3 ? attr3 : attr2;
-    if (smem > attr) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr = smem;
-    }
+    static SmemOptIn opt_in3, opt_in2;
+    OMM_CUDA_TRY(stages == 3 ? opt_in3(kern) : opt_in2(kern));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)ctas, 1, 1);
     cfg.blockDim = dim3(192, 1, 1);

@@ -34,6 +34,7 @@
 
 #include "omm_internal.cuh"
 #include "pdl.cuh"
+#include "smem_optin.cuh"
 #include "tc_ptx.cuh"
 #include "tc_units.cuh"
 
@@ -320,11 +321,8 @@ __global__ void __launch_bounds__(kUnitThreads, 1)
 template <bool PAIR, bool CRT>
 int launch_unit(const CUtensorMap &ma, const CUtensorMap &mb, const UnitArgs &a, int groups, cudaStream_t st) {
     const int smem = (PAIR ? 6 * 2 : 4 * 3) * kBox + 1024;
-    static int attr_bytes = 0;
-    if (smem > attr_bytes) {
-        OMM_CUDA_TRY(cudaFuncSetAttribute(tc_unit_kernel<PAIR, CRT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        attr_bytes = smem;
-    }
+    static SmemOptIn opt_in;
+    OMM_CUDA_TRY(opt_in(tc_unit_kernel<PAIR, CRT>));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(PAIR ? 2 * groups : groups), 1, 1);
     cfg.blockDim = dim3(kUnitThreads, 1, 1);
