@@ -32,6 +32,7 @@ namespace {
 
 constexpr int kChunkMax = 4096;             // 4096 * 64 * 64 = 2^24: exact FP32 integer sums
 constexpr int64_t kPlaneCap = 48ll << 20;   // words of level planes one launch may fill (192 MB)
+constexpr int64_t kSlabCols = 65280ll * 32;  // columns of one fold launch: 32 per block of a grid's y (at most 65535)
 
 // ------------------------------------------------------------------ level fold
 struct FoldArgs {
@@ -407,6 +408,7 @@ int exact_gemm(const CUtensorMap &mapA, const CUtensorMap &mapB, const ExactArgs
     f.eB_step = a.eB_step;
     f.state = a.state;
     int64_t slab = exact_plane_words(a.M, a.N, nbatch, s) / ((int64_t)s * nbatch * a.M);
+    if (slab > kSlabCols) slab = kSlabCols;
     if (slab < a.N) slab = slab / 256 * 256;
     for (int64_t c0 = 0; c0 < a.N; c0 += slab) {
         const int nc = (int)(a.N - c0 < slab ? a.N - c0 : slab);
