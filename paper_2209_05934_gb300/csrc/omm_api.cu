@@ -1526,14 +1526,6 @@ int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *patt
         return rc;
     }
     // last: what the handle cannot do without is allocated by now
-    if (h->sparse && h->opt.precision == OMM_PREC_FP64) {
-        if ((rc = omm::sp::fx_alloc(h->sh, h->sd)) == OMM_ERR_NOMEM) {
-            cudaGetLastError();   // the FP64 gathers need no fixed-point operands
-        } else if (rc != OMM_OK) {
-            free_handle(h);
-            return rc;
-        }
-    }
     if (!h->sparse && h->opt.precision == OMM_PREC_FP64 && (rc = crt_alloc(h))) {
         free_handle(h);
         return rc;

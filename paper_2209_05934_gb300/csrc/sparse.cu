@@ -446,12 +446,33 @@ struct VecGather {
 };
 __device__ __forceinline__ float4 ld4(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 
+// One output's sum.  SPLIT (the FP64 form): even and odd terms in two chains, which cuts
+// what a chain's rounding grows to over its length (the gradient keeps its two products apart as well);
+// the FP64 unit is the limit either way.  The mixed form keeps one chain: its FP32 first phase
+// turns a start that differs in the last bit into another trajectory (4e-6 in W after 24
+// steps of 1728 atoms).
+//
+// Fixed-point operands in integer arithmetic (rows and columns scaled to norms of 2^57, two
+// limbs, three 32 x 32 -> 64-bit multiply-adds a term) took 11.0 ms for 12 steps of 512 atoms
+// against 19.6 here, but their error follows the norms of the whole row and column: between
+// tails (products 1e-8 of the norms) they lost seven digits, and an orbital shifted up by 1e9
+// all but six.
+template <typename T, bool SPLIT>
+struct Sum {
+    T a = T(0), b = T(0);
+    __device__ __forceinline__ void add(int i, T x, T y) {
+        if (SPLIT && (i & 1)) b = fma(x, y, b);
+        else a = fma(x, y, a);
+    }
+    __device__ __forceinline__ T total() const { return SPLIT ? a + b : a; }
+};
+
 // ---- products: HD_o = sum H'_(I,K) D_(K,J), SD_o likewise; warp per P_HW block,
 // lanes 0..15 -> H'D element (r, c), lanes 16..31 -> SD element.
 // Screening (SCREEN): the block product H'_(I,K) D_(K,J) (or S_(I,K) D_(K,J)) is
 // skipped when ||H'_(I,K)||^2 ||D_(K,J)||^2 < eps^2, from the squared block norms
 // nHS ([nnzH][2]: H', S) and nB (one per D block).
-template <int BM, int BN, bool SCREEN, typename T = double>
+template <int BM, int BN, bool SCREEN, typename T = double, bool SPLIT = false>
 __global__ void __launch_bounds__(NT) products_kernel(int64_t nnzHW, const int64_t *__restrict__ Prp,
                                                        const int32_t *__restrict__ Ph, const int32_t *__restrict__ Pw,
                                                        const T *__restrict__ HS, const T *__restrict__ D,
@@ -502,7 +523,7 @@ __global__ void __launch_bounds__(NT) products_kernel(int64_t nnzHW, const int64
         const int r = e / BN, c = e % BN;
         const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
         for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5; o < nnzHW; o += nwarps) {
-            T acc = T(0);
+            Sum<T, SPLIT> acc;
 #pragma unroll 4
             for (int64_t t = Prp[o]; t < Prp[o + 1]; ++t) {
                 if (SCREEN && nHS[(int64_t)Ph[t] * 2 + which] * nB[Pw[t]] < eps2) continue;
@@ -510,10 +531,10 @@ __global__ void __launch_bounds__(NT) products_kernel(int64_t nnzHW, const int64
                 const T *B = D + (int64_t)Pw[t] * BM * BN + c;
                 if (active) {
 #pragma unroll
-                    for (int k = 0; k < BM; ++k) acc = fma(A[k], B[k * BN], acc);
+                    for (int k = 0; k < BM; ++k) acc.add(k, A[k], B[k * BN]);
                 }
             }
-            if (active) (which ? SD : HD)[o * NE + e] = acc;
+            if (active) (which ? SD : HD)[o * NE + e] = acc.total();
         }
     }
 }
@@ -522,7 +543,7 @@ __global__ void __launch_bounds__(NT) products_kernel(int64_t nnzHW, const int64
 // with two lanes each splitting the basis index k.
 // Screening: the pair (L block a, R block b) is skipped when ||L_a||^2 ||R_b||^2 < eps^2,
 // with L = W or D and R = H'D or SD as the output matrix takes them.
-template <int BM, int BN, bool SCREEN, typename T = double>
+template <int BM, int BN, bool SCREEN, typename T = double, bool SPLIT = false>
 __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_t *__restrict__ Crp,
                                                        const int32_t *__restrict__ Ca, const int32_t *__restrict__ Cb,
                                                        const T *__restrict__ W, const T *__restrict__ D,
@@ -612,7 +633,7 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
     } else {
     for (int64_t q = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5; q < nnzN; q += nwarps) {
         if (!SCREEN && Ntr != nullptr && Ntr[q] < q) {
-            T acc = T(0);
+            Sum<T, SPLIT> sum;
 #pragma unroll 4
             for (int64_t t = Crp[q]; t < Crp[q + 1]; ++t) {
                 const T *l = W + (int64_t)Ca[t] * BM * BN + a4;
@@ -620,9 +641,10 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
 #pragma unroll
                 for (int kk = 0; kk < BM / 4; ++kk) {
                     const int k = quarter * (BM / 4) + kk;
-                    acc = fma(l[k * BN], rr[k * BN], acc);
+                    sum.add(kk, l[k * BN], rr[k * BN]);
                 }
             }
+            T acc = sum.total();
             acc += __shfl_xor_sync(0xffffffffu, acc, 1);
             acc += __shfl_xor_sync(0xffffffffu, acc, 2);
             if (quarter == 0) out4[q * 4 + a4 * 2 + b4] = acc;
@@ -630,7 +652,7 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
         }
         // (16-byte vector loads measured slower here than these scalar ones: each
         // lane needs every other element of its block rows)
-        T acc = T(0);
+        Sum<T, SPLIT> sum;
 #pragma unroll 4
         for (int64_t t = Crp[q]; t < Crp[q + 1]; ++t) {
             if (SCREEN && nL[Ca[t]] * nR[Cb[t]] < eps2) continue;
@@ -639,9 +661,10 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
 #pragma unroll
             for (int kk = 0; kk < BM / 2; ++kk) {
                 const int k = half * (BM / 2) + kk;
-                acc = fma(l[k * BN], rr[k * BN], acc);
+                sum.add(kk, l[k * BN], rr[k * BN]);
             }
         }
+        T acc = sum.total();
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         if (half == 0) out[q * 4 + a * 2 + b] = acc;
     }
@@ -651,7 +674,7 @@ __global__ void __launch_bounds__(NT) contract_kernel(int64_t nnzN, const int64_
 // X = W^T H'W and Y = W^T S W alone (D = W: the start and the density matrices have no
 // h2, s2 of their own): sixteen lanes per P_N block, two blocks per warp, the lanes and
 // the order of the sums those of contract_kernel's X and Y.
-template <int BM, int BN, typename T = double>
+template <int BM, int BN, bool SPLIT, typename T = double>
 __global__ void __launch_bounds__(NT) contract_xy_kernel(int64_t nnzN, const int64_t *__restrict__ Crp,
                                                           const int32_t *__restrict__ Ca,
                                                           const int32_t *__restrict__ Cb, const T *__restrict__ W,
@@ -666,7 +689,7 @@ __global__ void __launch_bounds__(NT) contract_xy_kernel(int64_t nnzN, const int
     const int64_t nwarps = ((int64_t)gridDim.x * NT) >> 5;
     for (int64_t qb = (((int64_t)blockIdx.x * NT + threadIdx.x) >> 5) * 2; qb < nnzN; qb += nwarps * 2) {
         const int64_t q = qb + ((threadIdx.x >> 4) & 1);
-        T acc = T(0);
+        Sum<T, SPLIT> sum;
         const int64_t t1 = q < nnzN ? Crp[q + 1] : 0;
 #pragma unroll 4
         for (int64_t t = q < nnzN ? Crp[q] : 0; t < t1; ++t) {
@@ -675,9 +698,10 @@ __global__ void __launch_bounds__(NT) contract_xy_kernel(int64_t nnzN, const int
 #pragma unroll
             for (int kk = 0; kk < BM / 2; ++kk) {
                 const int k = half * (BM / 2) + kk;
-                acc = fma(l[k * BN], rr[k * BN], acc);
+                sum.add(kk, l[k * BN], rr[k * BN]);
             }
         }
+        T acc = sum.total();
         acc += __shfl_xor_sync(0xffffffffu, acc, 1);
         if (half == 0 && q < nnzN) out[q * 4 + a * 2 + b] = acc;
     }
@@ -791,7 +815,7 @@ __global__ void mirror_kernel(int64_t nnzN, const int32_t *__restrict__ Ntr, T *
 // half-warp per W block, one lane per element (r, c).
 // Screening: SW_(I,K) h0_(K,J) and H'W_(I,K) s0_(K,J) are skipped separately when
 // the product of their squared block norms is below eps^2.
-template <int BM, int BN, bool SCREEN, typename T = double>
+template <int BM, int BN, bool SCREEN, typename T = double, bool SPLIT = false>
 __global__ void __launch_bounds__(NT) gradient_kernel(int64_t nnzW, const int64_t *__restrict__ Grp,
                                                        const int32_t *__restrict__ Gb, const int32_t *__restrict__ Gq,
                                                        const int32_t *__restrict__ WtoHW, const T *__restrict__ HW,
@@ -840,6 +864,7 @@ __global__ void __launch_bounds__(NT) gradient_kernel(int64_t nnzW, const int64_
         const int64_t ngroups = ((int64_t)gridDim.x * NT) >> 4;
         for (int64_t o = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 4; o < nnzW; o += ngroups) {
             T acc = T(0);
+            Sum<T, true> ps, ph;   // SPLIT
 #pragma unroll 4
             for (int64_t t = Grp[o]; t < Grp[o + 1]; ++t) {
                 const T *sw = SW + (int64_t)Gb[t] * BM * BN + r * BN;
@@ -854,6 +879,12 @@ __global__ void __launch_bounds__(NT) gradient_kernel(int64_t nnzW, const int64_
                         if (use_s) acc = fma(sw[k], hq[k * BN], acc);
                         if (use_h) acc = fma(hw[k], sq[k * BN], acc);
                     }
+                } else if constexpr (SPLIT) {
+#pragma unroll
+                    for (int k = 0; k < BN; ++k) {
+                        ps.add(k, sw[k], hq[k * BN]);
+                        ph.add(k, hw[k], sq[k * BN]);
+                    }
                 } else {
 #pragma unroll
                     for (int k = 0; k < BN; ++k) {
@@ -862,6 +893,7 @@ __global__ void __launch_bounds__(NT) gradient_kernel(int64_t nnzW, const int64_
                     }
                 }
             }
+            if (SPLIT) acc = ps.total() + ph.total();
             G[o * BM * BN + e] = T(2) * (T(2) * HW[(int64_t)WtoHW[o] * BM * BN + e] - acc);
         }
     }
@@ -1381,7 +1413,6 @@ void release(Dev &d) {
                     d.Ndiag, d.HS, d.Hin, d.W, d.D, d.G, d.Gp, d.HW, d.SW, d.HD, d.SD, d.h0, d.s0, d.X,
                     d.Y, d.h2, d.s2, d.keep, d.nrm, d.fbuf, d.Nrp, d.WcolRp, d.WcolIdx, d.CaSlot, d.Nord};
     for (void *p : ptrs) cudaFree(p);
-    cudaFree(d.fx.base);
     d = Dev{};
 }
 
@@ -1401,16 +1432,12 @@ int set_HS(Dev &d, const double *H, const double *S, bool on_device, double eps,
     }
     shift_pack_kernel<<<blocks_for(d.nnzH * bb, 256), 256, 0, st>>>(d.nnzH, (int)bb, Hc, Sc, d.keep, state, d.HS);
     LAUNCHED();
-    if (d.fx.base != nullptr) {
-        const int rc = fx_set_HS(d, st);
-        if (rc != OMM_OK) return rc;
-    }
     return norms(d, NRM_HS, nullptr, st);
 }
 
-#define DISPATCH_BLOCKS(BMv, BNv, CALL)                              \
+#define DISPATCH_BLOCKS(BMv, BNv, ...)                               \
     do {                                                             \
-        if ((BMv) == 8 && (BNv) == 2) { constexpr int BM = 8, BN = 2; CALL; } \
+        if ((BMv) == 8 && (BNv) == 2) { constexpr int BM = 8, BN = 2; __VA_ARGS__; } \
         else return OMM_ERR_UNSUPPORTED;                             \
     } while (0)
 
@@ -1464,12 +1491,12 @@ int products(Dev &d, const double *Din, double *HDo, double *SDo, const double *
         DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, true><<<blocks_for(d.nnzHW * 32, NT), NT, 0, st>>>(
                                          d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS, Din, HDo, SDo, d.nHS, nDin,
                                          d.screen_eps2, state)));
-    } else if (d.fx.base != nullptr) {
-        return fx_products(d, Din, HDo, SDo, state, st);
     } else {
-        DISPATCH_BLOCKS(d.bm, d.bn, (products_kernel<BM, BN, false><<<blocks_for(d.nnzHW * 32, NT), NT, 0, st>>>(
-                                         d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS, Din, HDo, SDo, nullptr, nullptr, 0.0,
-                                         state)));
+        DISPATCH_BLOCKS(d.bm, d.bn, {
+            auto kern = d.mixed ? products_kernel<BM, BN, false> : products_kernel<BM, BN, false, double, true>;
+            kern<<<blocks_for(d.nnzHW * 32, NT), NT, 0, st>>>(d.nnzHW, d.Prp, d.Ph, d.Pw, d.HS, Din, HDo, SDo, nullptr,
+                                                              nullptr, 0.0, state);
+        });
     }
     LAUNCHED();
     return OMM_OK;
@@ -1489,19 +1516,19 @@ int contract(Dev &d, const double *Wl, const double *Dl, const double *HDr, cons
     // and mirrored to the lower one (H' and S are symmetric); with D = W (the start,
     // the density matrices) X and Y are all there is
     const bool sym = Dl != Wl;
-    if (d.fx.base != nullptr) {
-        const int rc = fx_contract(d, Wl, Dl, HDr, SDr, Xo, Yo, h2o, s2o, d.Ntr, state, st);
-        if (rc != OMM_OK) return rc;
-    } else if (!sym) {
-        DISPATCH_BLOCKS(d.bm, d.bn, (contract_xy_kernel<BM, BN><<<blocks_for(d.nnzN * 16, NT), NT, 0, st>>>(
-                                         d.nnzN, d.Crp, d.Ca, d.Cb, Wl, HDr, SDr, Xo, Yo, state)));
-        LAUNCHED();
+    if (!sym) {
+        DISPATCH_BLOCKS(d.bm, d.bn, {
+            auto kern = d.mixed ? contract_xy_kernel<BM, BN, false> : contract_xy_kernel<BM, BN, true>;
+            kern<<<blocks_for(d.nnzN * 16, NT), NT, 0, st>>>(d.nnzN, d.Crp, d.Ca, d.Cb, Wl, HDr, SDr, Xo, Yo, state);
+        });
     } else {
-        DISPATCH_BLOCKS(d.bm, d.bn, (contract_kernel<BM, BN, false><<<blocks_for(d.nnzN * 32, NT), NT, 0, st>>>(
-                                         d.nnzN, d.Crp, d.Ca, d.Cb, Wl, Dl, HDr, SDr, Xo, Yo, h2o, s2o, nullptr,
-                                         nullptr, nullptr, nullptr, 0.0, d.Ntr, state)));
-        LAUNCHED();
+        DISPATCH_BLOCKS(d.bm, d.bn, {
+            auto kern = d.mixed ? contract_kernel<BM, BN, false> : contract_kernel<BM, BN, false, double, true>;
+            kern<<<blocks_for(d.nnzN * 32, NT), NT, 0, st>>>(d.nnzN, d.Crp, d.Ca, d.Cb, Wl, Dl, HDr, SDr, Xo, Yo, h2o,
+                                                             s2o, nullptr, nullptr, nullptr, nullptr, 0.0, d.Ntr, state);
+        });
     }
+    LAUNCHED();
     if (sym) {
         mirror_kernel<double><<<blocks_for(d.nnzN * 4, 256), 256, 0, st>>>(d.nnzN, d.Ntr, h2o, s2o, state);
         LAUNCHED();
@@ -1553,12 +1580,12 @@ int gradient(Dev &d, const DevState *state, cudaStream_t st) {
         DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, true><<<blocks_for(d.nnzW * 16, NT), NT, 0, st>>>(
                                          d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW, d.SW, d.h0, d.s0, d.G, d.nHW,
                                          d.nSW, d.nh0, d.ns0, d.screen_eps2, state)));
-    } else if (d.fx.base != nullptr) {
-        return fx_gradient(d, state, st);
     } else {
-        DISPATCH_BLOCKS(d.bm, d.bn, (gradient_kernel<BM, BN, false><<<blocks_for(d.nnzW * 16, NT), NT, 0, st>>>(
-                                         d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW, d.SW, d.h0, d.s0, d.G, nullptr,
-                                         nullptr, nullptr, nullptr, 0.0, state)));
+        DISPATCH_BLOCKS(d.bm, d.bn, {
+            auto kern = d.mixed ? gradient_kernel<BM, BN, false> : gradient_kernel<BM, BN, false, double, true>;
+            kern<<<blocks_for(d.nnzW * 16, NT), NT, 0, st>>>(d.nnzW, d.Grp, d.Gb, d.Gq, d.WtoHW, d.HW, d.SW, d.h0, d.s0,
+                                                             d.G, nullptr, nullptr, nullptr, nullptr, 0.0, state);
+        });
     }
     LAUNCHED();
     return OMM_OK;

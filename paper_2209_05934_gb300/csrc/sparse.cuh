@@ -45,40 +45,6 @@ struct DensHost {
     std::vector<int32_t> Tw, Tq, Rt, Rw;
 };
 
-// Statistics of the vectors of a fixed-point operand: largest biased exponent and
-// sum of squares (in units of 2^-36 of the largest's power of two).
-struct FxStat {
-    unsigned long long *sq = nullptr;
-    int *mx = nullptr;
-};
-// Conversion of one block array: vectors are the blocks' scalar rows (by_row) or
-// columns, numbered by idx[block] * rows (or cols) + row (or column); block sizes as
-// powers of two, at most 8.
-struct FxJob {
-    const double *src;
-    int2 *dst;
-    int64_t nblk;
-    const int32_t *idx;
-    int lrows, lcols, by_row;
-    int64_t stride;   // elements from one block to the next
-    FxStat stat;
-};
-struct FxJobs {
-    FxJob j[4];
-    int n = 0;
-};
-// Fixed-point operands of the FP64 gathers (sparse_fx.cu), each value two limbs;
-// A and B hold H'D, SD (or the start's H'W, SW) for the contraction, by columns, and
-// then H'W, SW for the gradient, by rows.  base == nullptr: not allocated, the FP64
-// gathers run.
-struct Fx {
-    char *base = nullptr;
-    int32_t *Hrow = nullptr, *Wcol = nullptr, *HWrow = nullptr, *HWcol = nullptr, *Nrow = nullptr, *Ncol = nullptr;
-    int2 *HS = nullptr, *W = nullptr, *D = nullptr, *A = nullptr, *B = nullptr, *h0 = nullptr, *s0 = nullptr;
-    FxStat sH, sS, sW, sD, sA, sB, sh0, ss0;
-    char *z0 = nullptr, *z1 = nullptr, *z2 = nullptr, *z3 = nullptr;   // statistics: [H, S], [W, D], [the others]
-};
-
 // Device arrays of one sparse handle.
 struct Dev {
     int32_t bm = 0, bn = 0;
@@ -120,7 +86,6 @@ struct Dev {
     uint32_t *Nord = nullptr;
     int stage_rows = 0;
     int64_t stage_bytes = 0;
-    Fx fx;
 };
 
 // P_N's blocks (J, J2) by groups of `rows` rows J, each group in the order of J2 and
@@ -164,16 +129,6 @@ int contract(Dev &d, const double *Wl, const double *Dl, const double *HDr, cons
              double *Yo, double *h2o, double *s2o, const double *nWl, const double *nDl, const double *nHDr,
              const double *nSDr, const DevState *state, cudaStream_t st);
 int gradient(Dev &d, const DevState *state, cudaStream_t st);
-
-// The same in integer arithmetic on fixed-point operands (sparse_fx.cu); fx_products
-// converts W (and D), which fx_contract reads.  fx_alloc fails with OMM_ERR_NOMEM and
-// leaves the handle to the FP64 gathers.
-int fx_alloc(const Host &hs, Dev &d);
-int fx_set_HS(Dev &d, cudaStream_t st);
-int fx_products(Dev &d, const double *Din, double *HDo, double *SDo, const DevState *state, cudaStream_t st);
-int fx_contract(Dev &d, const double *Wl, const double *Dl, const double *HDr, const double *SDr, double *Xo, double *Yo,
-                double *h2o, double *s2o, const int32_t *Ntr, const DevState *state, cudaStream_t st);
-int fx_gradient(Dev &d, const DevState *state, cudaStream_t st);
 
 // Mixed form.  mixed_alloc: the FP32 arrays (about 60% of the FP64 ones).
 // mixed_shadow_HS: FP32 copies of H' and S (after set_HS).  mixed_begin: FP32
