@@ -72,14 +72,14 @@ struct ExactBufs {
     CUtensorMap mapHS_A, mapW, mapHWSW_B, mapSWHW_A, mapHSW_B;
 };
 
-// Residue planes of the FP64 form's products (crt.cu; 16 planes, row-scaled), each
-// with its per-row exponents:
-//   HSr   [16][2m][ldm]  rows of [H' ; S]         A of H'D, SD (and H'W, SW)
-//   WDr   [16][2n][ldm]  columns of [W | D]       B of those; A of Z
-//   HDSDr [16][2n][ldm]  columns of [H'D | SD]    B of Z (start: [SW | H'W])
-//   SWHWr [16][m][ld2n]  rows of [SW | H'W]       A of the gradient
-//   HSWr  [16][n][ld2n]  columns of [H_W ; S_W]   B of the gradient
-// words: the residue planes of a product; part: partial row norms.
+// Residue and magnitude planes of the FP64 form's products (crt.cu; 19 planes, row-scaled),
+// each with its per-row exponents:
+//   HSr   [19][2m][ldm]  rows of [H' ; S]         A of H'D, SD (and H'W, SW)
+//   WDr   [19][2n][ldm]  columns of [W | D]       B of those; A of Z
+//   HDSDr [19][2n][ldm]  columns of [H'D | SD]    B of Z (start: [SW | H'W])
+//   SWHWr [19][m][ld2n]  rows of [SW | H'W]       A of the gradient
+//   HSWr  [19][n][ld2n]  columns of [H_W ; S_W]   B of the gradient
+// words: the planes of a product; part: partial row norms.
 struct CrtBufs {
     int64_t ldm = 0, ld2n = 0;
     char *base = nullptr;   // one allocation holds them all
@@ -87,6 +87,7 @@ struct CrtBufs {
     __nv_bfloat16 *Pr = nullptr, *Gr = nullptr;   // preconditioner: rows of P, columns of G
     int *e = nullptr;
     int *eHS = nullptr, *eWD = nullptr, *eHDSD = nullptr, *eSWHW = nullptr, *eHSW = nullptr, *eP = nullptr, *eG = nullptr;
+    int *bal = nullptr;   // exponent of the energy unit in H' against S
     float2 *part = nullptr;
     uint32_t *words = nullptr;
     CUtensorMap mapHS, mapWD, mapHDSD, mapSWHW, mapHSW, mapP, mapG;
@@ -312,6 +313,7 @@ int64_t n_occ(const omm_handle *h) { return h->opt.n_occupied > 0 ? h->opt.n_occ
 // ---------------------------------------------------------------- FP64 form
 // The products run on the tensor cores through residue planes (crt.cu) where the
 // handle holds them, else on the CUDA cores (dense_fp64.cu).
+const omm::crt::Balance kNoBalance{};
 bool crt_on(const omm_handle *h) { return h->cr.words != nullptr; }
 
 omm::crt::Args crt_args(omm_handle *h, int64_t M, int64_t N, int64_t K) {
@@ -340,6 +342,12 @@ int crt_products(omm_handle *h, int b_row0, double *C, int64_t c_step) {
     a.eA = c.eHS;
     a.eA_step = m;
     a.eB = c.eWD + b_row0;
+    a.A = h->HS;
+    a.A_row = 1;
+    a.A_col = m;
+    a.A_step = m * m;
+    a.B = h->WD + (int64_t)b_row0 * m;
+    a.ldb = m;
     return omm::crt::gemm(c.mapHS, c.mapWD, a, s_identity(h) ? 1 : 2, h->stream);
 }
 
@@ -349,8 +357,10 @@ int dense_gradient(omm_handle *h) {
     cudaStream_t st = h->stream;
     if (crt_on(h)) {
         CrtBufs &c = h->cr;
-        TRY(omm::crt::pack_rows(m, 2 * n, h->SWHW, m, c.eSWHW, c.part, c.SWHWr, c.ld2n, m * c.ld2n, false, h->dstate, st));
-        TRY(omm::crt::pack_cols(2 * n, n, h->h0s0, 2 * n, c.eHSW, c.HSWr, c.ld2n, n * c.ld2n, true, h->dstate, st));
+        TRY(omm::crt::pack_rows(m, 2 * n, h->SWHW, m, c.eSWHW, c.part, c.SWHWr, c.ld2n, m * c.ld2n, false,
+                                omm::crt::Balance{c.bal, n, -1}, h->dstate, st));
+        TRY(omm::crt::pack_cols(2 * n, n, h->h0s0, 2 * n, c.eHSW, c.HSWr, c.ld2n, n * c.ld2n, true,
+                                omm::crt::Balance{c.bal, n, 1}, h->dstate, st));
         omm::crt::Args a = crt_args(h, m, n, 2 * n);
         a.alpha = -2.0;
         a.beta = 4.0;
@@ -360,6 +370,11 @@ int dense_gradient(omm_handle *h) {
         a.ldc = m;
         a.eA = c.eSWHW;
         a.eB = c.eHSW;
+        a.A = h->SWHW;
+        a.A_row = 1;
+        a.A_col = m;
+        a.B = h->h0s0;
+        a.ldb = 2 * n;
         return omm::crt::gemm(c.mapSWHW, c.mapHSW, a, 1, st);
     }
     omm::GemmBatch g{};
@@ -377,12 +392,17 @@ int dense_direction(omm_handle *h, int first) {
         StageTimer t(h, OMM_STAGE_PRECON);
         if (crt_on(h)) {
             CrtBufs &c = h->cr;
-            TRY(omm::crt::pack_cols(m, n, h->G, m, c.eG, c.Gr, c.ldm, n * c.ldm, false, h->dstate, st));
+            TRY(omm::crt::pack_cols(m, n, h->G, m, c.eG, c.Gr, c.ldm, n * c.ldm, false, kNoBalance, h->dstate, st));
             omm::crt::Args a = crt_args(h, m, n, m);
             a.C = h->PG;
             a.ldc = m;
             a.eA = c.eP;
             a.eB = c.eG;
+            a.A = h->P;
+            a.A_row = 1;
+            a.A_col = m;
+            a.B = h->G;
+            a.ldb = m;
             TRY(omm::crt::gemm(c.mapP, c.mapG, a, 1, st));
         } else {
             omm::GemmBatch p{};
@@ -406,7 +426,7 @@ int dense_iteration(omm_handle *h) {
         if (crt_on(h)) {
             // residues of W and D: D is the products' operand, both are the contraction's
             CrtBufs &c = h->cr;
-            TRY(omm::crt::pack_cols(m, 2 * n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, s, st));
+            TRY(omm::crt::pack_cols(m, 2 * n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, kNoBalance, s, st));
             TRY(crt_products(h, (int)n, h->HDSD, mn));
         } else {
             omm::GemmBatch b{};
@@ -422,12 +442,18 @@ int dense_iteration(omm_handle *h) {
         StageTimer t(h, OMM_STAGE_CONTRACT);
         if (crt_on(h)) {
             CrtBufs &c = h->cr;
-            TRY(omm::crt::pack_cols(m, 2 * n, h->HDSD, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, s, st));
+            TRY(omm::crt::pack_cols(m, 2 * n, h->HDSD, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, kNoBalance, s,
+                                    st));
             omm::crt::Args a = crt_args(h, 2 * n, 2 * n, m);
             a.C = h->Z;
             a.ldc = 2 * n;
             a.eA = c.eWD;
             a.eB = c.eHDSD;
+            a.A = h->WD;
+            a.A_row = m;
+            a.A_col = 1;
+            a.B = h->HDSD;
+            a.ldb = m;
             TRY(omm::crt::gemm(c.mapWD, c.mapHDSD, a, 1, st));
         } else {
             omm::GemmBatch z{};
@@ -456,7 +482,7 @@ int dense_start(omm_handle *h) {
     // SW = S W, H'W = H' W
     if (crt_on(h)) {
         CrtBufs &c = h->cr;
-        TRY(omm::crt::pack_cols(m, n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, s, st));
+        TRY(omm::crt::pack_cols(m, n, h->WD, m, c.eWD, c.WDr, c.ldm, 2 * n * c.ldm, false, kNoBalance, s, st));
         TRY(crt_products(h, 0, h->SWHW + mn, -mn));
     } else {
         omm::GemmBatch b{};
@@ -469,7 +495,8 @@ int dense_start(omm_handle *h) {
     // H_W = W^T H'W, S_W = W^T S W
     if (crt_on(h)) {
         CrtBufs &c = h->cr;
-        TRY(omm::crt::pack_cols(m, 2 * n, h->SWHW, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, s, st));
+        TRY(omm::crt::pack_cols(m, 2 * n, h->SWHW, m, c.eHDSD, c.HDSDr, c.ldm, 2 * n * c.ldm, true, kNoBalance, s,
+                                    st));
         omm::crt::Args a = crt_args(h, n, n, m);
         a.b_row0 = (int)n;          // z = 0: H'W -> rows [0, n) of h0s0;  z = 1: SW -> rows [n, 2n)
         a.b_row_step = -(int)n;
@@ -479,6 +506,12 @@ int dense_start(omm_handle *h) {
         a.eA = c.eWD;
         a.eB = c.eHDSD + n;
         a.eB_step = -n;
+        a.A = h->WD;
+        a.A_row = m;
+        a.A_col = 1;
+        a.B = h->SWHW + mn;
+        a.ldb = m;
+        a.B_step = -mn;
         TRY(omm::crt::gemm(c.mapWD, c.mapHDSD, a, 2, st));
     } else {
         omm::GemmBatch c{};
@@ -500,7 +533,7 @@ int dense_start(omm_handle *h) {
 int crt_alloc(omm_handle *h) {
     const int64_t m = h->m, n = h->n;
     CrtBufs &c = h->cr;
-    constexpr int64_t L = omm::crt::kModuli;
+    constexpr int64_t L = omm::crt::kPlanes;
     c.ldm = (m + 7) / 8 * 8;
     c.ld2n = (2 * n + 7) / 8 * 8;
     const bool pre = h->opt.precon != 0;
@@ -508,7 +541,7 @@ int crt_alloc(omm_handle *h) {
     const int64_t w1 = 2 * omm::crt::words_of(m, n), w2 = omm::crt::words_of(2 * n, 2 * n);
     const int64_t words = w1 > w2 ? w1 : w2;
     const int64_t nP = pre ? L * m * c.ldm : 0, nG = pre ? L * n * c.ldm : 0;
-    const int64_t nE = 2 * m + 4 * n + m + n + m + n, nPart = omm::crt::kRowSlices * m;
+    const int64_t nE = 2 * m + 4 * n + m + n + m + n + 1, nPart = omm::crt::kRowSlices * m;
     int64_t bytes = 0;
     auto take = [&](int64_t size) {   // 256-byte aligned offsets
         const int64_t at = bytes;
@@ -544,6 +577,7 @@ int crt_alloc(omm_handle *h) {
     c.eHSW = c.eSWHW + m;
     c.eP = c.eHSW + n;
     c.eG = c.eP + m;
+    c.bal = c.eG + n;
     const int l = (int)L;
     if ((rc = omm::tc::make_digit_map(&c.mapHS, c.HSr, m, 2 * m, c.ldm, 2 * m * c.ldm, l, 128)) ||
         (rc = omm::tc::make_digit_map(&c.mapWD, c.WDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128)) ||
@@ -1253,8 +1287,8 @@ int precon_build(omm_handle *h) {
             TRY(omm::tc::pack_cm(m, m, h->P, m, h->mx.Pd, h->mx.ldm, m * h->mx.ldm, kDig, nullptr, st));
     }
     if (crt_on(h))
-        TRY(omm::crt::pack_rows(m, m, h->P, m, h->cr.eP, h->cr.part, h->cr.Pr, h->cr.ldm, m * h->cr.ldm, true, nullptr,
-                                st));
+        TRY(omm::crt::pack_rows(m, m, h->P, m, h->cr.eP, h->cr.part, h->cr.Pr, h->cr.ldm, m * h->cr.ldm, true, kNoBalance,
+                                nullptr, st));
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
     if (h->hstate->status != OMM_OK) return h->hstate->status;
@@ -1324,10 +1358,12 @@ int dense_set(omm_handle *h, const double *H, const double *S, bool on_device) {
         // rows of H' and S; omm_set_H and the Cholesky variant's S = I repack H' only
         StageTimer t(h, OMM_STAGE_PACK);
         CrtBufs &c = h->cr;
-        TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, nullptr, st));
+        TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, kNoBalance, nullptr,
+                                st));
         if (S != nullptr && !s_identity(h))
             TRY(omm::crt::pack_rows(m, m, h->HS + mm, m, c.eHS + m, c.part, c.HSr + m * c.ldm, c.ldm, 2 * m * c.ldm, true,
-                                    nullptr, st));
+                                    kNoBalance, nullptr, st));
+        TRY(omm::crt::balance(m, c.eHS, s_identity(h) ? nullptr : c.eHS + m, c.bal, st));
     }
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaEventRecord(h->ev1, st));

@@ -244,6 +244,7 @@ __global__ void __launch_bounds__(kUnitThreads, 1)
                             const float x = __uint_as_float(r0[j]);
                             if (CRT) {
                                 // x - mod * rint(x / mod): exact, in [-mod/2 - 1, mod/2 + 1]
+                                // (mod = inv = 0: x)
                                 const float qf = fmaf(x, inv, kMagic) - kMagic;
                                 float r = fmaf(-mod, qf, x);
                                 if (k != 0) r += __uint_as_float(acc[c0 + j]);
@@ -276,6 +277,7 @@ __global__ void __launch_bounds__(kUnitThreads, 1)
 #pragma unroll
                             for (int j = 0; j < 4; ++j) {
                                 float r = __uint_as_float(acc[c + j]);
+                                if (mod == 0.f) r = (r >= kMagnitudeFloor || r == 0.f) ? 1.f : 0.f;
                                 if (nunits > 1) r = fmaf(-mod, fmaf(r, inv, kMagic) - kMagic, r);
                                 y[j] = __float_as_uint(r + kMagic);   // low byte: r mod 256
                             }

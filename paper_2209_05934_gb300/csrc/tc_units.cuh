@@ -9,7 +9,7 @@
 namespace omm {
 namespace tc {
 
-constexpr int kUnitMaxGroups = 16;   // planes of one launch
+constexpr int kUnitMaxGroups = 19;   // planes of one launch
 constexpr int kUnitMaxPairs = 36;
 
 // One launch computes `ngroups` integer planes of an M x N product (z-batched).
@@ -18,7 +18,11 @@ constexpr int kUnitMaxPairs = 36;
 //   digits (crt = 0): the sum as int32, plane g at out + g * plane words,
 //     element (i, j) of batch z at z * z_step + j * ldp + i;
 //   residues (crt = 1, one pair per group): the sum reduced modulo mod[g], a
-//     signed byte; four columns share a word: word (j / 4) * ldp + i.
+//     signed byte; four columns share a word: word (j / 4) * ldp + i.  A group with
+//     mod[g] = 0 multiplies magnitudes instead of integers: its byte is 1 where the sum
+//     is zero or at least kMagnitudeFloor, else 0.
+constexpr float kMagnitudeFloor = 1.f / 65536.f;
+
 struct UnitArgs {
     int M, N, K;
     int nbatch;
