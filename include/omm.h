@@ -59,11 +59,15 @@ enum {
 
 /* arithmetic of the solve */
 enum {
-    OMM_PREC_FP64 = 0,   /* every product accurate to FP64: dense handles find each from its
-                            residues on the tensor cores (about 60 bytes per element of
-                            [H; S] beside the arrays; a handle whose planes would exceed an
-                            eighth of the device's memory runs FP64 products on the CUDA
-                            cores instead), sparse handles in FP64 on the CUDA cores */
+    OMM_PREC_FP64 = 0,   /* every product at least as accurate as an FP64 multiply-add chain,
+                            element by element: dense handles find each from its residues on
+                            the tensor cores where that holds, else in FP64 (about 75 bytes
+                            per element of [H; S] beside the arrays, at most an eighth of
+                            the device's memory for all handles, kept between solves and
+                            given up, while no call is using it, for other handles and
+                            other allocations of this library; a solve without them runs
+                            FP64 products on the CUDA cores), sparse handles in FP64 on
+                            the CUDA cores */
     OMM_PREC_MIXED = 1   /* BF16-split tensor-core products for the bulk of the
                             CG, FP64 state, then an accurate refinement sweep */
 };

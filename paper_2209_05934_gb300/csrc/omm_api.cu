@@ -80,7 +80,14 @@ struct ExactBufs {
 //   SWHWr [19][m][ld2n]  rows of [SW | H'W]       A of the gradient
 //   HSWr  [19][n][ld2n]  columns of [H_W ; S_W]   B of the gradient
 // words: the planes of a product; part: partial row norms.
+//
+// A handle can do without them: they are kept between solves while there is room, and
+// taken again where another handle was given their memory (planes_take).
 struct CrtBufs {
+    int64_t bytes = 0;
+    int device = 0;
+    bool in_use = false;                                        // under g_planes.mu
+    bool packed_H = false, packed_S = false, packed_P = false;  // the planes hold the handle's matrices
     int64_t ldm = 0, ld2n = 0;
     char *base = nullptr;   // one allocation holds them all
     __nv_bfloat16 *HSr = nullptr, *WDr = nullptr, *HDSDr = nullptr, *SWHWr = nullptr, *HSWr = nullptr;
@@ -134,7 +141,9 @@ struct omm_handle {
     int graph_eager[kPhases] = {};
     MixedBufs mx;
     ExactBufs ex;
-    CrtBufs cr;               // FP64 form on the tensor cores (cr.words == nullptr: CUDA-core products)
+    CrtBufs cr;               // FP64 form on the tensor cores
+    bool planes_on = false;   // the handle is using its planes (else CUDA-core products)
+    bool graph_planes = false;  // planes_on of the captured chunk graphs
     HandleList lists[3];      // persistent tile lists of the step's split products (gemm_persistent)
     double *L = nullptr;      // Cholesky variant: factor of S (m x m)
     double *Wsave = nullptr;  // Cholesky variant: W in the original basis (m x n)
@@ -170,26 +179,80 @@ struct omm_handle {
 
 namespace {
 
+// Captured chunk graphs hold the launches of one choice of preconditioning and products.
+void drop_graphs(omm_handle *h) {
+    for (int i = 0; i < omm_handle::kPhases; ++i) {
+        if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
+        h->graph[i] = nullptr;
+        h->graph_kernels[i] = 0;
+        h->graph_eager[i] = 0;
+    }
+}
+
+// Handles that hold planes, least recently used first.  A handle's planes are in use from
+// planes_take to planes_release (a call, or a solve from begin to its last step); otherwise
+// any thread may give their memory to another allocation.
+struct PlaneHolders {
+    std::mutex mu;
+    std::vector<omm_handle *> list;
+} g_planes;
+
+void planes_free_locked(omm_handle *h) {
+    auto &l = g_planes.list;
+    l.erase(std::remove(l.begin(), l.end(), h), l.end());
+    drop_graphs(h);   // they hold the addresses
+    cudaFree(h->cr.base);
+    h->cr = CrtBufs{};
+}
+
+// Frees the planes of the least recently used handle of the device that is not using them
+bool planes_make_room_locked(int device) {
+    for (omm_handle *h : g_planes.list)
+        if (h->cr.device == device && !h->cr.in_use) {
+            planes_free_locked(h);
+            return true;
+        }
+    return false;
+}
+
+}  // namespace
+
+namespace omm {
+cudaError_t device_malloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    std::lock_guard<std::mutex> lock(g_planes.mu);
+    int dev = 0;
+    cudaGetDevice(&dev);
+    do {
+        cudaGetLastError();   // not left for a later launch's check
+        *p = nullptr;
+        if (!planes_make_room_locked(dev)) return cudaErrorMemoryAllocation;
+        e = cudaMalloc(p, bytes);
+    } while (e == cudaErrorMemoryAllocation);
+    return e;
+}
+}  // namespace omm
+
+namespace {
+
 template <class T>
 int dalloc(T **p, size_t count) {
     if (count == 0) count = 1;
-    if (cudaMalloc((void **)p, count * sizeof(T)) != cudaSuccess) {
+    if (omm::device_malloc((void **)p, count * sizeof(T)) != cudaSuccess) {
         *p = nullptr;
         return OMM_ERR_NOMEM;
     }
     return OMM_OK;
 }
 
-void crt_free(CrtBufs &c) {
-    cudaFree(c.base);
-    c = CrtBufs{};
-}
-
 void free_handle(omm_handle *h) {
     if (h == nullptr) return;
     if (h->stream) cudaStreamSynchronize(h->stream);
-    for (int i = 0; i < omm_handle::kPhases; ++i)
-        if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
+    {
+        std::lock_guard<std::mutex> lock(g_planes.mu);
+        planes_free_locked(h);
+    }
     for (int i = 0; i < omm_handle::kMaxEv; ++i)
         if (h->evs[i]) cudaEventDestroy(h->evs[i]);
     cudaFree(h->HS);
@@ -215,7 +278,6 @@ void free_handle(omm_handle *h) {
     cudaFree(h->mx.D32);
     cudaFree(h->mx.Df32);
     cudaFree(h->ex.base);
-    crt_free(h->cr);
     cudaFree(h->L);
     cudaFree(h->Wsave);
     cudaFree(h->S0);
@@ -312,9 +374,9 @@ int64_t n_occ(const omm_handle *h) { return h->opt.n_occupied > 0 ? h->opt.n_occ
 
 // ---------------------------------------------------------------- FP64 form
 // The products run on the tensor cores through residue planes (crt.cu) where the
-// handle holds them, else on the CUDA cores (dense_fp64.cu).
+// handle has them, else on the CUDA cores (dense_fp64.cu).
 const omm::crt::Balance kNoBalance{};
-bool crt_on(const omm_handle *h) { return h->cr.words != nullptr; }
+bool crt_on(const omm_handle *h) { return h->planes_on; }
 
 omm::crt::Args crt_args(omm_handle *h, int64_t M, int64_t N, int64_t K) {
     omm::crt::Args a{};
@@ -525,14 +587,9 @@ int dense_start(omm_handle *h) {
     return dense_direction(h, 1);
 }
 
-// Residue planes of an FP64 dense handle.  They take about 60 bytes per element of
-// [H' ; S] against 8 for the matrices themselves, so a handle whose planes would
-// exceed an eighth of the device's memory (m ~ 17000 at n = m / 4), or for which
-// the allocation fails, keeps the CUDA-core products.  There is no lower size limit:
-// a step takes 100 us against 104 at m = 8, 104 against 224 at m = 64.
-int crt_alloc(omm_handle *h) {
+// Sizes and addresses (from c.base) of a handle's planes
+void planes_layout(const omm_handle *h, CrtBufs &c) {
     const int64_t m = h->m, n = h->n;
-    CrtBufs &c = h->cr;
     constexpr int64_t L = omm::crt::kPlanes;
     c.ldm = (m + 7) / 8 * 8;
     c.ld2n = (2 * n + 7) / 8 * 8;
@@ -542,23 +599,16 @@ int crt_alloc(omm_handle *h) {
     const int64_t words = w1 > w2 ? w1 : w2;
     const int64_t nP = pre ? L * m * c.ldm : 0, nG = pre ? L * n * c.ldm : 0;
     const int64_t nE = 2 * m + 4 * n + m + n + m + n + 1, nPart = omm::crt::kRowSlices * m;
-    int64_t bytes = 0;
+    c.bytes = 0;
     auto take = [&](int64_t size) {   // 256-byte aligned offsets
-        const int64_t at = bytes;
-        bytes += (size + 255) / 256 * 256;
+        const int64_t at = c.bytes;
+        c.bytes += (size + 255) / 256 * 256;
         return at;
     };
     const int64_t oHS = take(2 * nHS), oWD = take(2 * nWD), oHDSD = take(2 * nWD), oSWHW = take(2 * nSWHW),
                   oHSW = take(2 * nHSW), oP = take(2 * nP), oG = take(2 * nG), oE = take(4 * nE), oPart = take(8 * nPart),
                   oWords = take(4 * words);
-    size_t free_b = 0, total_b = 0;
-    OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
-    if (bytes > (int64_t)(total_b / 8)) return OMM_OK;
-    if (cudaMalloc((void **)&c.base, (size_t)bytes) != cudaSuccess) {
-        cudaGetLastError();   // the handle works without them
-        c = CrtBufs{};
-        return OMM_OK;
-    }
+    if (c.base == nullptr) return;
     c.HSr = (__nv_bfloat16 *)(c.base + oHS);
     c.WDr = (__nv_bfloat16 *)(c.base + oWD);
     c.HDSDr = (__nv_bfloat16 *)(c.base + oHDSD);
@@ -569,7 +619,6 @@ int crt_alloc(omm_handle *h) {
     c.e = (int *)(c.base + oE);
     c.part = (float2 *)(c.base + oPart);
     c.words = (uint32_t *)(c.base + oWords);
-    int rc;
     c.eHS = c.e;
     c.eWD = c.eHS + 2 * m;
     c.eHDSD = c.eWD + 2 * n;
@@ -578,15 +627,103 @@ int crt_alloc(omm_handle *h) {
     c.eP = c.eHSW + n;
     c.eG = c.eP + m;
     c.bal = c.eG + n;
-    const int l = (int)L;
-    if ((rc = omm::tc::make_digit_map(&c.mapHS, c.HSr, m, 2 * m, c.ldm, 2 * m * c.ldm, l, 128)) ||
-        (rc = omm::tc::make_digit_map(&c.mapWD, c.WDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128)) ||
-        (rc = omm::tc::make_digit_map(&c.mapHDSD, c.HDSDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128)) ||
-        (rc = omm::tc::make_digit_map(&c.mapSWHW, c.SWHWr, 2 * n, m, c.ld2n, m * c.ld2n, l, 128)) ||
-        (rc = omm::tc::make_digit_map(&c.mapHSW, c.HSWr, 2 * n, n, c.ld2n, n * c.ld2n, l, 128)) ||
-        (pre && (rc = omm::tc::make_digit_map(&c.mapP, c.Pr, m, m, c.ldm, m * c.ldm, l, 128))) ||
-        (pre && (rc = omm::tc::make_digit_map(&c.mapG, c.Gr, m, n, c.ldm, n * c.ldm, l, 128))))
-        return rc;
+}
+
+int planes_maps(const omm_handle *h, CrtBufs &c) {
+    const int64_t m = h->m, n = h->n;
+    const int l = omm::crt::kPlanes;
+    TRY(omm::tc::make_digit_map(&c.mapHS, c.HSr, m, 2 * m, c.ldm, 2 * m * c.ldm, l, 128));
+    TRY(omm::tc::make_digit_map(&c.mapWD, c.WDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128));
+    TRY(omm::tc::make_digit_map(&c.mapHDSD, c.HDSDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128));
+    TRY(omm::tc::make_digit_map(&c.mapSWHW, c.SWHWr, 2 * n, m, c.ld2n, m * c.ld2n, l, 128));
+    TRY(omm::tc::make_digit_map(&c.mapHSW, c.HSWr, 2 * n, n, c.ld2n, n * c.ld2n, l, 128));
+    if (h->opt.precon != 0) {
+        TRY(omm::tc::make_digit_map(&c.mapP, c.Pr, m, m, c.ldm, m * c.ldm, l, 128));
+        TRY(omm::tc::make_digit_map(&c.mapG, c.Gr, m, n, c.ldm, n * c.ldm, l, 128));
+    }
+    return OMM_OK;
+}
+
+// Planes for an FP64 dense handle, before a call that packs or multiplies with them.  They
+// take about 75 bytes per element of [H' ; S] against 8 for the matrices themselves, so all
+// handles of a device together hold at most an eighth of its memory (one handle: m ~ 16000 at
+// n = m / 4): planes that no call is using give way to others, and to any other allocation
+// of the library (omm::device_malloc).  A handle beyond that, or one whose planes find no
+// memory, runs this solve's products on the CUDA cores.  There is no
+// lower size limit: a step takes 100 us against 104 at m = 8, 104 against 224 at m = 64.
+int planes_take(omm_handle *h) {
+    h->planes_on = false;
+    if (h->sparse || h->opt.precision != OMM_PREC_FP64) return OMM_OK;
+    std::lock_guard<std::mutex> lock(g_planes.mu);
+    auto &l = g_planes.list;
+    if (h->cr.base == nullptr) {
+        CrtBufs c;
+        planes_layout(h, c);
+        size_t free_b = 0, total_b = 0;
+        OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+        OMM_CUDA_TRY(cudaGetDevice(&c.device));
+        const int64_t most = (int64_t)(total_b / 8);
+        if (c.bytes > most) return OMM_OK;
+        for (;;) {
+            int64_t held = 0;
+            for (const omm_handle *o : l) held += o->cr.device == c.device ? o->cr.bytes : 0;
+            if (held + c.bytes <= most && cudaMalloc((void **)&c.base, (size_t)c.bytes) == cudaSuccess) break;
+            cudaGetLastError();
+            c.base = nullptr;
+            if (!planes_make_room_locked(c.device)) return OMM_OK;
+        }
+        planes_layout(h, c);
+        const int rc = planes_maps(h, c);
+        if (rc != OMM_OK) {
+            cudaFree(c.base);
+            return rc;
+        }
+        h->cr = c;
+    } else {
+        l.erase(std::remove(l.begin(), l.end(), h), l.end());
+    }
+    l.push_back(h);
+    h->cr.in_use = h->planes_on = true;
+    return OMM_OK;
+}
+
+void planes_release(omm_handle *h) {
+    if (!h->planes_on) return;
+    std::lock_guard<std::mutex> lock(g_planes.mu);
+    h->cr.in_use = h->planes_on = false;
+}
+
+// planes_release at the end of a call, unless the solve goes on
+struct PlaneUse {
+    omm_handle *h;
+    explicit PlaneUse(omm_handle *h_) : h(h_) {}
+    ~PlaneUse() {
+        if (h != nullptr) planes_release(h);
+    }
+    void keep() { h = nullptr; }
+};
+
+// What the planes do not hold yet of H', S (rows) and, with the preconditioner on, of P
+int planes_pack(omm_handle *h) {
+    if (!h->planes_on) return OMM_OK;
+    const int64_t m = h->m;
+    CrtBufs &c = h->cr;
+    cudaStream_t st = h->stream;
+    if (!c.packed_H || !c.packed_S) {
+        StageTimer t(h, OMM_STAGE_PACK);
+        if (!c.packed_H)
+            TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, kNoBalance, nullptr,
+                                    st));
+        if (!c.packed_S && !s_identity(h))
+            TRY(omm::crt::pack_rows(m, m, h->HS + m * m, m, c.eHS + m, c.part, c.HSr + m * c.ldm, c.ldm, 2 * m * c.ldm,
+                                    true, kNoBalance, nullptr, st));
+        TRY(omm::crt::balance(m, c.eHS, s_identity(h) ? nullptr : c.eHS + m, c.bal, st));
+        c.packed_H = c.packed_S = true;
+    }
+    if (h->precon_on && h->p_ready && !c.packed_P) {
+        TRY(omm::crt::pack_rows(m, m, h->P, m, c.eP, c.part, c.Pr, c.ldm, m * c.ldm, true, kNoBalance, nullptr, st));
+        c.packed_P = true;
+    }
     return OMM_OK;
 }
 
@@ -808,8 +945,8 @@ int run_split(omm_handle *h, const SplitCall &c, int slot) {
         TRY(tile_problem(c, mode, p));
         std::vector<omm::tc::TileRef> tiles;
         omm::tc::list_tiles(0, p.a, c.nbatch, mode, p.bn, tiles);
-        OMM_CUDA_TRY(cudaMalloc((void **)&L.probs, sizeof(p)));
-        OMM_CUDA_TRY(cudaMalloc((void **)&L.tiles, tiles.size() * sizeof(omm::tc::TileRef)));
+        OMM_CUDA_TRY(omm::device_malloc((void **)&L.probs, sizeof(p)));
+        OMM_CUDA_TRY(omm::device_malloc((void **)&L.tiles, tiles.size() * sizeof(omm::tc::TileRef)));
         OMM_CUDA_TRY(cudaMemcpy(L.probs, &p, sizeof(p), cudaMemcpyHostToDevice));
         OMM_CUDA_TRY(cudaMemcpy(L.tiles, tiles.data(), tiles.size() * sizeof(omm::tc::TileRef), cudaMemcpyHostToDevice));
         L.ntiles = (int)tiles.size();
@@ -1256,7 +1393,7 @@ int precon_alloc(omm_handle *h) {
     TRY(dalloc(&h->P, (size_t)(m * m)));
     TRY(dalloc(&h->PG, (size_t)(m * n)));
     TRY(dalloc(&h->cw.Linv, (size_t)omm::chol::linv_elems(m)));
-    if (cudaMalloc(&h->cw.ws, (size_t)h->cw.bytes) != cudaSuccess) {
+    if (omm::device_malloc(&h->cw.ws, (size_t)h->cw.bytes) != cudaSuccess) {
         h->cw.ws = nullptr;
         return OMM_ERR_NOMEM;
     }
@@ -1286,24 +1423,12 @@ int precon_build(omm_handle *h) {
         if (h->opt.precision == OMM_PREC_MIXED)
             TRY(omm::tc::pack_cm(m, m, h->P, m, h->mx.Pd, h->mx.ldm, m * h->mx.ldm, kDig, nullptr, st));
     }
-    if (crt_on(h))
-        TRY(omm::crt::pack_rows(m, m, h->P, m, h->cr.eP, h->cr.part, h->cr.Pr, h->cr.ldm, m * h->cr.ldm, true, kNoBalance,
-                                nullptr, st));
+    h->cr.packed_P = false;
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
     if (h->hstate->status != OMM_OK) return h->hstate->status;
     h->p_ready = true;
     return OMM_OK;
-}
-
-// Captured chunk graphs hold the launches of one choice of preconditioning.
-void drop_graphs(omm_handle *h) {
-    for (int i = 0; i < omm_handle::kPhases; ++i) {
-        if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
-        h->graph[i] = nullptr;
-        h->graph_kernels[i] = 0;
-        h->graph_eager[i] = 0;
-    }
 }
 
 // Dense setup for omm_set_HS (S given) and omm_set_H (S == nullptr: the
@@ -1354,17 +1479,12 @@ int dense_set(omm_handle *h, const double *H, const double *S, bool on_device) {
             TRY(omm::tc::exact_pack(p, nullptr, h->ex.s < 6 ? h->ex.s : 6, nullptr, st));
         }
     }
-    if (crt_on(h)) {
-        // rows of H' and S; omm_set_H and the Cholesky variant's S = I repack H' only
-        StageTimer t(h, OMM_STAGE_PACK);
-        CrtBufs &c = h->cr;
-        TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, kNoBalance, nullptr,
-                                st));
-        if (S != nullptr && !s_identity(h))
-            TRY(omm::crt::pack_rows(m, m, h->HS + mm, m, c.eHS + m, c.part, c.HSr + m * c.ldm, c.ldm, 2 * m * c.ldm, true,
-                                    kNoBalance, nullptr, st));
-        TRY(omm::crt::balance(m, c.eHS, s_identity(h) ? nullptr : c.eHS + m, c.bal, st));
-    }
+    // FP64 form: rows of H' and S; omm_set_H and the Cholesky variant's S = I repack H' only
+    PlaneUse use(h);
+    TRY(planes_take(h));
+    h->cr.packed_H = false;
+    if (S != nullptr) h->cr.packed_S = false;
+    TRY(planes_pack(h));
     OMM_CUDA_TRY(cudaMemcpyAsync(h->hstate, h->dstate, sizeof(omm::DevState), cudaMemcpyDeviceToHost, st));
     OMM_CUDA_TRY(cudaEventRecord(h->ev1, st));
     OMM_CUDA_TRY(cudaStreamSynchronize(st));
@@ -1547,7 +1667,7 @@ int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *patt
         if ((rc = dalloc(&h->L, (size_t)(m * m))) || (rc = dalloc(&h->Wsave, (size_t)mn)) ||
             (rc = dalloc(&h->S0, (size_t)(m * m))) ||
             (rc = dalloc(&h->cw.Linv, (size_t)omm::chol::linv_elems(m))) ||
-            (cudaMalloc(&h->cw.ws, (size_t)h->cw.bytes) != cudaSuccess ? (rc = OMM_ERR_NOMEM) : 0)) {
+            (omm::device_malloc(&h->cw.ws, (size_t)h->cw.bytes) != cudaSuccess ? (rc = OMM_ERR_NOMEM) : 0)) {
             free_handle(h);
             return rc;
         }
@@ -1562,10 +1682,11 @@ int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *patt
         return rc;
     }
     // last: what the handle cannot do without is allocated by now
-    if (!h->sparse && h->opt.precision == OMM_PREC_FP64 && (rc = crt_alloc(h))) {
+    if ((rc = planes_take(h))) {
         free_handle(h);
         return rc;
     }
+    planes_release(h);
     if (cudaMallocHost((void **)&h->hstate, sizeof(omm::DevState)) != cudaSuccess) {
         h->hstate = nullptr;
         free_handle(h);
@@ -1712,16 +1833,20 @@ int begin_setup(omm_handle *h, const double *W0, int32_t W0_on_device, double to
     if (h->opt.precon != 0 && !h->have_T) return OMM_ERR_STATE;
     const int64_t n = h->n;
     cudaStream_t st = h->stream;
+    PlaneUse use(h);
+    TRY(planes_take(h));
     OMM_CUDA_TRY(cudaEventRecord(h->ev0, st));
     h->precon_on = h->opt.precon < 0 || (h->opt.precon > 0 && h->precon_left > 0);
     if (h->precon_on) {
         if (!h->p_ready) TRY(precon_build(h));
         if (h->opt.precon > 0) --h->precon_left;
     }
-    if (h->precon_on != h->graph_precon) {
+    if (h->precon_on != h->graph_precon || h->planes_on != h->graph_planes) {
         drop_graphs(h);
         h->graph_precon = h->precon_on;
+        h->graph_planes = h->planes_on;
     }
+    TRY(planes_pack(h));
     if (h->opt.cholesky && !h->sparse) {
         // W~ = L^T W: W0, or the previous solution kept in the original basis
         if (W0 != nullptr)
@@ -1783,6 +1908,7 @@ int begin_setup(omm_handle *h, const double *W0, int32_t W0_on_device, double to
         { StageTimer t(h, OMM_STAGE_START); TRY(dense_start(h)); }
     }
     h->have_W = true;
+    use.keep();   // to the end of the solve
     return OMM_OK;
 }
 }  // namespace
@@ -1809,6 +1935,7 @@ int omm_solve_progress(omm_handle *h, int32_t blocking, int32_t *done) {
         omm::set_error("a bounded mbarrier wait in the tensor-core GEMM timed out");
         h->status = OMM_ERR_TIMEOUT;
         h->phase = PH_FINISHED;
+        planes_release(h);
         *done = 1;
         return OMM_OK;
     }
@@ -1864,6 +1991,7 @@ int omm_solve_progress(omm_handle *h, int32_t blocking, int32_t *done) {
     if (h->phase == PH_MIXED || h->phase == PH_SPARSE_MIXED) h->k_mixed = h->hstate->k;
     h->status = h->hstate->status;
     h->phase = PH_FINISHED;
+    planes_release(h);
     OMM_CUDA_TRY(cudaEventRecord(h->ev1, h->stream));
     *done = 1;
     return OMM_OK;
@@ -2016,8 +2144,8 @@ int build_group_list(omm_handle **hs, int count, int stage, int mode, GroupList 
     });
     std::vector<omm::tc::TileRef> tiles;
     for (int i : order) omm::tc::list_tiles(i, probs[i].a, nb[i], mode, probs[i].bn, tiles);
-    OMM_CUDA_TRY(cudaMalloc((void **)&L.probs, probs.size() * sizeof(omm::tc::TileProblem)));
-    OMM_CUDA_TRY(cudaMalloc((void **)&L.tiles, tiles.size() * sizeof(omm::tc::TileRef)));
+    OMM_CUDA_TRY(omm::device_malloc((void **)&L.probs, probs.size() * sizeof(omm::tc::TileProblem)));
+    OMM_CUDA_TRY(omm::device_malloc((void **)&L.tiles, tiles.size() * sizeof(omm::tc::TileRef)));
     OMM_CUDA_TRY(cudaMemcpy(L.probs, probs.data(), probs.size() * sizeof(omm::tc::TileProblem), cudaMemcpyHostToDevice));
     OMM_CUDA_TRY(cudaMemcpy(L.tiles, tiles.data(), tiles.size() * sizeof(omm::tc::TileRef), cudaMemcpyHostToDevice));
     L.ntiles = (int)tiles.size();
@@ -2111,7 +2239,7 @@ int build_group_glue(omm_handle **hs, int count, GroupGlue &G) {
     std::vector<char> host(bytes);
     memcpy(host.data(), sys.data(), sys.size() * sizeof(omm::GlueSys));
     for (int k = 0; k < omm::GLUE_KERNELS; ++k) memcpy(host.data() + off[k], list[k].data(), list[k].size() * sizeof(int2));
-    OMM_CUDA_TRY(cudaMalloc((void **)&G.mem, bytes));
+    OMM_CUDA_TRY(omm::device_malloc((void **)&G.mem, bytes));
     OMM_CUDA_TRY(cudaMemcpy(G.mem, host.data(), bytes, cudaMemcpyHostToDevice));
     G.sys = (const omm::GlueSys *)G.mem;
     for (int k = 0; k < omm::GLUE_KERNELS; ++k) G.blks[k] = (const int2 *)(G.mem + off[k]);
@@ -2356,7 +2484,7 @@ int omm_get_density(omm_handle *h, int32_t which, double *dst, int32_t on_device
         h->dWs_bytes = b1 > b2 ? b1 : b2;
         TRY(dalloc(&h->dK, (size_t)(3 * n * n)));   // K, then [H'_W ; S_W] (2n x n)
         TRY(dalloc(&h->dT, (size_t)(m * n)));
-        if (cudaMalloc(&h->dWs, (size_t)h->dWs_bytes) != cudaSuccess) return OMM_ERR_NOMEM;
+        if (omm::device_malloc(&h->dWs, (size_t)h->dWs_bytes) != cudaSuccess) return OMM_ERR_NOMEM;
     }
     double *out = dst;
     if (!on_device) {

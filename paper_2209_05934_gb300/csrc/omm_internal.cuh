@@ -81,6 +81,10 @@ int launch_coeffs_linemin(int n, const double *h0, const double *s0, int64_t ldh
                           int64_t ldz, double *scratch, unsigned int *counter, DevState *state,
                           double *coeffs_out, cudaStream_t st, bool do_linemin);
 
+// cudaMalloc for everything a handle cannot do without: where the device is full, what
+// idle handles hold beyond that (the planes of the FP64 products) is given up for it.
+cudaError_t device_malloc(void **p, size_t bytes);
+
 // Optional BF16 digit output of an elementwise kernel: planes of `plane`
 // elements, digit row stride `ld`; ptr == nullptr disables it.
 struct DigitOut {

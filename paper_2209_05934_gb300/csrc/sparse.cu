@@ -1372,7 +1372,7 @@ int upload(const Host &hs, Dev &d) {
     auto up = [](auto **dst, const auto &src) -> int {
         using T = typename std::remove_reference<decltype(src[0])>::type;
         const size_t n = src.size() ? src.size() : 1;
-        if (cudaMalloc((void **)dst, n * sizeof(T)) != cudaSuccess) return OMM_ERR_NOMEM;
+        if (device_malloc((void **)dst, n * sizeof(T)) != cudaSuccess) return OMM_ERR_NOMEM;
         if (!src.empty() && cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice) != cudaSuccess)
             return OMM_ERR_CUDA;
         return OMM_OK;
@@ -1394,7 +1394,7 @@ int upload(const Host &hs, Dev &d) {
         return rc;
     const int64_t bb = (int64_t)P.bm * P.bm, bw = (int64_t)P.bm * P.bn, bq = (int64_t)P.bn * P.bn;
     auto al = [](double **p, int64_t n) -> int {
-        return cudaMalloc((void **)p, (size_t)(n > 0 ? n : 1) * sizeof(double)) == cudaSuccess ? OMM_OK : OMM_ERR_NOMEM;
+        return device_malloc((void **)p, (size_t)(n > 0 ? n : 1) * sizeof(double)) == cudaSuccess ? OMM_OK : OMM_ERR_NOMEM;
     };
     if ((rc = al(&d.HS, 2 * d.nnzH * bb)) || (rc = al(&d.Hin, 2 * d.nnzH * bb)) || (rc = al(&d.W, d.nnzW * bw)) ||
         (rc = al(&d.D, d.nnzW * bw)) || (rc = al(&d.G, d.nnzW * bw)) || (rc = al(&d.Gp, d.nnzW * bw)) ||
@@ -1403,7 +1403,7 @@ int upload(const Host &hs, Dev &d) {
         (rc = al(&d.X, d.nnzN * bq)) || (rc = al(&d.Y, d.nnzN * bq)) || (rc = al(&d.h2, d.nnzN * bq)) ||
         (rc = al(&d.s2, d.nnzN * bq)))
         return rc;
-    if (cudaMalloc((void **)&d.keep, (size_t)(d.nnzH > 0 ? d.nnzH : 1)) != cudaSuccess) return OMM_ERR_NOMEM;
+    if (device_malloc((void **)&d.keep, (size_t)(d.nnzH > 0 ? d.nnzH : 1)) != cudaSuccess) return OMM_ERR_NOMEM;
     return OMM_OK;
 }
 
@@ -1444,7 +1444,7 @@ int set_HS(Dev &d, const double *H, const double *S, bool on_device, double eps,
 int screen_alloc(Dev &d, double eps) {
     if (!(eps > 0.0)) return OMM_OK;
     const int64_t total = 2 * d.nnzH + 2 * d.nnzW + 4 * d.nnzHW + 2 * d.nnzN;
-    if (cudaMalloc((void **)&d.nrm, (size_t)(total > 0 ? total : 1) * sizeof(double)) != cudaSuccess)
+    if (device_malloc((void **)&d.nrm, (size_t)(total > 0 ? total : 1) * sizeof(double)) != cudaSuccess)
         return OMM_ERR_NOMEM;
     d.screen_eps2 = eps * eps;
     d.nHS = d.nrm;
@@ -1538,12 +1538,12 @@ int contract(Dev &d, const double *Wl, const double *Dl, const double *HDr, cons
 
 int upload_density(const DensHost &dh, Dev &d) {
     auto up64 = [](int64_t **dst, const std::vector<int64_t> &v) -> int {
-        if (cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(int64_t)) != cudaSuccess) return OMM_ERR_NOMEM;
+        if (device_malloc((void **)dst, std::max<size_t>(1, v.size()) * sizeof(int64_t)) != cudaSuccess) return OMM_ERR_NOMEM;
         return cudaMemcpy(*dst, v.data(), v.size() * sizeof(int64_t), cudaMemcpyHostToDevice) == cudaSuccess
                    ? OMM_OK : OMM_ERR_CUDA;
     };
     auto up32 = [](int32_t **dst, const std::vector<int32_t> &v) -> int {
-        if (cudaMalloc(dst, std::max<size_t>(1, v.size()) * sizeof(int32_t)) != cudaSuccess) return OMM_ERR_NOMEM;
+        if (device_malloc((void **)dst, std::max<size_t>(1, v.size()) * sizeof(int32_t)) != cudaSuccess) return OMM_ERR_NOMEM;
         return cudaMemcpy(*dst, v.data(), v.size() * sizeof(int32_t), cudaMemcpyHostToDevice) == cudaSuccess
                    ? OMM_OK : OMM_ERR_CUDA;
     };
@@ -1551,8 +1551,8 @@ int upload_density(const DensHost &dh, Dev &d) {
     if ((rc = up64(&d.Trp, dh.Trp)) || (rc = up32(&d.Tw, dh.Tw)) || (rc = up32(&d.Tq, dh.Tq)) ||
         (rc = up64(&d.Rrp, dh.Rrp)) || (rc = up32(&d.Rt, dh.Rt)) || (rc = up32(&d.Rw, dh.Rw)))
         return rc;
-    if (cudaMalloc(&d.K, (size_t)(d.nnzN * d.bn * d.bn) * sizeof(double)) != cudaSuccess) return OMM_ERR_NOMEM;
-    if (cudaMalloc(&d.T, (size_t)(d.nnzHW * d.bm * d.bn) * sizeof(double)) != cudaSuccess) return OMM_ERR_NOMEM;
+    if (device_malloc((void **)&d.K, (size_t)(d.nnzN * d.bn * d.bn) * sizeof(double)) != cudaSuccess) return OMM_ERR_NOMEM;
+    if (device_malloc((void **)&d.T, (size_t)(d.nnzHW * d.bm * d.bn) * sizeof(double)) != cudaSuccess) return OMM_ERR_NOMEM;
     return OMM_OK;
 }
 
@@ -1646,7 +1646,7 @@ int mixed_alloc(const Host &hs, Dev &d) {
             for (size_t t = 0; t < hs.Ca.size(); ++t) slot[t] = wslot[hs.Ca[t]];
             auto up = [](auto **dst, const auto &v) -> int {
                 const size_t bytes = (v.empty() ? 1 : v.size()) * sizeof(v[0]);
-                if (cudaMalloc((void **)dst, bytes) != cudaSuccess) return OMM_ERR_NOMEM;
+                if (device_malloc((void **)dst, bytes) != cudaSuccess) return OMM_ERR_NOMEM;
                 if (!v.empty() && cudaMemcpy(*dst, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice) != cudaSuccess)
                     return OMM_ERR_CUDA;
                 return OMM_OK;
@@ -1662,7 +1662,7 @@ int mixed_alloc(const Host &hs, Dev &d) {
     const int64_t bb = (int64_t)d.bm * d.bm, bw = (int64_t)d.bm * d.bn, bq = (int64_t)d.bn * d.bn;
     const int64_t nHS = 2 * d.nnzH * bb, nW = d.nnzW * bw, nHW = d.nnzHW * bw, nN = d.nnzN * bq;
     const int64_t total = nHS + 4 * nW + 4 * nHW + 6 * nN;
-    if (cudaMalloc((void **)&d.fbuf, (size_t)(total > 0 ? total : 1) * sizeof(float)) != cudaSuccess)
+    if (device_malloc((void **)&d.fbuf, (size_t)(total > 0 ? total : 1) * sizeof(float)) != cudaSuccess)
         return OMM_ERR_NOMEM;
     float *p = d.fbuf;
     auto take = [&](float **dst, int64_t n) { *dst = p; p += n; };
