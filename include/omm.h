@@ -61,13 +61,8 @@ enum {
 enum {
     OMM_PREC_FP64 = 0,   /* every product at least as accurate as an FP64 multiply-add chain,
                             element by element: dense handles find each from its residues on
-                            the tensor cores where that holds, else in FP64 (about 75 bytes
-                            per element of [H; S] beside the arrays, at most an eighth of
-                            the device's memory for all handles, kept between solves and
-                            given up, while no call is using it, for other handles and
-                            other allocations of this library; a solve without them runs
-                            FP64 products on the CUDA cores), sparse handles in FP64 on
-                            the CUDA cores */
+                            the tensor cores where that holds, else in FP64 (omm_options.
+                            fp64_products), sparse handles in FP64 on the CUDA cores */
     OMM_PREC_MIXED = 1   /* BF16-split tensor-core products for the bulk of the
                             CG, FP64 state, then an accurate refinement sweep */
 };
@@ -177,7 +172,27 @@ typedef struct {
                               stays consistent to the split products' accuracy and the
                               converged result is held to the same bars.  0: D keeps
                               split_digits digits */
+    int32_t fp64_products; /* dense handles in OMM_PREC_FP64: where their products run
+                              (OMM_FP64_*).  The residue form takes about 75 bytes per element of
+                              [H; S] beside the arrays; that memory, at most an eighth of the
+                              device's for all handles, is kept between solves and given up, while
+                              no call is using it, for other handles and other allocations of
+                              this library */
 } omm_options;
+
+enum {
+    OMM_FP64_AUTO = 0,       /* residues, or the CUDA cores for a solve without the memory */
+    OMM_FP64_CUDA_CORES = 1, /* always the CUDA cores: no memory beyond the arrays */
+    OMM_FP64_RESIDUES = 2    /* always residues (the same bits whatever else runs): a solve
+                                without the memory ends in OMM_ERR_NOMEM */
+};
+
+/* where the products of a solve ran (omm_product_form) */
+enum {
+    OMM_PRODUCTS_NONE = 0,   /* no solve yet, or not a dense OMM_PREC_FP64 handle */
+    OMM_PRODUCTS_CUDA_CORES = 1,
+    OMM_PRODUCTS_RESIDUES = 2
+};
 
 enum {
     OMM_REFINE_EXACT = 0,  /* exact-digit BF16 tensor-core products (omm_op_exact_gemm) */
@@ -351,6 +366,9 @@ int omm_batch_last_tuning(int32_t *modes, float *ms);
 
 /* Diagnostics of the last set_HS / solve. */
 int omm_get_diag(omm_handle *h, omm_diag *d);
+
+/* OMM_PRODUCTS_* of the handle's last solve (as it began). */
+int omm_product_form(const omm_handle *h);
 
 /*
  * Copy one internal m x n or n x n FP64 array of the handle (for inspection

@@ -144,6 +144,7 @@ struct omm_handle {
     CrtBufs cr;               // FP64 form on the tensor cores
     bool planes_on = false;   // the handle is using its planes (else CUDA-core products)
     bool graph_planes = false;  // planes_on of the captured chunk graphs
+    int product_form = OMM_PRODUCTS_NONE;   // of the last solve
     HandleList lists[3];      // persistent tile lists of the step's split products (gemm_persistent)
     double *L = nullptr;      // Cholesky variant: factor of S (m x m)
     double *Wsave = nullptr;  // Cholesky variant: W in the original basis (m x n)
@@ -649,11 +650,11 @@ int planes_maps(const omm_handle *h, CrtBufs &c) {
 // handles of a device together hold at most an eighth of its memory (one handle: m ~ 16000 at
 // n = m / 4): planes that no call is using give way to others, and to any other allocation
 // of the library (omm::device_malloc).  A handle beyond that, or one whose planes find no
-// memory, runs this solve's products on the CUDA cores.  There is no
+// memory, runs this solve's products on the CUDA cores (h->product_form).  There is no
 // lower size limit: a step takes 100 us against 104 at m = 8, 104 against 224 at m = 64.
 int planes_take(omm_handle *h) {
     h->planes_on = false;
-    if (h->sparse || h->opt.precision != OMM_PREC_FP64) return OMM_OK;
+    if (h->sparse || h->opt.precision != OMM_PREC_FP64 || h->opt.fp64_products == OMM_FP64_CUDA_CORES) return OMM_OK;
     std::lock_guard<std::mutex> lock(g_planes.mu);
     auto &l = g_planes.list;
     if (h->cr.base == nullptr) {
@@ -1553,6 +1554,7 @@ void omm_default_options(omm_options *opt) {
     opt->gemm_pair = 1;
     opt->gemm_persistent = 0;
     opt->dir_digits = 1;
+    opt->fp64_products = OMM_FP64_AUTO;
 }
 
 const char *omm_status_str(int status) {
@@ -1602,7 +1604,7 @@ int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *patt
         (h->opt.n_occupied > 0 && h->opt.n_occupied < n && h->opt.eta_auto) ||
         (h->opt.precon != 0 && !(h->opt.tau_T > 0.0 && isfinite(h->opt.tau_T))) ||
         !(h->opt.screen_eps >= 0.0 && isfinite(h->opt.screen_eps)) || h->opt.dir_digits < 0 ||
-        h->opt.dir_digits > 1) {
+        h->opt.dir_digits > 1 || h->opt.fp64_products < OMM_FP64_AUTO || h->opt.fp64_products > OMM_FP64_RESIDUES) {
         delete h;
         return OMM_ERR_ARG;
     }
@@ -1835,6 +1837,13 @@ int begin_setup(omm_handle *h, const double *W0, int32_t W0_on_device, double to
     cudaStream_t st = h->stream;
     PlaneUse use(h);
     TRY(planes_take(h));
+    if (!h->sparse && h->opt.precision == OMM_PREC_FP64) {
+        if (!h->planes_on && h->opt.fp64_products == OMM_FP64_RESIDUES) {
+            omm::set_error("no memory for the residue planes of the FP64 products");
+            return OMM_ERR_NOMEM;
+        }
+        h->product_form = h->planes_on ? OMM_PRODUCTS_RESIDUES : OMM_PRODUCTS_CUDA_CORES;
+    }
     OMM_CUDA_TRY(cudaEventRecord(h->ev0, st));
     h->precon_on = h->opt.precon < 0 || (h->opt.precon > 0 && h->precon_left > 0);
     if (h->precon_on) {
@@ -2444,6 +2453,8 @@ int omm_batch_last_tuning(int32_t *modes, float *ms) {
     }
     return OMM_OK;
 }
+
+int omm_product_form(const omm_handle *h) { return h != nullptr ? h->product_form : OMM_PRODUCTS_NONE; }
 
 int omm_get_diag(omm_handle *h, omm_diag *d) {
     if (h == nullptr || d == nullptr) return OMM_ERR_ARG;

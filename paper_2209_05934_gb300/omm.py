@@ -20,6 +20,8 @@ ERR_ARG, ERR_NOMEM, ERR_CUDA, ERR_NOT_SPD, ERR_LINESEARCH = -1, -2, -3, -4, -5
 ERR_MAXITER, ERR_PATTERN, ERR_NONFINITE, ERR_TIMEOUT, ERR_STATE, ERR_UNSUPPORTED = -6, -7, -8, -9, -10, -11
 PREC_FP64, PREC_MIXED = 0, 1
 REFINE_EXACT, REFINE_FP64 = 0, 1
+FP64_AUTO, FP64_CUDA_CORES, FP64_RESIDUES = 0, 1, 2
+PRODUCTS_NONE, PRODUCTS_CUDA_CORES, PRODUCTS_RESIDUES = 0, 1, 2
 
 ARRAY_W, ARRAY_HW, ARRAY_SW, ARRAY_G, ARRAY_D, ARRAY_HW_N, ARRAY_SW_N = range(7)
 PATTERN_H, PATTERN_W, PATTERN_HW, PATTERN_N = range(4)
@@ -33,7 +35,8 @@ class Options(C.Structure):
                 ("exact_digits", C.c_int32), ("split_digits", C.c_int32), ("graphs", C.c_int32),
                 ("n_occupied", C.c_int32), ("precon", C.c_int32), ("tau_T", C.c_double),
                 ("screen_eps", C.c_double), ("gemm_pair", C.c_int32),
-                ("gemm_persistent", C.c_int32), ("dir_digits", C.c_int32)]
+                ("gemm_persistent", C.c_int32), ("dir_digits", C.c_int32),
+                ("fp64_products", C.c_int32)]
 
 
 class Pattern(C.Structure):
@@ -66,6 +69,7 @@ _SIGS = {
     "omm_selftest_bounded_wait": (C.c_int, [C.c_int64, C.POINTER(C.c_int32), C.c_void_p]),
     "omm_solve": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_double, C.c_void_p, C.c_int32,
                             C.POINTER(C.c_double), C.POINTER(C.c_int32)]),
+    "omm_product_form": (C.c_int, [C.c_void_p]),
     "omm_get_diag": (C.c_int, [C.c_void_p, C.POINTER(Diag)]),
     "omm_get_array": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_int32]),
     "omm_get_density": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_int32]),
@@ -276,6 +280,10 @@ class Solver:
         d = Diag()
         check(lib().omm_get_diag(self._h, C.byref(d)), "omm_get_diag")
         return d
+
+    def product_form(self) -> int:
+        """Where the products of the last solve ran (PRODUCTS_*)."""
+        return lib().omm_product_form(self._h)
 
     # asynchronous driver
     def begin(self, W0=None, tol: float = 1e-10):
