@@ -367,6 +367,11 @@ int omm_batch_last_tuning(int32_t *modes, float *ms);
 /* Diagnostics of the last set_HS / solve. */
 int omm_get_diag(omm_handle *h, omm_diag *d);
 
+/* Device memory that the residue form of the FP64 products adds to a dense handle (0: more
+ * than the eighth of the current device's memory that it may take, so the products run on the
+ * CUDA cores; without a device no such limit; -1: sizes that omm_create refuses). */
+int64_t omm_product_planes_bytes(int64_t m, int64_t n, int32_t cholesky, int32_t precon);
+
 /* OMM_PRODUCTS_* of the handle's last solve (as it began). */
 int omm_product_form(const omm_handle *h);
 

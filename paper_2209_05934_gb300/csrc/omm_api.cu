@@ -588,14 +588,13 @@ int dense_start(omm_handle *h) {
     return dense_direction(h, 1);
 }
 
-// Sizes and addresses (from c.base) of a handle's planes
-void planes_layout(const omm_handle *h, CrtBufs &c) {
-    const int64_t m = h->m, n = h->n;
+// Sizes and addresses (from c.base) of a handle's planes: with `pre`, of P and G too; with
+// S = I (s_one) of H' alone
+void planes_layout(int64_t m, int64_t n, bool pre, bool s_one, CrtBufs &c) {
     constexpr int64_t L = omm::crt::kPlanes;
     c.ldm = (m + 7) / 8 * 8;
     c.ld2n = (2 * n + 7) / 8 * 8;
-    const bool pre = h->opt.precon != 0;
-    const int64_t nHS = L * 2 * m * c.ldm, nWD = L * 2 * n * c.ldm, nSWHW = L * m * c.ld2n, nHSW = L * n * c.ld2n;
+    const int64_t nHS = L * (s_one ? 1 : 2) * m * c.ldm, nWD = L * 2 * n * c.ldm, nSWHW = L * m * c.ld2n, nHSW = L * n * c.ld2n;
     const int64_t w1 = 2 * omm::crt::words_of(m, n), w2 = omm::crt::words_of(2 * n, 2 * n);
     const int64_t words = w1 > w2 ? w1 : w2;
     const int64_t nP = pre ? L * m * c.ldm : 0, nG = pre ? L * n * c.ldm : 0;
@@ -630,10 +629,13 @@ void planes_layout(const omm_handle *h, CrtBufs &c) {
     c.bal = c.eG + n;
 }
 
+// rows of the planes of [H' ; S]
+int64_t hs_rows(const omm_handle *h) { return (s_identity(h) ? 1 : 2) * h->m; }
+
 int planes_maps(const omm_handle *h, CrtBufs &c) {
     const int64_t m = h->m, n = h->n;
     const int l = omm::crt::kPlanes;
-    TRY(omm::tc::make_digit_map(&c.mapHS, c.HSr, m, 2 * m, c.ldm, 2 * m * c.ldm, l, 128));
+    TRY(omm::tc::make_digit_map(&c.mapHS, c.HSr, m, hs_rows(h), c.ldm, hs_rows(h) * c.ldm, l, 128));
     TRY(omm::tc::make_digit_map(&c.mapWD, c.WDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128));
     TRY(omm::tc::make_digit_map(&c.mapHDSD, c.HDSDr, m, 2 * n, c.ldm, 2 * n * c.ldm, l, 128));
     TRY(omm::tc::make_digit_map(&c.mapSWHW, c.SWHWr, 2 * n, m, c.ld2n, m * c.ld2n, l, 128));
@@ -659,7 +661,7 @@ int planes_take(omm_handle *h) {
     auto &l = g_planes.list;
     if (h->cr.base == nullptr) {
         CrtBufs c;
-        planes_layout(h, c);
+        planes_layout(h->m, h->n, h->opt.precon != 0, s_identity(h), c);
         size_t free_b = 0, total_b = 0;
         OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
         OMM_CUDA_TRY(cudaGetDevice(&c.device));
@@ -673,7 +675,7 @@ int planes_take(omm_handle *h) {
             c.base = nullptr;
             if (!planes_make_room_locked(c.device)) return OMM_OK;
         }
-        planes_layout(h, c);
+        planes_layout(h->m, h->n, h->opt.precon != 0, s_identity(h), c);
         const int rc = planes_maps(h, c);
         if (rc != OMM_OK) {
             cudaFree(c.base);
@@ -713,7 +715,7 @@ int planes_pack(omm_handle *h) {
     if (!c.packed_H || !c.packed_S) {
         StageTimer t(h, OMM_STAGE_PACK);
         if (!c.packed_H)
-            TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, 2 * m * c.ldm, true, kNoBalance, nullptr,
+            TRY(omm::crt::pack_rows(m, m, h->HS, m, c.eHS, c.part, c.HSr, c.ldm, hs_rows(h) * c.ldm, true, kNoBalance, nullptr,
                                     st));
         if (!c.packed_S && !s_identity(h))
             TRY(omm::crt::pack_rows(m, m, h->HS + m * m, m, c.eHS + m, c.part, c.HSr + m * c.ldm, c.ldm, 2 * m * c.ldm,
@@ -2452,6 +2454,18 @@ int omm_batch_last_tuning(int32_t *modes, float *ms) {
         }
     }
     return OMM_OK;
+}
+
+int64_t omm_product_planes_bytes(int64_t m, int64_t n, int32_t cholesky, int32_t precon) {
+    if (m <= 0 || n <= 0 || n > m || n > 2147483647 / 2 || m > ((int64_t)1 << 31)) return -1;
+    CrtBufs c;
+    planes_layout(m, n, precon != 0, cholesky != 0, c);
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+        cudaGetLastError();   // no device: no limit
+        return c.bytes;
+    }
+    return c.bytes <= (int64_t)(total_b / 8) ? c.bytes : 0;
 }
 
 int omm_product_form(const omm_handle *h) { return h != nullptr ? h->product_form : OMM_PRODUCTS_NONE; }

@@ -70,6 +70,7 @@ _SIGS = {
     "omm_solve": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int32, C.c_double, C.c_void_p, C.c_int32,
                             C.POINTER(C.c_double), C.POINTER(C.c_int32)]),
     "omm_product_form": (C.c_int, [C.c_void_p]),
+    "omm_product_planes_bytes": (C.c_int64, [C.c_int64, C.c_int64, C.c_int32, C.c_int32]),
     "omm_get_diag": (C.c_int, [C.c_void_p, C.POINTER(Diag)]),
     "omm_get_array": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_int32]),
     "omm_get_density": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_int32]),
@@ -195,6 +196,11 @@ def selftest_bounded_wait(limit_ns: int, stream=None) -> int:
     check(lib().omm_selftest_bounded_wait(int(limit_ns), C.byref(st), C.c_void_p(stream) if stream else None),
           "omm_selftest_bounded_wait")
     return st.value
+
+
+def product_planes_bytes(m: int, n: int, cholesky: int = 0, precon: int = 0) -> int:
+    """Device memory of a dense FP64 handle's residue planes; see omm_product_planes_bytes."""
+    return lib().omm_product_planes_bytes(m, n, cholesky, precon)
 
 
 def default_options(**kw) -> Options:

@@ -67,11 +67,8 @@ class SolveRecord:
         return self.finish - self.submit
 
 
-DEVICE_BYTES = 284208 << 20   # HBM of one GB300
-
-
-def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7) -> int:
-    """Device memory of one dense handle (what omm_create allocates)."""
+def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7, cholesky: int = 0, precon: int = 0) -> int:
+    """Device memory of one dense handle's arrays and product operands."""
     f64 = 8 * (2 * m * m + 6 * m * n + 2 * n * n + 4 * n * n + 2 * m * n)
     if precision == omm.PREC_MIXED:
         ldm = (m + 7) // 8 * 8
@@ -81,10 +78,7 @@ def footprint_bytes(m: int, n: int, precision: int, exact_digits: int = 7) -> in
         f64 += 2 * exact_digits * (2 * m * ldm + 3 * n * ldm + m * ld2n + n * ld2n)  # exact digits
         f64 += 4 * min(12 * m * n, max(48 << 20, 12 * m * 256))                     # level planes
     else:
-        ldm, ld2n = (m + 7) // 8 * 8, (2 * n + 7) // 8 * 8
-        planes = 32 * (2 * m * ldm + 4 * n * ldm + m * ld2n + n * ld2n) + 16 * max(2 * m * n, 4 * n * n)
-        if planes <= DEVICE_BYTES // 8:                                             # residue planes
-            f64 += planes
+        f64 += omm.product_planes_bytes(m, n, cholesky, precon)                     # residue planes
     return int(f64)
 
 
@@ -107,7 +101,7 @@ class Server:
         self.max_inflight = 0
 
     def _admit(self, req: Request, now: float) -> bool:
-        need = footprint_bytes(req.m, req.n, req.precision)
+        need = footprint_bytes(req.m, req.n, req.precision, cholesky=req.cholesky)
         if self.active and self.used + need > self.budget:
             return False
         s = omm.Solver(req.m, req.n, 8, precision=req.precision, orth_tol=req.orth_tol, cholesky=req.cholesky,
@@ -159,7 +153,7 @@ class Server:
                     a.solver.begin(None, tol=a.req.tol)        # warm start from the resident W
                 else:
                     a.solver.close()
-                    self.used -= footprint_bytes(a.req.m, a.req.n, a.req.precision)
+                    self.used -= footprint_bytes(a.req.m, a.req.n, a.req.precision, cholesky=a.req.cholesky)
                     self.active.remove(a)
             if not progressed and poll_sleep > 0:
                 time.sleep(poll_sleep)
