@@ -223,13 +223,23 @@ __global__ void __launch_bounds__(256) pack_cols_kernel(int64_t K, int64_t R, co
 }
 
 // ------------------------------------------------------------------ packing, K along the rows' columns
-// Partial (code, S) of every row over one slice of the columns, a thread per row
-// (coalesced); S follows the code up as larger elements come.
-__device__ __forceinline__ float rescaled(float S, int from, int to) {   // S of one code in units of another
+// S of one code in units of another
+__device__ __forceinline__ float rescaled(float S, int from, int to) {
     const int d = 127 - 2 * (to - from);
     return d > 0 ? S * __uint_as_float((uint32_t)d << 23) : 0.f;
 }
 
+// (code, S) pairs combined in the order of their index
+__device__ __forceinline__ void norm_join(int &code, float &S, int code2, float S2) {
+    const int top = max(code, code2);
+    S = rescaled(S, code, top) + rescaled(S2, code2, top);
+    code = top;
+}
+
+// Partial (code, S) of every row over one slice of the columns, a thread per row
+// (coalesced); S follows the code up as larger elements come.  The columns on either side
+// of the balance's split are summed without a shift, which then goes to the code (with a
+// shift looked up for every element the kernel took 20 us at m = 1996 in place of 10).
 __global__ void __launch_bounds__(128) row_norm_kernel(int64_t R, int64_t K, const double *__restrict__ X, int64_t ld,
                                                        float2 *part, int64_t slice, const Balance bal,
                                                        const DevState *state) {
@@ -242,29 +252,32 @@ __global__ void __launch_bounds__(128) row_norm_kernel(int64_t R, int64_t K, con
     const uint64_t *xb = reinterpret_cast<const uint64_t *>(X) + r;
     int code = 0;
     float S = 0.f;
-    for (int64_t k = k0; k < k1; k += 8) {
-        uint64_t a[8];
-        int top = 0;
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+        const int64_t ka = half == 0 ? k0 : max(k0, sh.split), kb = half == 0 ? min(k1, sh.split) : k1;
+        int be = 0;
+        uint64_t any = 0;
+        float s = 0.f;
+        for (int64_t k = ka; k < kb; k += 8) {
+            uint64_t a[8];
+            int top = 0;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            a[u] = k + u < k1 ? xb[(k + u) * ld] & 0x7FFFFFFFFFFFFFFFull : 0;
-            top = max(top, fx_code(a[u], sh.at(k + u)));
-        }
-        if (top > code) {
-            S = rescaled(S, code, top);
-            code = top;
-        }
+            for (int u = 0; u < 8; ++u) {
+                a[u] = k + u < kb ? xb[(k + u) * ld] & 0x7FFFFFFFFFFFFFFFull : 0;
+                any |= a[u];
+                top = max(top, (int)(a[u] >> 52));
+            }
+            if (top > be) {
+                s = rescaled(s, be, top);
+                be = top;
+            }
 #pragma unroll
-        for (int u = 0; u < 8; ++u) S += fx_square(a[u], sh.at(k + u), code);
+            for (int u = 0; u < 8; ++u) s += fx_square(a[u], 0, be + kCodeBias);
+        }
+        const int c = be == 0x7FF ? kCodeInf : (be != 0 ? be + kCodeBias + (half != 0 ? sh.s : 0) : (any != 0 ? 1 : 0));
+        norm_join(code, S, c, s);
     }
     part[(int64_t)blockIdx.y * R + r] = make_float2(__int_as_float(code), S);
-}
-
-// (code, S) pairs combined in the order of their index
-__device__ __forceinline__ void norm_join(int &code, float &S, int code2, float S2) {
-    const int top = max(code, code2);
-    S = rescaled(S, code, top) + rescaled(S2, code2, top);
-    code = top;
 }
 
 // 32 rows x 64 columns per CTA, turned through shared memory so that both the reads
