@@ -640,7 +640,7 @@ def run_c3(args, quiet=False):
             else:
                 roof[name] = {"ms_per_launch": per, "fp64_tflops": tf, "frac_fp64": tf / fp64_peak,
                               "hbm_gbs": rows[name]["bytes"] / (per * 1e-3) / 1e9,
-                              "bound": "alu (wide integer multiplies of the fixed-point gathers; frac: against cuBLAS DGEMM in this run)"}
+                              "bound": "alu (FP64 pipe; frac: against cuBLAS DGEMM in this run)"}
     line = {"metric": "OMM solves/s & time-to-converge, linear-scaling form", "value": 1e3 / t_ms,
             "unit": "solves/s", "n_gpus": 1, "steps": args.steps, "warmup": 1, "ms_per_step": t_ms,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",

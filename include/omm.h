@@ -227,7 +227,9 @@ void omm_default_options(omm_options *opt);
  * nothing and may be 0.  pattern == NULL selects the dense form; otherwise
  * the pattern is validated (OMM_ERR_PATTERN) and copied.  opt == NULL takes
  * the defaults.  All device memory of the handle is allocated here
- * (OMM_ERR_NOMEM on failure).  *out receives the handle on OMM_OK.
+ * (OMM_ERR_NOMEM on failure); the operands of the residue products
+ * (omm_options.fp64_products) are allocated again by a later call where
+ * another handle was given their memory.  *out receives the handle on OMM_OK.
  */
 int omm_create(int64_t m, int64_t n, int32_t block_size, const omm_pattern *pattern,
                const omm_options *opt, omm_handle **out);

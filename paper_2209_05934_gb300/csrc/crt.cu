@@ -30,9 +30,10 @@
 //
 // 19 products at the BF16 rate against one at the FP64 rate (1/1500 of it) is why this is
 // the FP64 form's product: digits of a fixed-point split (tc_exact.cu) would take 55 pairs
-// for it.  A converged FP64 solve takes 4.4 ms at m = 144, 5.8 at m = 512 and 26 at m = 1996,
-// where CUDA-core products took 18, 70 and 763 (16 moduli without the comparison: 4.0, 5.2
-// and 22.6); W's error against 64 bits is the same.
+// for it.  A converged FP64 solve takes 4.4 ms at m = 144, 6.0 at m = 512 and 26.5 at m =
+// 1996, where CUDA-core products took 18, 70 and 763 (16 moduli without the comparison: 10 to
+// 14% less); W's error against 64 bits is the same.  Where every product is recomputed (W0 decaying
+// by a factor of 20 per Angstrom at m = 2016) 17 steps take 144 ms, the CUDA-core form 252.
 //
 // Reconstruction.  With q_i = (P / p_i)^-1 mod p_i folded into one operand's
 // residues, x / P = frac(sum_i y_i / p_i), y_i the residues of the product.  Two

@@ -1,6 +1,7 @@
 // FP64 GEMM on the CUDA cores: omm_op_dgemm (which has no workspace), the FP64
-// refinement of the mixed form, and dense FP64 handles too large for residue planes
-// (crt.cu, 4 to 33 times faster from m = 144 to 1996 and no slower at m = 8).
+// refinement of the mixed form, and dense FP64 solves that run without residue planes
+// (crt.cu, 4 to 29 times faster from m = 144 to 1996 and no slower at m = 8): by choice, or
+// for want of memory.
 //
 // GB300 executes FP64 on its CUDA cores only (no FP64 tensor-core kind in
 // tcgen05), at a small fraction of the BF16 tensor rate, so this kernel is

@@ -15,12 +15,12 @@
 // why it is a pass of its own over planes that mostly stay in L2.  An earlier form
 // combined the levels in tensor memory and had room for 128 columns only: it ran
 // the tensor pipe 36% of its active cycles.  W^T (H W) of 1024 x 1000 x 4096 with 7
-// digits (packing included) went from 621 to 255 us, the 6-digit gradient of a
-// 4096 x 1024 system from 498 to about 250 us, with the same bits.
+// digits (packing included) went from 621 to 187 us, the 6-digit gradient of a
+// 4096 x 1024 system from 494 to 228 us (fold included), with the same bits.
 //
 // One work item is one output tile of one plane.  Planes are independent, so a
-// product of few tiles still fills the chip: 16 residue planes (or 6 to 8 digit
-// levels) of a 512 x 128 product give 64 items.  Items are ordered heaviest plane
+// product of few tiles still fills the chip: 19 planes of residues and magnitudes (or
+// 6 to 8 digit levels) of a 512 x 128 product give 76 items.  Items are ordered heaviest plane
 // first and dealt out in alternating directions, CTAs (or CTA pairs) being
 // persistent; the shared-memory ring and the accumulators run on across items.
 //
