@@ -174,8 +174,9 @@ typedef struct {
                               split_digits digits */
     int32_t fp64_products; /* dense handles in OMM_PREC_FP64: where their products run
                               (OMM_FP64_*).  The residue form takes about 75 bytes per element of
-                              [H; S] beside the arrays; that memory, at most an eighth of the
-                              device's for all handles, is kept between solves and given up, while
+                              [H; S] beside the arrays: at most an eighth of the device's memory
+                              for a handle and, beyond an eighth, half for all handles, while a
+                              quarter stays free.  It is kept between solves and given up, while
                               no call is using it, for other handles and other allocations of
                               this library */
 } omm_options;

@@ -648,13 +648,17 @@ int planes_maps(const omm_handle *h, CrtBufs &c) {
 }
 
 // Planes for an FP64 dense handle, before a call that packs or multiplies with them.  They
-// take about 75 bytes per element of [H' ; S] against 8 for the matrices themselves, so all
-// handles of a device together hold at most an eighth of its memory (one handle: m ~ 16000 at
-// n = m / 4): planes that no call is using give way to others, and to any other allocation
-// of the library (omm::device_malloc).  A handle beyond that, or one whose planes find no
-// memory, runs this solve's products on the CUDA cores (h->product_form).  There is no
-// lower size limit: a step takes 85 us against 92 at m = 8, 91 against 208 at m = 64, 115
-// against 1383 at m = 512.
+// take about 75 bytes per element of [H' ; S] against 8 for the matrices themselves: at most
+// an eighth of the device's memory for one handle (m ~ 16000 at n = m / 4), and for all
+// handles together, beyond an eighth, at most half of it and only while a quarter stays
+// free.  kDriverReserve always stays free of them: the driver allocates for streams, graphs
+// and modules, and its cuStreamCreate was seen to corrupt the heap on a full device.  Planes
+// that no call is using give way to others, and to any other allocation of the
+// library (omm::device_malloc).  A handle whose planes find no room runs this solve's
+// products on the CUDA cores (h->product_form).  There is no lower size limit: a step takes
+// 85 us against 92 at m = 8, 91 against 208 at m = 64, 115 against 1383 at m = 512.
+constexpr int64_t kDriverReserve = 256ll << 20;
+
 int planes_take(omm_handle *h) {
     h->planes_on = false;
     if (h->sparse || h->opt.precision != OMM_PREC_FP64 || h->opt.fp64_products == OMM_FP64_CUDA_CORES) return OMM_OK;
@@ -663,15 +667,17 @@ int planes_take(omm_handle *h) {
     if (h->cr.base == nullptr) {
         CrtBufs c;
         planes_layout(h->m, h->n, h->opt.precon != 0, s_identity(h), c);
-        size_t free_b = 0, total_b = 0;
-        OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
         OMM_CUDA_TRY(cudaGetDevice(&c.device));
-        const int64_t most = (int64_t)(total_b / 8);
-        if (c.bytes > most) return OMM_OK;
         for (;;) {
-            int64_t held = 0;
+            size_t free_b = 0, total_b = 0;
+            OMM_CUDA_TRY(cudaMemGetInfo(&free_b, &total_b));
+            const int64_t eighth = (int64_t)(total_b / 8);
+            if (c.bytes > eighth) return OMM_OK;
+            int64_t held = c.bytes;
             for (const omm_handle *o : l) held += o->cr.device == c.device ? o->cr.bytes : 0;
-            if (held + c.bytes <= most && cudaMalloc((void **)&c.base, (size_t)c.bytes) == cudaSuccess) break;
+            const int64_t stays = held <= eighth ? kDriverReserve : 2 * eighth;
+            const bool room = held <= 4 * eighth && (int64_t)free_b >= c.bytes + stays;
+            if (room && cudaMalloc((void **)&c.base, (size_t)c.bytes) == cudaSuccess) break;
             cudaGetLastError();
             c.base = nullptr;
             if (!planes_make_room_locked(c.device)) return OMM_OK;

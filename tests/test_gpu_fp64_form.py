@@ -68,36 +68,26 @@ def test_cuda_core_products_reach_the_same_solution(omm, atoms, drop, variant):
 def test_without_memory_a_solve_reports_or_refuses(omm):
     _, H, S, W0 = system((4, 4, 4))
     m, n = W0.shape
-    E2, _, _, form = solved(omm, H, S, W0, fp64_products=omm.FP64_CUDA_CORES, graphs=0)   # its kernels loaded
+    E2, _, _, _ = solved(omm, H, S, W0, fp64_products=omm.FP64_CUDA_CORES)
+    w0 = dev(W0)
+    torch.cuda.empty_cache()
+    # room for the arrays, but not for planes beside what the driver is left with (256 MB)
+    fill = torch.empty(max(torch.cuda.mem_get_info()[0] - (200 << 20), 0), dtype=torch.uint8, device="cuda")
     res = omm.Solver(m, n, 8, fp64_products=omm.FP64_RESIDUES)
-    aut = omm.Solver(m, n, 8, graphs=0)
+    aut = omm.Solver(m, n, 8)
     res.set_HS(dev(H), dev(S))
     aut.set_HS(dev(H), dev(S))
-    w0 = dev(W0)
-    fill = lambda left: torch.empty(max(torch.cuda.mem_get_info()[0] - left, 0), dtype=torch.uint8, device="cuda")
-    torch.cuda.empty_cache()
-    keep = [fill(64 << 20)]
-    # idle planes go to the arrays of other handles until nothing is left of them
-    taken = []
-    while True:
-        try:
-            taken.append(omm.Solver(1024, 256, 8, fp64_products=omm.FP64_CUDA_CORES))
-        except omm.OmmError as e:
-            assert e.status == omm.ERR_NOMEM
-            break
-        assert len(taken) < 20
-    keep.append(fill(12 << 20))
     E1, _, _ = aut.solve(w0, tol=1e-12)
     assert aut.product_form() == omm.PRODUCTS_CUDA_CORES
     with pytest.raises(omm.OmmError) as err:
         res.solve(w0, tol=1e-12)
     assert err.value.status == omm.ERR_NOMEM
-    for s in taken:
-        s.close()
-    keep.clear()
+    del fill
     torch.cuda.empty_cache()
     E0, _, _ = res.solve(w0, tol=1e-12)                    # with memory again
     assert res.product_form() == omm.PRODUCTS_RESIDUES
-    assert E1 == E2 and abs(E0 - E1) <= 1e-10 * abs(E0)
+    E3, _, _ = aut.solve(w0, tol=1e-12)                    # the other form, after graphs of the first
+    assert aut.product_form() == omm.PRODUCTS_RESIDUES
+    assert E1 == E2 and E3 == E0 and abs(E0 - E1) <= 1e-10 * abs(E0)
     aut.close()
     res.close()
