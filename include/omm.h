@@ -59,8 +59,8 @@ enum {
 
 /* arithmetic of the solve */
 enum {
-    OMM_PREC_FP64 = 0,   /* every product at least as accurate as an FP64 multiply-add chain,
-                            element by element: dense handles find each from its residues on
+    OMM_PREC_FP64 = 0,   /* every product within the error bound of an FP64 multiply-add
+                            chain, element by element: dense handles find each from its residues on
                             the tensor cores where that holds, else in FP64 (omm_options.
                             fp64_products), sparse handles in FP64 on the CUDA cores */
     OMM_PREC_MIXED = 1   /* BF16-split tensor-core products for the bulk of the
